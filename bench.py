@@ -37,7 +37,7 @@ DEFAULT_WORKLOAD = "random_layered_V16384_D64"   # the largest configuration: sw
 
 FALLBACK_HBM_GBS = 6650.0
 # the kernel each variant runs for graphs that have a compact encoding (all benchmark workloads do)
-KERNEL_OF_VARIANT = {"shared": "pe_eval_lane_kernel<STATE_SMEM=true>", "global": "pe_eval_lane_kernel<STATE_SMEM=false>",
+KERNEL_OF_VARIANT = {"shared": "pe_eval_tile_kernel", "global": "pe_eval_lane_kernel",
                      "warp": "pe_eval_warp2_kernel", "team": "pe_eval_team_kernel"}
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per operator-evaluation of the evaluation kernel
@@ -47,7 +47,7 @@ KERNEL_SOURCES = {
     "team": ("pe_kernel_team.cuh", "pe_team.cu", "pe_team_launch.h", "pe_transpose.cuh"),
     "warp": ("pe_kernel_warp2.cuh", "pe_warp2_launch.h", "pe_device.cuh", "pe_kernel_lane.cuh"),
     "global": ("pe_kernel_lane.cuh", "pe_lane_launch.h", "pe_device.cuh"),
-    "shared": ("pe_kernel_lane.cuh", "pe_lane_launch.h", "pe_device.cuh"),
+    "shared": ("pe_kernel_tile.cuh", "pe_tile_launch.h", "pe_device.cuh"),
 }
 NCU_TRAFFIC = {
     # variant: (hash of its sources at capture time, DRAM bytes per operator-evaluation, captured workload)

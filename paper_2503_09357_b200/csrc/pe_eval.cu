@@ -233,53 +233,10 @@ static inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; 
 
 // exclusive: PE_COMM_EXCLUSIVE - the compact kernel keeps one more word per machine pair and candidate;
 // the generic shared-state kernel does not offer it.
-static bool plan_shared(const pe_graph* g, bool allow_compact, Plan* p, bool exclusive = false) {
+static bool plan_shared(const pe_graph* g, int64_t K, bool allow_compact, Plan* p, bool exclusive = false) {
+  if (allow_compact && plan_tile(g, K, exclusive, p)) return true;
   if (g->time_bound >= kPackedTimeLimit) return false;
   p->compact = false;
-  p->exclusive = exclusive;
-  if (g->narrow_ok && allow_compact) {  // compact graph staged in shared memory next to the state
-    const size_t fixed = (size_t)g->nview.bytes + 16;
-    // 16-bit state words when the machine id and every possible end time fit together (the all-ones time
-    // field marks "not scheduled"): half the state, so twice the candidates per SM where the state is what
-    // limits them.  Blocks are multiples of 64 threads there (two warps share the words of a row).
-    int jb = 1;
-    while ((1 << jb) < g->D) ++jb;
-    if (!exclusive && jb < 16 && g->time_bound < ((int64_t)1 << (16 - jb)) - 1) {
-      const size_t per16 = (size_t)2 * (g->V + 1) + (size_t)(g->has_weight ? 20 : 16) * g->D;
-      if (fixed + 64 * per16 <= g->smem_optin) {
-        size_t T = (g->smem_optin - fixed) / per16 / 64 * 64;
-        if (T > 256) T = 256;
-        p->variant = PE_VARIANT_SHARED;
-        p->threads = (int)T;
-        p->smem = fixed + T * per16;
-        p->graph_smem = true;
-        p->workspace = 0;
-        p->ws_x_off = 0;
-        p->compact = true;
-        p->state16 = true;
-        p->jbits = jb;
-        return true;
-      }
-    }
-    const size_t per = (size_t)4 * (g->V + 1) + (size_t)(g->has_weight ? 20 : 16) * g->D +
-                       (exclusive ? (size_t)4 * g->D * g->D : 0);
-    if (fixed + 32 * per <= g->smem_optin) {
-      // A block size that is a multiple of 32 keeps every lane's state column in its own bank.  That is
-      // given up only where rounding down would idle more than a sixth of the candidates that fit:
-      // with one or two warps per SM the kernel is bound by latency, not by bank conflicts.
-      size_t T = (g->smem_optin - fixed) / per;
-      if (T > 256) T = 256;
-      if (T / 32 * 32 * 6 >= T * 5) T = T / 32 * 32;
-      p->variant = PE_VARIANT_SHARED;
-      p->threads = (int)T;
-      p->smem = fixed + T * per;
-      p->graph_smem = true;
-      p->workspace = 0;
-      p->ws_x_off = 0;
-      p->compact = true;
-      return true;
-    }
-  }
   if (exclusive) return false;
   const size_t per_thread = (size_t)4 * g->V + (size_t)(g->has_weight ? 20 : 16) * g->D;
   const size_t budget = g->smem_optin;
@@ -432,6 +389,15 @@ static bool plan_global(const pe_graph* g, int64_t K, uint32_t flags, bool allow
   return true;
 }
 
+// Does a lane per candidate pay?  The tile kernel needs enough candidates per SM to make up for the latency of a
+// step (measured: 28 at V = 1536 / D = 32 take 2.6 ms against 3.3 ms of a warp per candidate; 20 of the MoE graph,
+// whose wide operators re-read the edge list, 6.2 ms against 2.1 ms of a block of warps per candidate; with exclusive
+// channels 20 at V = 1536 take 2.1 ms against 2.8 ms of the global-state kernel).
+static bool shared_pays(const pe_graph* g, const Plan& p) {
+  if (!p.tiled) return p.threads >= 48;
+  return p.tile_resident >= (p.exclusive ? 16 : (g->max_indeg > 3 ? 48 : 28));
+}
+
 // allow_compact: the call can use the compact-graph kernels (u16 orders; start and finish both
 // wanted or both absent).  Size queries pass true and false and take the larger workspace.
 static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_compact, Plan* p) {
@@ -441,8 +407,8 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
   const uint32_t want = flags & PE_VARIANT_MASK;
   if (g->hetero) {   // machine-dependent durations: the generic one-thread-per-candidate kernels
     if (want == PE_VARIANT_WARP || want == PE_VARIANT_TEAM) return PE_ERR_UNSUPPORTED;
-    if (!(flags & PE_COMM_EXCLUSIVE) && want != PE_VARIANT_GLOBAL && plan_shared(g, false, p) &&
-        (p->threads >= 48 || want == PE_VARIANT_SHARED))
+    if (!(flags & PE_COMM_EXCLUSIVE) && want != PE_VARIANT_GLOBAL && plan_shared(g, K, allow_compact, p) &&
+        (shared_pays(g, *p) || want == PE_VARIANT_SHARED))
       return PE_OK;
     if (want == PE_VARIANT_SHARED) return PE_ERR_UNSUPPORTED;
     return plan_global(g, K, flags, false, p) ? PE_OK : PE_ERR_UNSUPPORTED;
@@ -451,7 +417,7 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
     // exclusive channels: the compact shared-state kernel where a block of candidates still fits with one
     // more word per machine pair each, else the generic global-state kernel
     if (want == PE_VARIANT_AUTO || want == PE_VARIANT_SHARED) {
-      if (plan_shared(g, allow_compact, p, true) && (p->threads >= 48 || want == PE_VARIANT_SHARED)) return PE_OK;
+      if (plan_shared(g, K, allow_compact, p, true) && (shared_pays(g, *p) || want == PE_VARIANT_SHARED)) return PE_OK;
       if (want == PE_VARIANT_SHARED) return PE_ERR_UNSUPPORTED;
       *p = Plan();
     }
@@ -460,13 +426,11 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
   }
   switch (want) {
     case PE_VARIANT_AUTO: {
-      // Thread-per-candidate with everything on chip wins whenever about a warp and a half of
-      // candidates fit in shared memory (measured: 55 candidates per SM at V = 1024 beat the
-      // warp-per-candidate kernel by 1.35x, 44 did not).  Beyond that the state of a candidate is too
-      // large: a warp per candidate (state still on chip) wins while at least four warps fit on an SM;
-      // for the largest graphs the global-state kernel, which is bound by random DRAM accesses but
-      // keeps thousands of candidates in flight, is faster.
-      if (plan_shared(g, allow_compact, p) && p->threads >= 48) return PE_OK;
+      // A lane per candidate with everything on chip wins while enough candidates fit in shared memory.  Beyond
+      // that the state of a candidate is too large: a warp per candidate (state still on chip) wins while at
+      // least four warps fit on an SM; for the largest graphs the global-state kernel, which is bound by random
+      // DRAM accesses but keeps thousands of candidates in flight, is faster.
+      if (plan_shared(g, K, allow_compact, p) && shared_pays(g, *p)) return PE_OK;
       Plan w, gl, tm;
       const bool has_w = plan_warp(g, K, flags, allow_compact, &w);
       const bool has_g = plan_global(g, K, flags, allow_compact, &gl);
@@ -486,13 +450,13 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
       const bool warp_wins = w.threads >= 4 * 32 || (w.threads >= 3 * 32 && has_g && gl.smem == 0);
       if (has_w && (warp_wins || !has_g || !gl.compact)) { *p = w; return PE_OK; }
       if (has_g && gl.compact) { *p = gl; return PE_OK; }
-      if (plan_shared(g, allow_compact, p)) return PE_OK;
+      if (plan_shared(g, K, allow_compact, p)) return PE_OK;
       if (has_w) { *p = w; return PE_OK; }
       if (has_g) { *p = gl; return PE_OK; }
       return PE_ERR_UNSUPPORTED;
     }
     case PE_VARIANT_GLOBAL: return plan_global(g, K, flags, allow_compact, p) ? PE_OK : PE_ERR_UNSUPPORTED;
-    case PE_VARIANT_SHARED: return plan_shared(g, allow_compact, p) ? PE_OK : PE_ERR_UNSUPPORTED;
+    case PE_VARIANT_SHARED: return plan_shared(g, K, allow_compact, p) ? PE_OK : PE_ERR_UNSUPPORTED;
     case PE_VARIANT_WARP: return plan_warp(g, K, flags, allow_compact, p) ? PE_OK : PE_ERR_UNSUPPORTED;
     case PE_VARIANT_TEAM: return plan_team(g, K, allow_compact, p) ? PE_OK : PE_ERR_UNSUPPORTED;
     default: return PE_ERR_UNSUPPORTED;
@@ -510,6 +474,12 @@ static int launch_typed(const pe_graph* g, const Plan& p, int64_t K, const uint8
   if (p.compact) {
     if (sizeof(OrderT) != 2) return PE_ERR_INVALID_ARG;
     const uint16_t* ord16 = static_cast<const uint16_t*>(order);
+    if (p.tiled) {
+      const int rc = launch_tile(g, p, BY_POS, K, assign, ord16, flags, out, stream);
+      if (rc != PE_OK) return rc;
+      g_launches.fetch_add(1, std::memory_order_relaxed);
+      return cudaGetLastError() == cudaSuccess ? PE_OK : PE_ERR_CUDA;
+    }
     uint32_t* gstate = static_cast<uint32_t*>(workspace);
     if (p.variant == PE_VARIANT_TEAM) {
       if (p.staged && (((uintptr_t)assign | (uintptr_t)order) & 3u)) return PE_ERR_INVALID_ARG;   // word-wise transpositions

@@ -203,6 +203,79 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
     std::memcpy(nblob.data() + nv.cap, cap, (size_t)D * 4);
   }
 
+  // tile encoding
+  bool tile = V <= 65535 && L <= 2 && mdeg <= 255;
+  for (int32_t i = 0; tile && i < V; ++i)
+    tile = ops[i].dur <= 65535 && ops[i].mem_delta >= -128 && ops[i].mem_delta <= 127;
+  for (int64_t q = 0; tile && q < (int64_t)E * L; ++q) tile = comm[q] <= 65535;
+  if (g->hetero)
+    for (int64_t q = 0; tile && q < (int64_t)V * D; ++q) tile = d->dur_by_machine[q] <= 65535;
+  std::vector<uint8_t> tblob;
+  g->tile_ok = tile;
+  g->d_tblob = nullptr;
+  std::memset(&g->tview, 0, sizeof(g->tview));
+  if (tile) {
+    PeTileView& tv = g->tview;
+    tv.V = V; tv.D = D;
+    tv.has_weight = g->has_weight ? 1 : 0;
+    tv.max_indeg = mdeg;
+    bool cut = false;   // some pair of different machines has no channel
+    if (d->link_class)
+      for (int32_t a = 0; a < D * D; ++a) cut = cut || (d->link_class[a] == 0xFF && a / D != a % D);
+    tv.cls_kind = !cut && L == 1 ? 0 : (!cut && D <= 32 ? 2 : 1);
+    const bool listed = tv.cls_kind == 0 ? mdeg > 3 : mdeg > 2;
+    tv.list_edges = listed ? E : 0;
+    uint64_t tat = 0;
+    tv.ops = (uint32_t)tat;     tat = align16(tat + (uint64_t)(V + 1) * 16);
+    tv.edges = (uint32_t)tat;   tat = align16(tat + (listed ? (uint64_t)E * (tv.cls_kind == 0 ? 4 : 8) : 0));
+    tv.slot = (uint32_t)tat;    tat = align16(tat + (listed && tv.cls_kind != 0 ? (uint64_t)V * 4 : 0));
+    tv.cls = (uint32_t)tat;     tat = align16(tat + (tv.cls_kind == 1 ? (uint64_t)D * D : 0));
+    tv.cls_row = (uint32_t)tat; tat = align16(tat + (tv.cls_kind == 2 ? (uint64_t)D * 4 : 0));
+    tv.weight = (uint32_t)tat;  tat = align16(tat + (g->has_weight ? (uint64_t)V * 4 : 0));
+    tv.cap = (uint32_t)tat;     tat = align16(tat + (uint64_t)D * 4);
+    tv.durm = (uint32_t)tat;    tat = align16(tat + (g->hetero ? (uint64_t)(V + 1) * D * 2 : 0));
+    tv.bytes = (uint32_t)tat;
+    tblob.assign(tv.bytes, 0);
+    uint32_t* r = (uint32_t*)(tblob.data() + tv.ops);
+    const uint32_t none = (uint32_t)V;
+    auto delays = [&](int32_t q) {   // both classes of CSR edge q
+      const uint32_t c0 = (uint32_t)comm[(size_t)q * L];
+      return c0 | (L == 2 ? (uint32_t)comm[(size_t)q * L + 1] : c0) << 16;
+    };
+    for (int32_t i = 0; i <= V; ++i, r += 4) {
+      const int32_t b = i < V ? ops[i].edge_begin : 0, n = i < V ? ops[i].indeg : 0;
+      r[0] = i < V ? (uint32_t)(uint8_t)(int8_t)ops[i].mem_delta << 24 | (uint32_t)n << 16 | (uint32_t)(g->hetero ? 0 : ops[i].dur) : 0u;
+      if (tv.cls_kind == 0) {
+        auto edge = [&](int32_t q) { return (uint32_t)comm[q] << 16 | (uint32_t)pred[q]; };
+        r[1] = n > 0 ? edge(b) : none;
+        r[2] = n > 1 ? edge(b + 1) : none;
+        r[3] = n > 3 ? (uint32_t)b : (n > 2 ? edge(b + 2) : none);
+      } else {
+        r[1] = (n > 0 ? (uint32_t)pred[b] : none) | (n > 1 ? (uint32_t)pred[b + 1] : none) << 16;
+        r[2] = n > 0 ? delays(b) : 0u;
+        r[3] = n > 1 ? delays(b + 1) : 0u;
+      }
+    }
+    if (listed) {
+      uint32_t* te = (uint32_t*)(tblob.data() + tv.edges);
+      for (int32_t q = 0; q < E; ++q) {
+        if (tv.cls_kind == 0) te[q] = (uint32_t)comm[q] << 16 | (uint32_t)pred[q];
+        else { te[2 * (size_t)q] = (uint32_t)pred[q]; te[2 * (size_t)q + 1] = delays(q); }
+      }
+      if (tv.cls_kind != 0)
+        for (int32_t i = 0; i < V; ++i) ((uint32_t*)(tblob.data() + tv.slot))[i] = (uint32_t)ops[i].edge_begin;
+    }
+    if (tv.cls_kind == 1 && d->link_class) std::memcpy(tblob.data() + tv.cls, d->link_class, (size_t)D * D);
+    if (tv.cls_kind == 2 && d->link_class)
+      for (int32_t j = 0; j < D; ++j)
+        for (int32_t x = 0; x < D; ++x)
+          if (x != j && d->link_class[(size_t)x * D + j] == 1) ((uint32_t*)(tblob.data() + tv.cls_row))[j] |= 1u << x;
+    if (g->has_weight) std::memcpy(tblob.data() + tv.weight, d->mem_weight, (size_t)V * 4);
+    std::memcpy(tblob.data() + tv.cap, cap, (size_t)D * 4);
+    if (g->hetero)
+      for (int64_t q = 0; q < (int64_t)V * D; ++q) ((uint16_t*)(tblob.data() + tv.durm))[q] = (uint16_t)d->dur_by_machine[q];
+  }
+
   // forward view (successor lists) for priority-list decoding
   std::vector<uint8_t> fblob;
   g->fwd_ok = V <= 65536 && mdeg <= 255;
@@ -226,24 +299,34 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
     for (int32_t b = 0; b < E; ++b) fsucc[ffill[d->edge_src[b]]++] = (uint16_t)d->edge_dst[b];
   }
 
-  cudaDeviceProp prop;
-  int prev = -1;
+  // one allocation and one copy for all encodings (each on a 256-byte boundary), the status word last
+  std::vector<uint8_t> all;
+  auto place = [&](const std::vector<uint8_t>& part) {
+    const size_t at = (all.size() + 255) / 256 * 256;
+    all.resize(at);
+    all.insert(all.end(), part.begin(), part.end());
+    return at;
+  };
+  const size_t at_blob = place(blob), at_n = place(nblob), at_t = place(tblob), at_f = place(fblob);
+  const size_t at_err = place(std::vector<uint8_t>(256, 0));
+  int prev = -1, sms = 0, optin = 0, per_sm = 0;
   bool ok = cudaGetDevice(&prev) == cudaSuccess && cudaSetDevice(cuda_device) == cudaSuccess &&
-            cudaGetDeviceProperties(&prop, cuda_device) == cudaSuccess;
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cuda_device) == cudaSuccess &&
+            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, cuda_device) == cudaSuccess &&
+            cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, cuda_device) == cudaSuccess;
   if (ok) {
-    g->sm_count = prop.multiProcessorCount;
-    g->smem_optin = prop.sharedMemPerBlockOptin;
-    g->smem_per_sm = prop.sharedMemPerMultiprocessor;
-    ok = cudaMalloc((void**)&g->d_blob, lay.bytes) == cudaSuccess &&
-         cudaMalloc((void**)&g->d_error, 256) == cudaSuccess &&
-         cudaMemcpy(g->d_blob, blob.data(), lay.bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
-         cudaMemset(g->d_error, 0, 256) == cudaSuccess;
-    if (ok && narrow)
-      ok = cudaMalloc((void**)&g->d_nblob, nblob.size()) == cudaSuccess &&
-           cudaMemcpy(g->d_nblob, nblob.data(), nblob.size(), cudaMemcpyHostToDevice) == cudaSuccess;
-    if (ok && g->fwd_ok)
-      ok = cudaMalloc((void**)&g->d_fwd, fblob.size()) == cudaSuccess &&
-           cudaMemcpy(g->d_fwd, fblob.data(), fblob.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+    g->sm_count = sms;
+    g->smem_optin = (size_t)optin;
+    g->smem_per_sm = (size_t)per_sm;
+    ok = cudaMalloc((void**)&g->d_blob, all.size()) == cudaSuccess &&
+         cudaMemcpy(g->d_blob, all.data(), all.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+    if (ok) {
+      uint8_t* base = g->d_blob + at_blob;   // (= d_blob: the generic blob comes first)
+      g->d_nblob = narrow ? base + at_n : nullptr;
+      g->d_tblob = tile ? base + at_t : nullptr;
+      g->d_fwd = g->fwd_ok ? base + at_f : nullptr;
+      g->d_error = reinterpret_cast<int*>(base + at_err);
+    }
     if (ok) {
       ok = cudaStreamCreateWithFlags(&g->copy_in, cudaStreamNonBlocking) == cudaSuccess &&
            cudaStreamCreateWithFlags(&g->copy_out, cudaStreamNonBlocking) == cudaSuccess &&
@@ -263,9 +346,6 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
   if (!ok) {
     cudaGetLastError();
     if (g->d_blob) cudaFree(g->d_blob);
-    if (g->d_error) cudaFree(g->d_error);
-    if (g->d_nblob) cudaFree(g->d_nblob);
-    if (g->d_fwd) cudaFree(g->d_fwd);
     if (g->copy_in) cudaStreamDestroy(g->copy_in);
     if (g->copy_out) cudaStreamDestroy(g->copy_out);
     if (g->ev_begin) cudaEventDestroy(g->ev_begin);
@@ -299,9 +379,7 @@ extern "C" int pe_destroy(pe_graph* g) {
   for (int q = 0; q < 2; ++q) { cudaStreamDestroy(g->team_stream[q]); cudaEventDestroy(g->team_join[q]); }
   cudaEventDestroy(g->team_fork);
   for (int q = 0; q < pe_graph::kMaxChunks; ++q) { cudaEventDestroy(g->ev_in[q]); cudaEventDestroy(g->ev_done[q]); }
-  bool ok = cudaFree(g->d_blob) == cudaSuccess && cudaFree(g->d_error) == cudaSuccess;
-  if (g->d_nblob) ok = cudaFree(g->d_nblob) == cudaSuccess && ok;
-  if (g->d_fwd) ok = cudaFree(g->d_fwd) == cudaSuccess && ok;
+  const bool ok = cudaFree(g->d_blob) == cudaSuccess;
   if (prev >= 0) cudaSetDevice(prev);
   delete g;
   return ok ? PE_OK : PE_ERR_CUDA;

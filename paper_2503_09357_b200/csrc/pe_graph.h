@@ -63,6 +63,33 @@ struct PeNarrowView {
   uint32_t bytes;     // total, multiple of 16
 };
 
+// Tile encoding, the one that pe_eval_tile_kernel stages into shared memory (V <= 65535, durations and
+// delays below 65536, A in int8, L <= 2, in-degree <= 255; durations by machine allowed).  One 16-byte
+// record per operator plus a record for the sentinel operator V:
+//   x = (uint8)A << 24 | indeg << 16 | dur
+//   one class, every pair connected (cls_kind 0):  y, z, w = incoming edges 0, 1, 2 as delay << 16 | pred;
+//     w = slot of the first incoming edge in the edge list when indeg > 3 (edges 2.. are read from there)
+//   otherwise:  y = pred 0 | pred 1 << 16,  z, w = delay of edge 0, 1:  class 0 | class 1 << 16;
+//     edges 2.. are in the edge list, the first incoming edge of operator i at slot[i]
+// Missing edges name the sentinel with zero delay.  The edge list (delay << 16 | pred, or
+// {pred, class 0 | class 1 << 16}) is present only if some operator has more edges than a record holds.
+struct PeTileView {
+  int32_t V, D;
+  int32_t has_weight;
+  int32_t cls_kind;    // 0: one class, all connected; 1: class table; 2: two classes, all connected, D <= 32: row bits
+  int32_t max_indeg;
+  int32_t list_edges;  // edges in the list (0 or E)
+  uint32_t ops;        // uint4[V + 1]
+  uint32_t edges;      // uint32[E] or uint2[E]
+  uint32_t slot;       // uint32[V] (class kinds 1 and 2 with an edge list)
+  uint32_t cls;        // uint8[D*D] (kind 1)
+  uint32_t cls_row;    // uint32[D] (kind 2): bit x of row j = class of the channel x -> j
+  uint32_t weight;     // int32[V] if has_weight
+  uint32_t cap;        // int32[D]
+  uint32_t durm;       // uint16[V*D] duration of operator i on machine j at i*D + j (heterogeneous machines; row V = 0 follows)
+  uint32_t bytes;      // total, multiple of 16
+};
+
 // Forward view of the DAG for priority-list decoding, built when V <= 65536 and no operator has
 // more than 255 incoming edges: successors of operator i are succ[ptr[i] .. ptr[i+1]).
 struct PeFwdView {
@@ -82,10 +109,13 @@ struct pe_graph {
   int64_t mem_bound;   // sum |A| + sum W
   int32_t max_indeg;
   PeBlobLayout lay;
-  uint8_t* d_blob;     // device copy of the blob
+  uint8_t* d_blob;     // device copy of the blob; one allocation that also holds the encodings below and d_error
   bool narrow_ok;      // the compact encoding exists
   PeNarrowView nview;
   uint8_t* d_nblob;    // device copy of the compact encoding (nullptr if !narrow_ok)
+  bool tile_ok;        // the tile encoding exists
+  PeTileView tview;
+  uint8_t* d_tblob;    // device copy of the tile encoding (nullptr if !tile_ok)
   bool fwd_ok;         // the forward view exists
   PeFwdView fview;
   uint8_t* d_fwd;      // device copy of the forward view (nullptr if !fwd_ok)

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "pe_graph.h"
+#include "pe_tile_shape.h"
 
 namespace pe {
 
@@ -20,9 +21,13 @@ struct Plan {
   int warp_words = 0;     // WARP: 32-bit words of shared memory per candidate
   bool compact = false;   // SHARED / GLOBAL / WARP: the compact-graph kernels
   bool exclusive = false; // SHARED (compact): PE_COMM_EXCLUSIVE, one more word per machine pair and candidate
-  bool state16 = false;   // SHARED (compact): 16-bit state words, end << jbits | machine
-  int jbits = 8;          // bits of the machine field of a state word
   bool slab = false;      // WARP (compact): order entries and times go through shared tiles, a slab at a time
+  // SHARED over the tile encoding (pe_eval_tile_kernel)
+  bool tiled = false;
+  int tile_mode = 0;
+  int tile_resident = 0;    // candidates an SM holds at once
+  int64_t grid = 0;
+  TileShape tile = {};
   // TEAM: inputs and times go through candidate-major staging copies in the workspace, a chunk of candidates at a time
   bool staged = false;
   int64_t team_chunk = 0;   // candidates per chunk (multiple of 4)
@@ -42,7 +47,12 @@ static bool set_smem(Kern kern, size_t bytes) {
   return raise_smem_limit(reinterpret_cast<const void*>(kern), bytes);
 }
 
-// pe_eval_lane_kernel: state in shared memory (plan variant SHARED) or in `gstate` (GLOBAL).
+// pe_eval_tile_kernel (plan variant SHARED over the tile encoding).
+bool plan_tile(const pe_graph* g, int64_t K, bool exclusive, Plan* p);
+int launch_tile(const pe_graph* g, const Plan& p, bool by_pos, int64_t K, const uint8_t* assign, const uint16_t* order,
+                uint32_t flags, const pe_outputs& out, cudaStream_t stream);
+
+// pe_eval_lane_kernel (plan variant GLOBAL over the compact encoding; state in `gstate`).
 int launch_lane(const pe_graph* g, const Plan& p, bool by_pos, int64_t K, const uint8_t* assign, const uint16_t* order,
                 uint32_t flags, const pe_outputs& out, uint32_t* gstate, unsigned grid, cudaStream_t stream);
 

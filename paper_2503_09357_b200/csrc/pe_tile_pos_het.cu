@@ -1,0 +1,8 @@
+// pe_eval_tile_kernel: instantiations of one assignment layout and mode.
+#include "pe_tile_launch.h"
+
+namespace pe {
+
+int launch_tile_pos_het(const TileCall& t) { return launch_tile_mode<true, kTileHet>(t); }
+
+}  // namespace pe

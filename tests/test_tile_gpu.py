@@ -1,0 +1,55 @@
+"""The lane-per-candidate kernel at the edges of its tiles: batches around a tile of 32 (or fewer) candidates and one
+that no four-candidate load divides, orders whose length leaves every kind of remainder of the request blocks, 16- and
+32-bit state words, tiles narrower than a warp, each form of the link-class encoding, candidates that are invalid in
+one lane only.  Integers: bit-exact against the oracle."""
+import numpy as np
+import pytest
+
+from paper_2503_09357_b200 import workloads as wl
+from tests import checkers as ck
+from tests import gpu_util as gu
+
+pytestmark = pytest.mark.gpu
+
+
+def chain_graph(V, D, indeg, classes, scale, seed=0):
+    rs = np.random.RandomState(seed + V)
+    edges = [(int(p), i) for i in range(1, V) for p in rs.choice(i, size=min(i, indeg), replace=False)]
+    cls = None if classes == 1 else rs.randint(0, 2, (D, D)).astype(np.uint8)
+    if classes == 3:
+        cls[0, D - 1] = 0xFF
+    L = 1 if classes == 1 else 2
+    w = ck.problem(V, edges, rs.randint(0, scale, V), D, comm=rs.randint(0, scale, (len(edges), L)) if edges else None,
+                   L=L, link_class=cls, A=rs.randint(-4, 5, V), W=rs.randint(0, 3, V) if V % 2 else None,
+                   cap=rs.randint(5, 60, D))
+    w.assign_mode, w.group = "per_op", None
+    return w
+
+
+@pytest.mark.parametrize("V,D,indeg,classes,scale,K", [
+    (15, 3, 2, 1, 4, 31), (16, 3, 2, 1, 4, 33), (17, 4, 3, 1, 4, 64), (47, 8, 3, 1, 200, 128), (48, 8, 2, 2, 200, 129),
+    (49, 40, 3, 2, 30, 96), (63, 32, 5, 2, 30, 97), (65, 5, 6, 1, 300, 1), (80, 6, 3, 3, 30, 4740), (1500, 8, 3, 1, 40, 300),
+    (1600, 8, 2, 2, 40, 299)])
+def test_tile_edges_match_the_oracle(V, D, indeg, classes, scale, K):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2503_09357_b200 import binding as pe
+    w = chain_graph(V, D, indeg, classes, scale)
+    assign, order = wl.make_candidates(w, K=K)
+    if K > 40:                                          # one lane each: an operator twice in a row, a predecessor late,
+        order[5, 3] = order[4, 3]                       # no operator, a machine that does not exist
+        order[:, 6] = order[::-1, 6].copy()
+        order[7, 9] = 65535
+        assign[int(order[V // 2, 11]), 11] = 255
+    g = pe.Graph(w)
+    try:
+        for flags in (0, pe.PE_ASSIGN_BY_POS | pe.PE_TIMES_BY_OP, pe.PE_COMM_EXCLUSIVE):
+            a = assign
+            if flags & pe.PE_ASSIGN_BY_POS:
+                a = np.take_along_axis(assign, np.minimum(order, V - 1).astype(np.int64), axis=0)
+            if pe.pe_eval_variant(g.handle, K, flags | pe.PE_VARIANT_SHARED) < 0:
+                continue
+            gu.check(g, w, a, order, flags=flags | pe.PE_VARIANT_SHARED, label=f"flags {flags}")
+    finally:
+        g.close()
