@@ -7,20 +7,32 @@
 // one of smallest rank comes next (Kahn's algorithm with the ranks as priorities).  The result is
 // a topological order of G_m, i.e. a valid `order` argument of pe_eval_batch.
 //
-// One thread per candidate.  Because the priorities are the ranks 0..V-1, the set of available
-// operators is a bitmap over ranks with two summary levels above it (one bit per 32-bit word of
-// the level below; the top level is a 64-bit register, which is why V <= 65536): "take the
-// smallest" is three find-first-set steps, "add" is three bit sets - no heap, no comparisons of
-// keys.  Per candidate:
-//   word[i]   rank of operator i (bits 0..15) | predecessors still missing (bits 16..23) |
-//             seen in the list (bit 31)
-//   L0, L1    the bitmap over ranks and its first summary level
-//   list      (shared-state variant only) the list itself, two 16-bit entries per word; the
-//             global-state variant reads list[r] back from the input when rank r is taken
-// The shared-state variant keeps these as [row][thread] in shared memory (a lane's accesses stay in
-// its own bank) next to the graph's successor lists, staged by bulk copy; the global-state
-// variant keeps them in the caller's workspace in tiles of 32 candidates, [tile][row][32], and
-// reads the successor lists through the cache.
+// The set of available operators is kept by rank.  Two kernels:
+//
+// Warp per candidate (pe_decode_warp_kernel; per-operator state on chip).  Placing an operator is a chain of
+// dependent steps (smallest rank -> operator -> successors -> their counts -> new ranks), so the work is spread
+// over the lanes only where that shortens the chain:
+//   word[i]   shared memory: rank of operator i (bits 0..15) | predecessors still missing (bits 16..31)
+//   bitmap    shared memory: available operators of rank >= T
+//   pool      registers: every available operator of rank < T, one per lane as rank << 16 | operator
+// The smallest available rank is then one warp-wide minimum over the pool; an operator's successors are handled by
+// the lanes whose pool place is free, so a released operator of rank < T stays where it was found, one of rank >= T
+// sets its bit.  When the pool is empty the next bitmap words that together hold up to kFill operators are loaded into
+// it and T moves behind those words; all words below T stay empty, so the scan over the bitmap is monotone.  If more
+// operators are released than the pool has places, the pool goes back to the bitmap (T = 0) and fills again.
+// What bounds it: instruction issue (52 warp instructions a placement, 85 % of the issue slots used at V = 480) while
+// many warps fit, the chain (~270 cycles a placement with the records on chip) when few do.  Measured (before: a
+// thread per candidate, state in shared memory up to V ~ 1100, else in the workspace): V = 480, K = 65536 2.21 -> 1.65
+// ms, K = 1024 318 -> 78 us; V = 1536, K = 8192 3.14 -> 0.83 ms; V = 2816, K = 8192 9.97 -> 2.8 ms; V = 4096, K = 8192
+// 27.5 -> 5.9 ms; V = 16384, K = 2048 125 -> 23.5 ms.  Candidate-major copies of list and order, and records brought
+// to the pool's places by asynchronous copies, were measured and changed nothing or cost up to 15 %.
+//
+// Thread per candidate (pe_decode_kernel; for graphs whose per-candidate state does not fit on chip, V above
+// ~55000, or on request).  The bitmap has two summary levels above it (one bit per 32-bit word of the level below;
+// the top level is a 64-bit register, which is why V <= 65536): "take the smallest" is three find-first-set steps.
+// Words and bitmaps are in the caller's workspace in tiles of 32 candidates, [tile][row][32]; the list is read back
+// from the input when a rank is taken, the successor lists through the cache.
+#include <algorithm>
 #include <atomic>
 #include <climits>
 
@@ -48,38 +60,27 @@ __device__ __forceinline__ FwdPtrs fwd_ptrs(const uint8_t* base, const PeFwdView
 }
 
 constexpr uint32_t kSeen = 0x80000000u;
+constexpr uint32_t kFill = 16;              // operators that an empty pool is filled with: as many places stay free
+constexpr size_t kDecodeRecBytes = 32768;   // operator records up to this size are kept in shared memory
 constexpr int kListAhead = 8;  // rows of the list requested ahead of the one being placed
 
-template <bool STATE_SMEM>
 __global__ void __launch_bounds__(256) pe_decode_kernel(PeFwdView f, const uint8_t* __restrict__ fblob, int64_t K,
                                                         const uint16_t* __restrict__ list, uint16_t* __restrict__ order,
-                                                        uint32_t* __restrict__ status, uint32_t* __restrict__ gstate,
-                                                        int* err) {
-  extern __shared__ __align__(16) uint8_t smem_raw[];
+                                                        uint32_t* __restrict__ status, uint32_t* __restrict__ gstate) {
   const int T = blockDim.x;
   const int t = threadIdx.x;
   const int V = f.V;
-  const uint8_t* fbase = fblob;
-  uint8_t* sm = smem_raw;
-  if (STATE_SMEM) {
-    uint64_t* bar = reinterpret_cast<uint64_t*>(sm + f.bytes);
-    if (!stage_blob(sm, fblob, f.bytes, bar, err)) return;
-    fbase = sm;
-    sm += f.bytes + 16;
-  }
-  const FwdPtrs fp = fwd_ptrs(fbase, f);
+  const FwdPtrs fp = fwd_ptrs(fblob, f);
   const int64_t c = (int64_t)blockIdx.x * T + t;
   if (c >= K) return;
   const size_t Ks = (size_t)K;
   const int n0 = (V + 31) >> 5, n1 = (n0 + 31) >> 5;
   // row r of this candidate's state is st[r * pitch]
-  uint32_t* st = STATE_SMEM ? reinterpret_cast<uint32_t*>(sm) + t
-                            : gstate + (size_t)(c >> 5) * (size_t)(V + n0 + n1) * 32 + (c & 31);
-  const uint32_t pitch = STATE_SMEM ? (uint32_t)T : 32u;
+  uint32_t* st = gstate + (size_t)(c >> 5) * (size_t)(V + n0 + n1) * 32 + (c & 31);
+  constexpr uint32_t pitch = 32u;
   uint32_t* word = st;
   uint32_t* L0 = st + (size_t)V * pitch;
   uint32_t* L1 = L0 + (size_t)n0 * pitch;
-  uint32_t* lst = L1 + (size_t)n1 * pitch;   // shared-state variant only: [ceil(V / 2)] pairs of entries
   uint64_t L2 = 0;
 
   auto add = [&](uint32_t r) {   // rank r becomes available
@@ -114,7 +115,6 @@ __global__ void __launch_bounds__(256) pe_decode_kernel(PeFwdView f, const uint8
         const int r = r0 + u;
         if (r < V) {
           const uint32_t i = cur[u];
-          if (STATE_SMEM) reinterpret_cast<uint16_t*>(lst + (uint32_t)(r >> 1) * pitch)[r & 1] = (uint16_t)i;
           if (i >= (uint32_t)V) {
             bad = true;
           } else {
@@ -167,8 +167,7 @@ __global__ void __launch_bounds__(256) pe_decode_kernel(PeFwdView f, const uint8
         L1[b2 * pitch] = w1;
         if (w1 == 0u) L2 &= ~(1ull << b2);
       }
-      const uint32_t i = STATE_SMEM ? (uint32_t) reinterpret_cast<const uint16_t*>(lst + (r >> 1) * pitch)[r & 1u]
-                                    : (uint32_t)list_col[(size_t)r * Ks];
+      const uint32_t i = (uint32_t)list_col[(size_t)r * Ks];
       order_col[(size_t)k * Ks] = (uint16_t)i;
       ++k;
       e = fp.ptr[i];
@@ -177,32 +176,208 @@ __global__ void __launch_bounds__(256) pe_decode_kernel(PeFwdView f, const uint8
   }
 }
 
+constexpr uint32_t kNoKey = 0xFFFFFFFFu;   // an empty pool place (V <= 65535: no key equals it)
+
+// REC_SMEM: the operator records are copied to shared memory in front of the warps' words.
+template <bool REC_SMEM>
+__global__ void __launch_bounds__(256) pe_decode_warp_kernel(PeFwdView f, const uint8_t* __restrict__ fblob, int64_t K,
+                                                             const uint16_t* __restrict__ list, uint16_t* __restrict__ order,
+                                                             uint32_t* __restrict__ status, uint32_t words) {
+  extern __shared__ __align__(16) uint32_t smem_words[];
+  constexpr uint32_t FULL = 0xFFFFFFFFu;
+  constexpr uint32_t kOne = 1u << 16;   // one missing predecessor
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+  const int V = f.V;
+  const uint32_t rb = f.rec_bytes, inl2 = f.rec_bytes - 4u;   // bytes of a record, of its inline successors
+  const uint8_t* indeg = fblob + f.indeg;
+  const uint8_t* rec_g = fblob + f.rec;
+  const uint16_t* more = reinterpret_cast<const uint16_t*>(fblob + f.more);
+  if (REC_SMEM) {
+    uint4* copy = reinterpret_cast<uint4*>(smem_words);
+    const int n16 = V * (int)(rb >> 4);
+    for (int i = threadIdx.x; i < n16; i += blockDim.x) copy[i] = __ldg(reinterpret_cast<const uint4*>(rec_g) + i);
+    __syncthreads();
+  }
+  if (c >= K) return;
+  const uint32_t rec_a = smem_u32(smem_words);
+  // word[V] is the operator that empty record places name: it misses more predecessors than there are placements, and
+  // each placement takes off one at most
+  uint32_t* word = smem_words + (REC_SMEM ? (size_t)V * (rb >> 2) : 0) + (size_t)warp * words;
+  uint32_t* bitmap = word + V + 1;
+  uint32_t* found = bitmap + ((V + 31) >> 5);   // ranks on their way from the bitmap to the pool
+  const uint32_t word_a = smem_u32(word);
+  const int nb = (V + 31) >> 5;
+  const size_t row = (size_t)K;
+  const uint16_t* list_c = list + c;
+  uint16_t* order_c = order + c;
+  const uint32_t lt_mask = (1u << lane) - 1u;
+
+  for (int i = lane; i <= V; i += 32) word[i] = 0xFFFFFFFFu;
+  __syncwarp();
+  // ranks into the operators' words; operators without predecessors are available
+  bool bad = false;
+  constexpr int kBatch = 8;
+  for (int b = 0; b < nb; b += kBatch) {
+    uint32_t i[kBatch], m[kBatch];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int r = (b + q) * 32 + lane;
+      i[q] = r < V ? (uint32_t)list_c[(size_t)r * row] : 0xFFFFFFFFu;
+      bad = bad || (r < V && i[q] >= (uint32_t)V);
+    }
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) m[q] = i[q] < (uint32_t)V ? (uint32_t)__ldg(indeg + i[q]) : 1u;
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      if (i[q] < (uint32_t)V) word[i[q]] = m[q] * kOne | (uint32_t)((b + q) * 32 + lane);
+      const uint32_t avail = __ballot_sync(FULL, m[q] == 0u);
+      if (lane == 0 && b + q < nb) bitmap[b + q] = avail;
+    }
+  }
+  __syncwarp();
+  for (int i = lane; i < V; i += 32) bad = bad || word[i] == 0xFFFFFFFFu;   // an operator twice leaves another one out
+  bad = __any_sync(FULL, bad);
+  if (status && lane == 0) status[c] = bad ? (uint32_t)PE_STATUS_ORDER_INVALID : 0u;
+  if (bad) return;   // not a permutation: the order of this candidate stays unwritten
+
+  uint32_t hot = kNoKey;      // this lane's pool place
+  uint32_t T = 0;             // ranks below T are in the pool, the others in the bitmap
+  int scan = 0;               // bitmap words below are empty
+  // one successor: one predecessor fewer; released (its word is its rank now), it takes this lane's place or its bit
+  auto handle = [&](uint32_t s) {
+    const uint32_t at = word_a + s * 4u;
+    uint32_t w;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(at));
+    w -= kOne;
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(at), "r"(w) : "memory");
+    if (w < T) hot = __byte_perm(w, s, 0x1054);
+    if (w - T < kOne - T) atomicOr(&bitmap[w >> 5], 1u << (w & 31u));
+  };
+  // (every turn places an operator or fills an empty pool, which the next turn takes from: at most 2 V turns)
+  while (true) {
+    // free places and this lane's number among them (the place of the operator taken now counts from the next turn on)
+    const uint32_t open = __ballot_sync(FULL, hot == kNoKey);
+    const uint32_t key = __reduce_min_sync(FULL, hot);
+    if (key == kNoKey) {      // the next words of the bitmap that hold up to kFill operators (or more in the first one)
+      uint32_t total = 0;
+      while (total == 0u && scan < nb) {
+        uint32_t x = scan + lane < nb ? bitmap[scan + lane] : 0u;
+        if (!__any_sync(FULL, x != 0u)) { scan += 32; continue; }
+        const uint32_t cnt = (uint32_t)__popc(x);
+        uint32_t incl = cnt;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const uint32_t o = __shfl_up_sync(FULL, incl, off);
+          incl += lane >= off ? o : 0u;
+        }
+        const bool take = incl <= kFill || incl == cnt;   // a prefix of the words
+        const int nw = __popc(__ballot_sync(FULL, take));
+        total = __shfl_sync(FULL, incl, nw - 1);
+        if (take && x != 0u) {
+          bitmap[scan + lane] = 0u;
+          for (uint32_t at = incl - cnt; x != 0u; x &= x - 1u) found[at++] = 32u * (uint32_t)(scan + lane) + (uint32_t)__ffs((int)x) - 1u;
+        }
+        scan = min(scan + nw, nb);
+      }
+      if (total == 0u) break;   // all placed
+      T = 32u * (uint32_t)scan;
+      __syncwarp();
+      if ((uint32_t)lane < total) {
+        const uint32_t r = found[lane];
+        hot = (r << 16) | (uint32_t)list_c[(size_t)r * row];
+      }
+      __syncwarp();
+      continue;
+    }
+    const uint32_t i = key & 0xFFFFu;
+    const bool mine = hot == kNoKey;
+    uint32_t t = mine ? (uint32_t)__popc(open & lt_mask) * 2u : inl2;
+    t = min(t, inl2);
+    uint32_t n, s;
+    if (REC_SMEM) {
+      const uint32_t at = rec_a + i * rb;
+      uint16_t h, g;
+      asm volatile("ld.shared.u16 %0, [%1];" : "=h"(h) : "r"(at));
+      asm volatile("ld.shared.u16 %0, [%1];" : "=h"(g) : "r"(at + t + 2u));
+      n = h; s = g;
+    } else {
+      const uint8_t* at = rec_g + i * rb;
+      n = __ldg(reinterpret_cast<const uint16_t*>(at));
+      s = __ldg(reinterpret_cast<const uint16_t*>(at + t + 2u));
+    }
+    if (lane == 0) *order_c = (uint16_t)i;
+    order_c += row;
+    if (hot == key) hot = kNoKey;
+    if (n <= (uint32_t)__popc(open)) {   // (n is 64 in the record of an operator with a longer list)
+      handle(s);
+      __syncwarp();
+      continue;
+    }
+    // an operator with a longer list, or fewer free places than successors
+    const uint16_t* r8 = reinterpret_cast<const uint16_t*>(rec_g + (size_t)i * rb);
+    const bool listed = n > 32u;
+    const uint16_t* list_s = listed ? more + ((uint32_t)__ldg(r8 + 2) | (uint32_t)__ldg(r8 + 3) << 16) : r8 + 1;
+    if (listed) n = __ldg(r8 + 1);
+    for (uint32_t done = 0; done < n;) {
+      uint32_t free_now = __ballot_sync(FULL, hot == kNoKey);
+      if (free_now == 0u) {   // the pool is full: back to the bitmap with it
+        const uint32_t r = hot >> 16;
+        atomicOr(&bitmap[r >> 5], 1u << (r & 31u));
+        hot = kNoKey;
+        T = 0u;
+        scan = 0;
+        free_now = FULL;
+        __syncwarp();
+      }
+      const uint32_t q = done + (uint32_t)__popc(free_now & lt_mask);
+      if (hot == kNoKey && q < n) handle((uint32_t)__ldg(list_s + q));
+      done += (uint32_t)__popc(free_now);
+      __syncwarp();
+    }
+  }
+}
+
 struct DecodePlan {
-  bool shared = false;
+  bool shared = false;      // pe_decode_warp_kernel
+  bool rec_smem = false;    // operator records in shared memory
   int threads = 0;
+  uint32_t words = 0;       // shared words per warp
   size_t smem = 0;
   size_t workspace = 0;
 };
+
+static bool plan_decode_warp(const pe_graph* g, int64_t K, DecodePlan* p) {
+  const size_t V = (size_t)g->V, n0 = (V + 31) / 32, rb = g->fview.rec_bytes;
+  if (V > 65535) return false;
+  // the block size that keeps most warps on an SM, and no more warps per block than spread the batch over the SMs
+  size_t best = 0;
+  for (size_t nw = 1; nw <= 8; nw *= 2) {
+    if (nw > 1 && (int64_t)nw * g->sm_count > K) break;
+    const bool with = V * rb <= kDecodeRecBytes;
+    const size_t words = (V + 1 + n0 + 32 + 3) / 4 * 4;
+    const size_t bytes = nw * words * 4 + (with ? V * rb : 0);
+    if (bytes > g->smem_optin) break;
+    size_t blocks = g->smem_per_sm / (bytes + 1024);
+    if (blocks > 32) blocks = 32;
+    const size_t warps = std::min<size_t>(blocks * nw, 64);
+    if (warps <= best) continue;
+    best = warps;
+    p->rec_smem = with;
+    p->threads = (int)(32 * nw);
+    p->words = (uint32_t)words;
+    p->smem = bytes;
+  }
+  p->shared = best > 0;
+  return p->shared;
+}
 
 static bool decode_plan(const pe_graph* g, int64_t K, uint32_t flags, DecodePlan* p) {
   if (!g->fwd_ok) return false;
   const uint32_t want = flags & PE_VARIANT_MASK;
   const size_t V = (size_t)g->V, n0 = (V + 31) / 32, n1 = (n0 + 31) / 32;
   if (want == PE_VARIANT_AUTO || want == PE_VARIANT_SHARED) {
-    const size_t per = 4 * (V + n0 + n1 + (V + 1) / 2);
-    const size_t fixed = (size_t)g->fview.bytes + 16;
-    // with a single warp per SM the shared-state variant loses to the global-state one (measured at
-    // V = 1024: 3.2e9 against ~7e9 operators/s), so it needs room for two warps unless it was asked for
-    if (fixed + (want == PE_VARIANT_SHARED ? 32 : 64) * per <= g->smem_optin) {
-      size_t T = (g->smem_optin - fixed) / per;
-      if (T > 256) T = 256;
-      T = T / 32 * 32;
-      p->shared = true;
-      p->threads = (int)T;
-      p->smem = fixed + T * per;
-      p->workspace = 0;
-      return true;
-    }
+    if (plan_decode_warp(g, K, p)) return true;
     if (want == PE_VARIANT_SHARED) return false;
   }
   if (want != PE_VARIANT_AUTO && want != PE_VARIANT_GLOBAL) return false;
@@ -240,23 +415,23 @@ extern "C" int pe_decode_priority(pe_graph* g, int64_t K, const void* list, int 
   if (!pe::decode_plan(g, K, flags, &p)) return PE_ERR_UNSUPPORTED;
   if (K == 0) return PE_OK;
   if (!list || !order) return PE_ERR_INVALID_ARG;
-  if ((K + p.threads - 1) / p.threads > (int64_t)INT_MAX) return PE_ERR_INVALID_ARG;
+  if (K > (int64_t)INT_MAX) return PE_ERR_INVALID_ARG;
   if (p.workspace > 0 && (!workspace || workspace_bytes < p.workspace)) return PE_ERR_WORKSPACE;
   int prev = -1;
   if (cudaGetDevice(&prev) != cudaSuccess) return PE_ERR_CUDA;
   if (prev != g->device && cudaSetDevice(g->device) != cudaSuccess) return PE_ERR_CUDA;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  const unsigned grid = (unsigned)((K + p.threads - 1) / p.threads);
+  const uint16_t* list16 = static_cast<const uint16_t*>(list);
+  uint16_t* order16 = static_cast<uint16_t*>(order);
   int ret = PE_OK;
   if (p.shared) {
-    auto kern = pe::pe_decode_kernel<true>;
+    const int64_t nw = p.threads / 32;
+    auto kern = p.rec_smem ? pe::pe_decode_warp_kernel<true> : pe::pe_decode_warp_kernel<false>;
     if (!pe::set_smem(kern, p.smem)) ret = PE_ERR_CUDA;
-    else kern<<<grid, p.threads, p.smem, stream>>>(g->fview, g->d_fwd, K, static_cast<const uint16_t*>(list),
-                                                    static_cast<uint16_t*>(order), status, nullptr, g->d_error);
+    else kern<<<(unsigned)((K + nw - 1) / nw), p.threads, p.smem, stream>>>(g->fview, g->d_fwd, K, list16, order16, status, p.words);
   } else {
-    pe::pe_decode_kernel<false><<<grid, p.threads, 0, stream>>>(g->fview, g->d_fwd, K, static_cast<const uint16_t*>(list),
-                                                                static_cast<uint16_t*>(order), status,
-                                                                static_cast<uint32_t*>(workspace), g->d_error);
+    pe::pe_decode_kernel<<<(unsigned)((K + p.threads - 1) / p.threads), p.threads, 0, stream>>>(
+        g->fview, g->d_fwd, K, list16, order16, status, static_cast<uint32_t*>(workspace));
   }
   if (ret == PE_OK) {
     pe::g_decode_launches.fetch_add(1, std::memory_order_relaxed);

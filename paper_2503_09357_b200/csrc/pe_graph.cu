@@ -1,4 +1,5 @@
 // Host side of the library: description checks, by-predecessor CSR, upload, teardown.
+#include <algorithm>
 #include <climits>
 #include <cstdlib>
 #include <cstring>
@@ -283,20 +284,58 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
   std::memset(&g->fview, 0, sizeof(g->fview));
   if (g->fwd_ok) {
     PeFwdView& fv = g->fview;
-    fv.V = V; fv.E = E;
+    std::vector<uint32_t> sptr(V + 1, 0);
+    for (int32_t b = 0; b < E; ++b) sptr[d->edge_src[b] + 1]++;
+    for (int32_t i = 0; i < V; ++i) sptr[i + 1] += sptr[i];
+    std::vector<uint16_t> succ(E);
+    std::vector<uint32_t> fill(sptr.begin(), sptr.end() - 1);
+    for (int32_t b = 0; b < E; ++b) succ[fill[d->edge_src[b]]++] = (uint16_t)d->edge_dst[b];
+    std::vector<uint8_t> uindeg(V, 0);
+    std::vector<uint32_t> uptr(V + 1, 0);
+    std::vector<uint16_t> usucc, more;
+    usucc.reserve(E);
+    int32_t seven = 0;
+    for (int32_t i = 0; i < V; ++i) {
+      std::sort(succ.begin() + sptr[i], succ.begin() + sptr[i + 1]);
+      const auto end = std::unique(succ.begin() + sptr[i], succ.begin() + sptr[i + 1]);
+      usucc.insert(usucc.end(), succ.begin() + sptr[i], end);
+      uptr[i + 1] = (uint32_t)usucc.size();
+      const uint32_t n = uptr[i + 1] - uptr[i];
+      seven += n > 6 && n <= 14;
+    }
+    fv.rec_bytes = seven > V / 50 ? 32 : 16;
+    const uint32_t halves = fv.rec_bytes / 2, inl = halves - 2;
+    std::vector<uint16_t> rec((size_t)V * halves, (uint16_t)V);
+    for (int32_t i = 0; i < V; ++i) {
+      const uint32_t n = uptr[i + 1] - uptr[i];
+      uint16_t* r = rec.data() + (size_t)i * halves;
+      r[0] = (uint16_t)n;
+      for (uint32_t q = 0; q < n; ++q) {
+        uindeg[usucc[uptr[i] + q]]++;
+        if (n <= inl) r[1 + q] = usucc[uptr[i] + q];
+      }
+      if (n > inl) {
+        r[0] = 64;
+        r[1] = (uint16_t)n;
+        r[2] = (uint16_t)(more.size() & 0xFFFFu);
+        r[3] = (uint16_t)(more.size() >> 16);
+        more.insert(more.end(), usucc.begin() + uptr[i], usucc.begin() + uptr[i + 1]);
+      }
+    }
+    fv.V = V; fv.E = (int32_t)usucc.size();
     uint64_t fat = 0;
     fv.ptr = (uint32_t)fat;   fat = align16(fat + (uint64_t)(V + 1) * 4);
-    fv.succ = (uint32_t)fat;  fat = align16(fat + (uint64_t)E * 2);
+    fv.succ = (uint32_t)fat;  fat = align16(fat + (uint64_t)usucc.size() * 2);
     fv.indeg = (uint32_t)fat; fat = align16(fat + (uint64_t)V);
-    fv.bytes = (uint32_t)fat;
-    fblob.assign(fv.bytes, 0);
-    uint32_t* fptr = (uint32_t*)(fblob.data() + fv.ptr);
-    uint16_t* fsucc = (uint16_t*)(fblob.data() + fv.succ);
-    uint8_t* findeg = fblob.data() + fv.indeg;
-    for (int32_t b = 0; b < E; ++b) fptr[d->edge_src[b] + 1]++;
-    for (int32_t i = 0; i < V; ++i) { fptr[i + 1] += fptr[i]; findeg[i] = (uint8_t)ops[i].indeg; }
-    std::vector<uint32_t> ffill(fptr, fptr + V);
-    for (int32_t b = 0; b < E; ++b) fsucc[ffill[d->edge_src[b]]++] = (uint16_t)d->edge_dst[b];
+    fv.rec = (uint32_t)fat;   fat = align16(fat + (uint64_t)V * fv.rec_bytes);
+    fv.more = (uint32_t)fat;  fat = align16(fat + (uint64_t)more.size() * 2);
+    fblob.assign((size_t)fat, 0);
+    auto put = [&](uint32_t at, const void* from, size_t n) { if (n) std::memcpy(fblob.data() + at, from, n); };
+    put(fv.ptr, uptr.data(), (size_t)(V + 1) * 4);
+    put(fv.succ, usucc.data(), usucc.size() * 2);
+    put(fv.indeg, uindeg.data(), (size_t)V);
+    put(fv.rec, rec.data(), (size_t)V * fv.rec_bytes);
+    put(fv.more, more.data(), more.size() * 2);
   }
 
   // one allocation and one copy for all encodings (each on a 256-byte boundary), the status word last

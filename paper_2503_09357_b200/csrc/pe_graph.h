@@ -90,14 +90,19 @@ struct PeTileView {
   uint32_t bytes;      // total, multiple of 16
 };
 
-// Forward view of the DAG for priority-list decoding, built when V <= 65536 and no operator has
-// more than 255 incoming edges: successors of operator i are succ[ptr[i] .. ptr[i+1]).
+// Forward view of the DAG for priority-list decoding, built when V <= 65536 and no operator has more than
+// 255 incoming edges.  Parallel edges count once (a predecessor is placed once).  One record per operator of
+// rec_bytes / 2 uint16: {n, successors 0 .. inl - 1, V} with inl = rec_bytes / 2 - 2, places without a successor hold V;
+// with n > inl: {64, n, first entry in `more` as two halves, ...}, all n successors in `more`.  ptr / succ hold the
+// same lists in CSR form.
 struct PeFwdView {
-  int32_t V, E;
+  int32_t V, E;    // E: edges without repetitions
   uint32_t ptr;    // uint32[V + 1]
   uint32_t succ;   // uint16[E]
   uint32_t indeg;  // uint8[V]
-  uint32_t bytes;  // total, multiple of 16
+  uint32_t rec;    // uint16[V][rec_bytes / 2]
+  uint32_t rec_bytes;   // 16, or 32 where a fiftieth of the operators has 7 to 14 successors
+  uint32_t more;   // uint16[]
 };
 
 struct pe_graph {
