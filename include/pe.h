@@ -105,7 +105,8 @@ enum {
                                   warps prepare windows of the order side by side and only the recurrence of
                                   Eqs. 3, 7-8, 11-13 runs window after window.  For graphs with in-degree <= 8 and
                                   16-bit orders, with start and finish both wanted or both absent; otherwise
-                                  PE_ERR_UNSUPPORTED.  Uses workspace (staging copies) when K is a multiple of 4 */
+                                  PE_ERR_UNSUPPORTED.  Uses workspace (staging copies) from K = 64 on; a K that is no multiple of 4
+                                  also runs, slower, without it */
   PE_VARIANT_MASK = 15u << 8
 };
 

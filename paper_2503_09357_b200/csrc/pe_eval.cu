@@ -301,9 +301,8 @@ static bool plan_warp(const pe_graph* g, int64_t K, uint32_t flags, bool allow_c
   return true;
 }
 
-// TEAM: one block per candidate; plan.threads / 32 warps share the candidate's windows.  With K a multiple of 4
-// (the transpositions move 32-bit words) the inputs and the times go through candidate-major staging copies
-// in the workspace, a chunk of candidates at a time; a chunk is sixteen times what the GPU holds at once.
+// TEAM: one block per candidate; plan.threads / 32 warps share the candidate's windows.  The inputs and the times
+// go through candidate-major staging copies in the workspace, a chunk of candidates at a time.
 static bool plan_team(const pe_graph* g, int64_t K, bool allow_compact, Plan* p) {
   if (!g->narrow_ok || !allow_compact || g->max_indeg > 8 || g->time_bound >= (int64_t)1 << 23) return false;
   const size_t smem = round_up((size_t)4 * (g->V + 2) + (size_t)4 * (5 * g->D + 2), 16);
@@ -313,7 +312,10 @@ static bool plan_team(const pe_graph* g, int64_t K, bool allow_compact, Plan* p)
   // reserves two named barriers per warp, an SM has 64 of them, and more chains beat deeper pipelines there
   // (measured at V = 4096 / D = 64: 4.46e10 with two warps, 4.36e10 with four, 3.3e10 with six; the MoE graph:
   // 2.03e10 against 1.96e10 and 1.63e10).
+  // A batch that leaves SMs with fewer blocks than fit is bound by the latency of one block: more warps then.
   size_t per_sm = (g->smem_per_sm ? g->smem_per_sm : g->smem_optin) / (smem + 1024);
+  const size_t fair = (size_t)((K + g->sm_count - 1) / g->sm_count);
+  if (per_sm > fair) per_sm = fair;
   if (per_sm < 1) per_sm = 1;
   const int nw = per_sm <= 4 ? 6 : (per_sm <= 7 ? 4 : 2);
   const size_t by_barriers = (size_t)64 / (nw == 6 ? 16 : 2 * nw + 1);
@@ -326,7 +328,7 @@ static bool plan_team(const pe_graph* g, int64_t K, bool allow_compact, Plan* p)
   p->workspace = 0;
   p->ws_x_off = 0;
   p->compact = true;
-  p->staged = K >= 64 && K % 4 == 0;
+  p->staged = K >= 64;
   if (p->staged) {
     // a chunk is eight times what the GPU holds at once (measured at V = 16384: 4, 8 and 16 times are
     // within 2 % of each other; two chunks are in flight)
@@ -482,7 +484,6 @@ static int launch_typed(const pe_graph* g, const Plan& p, int64_t K, const uint8
     }
     uint32_t* gstate = static_cast<uint32_t*>(workspace);
     if (p.variant == PE_VARIANT_TEAM) {
-      if (p.staged && (((uintptr_t)assign | (uintptr_t)order) & 3u)) return PE_ERR_INVALID_ARG;   // word-wise transpositions
       int64_t n = 0;
       const int rc = launch_team(g, p, BY_POS, K, assign, ord16, flags, out, workspace, stream, &n);
       if (rc != PE_OK) return rc;
@@ -564,6 +565,10 @@ extern "C" int pe_eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, cons
   if (K == 0) return PE_OK;
   if (!assign || !order) return PE_ERR_INVALID_ARG;
   if ((K + p.threads - 1) / p.threads > (int64_t)INT_MAX) return PE_ERR_INVALID_ARG;
+  if (p.variant == PE_VARIANT_TEAM && p.staged && K % 4 != 0 && (!workspace || workspace_bytes < p.workspace)) {
+    p.staged = false;   // batches that are no multiple of 4 also run without staging copies
+    p.workspace = 0;
+  }
   if (p.workspace > 0 && (!workspace || workspace_bytes < p.workspace)) return PE_ERR_WORKSPACE;
   int prev = -1;
   if (cudaGetDevice(&prev) != cudaSuccess) return PE_ERR_CUDA;

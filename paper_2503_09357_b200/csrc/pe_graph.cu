@@ -88,6 +88,11 @@ int check_desc(const pe_graph_desc* d, int64_t* time_bound, int64_t* mem_bound, 
   return PE_OK;
 }
 
+std::vector<cudaEvent_t*> team_events(pe_graph* g) {
+  return {&g->team_fork,    &g->team_join[0], &g->team_join[1], &g->team_join[2], &g->team_in[0],
+          &g->team_in[1],   &g->team_done[0], &g->team_done[1], &g->team_back[0], &g->team_back[1]};
+}
+
 }  // namespace
 
 extern "C" int pe_graph_validate(const pe_graph_desc* desc) { return check_desc(desc, nullptr, nullptr, nullptr); }
@@ -372,10 +377,11 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
            cudaEventCreateWithFlags(&g->ev_begin, cudaEventDisableTiming) == cudaSuccess &&
            cudaEventCreateWithFlags(&g->ev_end, cudaEventDisableTiming) == cudaSuccess &&
            cudaStreamCreateWithFlags(&g->team_stream[0], cudaStreamNonBlocking) == cudaSuccess &&
-           cudaStreamCreateWithFlags(&g->team_stream[1], cudaStreamNonBlocking) == cudaSuccess &&
-           cudaEventCreateWithFlags(&g->team_fork, cudaEventDisableTiming) == cudaSuccess &&
-           cudaEventCreateWithFlags(&g->team_join[0], cudaEventDisableTiming) == cudaSuccess &&
-           cudaEventCreateWithFlags(&g->team_join[1], cudaEventDisableTiming) == cudaSuccess;
+           cudaStreamCreateWithFlags(&g->team_stream[1], cudaStreamNonBlocking) == cudaSuccess;
+      int least = 0, greatest = 0;
+      ok = ok && cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess &&
+           cudaStreamCreateWithPriority(&g->team_copy, cudaStreamNonBlocking, greatest) == cudaSuccess;
+      for (cudaEvent_t* e : team_events(g)) ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
       for (int q = 0; ok && q < pe_graph::kMaxChunks; ++q)
         ok = cudaEventCreateWithFlags(&g->ev_in[q], cudaEventDisableTiming) == cudaSuccess &&
              cudaEventCreateWithFlags(&g->ev_done[q], cudaEventDisableTiming) == cudaSuccess;
@@ -389,11 +395,10 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
     if (g->copy_out) cudaStreamDestroy(g->copy_out);
     if (g->ev_begin) cudaEventDestroy(g->ev_begin);
     if (g->ev_end) cudaEventDestroy(g->ev_end);
-    for (int q = 0; q < 2; ++q) {
-      if (g->team_stream[q]) cudaStreamDestroy(g->team_stream[q]);
-      if (g->team_join[q]) cudaEventDestroy(g->team_join[q]);
-    }
-    if (g->team_fork) cudaEventDestroy(g->team_fork);
+    for (cudaStream_t s : {g->team_stream[0], g->team_stream[1], g->team_copy})
+      if (s) cudaStreamDestroy(s);
+    for (cudaEvent_t* e : team_events(g))
+      if (*e) cudaEventDestroy(*e);
     for (int q = 0; q < pe_graph::kMaxChunks; ++q) {
       if (g->ev_in[q]) cudaEventDestroy(g->ev_in[q]);
       if (g->ev_done[q]) cudaEventDestroy(g->ev_done[q]);
@@ -415,8 +420,8 @@ extern "C" int pe_destroy(pe_graph* g) {
   cudaStreamDestroy(g->copy_out);
   cudaEventDestroy(g->ev_begin);
   cudaEventDestroy(g->ev_end);
-  for (int q = 0; q < 2; ++q) { cudaStreamDestroy(g->team_stream[q]); cudaEventDestroy(g->team_join[q]); }
-  cudaEventDestroy(g->team_fork);
+  for (cudaStream_t s : {g->team_stream[0], g->team_stream[1], g->team_copy}) cudaStreamDestroy(s);
+  for (cudaEvent_t* e : team_events(g)) cudaEventDestroy(*e);
   for (int q = 0; q < pe_graph::kMaxChunks; ++q) { cudaEventDestroy(g->ev_in[q]); cudaEventDestroy(g->ev_done[q]); }
   const bool ok = cudaFree(g->d_blob) == cudaSuccess;
   if (prev >= 0) cudaSetDevice(prev);

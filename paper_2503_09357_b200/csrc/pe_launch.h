@@ -30,7 +30,7 @@ struct Plan {
   TileShape tile = {};
   // TEAM: inputs and times go through candidate-major staging copies in the workspace, a chunk of candidates at a time
   bool staged = false;
-  int64_t team_chunk = 0;   // candidates per chunk (multiple of 4)
+  int64_t team_chunk = 0;   // candidates per chunk
   int64_t team_vp = 0;      // row length of the staging copies: V rounded up to a multiple of 64
   size_t team_off_order = 0, team_off_assign = 0, team_off_start = 0, team_off_finish = 0;   // offsets in a half
   size_t team_half = 0;     // bytes of one half of the workspace (two chunks are in flight)

@@ -22,9 +22,13 @@ int launch1(const TeamCall& t) {
 template <int S>
 void transpose(const void* in, void* out, int64_t R, int64_t C, int64_t in_ld, int64_t out_ld, cudaStream_t stream) {
   constexpr int TR = 32 * (4 / S);
-  const dim3 grid((unsigned)((C + TR - 1) / TR), (unsigned)((R + TR - 1) / TR));
-  pe_transpose_kernel<S><<<grid, 256, 0, stream>>>(static_cast<const uint8_t*>(in), static_cast<uint8_t*>(out), R, C, in_ld,
-                                                   out_ld);
+  const dim3 grid((unsigned)((C + 31) / 32), (unsigned)((R + TR - 1) / TR));
+  const uint8_t* from = static_cast<const uint8_t*>(in);
+  uint8_t* to = static_cast<uint8_t*>(out);
+  if (((uintptr_t)in & 3u) == 0 && in_ld * S % 4 == 0)
+    pe_transpose_kernel<S, true><<<grid, 128, 0, stream>>>(from, to, R, C, in_ld, out_ld);
+  else
+    pe_transpose_kernel<S, S == 4><<<grid, 128, 0, stream>>>(from, to, R, C, in_ld, out_ld);
 }
 
 }  // namespace
@@ -39,9 +43,10 @@ int launch_team(const pe_graph* g, const Plan& p, bool by_pos, int64_t K, const 
     *launches += 1;
     return by_pos ? launch1<true>(t) : launch1<false>(t);
   }
-  // staged: chunks of candidates go through candidate-major copies in the workspace.  Consecutive chunks
-  // use the two halves of the workspace and the graph's two side streams, so the transpositions of one
-  // chunk run while the other is evaluated, and the tail of one evaluation overlaps the head of the next.
+  // staged: chunks of candidates go through candidate-major copies in the workspace, which has room for two
+  // chunks.  Evaluations alternate between two streams, so that the tail of one overlaps the head of the next; the
+  // transpositions have a stream of higher priority of their own: their blocks are placed in what the evaluation's
+  // blocks leave free of an SM (at the same priority they wait until every block of an evaluation is placed).
   const int64_t V = g->V, Vp = p.team_vp;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   const bool times = out.start != nullptr;
@@ -49,47 +54,57 @@ int launch_team(const pe_graph* g, const Plan& p, bool by_pos, int64_t K, const 
   pe_graph* gm = const_cast<pe_graph*>(g);
   std::unique_lock<std::mutex> lock(gm->team_mutex, std::defer_lock);
   bool ok = true;
-  if (fork) {
-    lock.lock();
-    ok = cudaEventRecord(gm->team_fork, stream) == cudaSuccess &&
-         cudaStreamWaitEvent(gm->team_stream[0], gm->team_fork, 0) == cudaSuccess &&
-         cudaStreamWaitEvent(gm->team_stream[1], gm->team_fork, 0) == cudaSuccess;
-  }
-  int rc = ok ? PE_OK : PE_ERR_CUDA;
+  auto record = [&](cudaEvent_t e, cudaStream_t s) { if (fork) ok = cudaEventRecord(e, s) == cudaSuccess && ok; };
+  auto wait = [&](cudaStream_t s, cudaEvent_t e) { if (fork) ok = cudaStreamWaitEvent(s, e, 0) == cudaSuccess && ok; };
+  const cudaStream_t copies = fork ? gm->team_copy : stream;
+  if (fork) lock.lock();
+  record(gm->team_fork, stream);
+  wait(gm->team_stream[0], gm->team_fork);
+  wait(gm->team_stream[1], gm->team_fork);
+  wait(gm->team_copy, gm->team_fork);
+  auto half_of = [&](int q) { return ws + (size_t)(q & 1) * p.team_half; };
+  auto copy_back = [&](int q, int64_t c0) {   // times of chunk q, once it is evaluated
+    const int64_t kc = K - c0 < p.team_chunk ? K - c0 : p.team_chunk;
+    wait(copies, gm->team_done[q & 1]);
+    transpose<4>(half_of(q) + p.team_off_start, out.start + c0, kc, V, Vp, K, copies);
+    transpose<4>(half_of(q) + p.team_off_finish, out.finish + c0, kc, V, Vp, K, copies);
+    record(gm->team_back[q & 1], copies);
+    *launches += 2;
+  };
+  int rc = PE_OK;
   int q = 0;
   for (int64_t c0 = 0; c0 < K && rc == PE_OK; c0 += p.team_chunk, ++q) {
     const int64_t kc = K - c0 < p.team_chunk ? K - c0 : p.team_chunk;
-    uint8_t* half = ws + (size_t)(q & 1) * p.team_half;
+    uint8_t* half = half_of(q);
     uint16_t* ord_t = reinterpret_cast<uint16_t*>(half + p.team_off_order);
     uint8_t* asg_t = half + p.team_off_assign;
-    int32_t* start_t = reinterpret_cast<int32_t*>(half + p.team_off_start);
-    int32_t* finish_t = reinterpret_cast<int32_t*>(half + p.team_off_finish);
     t.stream = fork ? gm->team_stream[q & 1] : stream;
-    transpose<2>(order + c0, ord_t, V, kc, K, Vp, t.stream);
-    transpose<1>(assign + c0, asg_t, V, kc, K, Vp, t.stream);
+    if (q >= 2) wait(copies, gm->team_done[q & 1]);     // chunk q - 2 has read its inputs
+    transpose<2>(order + c0, ord_t, V, kc, K, Vp, copies);
+    transpose<1>(assign + c0, asg_t, V, kc, K, Vp, copies);
+    record(gm->team_in[q & 1], copies);
+    wait(t.stream, gm->team_in[q & 1]);
+    if (q >= 2 && times) wait(t.stream, gm->team_back[q & 1]);   // the times of chunk q - 2 have left
     t.kc = kc; t.assign = asg_t; t.order = ord_t;
-    t.out.start = times ? start_t : nullptr;
-    t.out.finish = times ? finish_t : nullptr;
+    t.out.start = times ? reinterpret_cast<int32_t*>(half + p.team_off_start) : nullptr;
+    t.out.finish = times ? reinterpret_cast<int32_t*>(half + p.team_off_finish) : nullptr;
     t.out.makespan = out.makespan ? out.makespan + c0 : nullptr;
     t.out.status = out.status ? out.status + c0 : nullptr;
     t.out.busy = out.busy ? out.busy + c0 : nullptr;
     t.out.peak_mem = out.peak_mem ? out.peak_mem + c0 : nullptr;
     t.sd.in_row = 1; t.sd.in_cand = (size_t)Vp; t.sd.out_row = 1; t.sd.out_cand = (size_t)Vp;
     rc = by_pos ? launch1<true>(t) : launch1<false>(t);
-    if (rc != PE_OK) break;
+    record(gm->team_done[q & 1], t.stream);
     *launches += 3;
-    if (times) {
-      transpose<4>(start_t, out.start + c0, kc, V, Vp, K, t.stream);
-      transpose<4>(finish_t, out.finish + c0, kc, V, Vp, K, t.stream);
-      *launches += 2;
-    }
+    if (rc == PE_OK && times && q >= 1) copy_back(q - 1, c0 - p.team_chunk);
   }
-  if (fork) {   // join, also after an error: nothing of this call may stay unordered on the side streams
-    for (int b = 0; b < 2; ++b)
-      if (cudaEventRecord(gm->team_join[b], gm->team_stream[b]) != cudaSuccess ||
-          cudaStreamWaitEvent(stream, gm->team_join[b], 0) != cudaSuccess)
-        rc = rc == PE_OK ? PE_ERR_CUDA : rc;
-  }
+  if (rc == PE_OK && times) copy_back(q - 1, (int64_t)(q - 1) * p.team_chunk);
+  // join, also after an error: nothing of this call may stay unordered on the side streams
+  record(gm->team_join[0], gm->team_stream[0]);
+  record(gm->team_join[1], gm->team_stream[1]);
+  record(gm->team_join[2], gm->team_copy);
+  for (int b = 0; b < 3; ++b) wait(stream, gm->team_join[b]);
+  if (!ok && rc == PE_OK) rc = PE_ERR_CUDA;
   return rc;
 }
 

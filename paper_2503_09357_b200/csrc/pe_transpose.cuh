@@ -1,8 +1,8 @@
 // Tiled transposition between the candidate-interleaved arrays of the interface ([rows][K]) and
 // candidate-major staging copies ([K][rows padded]).  A block of pe_eval_team_kernel works on one
 // candidate; with the interleaved layout every one of its loads and stores would touch its own
-// 32-byte sector (2 or 4 useful bytes each), with the staging copy it moves whole lines.  The
-// transposition itself reads and writes 128 contiguous bytes per warp instruction on both sides.
+// 32-byte sector (2 or 4 useful bytes each), with the staging copy it moves whole lines. The
+// transposition itself reads whole 32-byte sectors (or more) and writes 128 contiguous bytes per warp instruction.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -10,38 +10,52 @@
 namespace pe {
 
 // in:  [R][in_ld] elements of S bytes, columns 0..C-1 used; out: [C][out_ld], columns 0..R-1 written
-// (and zeros up to the next multiple of 4 / S).  C * S, in_ld * S and out_ld * S must be multiples of 4
-// and both bases 4-byte aligned.  One block moves a tile of 32*G rows by 32*G columns (G = 4 / S
-// elements per 32-bit word) through shared memory; word (r, cw) of the tile is kept at column
-// (cw + r / G) mod 32, which makes both the row-wise writes and the G-rows-per-lane reads free of bank
-// conflicts.  grid = (ceil(C / (32 G)), ceil(R / (32 G))), 256 threads.
-template <int S>
-__global__ void __launch_bounds__(256) pe_transpose_kernel(const uint8_t* __restrict__ in, uint8_t* __restrict__ out,
+// (and zeros up to the next multiple of 4 / S).  out_ld * S must be a multiple of 4 and `out` 4-byte aligned; `in` and
+// its rows may start anywhere when !ALIGNED (odd batches: a word is put together from two aligned ones).
+// One block of 128 threads moves a tile of 32 G rows by 32 columns (G = 4 / S elements per 32-bit word) through 4 KB of
+// shared memory; word (r, cw) of the tile is kept at word (cw + r / G) mod (32 / G) of its row, which keeps the
+// G-rows-per-lane reads to few lanes a bank.  grid = (ceil(C / 32), ceil(R / (32 G))).
+// Bound by DRAM.  The tile is this small so that a few blocks fit next to the evaluation's blocks, which leave ~25 KB
+// of an SM's shared memory and most of its threads free: the copies of one chunk then run while another is evaluated.
+template <int S, bool ALIGNED>
+__global__ void __launch_bounds__(128) pe_transpose_kernel(const uint8_t* __restrict__ in, uint8_t* __restrict__ out,
                                                            int64_t R, int64_t C, int64_t in_ld, int64_t out_ld) {
   constexpr int G = 4 / S;
-  constexpr int TR = 32 * G;   // tile rows = tile columns (elements)
-  __shared__ uint32_t tile[TR][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t r0 = (int64_t)blockIdx.y * TR, c0 = (int64_t)blockIdx.x * TR;
-  const uint32_t* in_w = reinterpret_cast<const uint32_t*>(in);
+  constexpr int TR = 32 * G;   // tile rows (elements)
+  constexpr int TW = 32 / G;   // words of a tile row
+  __shared__ uint32_t tile[TR][TW];
+  const int64_t r0 = (int64_t)blockIdx.y * TR, c0 = (int64_t)blockIdx.x * 32;
   uint32_t* out_w = reinterpret_cast<uint32_t*>(out);
-  const int64_t in_ldw = in_ld / G, out_ldw = out_ld / G;   // row pitches in words
-  const int64_t cw0 = c0 / G, rw0 = r0 / G;
-  const int64_t Cw = C / G;                                  // words per input row
+  const int64_t out_ldw = out_ld / G, rw0 = r0 / G;          // in words
   const int64_t Rw = (R + G - 1) / G;                        // words per output row
-  // load: row r of the tile, lanes over the 32 words of the row
-  for (int r = warp; r < TR; r += 8) {
-    const int64_t rr = r0 + r;
+  const int64_t width = (C - c0) * S;                        // bytes of a row from the tile's first column on
+  // load: consecutive threads take consecutive words of a row, then the next row
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int idx = q * 128 + threadIdx.x;
+    const int r = idx / TW, cw = idx % TW;
     uint32_t w = 0;
-    if (rr < R && cw0 + lane < Cw) w = in_w[rr * in_ldw + cw0 + lane];
-    tile[r][(lane + r / G) & 31] = w;
+    if (r0 + r < R && 4 * cw < width) {
+      const uint8_t* at = in + ((r0 + r) * in_ld + c0) * S + 4 * cw;
+      if (ALIGNED) {
+        w = __ldg(reinterpret_cast<const uint32_t*>(at));
+      } else {
+        const uint32_t a = (uint32_t)(uintptr_t)at & 3u;
+        const uint32_t* base = reinterpret_cast<const uint32_t*>(at - a);
+        const uint32_t lo = __ldg(base), hi = (a != 0 && 4 * cw + 4 - (int)a < width) ? __ldg(base + 1) : 0u;
+        w = __funnelshift_r(lo, hi, 8u * a);
+      }
+    }
+    tile[r][(cw + r / G) % TW] = w;
   }
   __syncthreads();
   // store: word column cw of the tile holds G input columns; lane t owns input rows G t .. G t + G - 1
-  for (int cw = warp; cw < 32; cw += 8) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int cw = warp; cw < TW; cw += 4) {
     uint32_t v[G];
 #pragma unroll
-    for (int q = 0; q < G; ++q) v[q] = tile[G * lane + q][(cw + lane) & 31];
+    for (int q = 0; q < G; ++q) v[q] = tile[G * lane + q][(cw + lane) % TW];
     uint32_t o[G];
     if constexpr (G == 1) {
       o[0] = v[0];
