@@ -328,7 +328,9 @@ static bool plan_team(const pe_graph* g, int64_t K, bool allow_compact, Plan* p)
   p->workspace = 0;
   p->ws_x_off = 0;
   p->compact = true;
-  p->staged = K >= 64;
+  // the four extra launches pay from about a million operator-evaluations on (measured: bidirectional pipeline K = 1023
+  // 29 us direct, 39 us staged; multi-modal graph K = 1023 92 and 88 us; V = 16384, K = 443 289 and 241 us)
+  p->staged = K >= 64 && (int64_t)g->V * K >= ((int64_t)1 << 20);
   if (p->staged) {
     // a chunk is eight times what the GPU holds at once (measured at V = 16384: 4, 8 and 16 times are
     // within 2 % of each other; two chunks are in flight)
@@ -400,6 +402,19 @@ static bool shared_pays(const pe_graph* g, const Plan& p) {
   return p.tile_resident >= (p.exclusive ? 16 : (g->max_indeg > 3 ? 48 : 28));
 }
 
+// Is a block of warps per candidate (TEAM) sooner done than a lane per candidate?  A lane takes ~0.1 us a position
+// however few candidates there are; a block of warps ~0.026 us a position, and an SM full of blocks ~4 us per 1000
+// candidate positions.  Measured (lane / team, us): V = 480 K = 1023 50 / 29, K = 3551 50 / 77; V = 1536 K = 64 191 / 64,
+// K = 1024 197 / 84, K = 2664 171 / 177; V = 1024 D = 8 K = 1000 105 / 49, K = 3000 92 / 107; V = 64 K = 1024 12 / 26.
+static bool team_sooner(const pe_graph* g, int64_t K, const Plan& lane) {
+  if (!lane.tiled) return false;
+  const double V = g->V, work = V * (double)K;
+  const double rounds = (double)K / ((double)lane.tile_resident * g->sm_count);
+  const double t_lane = 8.0 + 0.1 * V * (rounds > 1.0 ? rounds : 1.0);
+  const double t_team = 12.0 + 0.026 * V + work / 36000.0;
+  return t_team < t_lane;
+}
+
 // allow_compact: the call can use the compact-graph kernels (u16 orders; start and finish both
 // wanted or both absent).  Size queries pass true and false and take the larger workspace.
 static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_compact, Plan* p) {
@@ -432,8 +447,12 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
       // that the state of a candidate is too large: a warp per candidate (state still on chip) wins while at
       // least four warps fit on an SM; for the largest graphs the global-state kernel, which is bound by random
       // DRAM accesses but keeps thousands of candidates in flight, is faster.
-      if (plan_shared(g, K, allow_compact, p) && shared_pays(g, *p)) return PE_OK;
       Plan w, gl, tm;
+      const bool has_s = plan_shared(g, K, allow_compact, p) && shared_pays(g, *p);
+      const bool has_t = plan_team(g, K, allow_compact, &tm);
+      // A batch so small that the lanes of the first round are not filled takes a lane's time over the whole order
+      // whatever its size; a block of warps per candidate is done sooner.
+      if (has_s && !(has_t && team_sooner(g, K, *p))) return PE_OK;
       const bool has_w = plan_warp(g, K, flags, allow_compact, &w);
       const bool has_g = plan_global(g, K, flags, allow_compact, &gl);
       // Once fewer than about twenty single-warp candidates fit on an SM, a block of warps per candidate
@@ -442,7 +461,7 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
       // (global); at V = 1024 the single-warp kernel still wins, 4.0e10 against 3.0e10).
       // Graphs with operators of more than three incoming edges take the single-warp kernel off its register
       // slots; there the block of warps wins as well (measured on the MoE graph: 1.7e10 against 0.9e10).
-      if (plan_team(g, K, allow_compact, &tm) && (!has_w || w.threads < 20 * 32 || (g->max_indeg > 3 && w.threads < 24 * 32))) {
+      if (has_t && (has_s || !has_w || w.threads < 20 * 32 || (g->max_indeg > 3 && w.threads < 24 * 32))) {
         *p = tm;
         return PE_OK;
       }
