@@ -571,9 +571,10 @@ extern "C" int64_t pe_kernel_launches(void) {
   return pe::g_launches.load(std::memory_order_relaxed) + pe::g_decode_launches.load(std::memory_order_relaxed);
 }
 
-extern "C" int pe_eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, const void* order, int order_bytes,
-                             uint32_t flags, const pe_outputs* out, void* workspace, size_t workspace_bytes,
-                             void* cuda_stream) {
+// direct_ok: a TEAM batch whose staging copies do not fit the workspace runs without them.
+static int eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, const void* order, int order_bytes,
+                      uint32_t flags, const pe_outputs* out, void* workspace, size_t workspace_bytes,
+                      void* cuda_stream, bool direct_ok) {
   if (!g || !out || K < 0) return PE_ERR_INVALID_ARG;
   if (order_bytes != 2 && order_bytes != 4) return PE_ERR_INVALID_ARG;
   if (order_bytes == 2 && g->V > 65536) return PE_ERR_INVALID_ARG;
@@ -584,8 +585,8 @@ extern "C" int pe_eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, cons
   if (K == 0) return PE_OK;
   if (!assign || !order) return PE_ERR_INVALID_ARG;
   if ((K + p.threads - 1) / p.threads > (int64_t)INT_MAX) return PE_ERR_INVALID_ARG;
-  if (p.variant == PE_VARIANT_TEAM && p.staged && K % 4 != 0 && (!workspace || workspace_bytes < p.workspace)) {
-    p.staged = false;   // batches that are no multiple of 4 also run without staging copies
+  if (p.variant == PE_VARIANT_TEAM && p.staged && direct_ok && (!workspace || workspace_bytes < p.workspace)) {
+    p.staged = false;
     p.workspace = 0;
   }
   if (p.workspace > 0 && (!workspace || workspace_bytes < p.workspace)) return PE_ERR_WORKSPACE;
@@ -603,6 +604,12 @@ extern "C" int pe_eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, cons
                  : pe::launch_typed<uint32_t, false>(g, p, K, assign, order, flags, *out, workspace, stream);
   if (prev != g->device) cudaSetDevice(prev);
   return ret;
+}
+
+extern "C" int pe_eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, const void* order, int order_bytes,
+                             uint32_t flags, const pe_outputs* out, void* workspace, size_t workspace_bytes,
+                             void* cuda_stream) {
+  return eval_batch(g, K, assign, order, order_bytes, flags, out, workspace, workspace_bytes, cuda_stream, K % 4 != 0);
 }
 
 extern "C" int pe_eval_batch_host(pe_graph* g, int64_t K, const uint8_t* host_assign, const void* host_order,
@@ -637,11 +644,22 @@ extern "C" int pe_eval_batch_host(pe_graph* g, int64_t K, const uint8_t* host_as
   // directions use separate DMA engines).  A chunk of Kc candidates lives in the staging buffers
   // as a dense [rows][Kc] block at element offset rows * first; the strided host side is handled
   // by 2-D copies.
-  // (measured on the default workload: 16 chunks 6.1e9, 8 chunks 5.8e9, 4 chunks 5.3e9 operator-evaluations/s
-  // end to end - shorter chunks shorten the ramp before the first download and after the last upload)
-  int nchunks = K >= 16 * 4096 ? 16 : (K >= 8 * 4096 ? 8 : 1);
-  const int64_t per = ((K + nchunks - 1) / nchunks + 255) / 256 * 256;
-  nchunks = (int)((K + per - 1) / per);
+  // Shorter chunks shorten the ramp before the first download and after the last upload (the first and the last chunk
+  // are half the others for the same reason), but every chunk costs launches, and narrow rows copy more slowly.
+  // Measured (ms, 1 / 3 / 5 / 8 / 16 chunks): MoE graph K = 16384 (500 MB moved) 11.3 / 8.5 / 8.2 / 8.5 / 8.8,
+  // bidirectional pipeline K = 65536 (350 MB) 6.6 / 5.4 / 5.3 / 5.3 / 6.1, K = 8192 (44 MB) 0.88 / 0.81 / 0.84 / 0.93 /
+  // 1.09, K = 1024 (5 MB) 0.18 / 0.20 / 0.25 / 0.31 / 0.46; V = 16384 K = 65536 (12 GB): 16 beat 8 and 4.
+  const size_t moved = V * Ks * (1 + ob + (host_out->start ? 4 : 0) + (host_out->finish ? 4 : 0));
+  int nchunks = moved < ((size_t)24 << 20) ? 1 : (moved < ((size_t)64 << 20) ? 3 : 5);
+  if (K >= 32768) nchunks = 8;   // (rows stay wide)
+  if (moved >= ((size_t)4 << 30)) nchunks = 16;
+  if (nchunks > (K + 63) / 64) nchunks = (int)((K + 63) / 64);
+  int64_t begin[pe_graph::kMaxChunks + 1];
+  const int64_t halves = nchunks > 3 ? 2 * nchunks - 2 : 2 * nchunks;
+  for (int q = 0; q <= nchunks; ++q) {
+    const int64_t at = nchunks > 3 ? (q == 0 ? 0 : 2 * q - 1) : 2 * q;
+    begin[q] = q == nchunks ? K : K * at / halves / 64 * 64;
+  }
   std::lock_guard<std::mutex> lock(g->host_mutex);
   int ret = PE_OK;
   auto ok = [&](cudaError_t e) { if (e != cudaSuccess && ret == PE_OK) ret = PE_ERR_CUDA; };
@@ -649,8 +667,9 @@ extern "C" int pe_eval_batch_host(pe_graph* g, int64_t K, const uint8_t* host_as
   ok(cudaStreamWaitEvent(g->copy_in, g->ev_begin, 0));
   ok(cudaStreamWaitEvent(g->copy_out, g->ev_begin, 0));
   for (int q = 0; q < nchunks && ret == PE_OK; ++q) {
-    const size_t first = (size_t)q * (size_t)per;
-    const size_t Kc = (size_t)(K - (int64_t)first < per ? K - (int64_t)first : per);
+    const size_t first = (size_t)begin[q];
+    const size_t Kc = (size_t)(begin[q + 1] - begin[q]);
+    if (Kc == 0) continue;
     uint8_t* d_as = dev_assign + V * first;
     uint8_t* d_or = static_cast<uint8_t*>(dev_order) + V * first * ob;
     ok(cudaMemcpy2DAsync(d_as, Kc, host_assign + first, Ks, Kc, V, cudaMemcpyHostToDevice, g->copy_in));
@@ -666,7 +685,8 @@ extern "C" int pe_eval_batch_host(pe_graph* g, int64_t K, const uint8_t* host_as
     run.peak_mem = want.peak_mem ? want.peak_mem + D * first : nullptr;
     run.status = want.status ? want.status + first : nullptr;
     if (ret == PE_OK)
-      ret = pe_eval_batch(g, (int64_t)Kc, d_as, d_or, order_bytes, flags, &run, workspace, workspace_bytes, cuda_stream);
+      // (a chunk may take another kernel than the whole batch, which the workspace was sized for)
+      ret = eval_batch(g, (int64_t)Kc, d_as, d_or, order_bytes, flags, &run, workspace, workspace_bytes, cuda_stream, true);
     ok(cudaEventRecord(g->ev_done[q], stream));
     ok(cudaStreamWaitEvent(g->copy_out, g->ev_done[q], 0));
     auto back = [&](void* h, const void* d, size_t rows, size_t elem) {  // [rows][Kc] block -> columns first.. of [rows][K]
