@@ -27,6 +27,11 @@
 // 27.5 -> 5.9 ms; V = 16384, K = 2048 125 -> 23.5 ms.  Candidate-major copies of list and order, and records brought
 // to the pool's places by asynchronous copies, were measured and changed nothing or cost up to 15 %.
 //
+// Lane per candidate (pe_decode_lane_kernel; V <= 256, large batches).  The set of available operators is a bitmap
+// with one summary word in a register; 3.1 bytes of state per operator (rank and missing predecessors in 16 bits, the
+// list in 8) let up to ~1000 candidates share an SM and hide the chain of a placement, bitmap -> list -> successor
+// list -> counts, about five shared-memory round trips.
+//
 // Thread per candidate (pe_decode_kernel; for graphs whose per-candidate state does not fit on chip, V above
 // ~55000, or on request).  The bitmap has two summary levels above it (one bit per 32-bit word of the level below;
 // the top level is a 64-bit register, which is why V <= 65536): "take the smallest" is three find-first-set steps.
@@ -338,8 +343,98 @@ __global__ void __launch_bounds__(256) pe_decode_warp_kernel(PeFwdView f, const 
   }
 }
 
+// The block's threads keep word[i] (rank of operator i | missing predecessors << 8) and list[r] as [row][thread]; two
+// (four) warps share the 32-bit words of a row, so that the lanes of a warp fall into different banks.
+constexpr int kLaneThreads = 128;
+__global__ void __launch_bounds__(kLaneThreads) pe_decode_lane_kernel(PeFwdView f, const uint8_t* __restrict__ fblob, int64_t K,
+                                                                      const uint16_t* __restrict__ list,
+                                                                      uint16_t* __restrict__ order, uint32_t* __restrict__ status) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int V = f.V, E = f.E, t = threadIdx.x;
+  const FwdPtrs fp = fwd_ptrs(fblob, f);
+  uint32_t* head = reinterpret_cast<uint32_t*>(smem_raw);   // first successor | how many << 16 | missing predecessors << 24
+  uint32_t* bits = head + V;                                // [(V + 31) / 32][thread]
+  const int nb = (V + 31) >> 5;
+  uint16_t* words = reinterpret_cast<uint16_t*>(bits + nb * kLaneThreads);
+  uint8_t* lists = reinterpret_cast<uint8_t*>(words + V * kLaneThreads);
+  uint8_t* succ = lists + V * kLaneThreads;
+  for (int i = t; i < V; i += kLaneThreads) {
+    const uint32_t b = fp.ptr[i];
+    head[i] = b | (fp.ptr[i + 1] - b) << 16 | (uint32_t)fp.indeg[i] << 24;   // (a predecessor list is at most 255 long)
+  }
+  for (int e = t; e < E; e += kLaneThreads) succ[e] = (uint8_t)fp.succ[e];
+  __syncthreads();
+  const int64_t c = (int64_t)blockIdx.x * kLaneThreads + t;
+  if (c >= K) return;
+  const size_t Ks = (size_t)K;
+  uint16_t* word = words + 2 * (32 * (t >> 6) + (t & 31)) + ((t >> 5) & 1);
+  uint8_t* lst = lists + 4 * (t & 31) + (t >> 5);
+  uint32_t* bit = bits + t;
+  uint32_t some = 0;   // bitmap words that are not empty
+  auto add = [&](uint32_t r) {
+    bit[(r >> 5) * kLaneThreads] |= 1u << (r & 31u);
+    some |= 1u << (r >> 5);
+  };
+  for (int q = 0; q < nb; ++q) bit[q * kLaneThreads] = 0u;
+  for (int i = 0; i < V; ++i) word[i * kLaneThreads] = 0xFFFFu;
+  bool bad = false;
+  const uint16_t* list_c = list + c;
+  constexpr int kBatch = 16;
+  for (int r0 = 0; r0 < V; r0 += kBatch) {
+    uint32_t i[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) i[u] = (uint32_t)list_c[(size_t)min(r0 + u, V - 1) * Ks];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const int r = r0 + u;
+      if (r < V) {
+        bad = bad || i[u] >= (uint32_t)V;
+        const uint32_t op = min(i[u], (uint32_t)(V - 1));
+        const uint32_t missing = head[op] >> 24;
+        bad = bad || word[op * kLaneThreads] != 0xFFFFu;   // twice (rank and count are never both 255: 255 missing need a 256th operator)
+        lst[r * kLaneThreads] = (uint8_t)op;
+        word[op * kLaneThreads] = (uint16_t)(missing << 8 | (uint32_t)r);
+        if (missing == 0u) add((uint32_t)r);
+      }
+    }
+  }
+  if (status) status[c] = bad ? (uint32_t)PE_STATUS_ORDER_INVALID : 0u;
+  if (bad) return;   // not a permutation: the order of this candidate stays unwritten
+
+  // Every iteration hands one successor of the operator placed last its "one predecessor fewer" and, once that
+  // operator's list is used up, places the next one: all lanes need the same number of either in total.
+  uint16_t* order_c = order + c;
+  uint32_t e = 0, e_end = 0;
+  int k = 0;
+  for (int it = 0; it < V + E + 2; ++it) {   // (bound: V placements, E successor steps)
+    if (e < e_end) {
+      const uint32_t s = succ[e++];
+      const uint32_t w = (uint32_t)word[s * kLaneThreads] - 0x100u;
+      word[s * kLaneThreads] = (uint16_t)w;
+      if ((w >> 8) == 0u) add(w & 0xFFu);
+    }
+    if (e == e_end) {
+      if (k == V) break;
+      if (some == 0u) break;   // (cannot happen for a permutation over a DAG)
+      const uint32_t q = (uint32_t)__ffs((int)some) - 1u;
+      const uint32_t x = bit[q * kLaneThreads];
+      const uint32_t r = 32u * q + (uint32_t)__ffs((int)x) - 1u;
+      bit[q * kLaneThreads] = x & (x - 1u);
+      if ((x & (x - 1u)) == 0u) some &= some - 1u;
+      const uint32_t i = lst[r * kLaneThreads];
+      *order_c = (uint16_t)i;
+      order_c += Ks;
+      ++k;
+      const uint32_t h = head[i];
+      e = h & 0xFFFFu;
+      e_end = e + ((h >> 16) & 0xFFu);
+    }
+  }
+}
+
 struct DecodePlan {
-  bool shared = false;      // pe_decode_warp_kernel
+  bool shared = false;      // per-operator state on chip
+  bool lane = false;        // pe_decode_lane_kernel, otherwise pe_decode_warp_kernel
   bool rec_smem = false;    // operator records in shared memory
   int threads = 0;
   uint32_t words = 0;       // shared words per warp
@@ -372,12 +467,28 @@ static bool plan_decode_warp(const pe_graph* g, int64_t K, DecodePlan* p) {
   return p->shared;
 }
 
+static bool plan_decode_lane(const pe_graph* g, int64_t K, DecodePlan* p) {
+  const size_t V = (size_t)g->V, E = (size_t)g->fview.E;
+  if (V > 256 || E > 65535 || !g->fview.short_lists) return false;
+  const size_t bytes = V * 4 + (V + 31) / 32 * kLaneThreads * 4 + V * kLaneThreads * 3 + (E + 3) / 4 * 4;
+  if (bytes > g->smem_optin) return false;
+  // A lane takes ~0.1 us a placement and ~0.3 us a successor however few candidates there are; the warp kernel places
+  // ~18000 operators a microsecond.  Measured (lane / warp, us): V = 64 K = 8192 46 / 39, K = 32768 48 / 129; V = 256
+  // K = 8192 179 / 132, K = 32768 187 / 449, K = 131072 757 / 1706; tiny pipeline (one successor an operator)
+  // K = 1024 25 / 18, K = 8192 25 / 38.
+  if (0.1 * (double)V + 0.3 * (double)E > 6.0 + (double)V * (double)K / 18000.0) return false;
+  p->shared = p->lane = true;
+  p->threads = kLaneThreads;
+  p->smem = bytes;
+  return true;
+}
+
 static bool decode_plan(const pe_graph* g, int64_t K, uint32_t flags, DecodePlan* p) {
   if (!g->fwd_ok) return false;
   const uint32_t want = flags & PE_VARIANT_MASK;
   const size_t V = (size_t)g->V, n0 = (V + 31) / 32, n1 = (n0 + 31) / 32;
   if (want == PE_VARIANT_AUTO || want == PE_VARIANT_SHARED) {
-    if (plan_decode_warp(g, K, p)) return true;
+    if (plan_decode_lane(g, K, p) || plan_decode_warp(g, K, p)) return true;
     if (want == PE_VARIANT_SHARED) return false;
   }
   if (want != PE_VARIANT_AUTO && want != PE_VARIANT_GLOBAL) return false;
@@ -424,7 +535,11 @@ extern "C" int pe_decode_priority(pe_graph* g, int64_t K, const void* list, int 
   const uint16_t* list16 = static_cast<const uint16_t*>(list);
   uint16_t* order16 = static_cast<uint16_t*>(order);
   int ret = PE_OK;
-  if (p.shared) {
+  if (p.lane) {
+    auto kern = pe::pe_decode_lane_kernel;
+    if (!pe::set_smem(kern, p.smem)) ret = PE_ERR_CUDA;
+    else kern<<<(unsigned)((K + p.threads - 1) / p.threads), p.threads, p.smem, stream>>>(g->fview, g->d_fwd, K, list16, order16, status);
+  } else if (p.shared) {
     const int64_t nw = p.threads / 32;
     auto kern = p.rec_smem ? pe::pe_decode_warp_kernel<true> : pe::pe_decode_warp_kernel<false>;
     if (!pe::set_smem(kern, p.smem)) ret = PE_ERR_CUDA;

@@ -10,6 +10,7 @@
 #include <map>
 #include <mutex>
 #include <utility>
+#include <algorithm>
 #include <climits>
 #include <cstdio>
 
@@ -393,26 +394,33 @@ static bool plan_global(const pe_graph* g, int64_t K, uint32_t flags, bool allow
   return true;
 }
 
-// Does a lane per candidate pay?  The tile kernel needs enough candidates per SM to make up for the latency of a
-// step (measured: 28 at V = 1536 / D = 32 take 2.6 ms against 3.3 ms of a warp per candidate; 20 of the MoE graph,
-// whose wide operators re-read the edge list, 6.2 ms against 2.1 ms of a block of warps per candidate; with exclusive
-// channels 20 at V = 1536 take 2.1 ms against 2.8 ms of the global-state kernel).
-static bool shared_pays(const pe_graph* g, const Plan& p) {
-  if (!p.tiled) return p.threads >= 48;
-  return p.tile_resident >= (p.exclusive ? 16 : (g->max_indeg > 3 ? 48 : 28));
+// Which of a lane (SHARED over the tile encoding), a block of warps (TEAM) and, for graphs that TEAM does not serve, a
+// warp per candidate is done first.  A lane takes ~0.1 us a position however few candidates there are, an SM holds
+// tile_resident of them; a block of warps takes ~0.026 us a position, and all SMs together evaluate `rate` positions a
+// microsecond, the fewer the deeper a window of 32 positions is (few operators per level of the graph, few machines) and
+// the more sources an operator has.  Measured (lane / team, us): V = 480 K = 1023 50 / 29, K = 3551 50 / 77; V = 1536
+// K = 1024 197 / 84, K = 65536 2554 / 3149; V = 1024 D = 8 K = 1000 105 / 49, K = 3000 92 / 107; V = 1024 D = 64
+// K = 524288 8578 / 10558; V = 1600 D = 64 K = 65536 2752 / 2030; V = 2116 D = 8 K = 65536 4186 / 3354; MoE graph
+// K = 16384 6200 / 2080.
+static double team_us(const pe_graph* g, int64_t K) {
+  const double V = g->V, width = V / g->levels;
+  const double rate = g->max_indeg > 3 ? 20000.0 : (width < 24.0 ? 32000.0 : (g->D < 32 ? 42000.0 : 51000.0));
+  return 10.0 + 0.026 * V + V * (double)K / rate;
+}
+static double lane_us(const pe_graph* g, int64_t K, const Plan& lane) {
+  const double V = g->V, rounds = (double)K / ((double)lane.tile_resident * g->sm_count);
+  return 8.0 + (g->max_indeg > 3 ? 0.15 : 0.103) * V * (rounds > 1.0 ? rounds : 1.0);
 }
 
-// Is a block of warps per candidate (TEAM) sooner done than a lane per candidate?  A lane takes ~0.1 us a position
-// however few candidates there are; a block of warps ~0.026 us a position, and an SM full of blocks ~4 us per 1000
-// candidate positions.  Measured (lane / team, us): V = 480 K = 1023 50 / 29, K = 3551 50 / 77; V = 1536 K = 64 191 / 64,
-// K = 1024 197 / 84, K = 2664 171 / 177; V = 1024 D = 8 K = 1000 105 / 49, K = 3000 92 / 107; V = 64 K = 1024 12 / 26.
-static bool team_sooner(const pe_graph* g, int64_t K, const Plan& lane) {
-  if (!lane.tiled) return false;
-  const double V = g->V, work = V * (double)K;
+// Exclusive channels: a lane per candidate (~0.3 us a position where the channel words leave few lanes per SM) or the
+// global-state kernel (latency ~2.4 us a position, ~4500 positions a microsecond).  Measured (lane / global, us):
+// V = 2304 D = 64 K = 32 641 / 5600, K = 16384 18045 / 11126; V = 4096 D = 8 K = 16384 16668 / 13345; V = 1536 D = 32
+// K = 16384 2049 / 2743; V = 400 D = 64 K = 8192 939 / 1348.
+static bool lane_pays_exclusive(const pe_graph* g, int64_t K, const Plan& lane) {
+  if (!lane.tiled) return lane.threads >= 48;
+  if (lane.tile_resident >= 16) return true;
   const double rounds = (double)K / ((double)lane.tile_resident * g->sm_count);
-  const double t_lane = 8.0 + 0.1 * V * (rounds > 1.0 ? rounds : 1.0);
-  const double t_team = 12.0 + 0.026 * V + work / 36000.0;
-  return t_team < t_lane;
+  return 0.3 * (rounds > 1.0 ? rounds : 1.0) < std::max(2.4, (double)K / 4500.0);
 }
 
 // allow_compact: the call can use the compact-graph kernels (u16 orders; start and finish both
@@ -425,7 +433,7 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
   if (g->hetero) {   // machine-dependent durations: the generic one-thread-per-candidate kernels
     if (want == PE_VARIANT_WARP || want == PE_VARIANT_TEAM) return PE_ERR_UNSUPPORTED;
     if (!(flags & PE_COMM_EXCLUSIVE) && want != PE_VARIANT_GLOBAL && plan_shared(g, K, allow_compact, p) &&
-        (shared_pays(g, *p) || want == PE_VARIANT_SHARED))
+        (p->tiled || p->threads >= 48 || want == PE_VARIANT_SHARED))
       return PE_OK;
     if (want == PE_VARIANT_SHARED) return PE_ERR_UNSUPPORTED;
     return plan_global(g, K, flags, false, p) ? PE_OK : PE_ERR_UNSUPPORTED;
@@ -434,7 +442,7 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
     // exclusive channels: the compact shared-state kernel where a block of candidates still fits with one
     // more word per machine pair each, else the generic global-state kernel
     if (want == PE_VARIANT_AUTO || want == PE_VARIANT_SHARED) {
-      if (plan_shared(g, K, allow_compact, p, true) && (shared_pays(g, *p) || want == PE_VARIANT_SHARED)) return PE_OK;
+      if (plan_shared(g, K, allow_compact, p, true) && (want == PE_VARIANT_SHARED || lane_pays_exclusive(g, K, *p))) return PE_OK;
       if (want == PE_VARIANT_SHARED) return PE_ERR_UNSUPPORTED;
       *p = Plan();
     }
@@ -443,28 +451,17 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
   }
   switch (want) {
     case PE_VARIANT_AUTO: {
-      // A lane per candidate with everything on chip wins while enough candidates fit in shared memory.  Beyond
-      // that the state of a candidate is too large: a warp per candidate (state still on chip) wins while at
-      // least four warps fit on an SM; for the largest graphs the global-state kernel, which is bound by random
-      // DRAM accesses but keeps thousands of candidates in flight, is faster.
       Plan w, gl, tm;
-      const bool has_s = plan_shared(g, K, allow_compact, p) && shared_pays(g, *p);
+      const bool has_s = plan_shared(g, K, allow_compact, p) && (p->tiled || p->threads >= 48);
       const bool has_t = plan_team(g, K, allow_compact, &tm);
-      // A batch so small that the lanes of the first round are not filled takes a lane's time over the whole order
-      // whatever its size; a block of warps per candidate is done sooner.
-      if (has_s && !(has_t && team_sooner(g, K, *p))) return PE_OK;
+      if (has_s && !p->tiled) return PE_OK;
+      if (has_s && (!has_t || lane_us(g, K, *p) <= team_us(g, K)) && (has_t || p->tile_resident >= 28)) return PE_OK;
+      if (has_t) { *p = tm; return PE_OK; }
       const bool has_w = plan_warp(g, K, flags, allow_compact, &w);
       const bool has_g = plan_global(g, K, flags, allow_compact, &gl);
-      // Once fewer than about twenty single-warp candidates fit on an SM, a block of warps per candidate
-      // is faster (measured at V = 4096: 3.6e10 against 2.6e10 operator-evaluations/s at D = 64, 2.7e10
-      // against 2.0e10 at D = 8; at V = 16384: 3.1e10 against 1.0e10 (warp) and 2.3e10 against 1.25e10
-      // (global); at V = 1024 the single-warp kernel still wins, 4.0e10 against 3.0e10).
-      // Graphs with operators of more than three incoming edges take the single-warp kernel off its register
-      // slots; there the block of warps wins as well (measured on the MoE graph: 1.7e10 against 0.9e10).
-      if (has_t && (has_s || !has_w || w.threads < 20 * 32 || (g->max_indeg > 3 && w.threads < 24 * 32))) {
-        *p = tm;
-        return PE_OK;
-      }
+      // Graphs that TEAM does not serve (operators with more than eight sources, 32-bit orders, one of the times only):
+      // a warp per candidate (state on chip) wins while at least four warps fit on an SM; for the largest graphs the
+      // global-state kernel, which is bound by random DRAM accesses but keeps thousands of candidates in flight.
       // With three warps per SM the two are close; the global-state kernel loses once it has to keep the
       // per-machine records in the workspace as well (measured at V = 16384: 1.25e10 against 0.84e10
       // operator-evaluations/s at D = 8, 0.93e10 against 1.01e10 at D = 64).

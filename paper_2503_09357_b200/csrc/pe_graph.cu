@@ -14,7 +14,7 @@ namespace {
 inline uint32_t align16(uint64_t x) { return (uint32_t)((x + 15u) & ~(uint64_t)15u); }
 
 // Ranges, acyclicity and overflow bounds; fills the bounds when asked.
-int check_desc(const pe_graph_desc* d, int64_t* time_bound, int64_t* mem_bound, int32_t* max_indeg) {
+int check_desc(const pe_graph_desc* d, int64_t* time_bound, int64_t* mem_bound, int32_t* max_indeg, int32_t* levels) {
   if (!d) return PE_ERR_INVALID_ARG;
   const int32_t V = d->num_ops, E = d->num_edges, D = d->num_devices, L = d->num_link_classes;
   if (V < 1 || E < 0 || D < 1 || D > 255 || L < 1 || L > 254) return PE_ERR_INVALID_ARG;
@@ -72,19 +72,24 @@ int check_desc(const pe_graph_desc* d, int64_t* time_bound, int64_t* mem_bound, 
   for (int32_t b = 0; b < E; ++b) succ[fill[d->edge_src[b]]++] = d->edge_dst[b];
   for (int32_t i = 0; i < V; ++i)
     if (deg[i] == 0) stack.push_back(i);
-  int32_t removed = 0;
+  std::vector<int32_t> level(V, 1);
+  int32_t removed = 0, deepest = 1;
   while (!stack.empty()) {
     const int32_t i = stack.back();
     stack.pop_back();
     ++removed;
-    for (int32_t q = succ_ptr[i]; q < succ_ptr[i + 1]; ++q)
+    if (level[i] > deepest) deepest = level[i];
+    for (int32_t q = succ_ptr[i]; q < succ_ptr[i + 1]; ++q) {
+      if (level[succ[q]] <= level[i]) level[succ[q]] = level[i] + 1;
       if (--deg[succ[q]] == 0) stack.push_back(succ[q]);
+    }
   }
   if (removed != V) return PE_ERR_CYCLE;
 
   if (time_bound) *time_bound = tsum;
   if (mem_bound) *mem_bound = msum;
   if (max_indeg) *max_indeg = mdeg;
+  if (levels) *levels = deepest;
   return PE_OK;
 }
 
@@ -95,14 +100,14 @@ std::vector<cudaEvent_t*> team_events(pe_graph* g) {
 
 }  // namespace
 
-extern "C" int pe_graph_validate(const pe_graph_desc* desc) { return check_desc(desc, nullptr, nullptr, nullptr); }
+extern "C" int pe_graph_validate(const pe_graph_desc* desc) { return check_desc(desc, nullptr, nullptr, nullptr, nullptr); }
 
 extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph** out) {
   if (!out) return PE_ERR_INVALID_ARG;
   *out = nullptr;
   int64_t tb = 0, mb = 0;
-  int32_t mdeg = 0;
-  const int rc = check_desc(d, &tb, &mb, &mdeg);
+  int32_t mdeg = 0, levels = 1;
+  const int rc = check_desc(d, &tb, &mb, &mdeg, &levels);
   if (rc != PE_OK) return rc;
   const int32_t V = d->num_ops, E = d->num_edges, D = d->num_devices, L = d->num_link_classes;
 
@@ -112,7 +117,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
   g->device = cuda_device;
   g->has_weight = d->mem_weight != nullptr;
   g->hetero = d->dur_by_machine != nullptr;
-  g->time_bound = tb; g->mem_bound = mb; g->max_indeg = mdeg;
+  g->time_bound = tb; g->mem_bound = mb; g->max_indeg = mdeg; g->levels = levels;
   g->d_blob = nullptr; g->d_error = nullptr;
 
   PeBlobLayout& lay = g->lay;
@@ -300,6 +305,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
     std::vector<uint16_t> usucc, more;
     usucc.reserve(E);
     int32_t seven = 0;
+    fv.short_lists = 1;
     for (int32_t i = 0; i < V; ++i) {
       std::sort(succ.begin() + sptr[i], succ.begin() + sptr[i + 1]);
       const auto end = std::unique(succ.begin() + sptr[i], succ.begin() + sptr[i + 1]);
@@ -307,6 +313,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
       uptr[i + 1] = (uint32_t)usucc.size();
       const uint32_t n = uptr[i + 1] - uptr[i];
       seven += n > 6 && n <= 14;
+      if (n > 255) fv.short_lists = 0;
     }
     fv.rec_bytes = seven > V / 50 ? 32 : 16;
     const uint32_t halves = fv.rec_bytes / 2, inl = halves - 2;

@@ -103,6 +103,7 @@ struct PeFwdView {
   uint32_t rec;    // uint16[V][rec_bytes / 2]
   uint32_t rec_bytes;   // 16, or 32 where a fiftieth of the operators has 7 to 14 successors
   uint32_t more;   // uint16[]
+  int32_t short_lists;  // no operator has more than 255 successors
 };
 
 struct pe_graph {
@@ -113,6 +114,7 @@ struct pe_graph {
   int64_t time_bound;  // sum dur + sum_e max_l comm: no start/end time exceeds it
   int64_t mem_bound;   // sum |A| + sum W
   int32_t max_indeg;
+  int32_t levels;      // operators on the longest path
   PeBlobLayout lay;
   uint8_t* d_blob;     // device copy of the blob; one allocation that also holds the encodings below and d_error
   bool narrow_ok;      // the compact encoding exists
