@@ -3,6 +3,7 @@
 #include <climits>
 
 #include "pe.h"
+#include "pe_launch.h"
 #include <cuda_runtime.h>
 
 namespace pe {
@@ -59,6 +60,46 @@ __global__ void __launch_bounds__(256) pe_select_kernel(int64_t K, const int32_t
   }
 }
 
+constexpr int64_t kOneBlock = 32768;   // batches up to this size are handled by one block: no state to set up, one launch
+
+__global__ void __launch_bounds__(1024) pe_select_one_kernel(int K, const int32_t* __restrict__ makespan,
+                                                             const uint32_t* __restrict__ status, uint32_t reject_mask,
+                                                             int64_t* result) {
+  unsigned long long best = kNoKey;
+  unsigned int count = 0;
+#pragma unroll 8
+  for (int c = threadIdx.x; c < K; c += 1024) {
+    const uint32_t s = status[c];
+    const int32_t m = makespan[c];
+    if ((s & reject_mask) == 0) {
+      ++count;
+      const unsigned long long key = ((unsigned long long)(unsigned)m << 32) | (unsigned long long)c;
+      best = key < best ? key : best;
+    }
+  }
+  __shared__ unsigned long long s_best[32];
+  __shared__ unsigned int s_count[32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int round = 0; round < 2; ++round) {
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, best, off);
+      best = o < best ? o : best;
+    }
+    count = __reduce_add_sync(0xFFFFFFFFu, count);
+    if (round == 1 || warp >= 32) break;
+    if (lane == 0) { s_best[warp] = best; s_count[warp] = count; }
+    __syncthreads();
+    best = s_best[lane];
+    count = s_count[lane];
+  }
+  if (threadIdx.x == 0) {
+    result[0] = best == kNoKey ? -1 : (int64_t)(best & 0xFFFFFFFFull);
+    result[1] = best == kNoKey ? (int64_t)INT32_MAX : (int64_t)(best >> 32);
+    result[2] = (int64_t)count;
+    result[3] = 0;
+  }
+}
+
 }  // namespace pe
 
 extern "C" int pe_select_best(int64_t K, const int32_t* makespan, const uint32_t* status, uint32_t reject_mask,
@@ -77,11 +118,14 @@ extern "C" int pe_select_best(int64_t K, const int32_t* makespan, const uint32_t
   if (prev != attr.device && cudaSetDevice(attr.device) != cudaSuccess) return PE_ERR_CUDA;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   unsigned long long* scratch = reinterpret_cast<unsigned long long*>(result);
-  pe::pe_select_init_kernel<<<1, 1, 0, stream>>>(scratch);
-  int blocks = (int)((K + 255) / 256);
-  if (blocks > 1184) blocks = 1184;  // 148 SMs x 8 resident blocks: a grid-stride loop covers the rest
-  if (blocks < 1) blocks = 1;
-  pe::pe_select_kernel<<<blocks, 256, 0, stream>>>(K, makespan, status, reject_mask, scratch);
+  if (K <= pe::kOneBlock) {
+    pe::pe_select_one_kernel<<<1, 1024, 0, stream>>>((int)K, makespan, status, reject_mask, result);
+  } else {
+    pe::pe_select_init_kernel<<<1, 1, 0, stream>>>(scratch);
+    const int64_t want = (K + 255) / 256;
+    const int blocks = (int)(want < 1184 ? want : 1184);  // 148 SMs x 8 resident blocks: a grid-stride loop covers the rest
+    pe::pe_select_kernel<<<blocks, 256, 0, stream>>>(K, makespan, status, reject_mask, scratch);
+  }
   const int ret = cudaGetLastError() == cudaSuccess ? PE_OK : PE_ERR_CUDA;
   if (prev != attr.device) cudaSetDevice(prev);
   return ret;
@@ -296,6 +340,104 @@ __global__ void pe_topk_fill_kernel(int32_t* out_index, int32_t k) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < k; i += gridDim.x * blockDim.x) out_index[i] = -1;
 }
 
+// The whole selection in one block, for batches whose keys fit in shared memory.  Bound by the latency of a few block
+// barriers (a launch of its own per step, eleven in all, cost ~2 us each).  The histogram covers the range the values
+// have, not 32 bits: most batches need one or two rounds, and neighbouring values do not meet in one bin.
+__global__ void __launch_bounds__(1024) pe_topk_one_kernel(int K, const int32_t* __restrict__ makespan,
+                                                           const uint32_t* __restrict__ status, uint32_t reject_mask, int32_t k,
+                                                           int32_t* __restrict__ out_index, int32_t* __restrict__ out_count) {
+  extern __shared__ unsigned int keys[];   // makespan, or kNone where the candidate does not qualify
+  constexpr unsigned int kNone = 0xFFFFFFFFu, FULL = 0xFFFFFFFFu;
+  __shared__ unsigned int hist[kTopkBins];
+  __shared__ unsigned int wa[32], wb[32], wc[32];
+  __shared__ unsigned int sh_bin, sh_below;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  unsigned int lo = kNone, hi = 0, n = 0;
+#pragma unroll 8
+  for (int c = t; c < K; c += 1024) {
+    const unsigned int m = (unsigned int)makespan[c];
+    const unsigned int v = (status[c] & reject_mask) == 0 ? m : kNone;
+    keys[c] = v;
+    if (v != kNone) { lo = min(lo, v); hi = max(hi, v); ++n; }
+  }
+  lo = __reduce_min_sync(FULL, lo); hi = __reduce_max_sync(FULL, hi); n = __reduce_add_sync(FULL, n);
+  if (lane == 0) { wa[warp] = lo; wb[warp] = hi; wc[warp] = n; }
+  __syncthreads();
+  lo = __reduce_min_sync(FULL, wa[lane]); hi = __reduce_max_sync(FULL, wb[lane]); n = __reduce_add_sync(FULL, wc[lane]);
+  // T: the k-th smallest key; everything qualifying is better than it when at most k qualify
+  unsigned int T = kNone, take_equal = 0;
+  if (k > 0 && n > (unsigned int)k) {
+    unsigned int base = lo, rem = (unsigned int)k;
+    int bits = 32 - __clz((int)(hi - lo));
+    while (true) {   // (each round fixes up to 11 bits: at most three)
+      const int shift = bits > 11 ? bits - 11 : 0;
+      __syncthreads();
+      hist[t] = 0; hist[t + 1024] = 0;
+      __syncthreads();
+      const unsigned int range = bits >= 32 ? kNone : (1u << bits) - 1u;
+      for (int c = t; c < K; c += 1024) {
+        const unsigned int d = keys[c] - base;
+        if (keys[c] != kNone && keys[c] >= base && d <= range) atomicAdd(&hist[d >> shift], 1u);
+      }
+      __syncthreads();
+      const unsigned int h0 = hist[2 * t], h1 = hist[2 * t + 1];
+      unsigned int incl = h0 + h1;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const unsigned int o = __shfl_up_sync(FULL, incl, off);
+        incl += lane >= off ? o : 0u;
+      }
+      if (lane == 31) wa[warp] = incl;
+      __syncthreads();
+      incl += __reduce_add_sync(FULL, lane < warp ? wa[lane] : 0u);
+      const unsigned int excl = incl - h0 - h1;
+      if (excl < rem && incl >= rem) {   // exactly one thread: the bin that holds the rem-th smallest
+        const bool first = excl + h0 >= rem;
+        sh_bin = 2u * (unsigned int)t + (first ? 0u : 1u);
+        sh_below = first ? excl : excl + h0;
+      }
+      __syncthreads();
+      base += sh_bin << shift;
+      rem -= sh_below;
+      if (shift == 0) break;
+      bits = shift;
+    }
+    T = base;
+    take_equal = rem;
+  }
+  // ordered compaction: thread t owns consecutive candidates
+  __syncthreads();
+  const int per = ((K + 1023) / 1024) | 1;   // (odd: a warp's threads read different banks)
+  const int c0 = min(t * per, K), c1 = min(c0 + per, K);
+  unsigned int nb = 0, ne = 0;
+  for (int c = c0; c < c1; ++c) { nb += keys[c] < T; ne += keys[c] == T && T != kNone; }
+  unsigned int ib = nb, ie = ne;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const unsigned int ob = __shfl_up_sync(FULL, ib, off), oe = __shfl_up_sync(FULL, ie, off);
+    ib += lane >= off ? ob : 0u;
+    ie += lane >= off ? oe : 0u;
+  }
+  if (lane == 31) { wb[warp] = ib; wc[warp] = ie; }
+  __syncthreads();
+  const unsigned int xb = lane < 32 ? wb[lane] : 0u, xe = wc[lane];
+  const unsigned int all = min((unsigned int)k, __reduce_add_sync(FULL, xb) + min(__reduce_add_sync(FULL, xe), take_equal));
+  unsigned int before_b = ib - nb + __reduce_add_sync(FULL, lane < warp ? xb : 0u);
+  unsigned int before_e = ie - ne + __reduce_add_sync(FULL, lane < warp ? xe : 0u);
+  if (nb + ne)
+    for (int c = c0; c < c1; ++c) {
+      const bool better = keys[c] < T, equal = keys[c] == T && T != kNone;
+      if (better || (equal && before_e < take_equal)) {
+        const unsigned int at = before_b + min(before_e, take_equal);
+        if (at < (unsigned int)k) out_index[at] = c;
+      }
+      before_b += better;
+      before_e += equal;
+    }
+  for (int i = (int)all + t; i < k; i += 1024) out_index[i] = -1;
+  if (t == 0) *out_count = (int32_t)all;
+}
+
 static size_t topk_blocks(int64_t K) { return (size_t)((K + kTopkPerBlock - 1) / kTopkPerBlock); }
 
 }  // namespace pe
@@ -329,6 +471,15 @@ extern "C" int pe_select_topk(int64_t K, const int32_t* makespan, const uint32_t
   int grid = (int)((K + pe::kTopkBlock - 1) / pe::kTopkBlock);
   if (grid > 1184) grid = 1184;
   if (grid < 1) grid = 1;
+  if (K <= pe::kOneBlock) {
+    int ret = PE_OK;
+    const size_t bytes = sizeof(unsigned int) * (size_t)(K > 0 ? K : 1);
+    if (!pe::set_smem(pe::pe_topk_one_kernel, bytes)) ret = PE_ERR_CUDA;
+    else pe::pe_topk_one_kernel<<<1, 1024, bytes, stream>>>((int)K, makespan, status, reject_mask, k, out_index, out_count);
+    if (cudaGetLastError() != cudaSuccess) ret = PE_ERR_CUDA;
+    if (prev != attr.device) cudaSetDevice(prev);
+    return ret;
+  }
   if (k > 0) pe::pe_topk_fill_kernel<<<(k + 255) / 256 > 256 ? 256 : (k + 255) / 256, 256, 0, stream>>>(out_index, k);
   pe::pe_topk_init_kernel<<<1, 256, 0, stream>>>(st, hist, (unsigned int)k);
   const int shifts[3] = {21, 10, 0}, bits[3] = {11, 11, 10};
@@ -337,13 +488,11 @@ extern "C" int pe_select_topk(int64_t K, const int32_t* makespan, const uint32_t
                                                                  bits[p], p == 0);
     pe::pe_topk_pick_kernel<<<1, pe::kTopkBlock, 0, stream>>>(st, hist, shifts[p], bits[p], p == 0, p == 2);
   }
-  if (nblocks > 0) {
+  {
     pe::pe_topk_count_kernel<<<nblocks, pe::kTopkBlock, 0, stream>>>(K, makespan, status, reject_mask, st, blk);
     pe::pe_topk_scan_kernel<<<1, pe::kTopkBlock, 0, stream>>>(blk, nblocks);
     pe::pe_topk_write_kernel<<<nblocks, pe::kTopkBlock, 0, stream>>>(K, makespan, status, reject_mask, st, blk, k,
                                                                       out_index, out_count);
-  } else {
-    cudaMemsetAsync(out_count, 0, sizeof(int32_t), stream);
   }
   const int ret = cudaGetLastError() == cudaSuccess ? PE_OK : PE_ERR_CUDA;
   if (prev != attr.device) cudaSetDevice(prev);
