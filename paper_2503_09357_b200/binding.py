@@ -256,6 +256,12 @@ def pe_kernel_launches() -> int:
     return int(_lib.pe_kernel_launches())
 
 
+def _raw_stream(device):
+    """Handle of torch's current stream on a device (an int; without building a Stream object)."""
+    import torch
+    return torch._C._cuda_getCurrentRawStream(device)
+
+
 class Graph:
     """Owner of a pe_graph handle with torch-tensor conveniences (allocation and pointers only)."""
 
@@ -264,6 +270,21 @@ class Graph:
         self.V, self.D = int(workload.num_ops), int(workload.num_devices)
         self.device = int(device)
         self.handle = pe_graph_create(desc, device)
+        self._bytes = {}                      # workspace sizes by (call, K, flags)
+
+    def _workspace(self, call, K, flags):
+        """A workspace for one call: (tensor or None, pointer, bytes)."""
+        n = self._bytes.get((call, K, flags))
+        if n is None:
+            n = pe_workspace_bytes(self.handle, K, flags) if call == "eval" else pe_decode_workspace_bytes(self.handle, K, flags)
+            if len(self._bytes) >= 256:
+                self._bytes.clear()
+            self._bytes[(call, K, flags)] = n
+        if n == 0:
+            return None, 0, 0
+        import torch
+        ws = torch.empty(n, dtype=torch.uint8, device=f"cuda:{self.device}")
+        return ws, ws.data_ptr(), n
 
     def close(self):
         if getattr(self, "handle", None):
@@ -303,7 +324,7 @@ class Graph:
         """Index, makespan and count of the best qualifying candidate of an eval_batch result (host ints)."""
         import torch
         res = torch.empty(4, dtype=torch.int64, device=out["makespan"].device)
-        s = torch.cuda.current_stream(self.device).cuda_stream if stream is None else stream
+        s = _raw_stream(self.device) if stream is None else stream
         rc = pe_select_best(out["makespan"].numel(), out["makespan"].data_ptr(), out["status"].data_ptr(), reject_mask,
                             res.data_ptr(), s)
         if rc != PE_OK:
@@ -321,7 +342,7 @@ class Graph:
         cnt = torch.empty(1, dtype=torch.int32, device=dev)
         n = pe_select_topk_workspace_bytes(K)
         ws = torch.empty(n, dtype=torch.uint8, device=dev)
-        s = torch.cuda.current_stream(self.device).cuda_stream if stream is None else stream
+        s = _raw_stream(self.device) if stream is None else stream
         rc = pe_select_topk(K, out["makespan"].data_ptr(), out["status"].data_ptr(), reject_mask, k, idx.data_ptr(),
                             cnt.data_ptr(), ws.data_ptr(), n, s)
         if rc != PE_OK:
@@ -340,14 +361,13 @@ class Graph:
         dev = torch.device("cuda", self.device)
         order = torch.empty_like(plist)
         status = torch.empty(K, dtype=torch.int32, device=dev)
-        n = pe_decode_workspace_bytes(self.handle, K, flags)
-        ws = torch.empty(max(n, 256), dtype=torch.uint8, device=dev)
-        s = torch.cuda.current_stream(self.device).cuda_stream if stream is None else stream
+        ws, ws_ptr, n = self._workspace("decode", K, flags)
+        s = _raw_stream(self.device) if stream is None else stream
         rc = pe_decode_priority(self.handle, K, plist.data_ptr(), 2, flags, order.data_ptr(), status.data_ptr(),
-                                ws.data_ptr(), n, s)
+                                ws_ptr, n, s)
         if rc != PE_OK:
             raise PeError(rc, "pe_decode_priority")
-        if stream is not None:        # the workspace dies here: keep the allocator from reusing it under the kernel
+        if stream is not None and ws is not None:        # the workspace dies here: keep the allocator from reusing it under the kernel
             ws.record_stream(torch.cuda.ExternalStream(stream, device=dev))
         return order, status
 
@@ -361,14 +381,16 @@ class Graph:
         if out is None:
             out = self.alloc_outputs(K, want_times)
         if workspace is None:
-            workspace = self.alloc_workspace(K, flags)
-        ws, ws_bytes = workspace
+            ws, ws_ptr, ws_bytes = self._workspace("eval", K, flags)
+        else:
+            ws, ws_bytes = workspace
+            ws_ptr = ws.data_ptr()
         o = make_outputs(**{k: v.data_ptr() for k, v in out.items()})
-        s = torch.cuda.current_stream(self.device).cuda_stream if stream is None else stream
+        s = _raw_stream(self.device) if stream is None else stream
         rc = pe_eval_batch(self.handle, K, assign.data_ptr(), order.data_ptr(), order.element_size(), flags, o,
-                           ws.data_ptr(), ws_bytes, s)
+                           ws_ptr, ws_bytes, s)
         if rc != PE_OK:
             raise PeError(rc, "pe_eval_batch")
-        if stream is not None:        # a workspace allocated here dies here: keep the allocator from reusing it
+        if stream is not None and ws is not None:        # a workspace allocated here dies here: keep the allocator from reusing it
             ws.record_stream(torch.cuda.ExternalStream(stream, device=torch.device("cuda", self.device)))
         return out
