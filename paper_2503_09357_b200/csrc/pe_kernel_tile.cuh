@@ -20,9 +20,10 @@
 //     own word scheduled; an entry that is no operator is clamped to the sentinel row V, which counts as
 //     scheduled.
 // Measured on B200 (before: the thread-per-candidate kernel this one replaces, 92 instructions and ~370 cycles a
-// step at V = 256; now 69 and ~240): V = 256 / D = 8, K = 2^20: 1.85 -> 1.25 ms; bidirectional pipeline (V = 480),
-// K = 65536: 352 -> 166 us, with durations by machine, K = 16384: 490 -> 137 us (generic kernel before); multi-modal
-// graph with exclusive channels, K = 16384: 2.74 -> 2.09 ms (global-state kernel before).
+// step at V = 256; now 68 and ~230): V = 256 / D = 8, K = 2^20: 1.85 -> 1.19 ms; bidirectional pipeline (V = 480),
+// K = 65536: 352 -> 166 us, with durations by machine, K = 16384: 490 -> 113 us (generic kernel before); multi-modal
+// graph K = 65536: 3.34 -> 2.42 ms (warp per candidate), with exclusive channels, K = 16384: 2.74 -> 1.75 ms
+// (global-state kernel before).
 //
 // State word: uint32_t time << 8 | machine, or uint16_t time << jb | machine when the graph's time bound
 // and machine count fit 16 bits (two warps then share the 32-bit words of a row, one the low and one the
@@ -79,6 +80,17 @@ __device__ __forceinline__ uint32_t lds8(uint32_t a) {
   asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
   return v;
 }
+// Order entries and by-position machine ids: volatile, so that a block's requests stay in front of its steps.
+__device__ __forceinline__ uint32_t ldg_u16(const void* p) {
+  uint16_t v;
+  asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t ldg_u8(const void* p) {
+  uint32_t v;
+  asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -98,7 +110,7 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
   constexpr uint32_t FULL = 0xFFFFFFFFu;
   constexpr bool S16 = MODE == kTileS16, EXCL = MODE == kTileExcl, HET = MODE == kTileHet;
   using StateT = typename std::conditional<S16, uint16_t, uint32_t>::type;
-  constexpr int kRing = BY_POS ? 8 : 16;   // order entries (and by-position machine ids) per request
+  constexpr int kRing = BY_POS || EXCL || HET ? 8 : 16;   // order entries (and by-position machine ids) per request
   constexpr int NIN = CLS == 0 ? (EDGES == 2 ? 2 : 3) : 2;   // edges that the record carries inline
   const int V = g.V, D = g.D;
   const int lane = threadIdx.x & 31;
@@ -278,7 +290,7 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
 
     // ---- main loop ----
     uint32_t st = 0;
-    uint32_t z = 0, own_min = 0xFFFFFFFFu, dev_max = 0;
+    uint32_t own_min = 0xFFFFFFFFu, dev_max = 0;
     uint8_t* start_b = reinterpret_cast<uint8_t*>(out.start) + (size_t)cc * 4;     // this position's row
     uint8_t* finish_b = reinterpret_cast<uint8_t*>(out.finish) + (size_t)cc * 4;
 
@@ -388,7 +400,6 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
       const uint32_t bz = HET ? dv.y + dur_het : __dp2a_lo(r4.x, 1u, dv.y);                     // + D^o_i (low half)
       sts_state<S16>(st_a + i * pitch, e);
       sts128(dv_a + j * dpitch, make_uint4(e, bz, (uint32_t)lv, (uint32_t)max((int32_t)dv.w, lv)));
-      z = max(z, e);
       if (TIMES) {
         if (TIMES == 1) {
           *reinterpret_cast<int32_t*>(start_b) = (int32_t)(rt >> jb);
@@ -414,7 +425,10 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
     // The next block's order entries are requested together at the start of a block: a wait for one load waits
     // for every load that shares its scoreboard (a warp has six), so loads spread over the steps would be waited
     // for a step or two after they were issued.  Measured at V = 256, D = 8 (K = 2^20): entries requested one a
-    // step 1583 us, blocks of 16 1242 us, two alternating register sets of 8 1558 us.
+    // step 1583 us, blocks of 16 1242 us, two alternating register sets of 8 1558 us; entries brought to a shared ring by asynchronous
+    // copies 1517 us (11 more instructions a step).  With exclusive channels or durations by machine the step is so
+    // long that sixteen of them unrolled overflow the instruction cache: blocks of 8 (238 -> 185 us and 138 -> 113 us on
+    // the bidirectional pipeline, K = 16384).
     for (int kb = 0; kb < V; kb += kRing) {
       ord_b += (size_t)kRing * K2;
       asg_b += (size_t)kRing * K1;
@@ -422,15 +436,15 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
       if (kb + 2 * kRing <= V) {
 #pragma unroll
         for (int u = 0; u < kRing; ++u) {
-          nxt[u] = *reinterpret_cast<const uint16_t*>(ord_b + (size_t)u * K2);
-          anxt[u] = BY_POS ? (uint32_t)asg_b[(size_t)u * K1] : 0u;
+          nxt[u] = ldg_u16(ord_b + (size_t)u * K2);
+          anxt[u] = BY_POS ? ldg_u8(asg_b + (size_t)u * K1) : 0u;
         }
       } else {   // rows that do not exist are not read
 #pragma unroll
         for (int u = 0; u < kRing; ++u) {
           const bool have = kb + kRing + u < V;
-          nxt[u] = have ? (uint32_t)*reinterpret_cast<const uint16_t*>(ord_b + (size_t)u * K2) : 0u;
-          anxt[u] = BY_POS && have ? (uint32_t)asg_b[(size_t)u * K1] : 0u;
+          nxt[u] = have ? ldg_u16(ord_b + (size_t)u * K2) : 0u;
+          anxt[u] = BY_POS && have ? ldg_u8(asg_b + (size_t)u * K1) : 0u;
         }
       }
       if (kb + kRing <= V) {
@@ -452,6 +466,10 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
 
     // ---- results of the tile ----
     if (own_min < unsched) st |= PE_STATUS_ORDER_INVALID;   // an operator twice, or an entry that is no operator
+    // a machine's end times rise: the largest last one is the makespan (formed here, not in the loop below: 1185 against
+    // 1248 us at V = 256, D = 8)
+    uint32_t z = 0;
+    for (int j = 0; j < D; ++j) z = max(z, (uint32_t)dev((uint32_t)j).x);
     if (z >= unsched) st |= PE_STATUS_ORDER_INVALID;        // an operator ahead of one of its predecessors
     if (BY_POS) {
       if (dev_max > dmax) st |= PE_STATUS_ASSIGN_RANGE;
