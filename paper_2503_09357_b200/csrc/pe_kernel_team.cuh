@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
   constexpr bool NEED_CLS = CLS != 0;
   constexpr int NT = NW * 32;
   constexpr bool IMMBAR = NW < 6;   // six warps per block go with large states, where few blocks fit anyway
-  constexpr int32_t kNever = -(1 << 29);   // delay of an empty slot: never wins the maximum
+  constexpr int32_t kNever = -(1 << 25);   // delay of an empty slot: never wins the maximum (times stay below 2^23)
   const int tid = threadIdx.x;
   const int lane = tid & 31;
   const int warp = tid >> 5;
@@ -272,17 +272,20 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
     const bool has_prev = below != 0;
     const bool last_on_dev = (same_dev >> lane) == 1u;
 
-    // Incoming edges: edge q owns slot q.  A source inside the window becomes (lane, delay) for the
-    // relaxation; any other becomes (state address, delay) for the gather under the baton.  The unused
-    // half of a slot is neutral: lane = own lane with delay kNever, address = sentinel with delay kNever.
+    // Incoming edges.  With six warps (where the serial part limits) a source that is final already contributes its end
+    // time to r_pre at once and stays out of the gather under the baton, whose lanes then meet in one word; with fewer
+    // warps issue limits and the extra instructions cost 3 % at V = 4096.  A source inside the window becomes a slot
+    // word (delay << 5 | lane) for the relaxation; any other becomes (state address, delay) for the gather under the
+    // baton.  What a lane does not use is neutral: slot word kNever << 5 | own lane, address = sentinel with delay kNever.
     // `rel` is the source's position relative to the window when its word is pending; a final word
     // (bit 31 clear) wraps to a huge value, so one unsigned compare tells "inside the window, before me".
     const uint32_t pend_base = (kTeamPending >> 8) + (uint32_t)base;
+    const int32_t empty = (int32_t)((uint32_t)(kNever << 5) | (uint32_t)lane);
     uint32_t depmask = 0;
     uint32_t a0, a1, a2;
-    int32_t g0, g1, g2, d0, d1, d2;
-    int l0, l1, l2;
-    auto classify = [&](uint32_t lo, uint32_t hi, uint32_t& addr, int32_t& gdel, int& lsl, int32_t& ldel) {
+    int32_t g0, g1, g2, x0, x1, x2, x3;
+    int32_t r_pre = 0;
+    auto classify = [&](uint32_t lo, uint32_t hi, uint32_t& addr, int32_t& gdel, int32_t& x) {
       const uint32_t p = lo & 0xFFFFu;
       const uint32_t w = state[p];
       const uint32_t xp = w & 0xFFu;
@@ -297,12 +300,13 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
       }
       const int32_t dly = xp != j ? (int32_t)delay : 0;
       const uint32_t rel = (w >> 8) - pend_base;
-      const bool inw = rel < (uint32_t)lane;
+      const bool inw = rel < (uint32_t)lane, final = NW == 6 && !WIDE && (int32_t)w >= 0;   // (otherwise the gather sees to it)
       if (!inw && rel < 0x10000u) st |= PE_STATUS_ORDER_INVALID;   // pending, but not before this operator
-      addr = inw ? none : p;
-      gdel = inw ? kNever : dly;
-      lsl = inw ? (int)rel : lane;
-      ldel = (inw ? dly : kNever) + dur;   // D^o folded into the in-window delays (Eq. 3)
+      if (final) r_pre = __viaddmax_s32((int32_t)(w >> 8), dly, r_pre);
+      const bool later = !inw && !final;
+      addr = later ? p : none;
+      gdel = later ? dly : kNever;
+      x = inw ? (int32_t)((uint32_t)dly << 5 | rel) : empty;
       depmask |= inw ? 1u << rel : 0u;
     };
     // (a lane beyond the end of the order goes through the same code on operator 0's record; what it
@@ -311,44 +315,62 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
     // WIDE: operators with four to eight incoming edges; edges 3.. take the extra slots
     constexpr int kExtra = WIDE ? 5 : 1;
     uint32_t xa[kExtra];
-    int32_t xg[kExtra], xd[kExtra];
-    int xl[kExtra];
+    int32_t xg[kExtra], xx[kExtra];
 #pragma unroll
-    for (int q = 0; q < kExtra; ++q) { xa[q] = none; xg[q] = kNever; xl[q] = lane; xd[q] = kNever + dur; }
-    classify(rec.z, rec.w, a0, g0, l0, d0);
+    for (int q = 0; q < kExtra; ++q) { xa[q] = none; xg[q] = kNever; xx[q] = empty; }
+    classify(rec.z, rec.w, a0, g0, x0);
     if (TWO_CLASS) {
-      a1 = none; a2 = none; g1 = kNever; g2 = kNever; l1 = lane; l2 = lane; d1 = kNever + dur; d2 = kNever + dur;
+      a1 = none; a2 = none; g1 = kNever; g2 = kNever; x1 = empty; x2 = empty;
       const uint2* ed = reinterpret_cast<const uint2*>(gp.edges) + rec.x;
-      if (indeg > 1) { const uint2 e1 = __ldg(ed + 1); classify(e1.x, e1.y, a1, g1, l1, d1); }
-      if (indeg > 2) { const uint2 e2 = __ldg(ed + 2); classify(e2.x, e2.y, a2, g2, l2, d2); }
+      if (indeg > 1) { const uint2 e1 = __ldg(ed + 1); classify(e1.x, e1.y, a1, g1, x1); }
+      if (indeg > 2) { const uint2 e2 = __ldg(ed + 2); classify(e2.x, e2.y, a2, g2, x2); }
       if constexpr (WIDE) {
 #pragma unroll
         for (int q = 0; q < kExtra; ++q)
-          if (indeg > 3 + q) { const uint2 eq = __ldg(ed + 3 + q); classify(eq.x, eq.y, xa[q], xg[q], xl[q], xd[q]); }
+          if (indeg > 3 + q) { const uint2 eq = __ldg(ed + 3 + q); classify(eq.x, eq.y, xa[q], xg[q], xx[q]); }
       }
     } else {
-      classify(rec.w, 0u, a1, g1, l1, d1);
+      classify(rec.w, 0u, a1, g1, x1);
       if constexpr (WIDE) {
         // with more than three incoming edges the record's first word is the edge list's slot, not edge 2
         const uint32_t* ed = gp.edges + rec.x;
         const bool many = indeg > 3;
-        classify(many ? __ldg(ed + 2) : rec.x, 0u, a2, g2, l2, d2);
+        classify(many ? __ldg(ed + 2) : rec.x, 0u, a2, g2, x2);
 #pragma unroll
         for (int q = 0; q < kExtra; ++q)
-          if (indeg > 3 + q) classify(__ldg(ed + 3 + q), 0u, xa[q], xg[q], xl[q], xd[q]);
+          if (indeg > 3 + q) classify(__ldg(ed + 3 + q), 0u, xa[q], xg[q], xx[q]);
       } else {
-        classify(rec.x, 0u, a2, g2, l2, d2);
+        classify(rec.x, 0u, a2, g2, x2);
       }
     }
     if (!act) {
-      st = st_before; depmask = 0; a0 = a1 = a2 = none;
+      st = st_before; depmask = 0; r_pre = 0; a0 = a1 = a2 = none; x0 = x1 = x2 = empty;
 #pragma unroll
-      for (int q = 0; q < kExtra; ++q) xa[q] = none;
+      for (int q = 0; q < kExtra; ++q) { xa[q] = none; xx[q] = empty; }
     }
     const int prev = 31 - __clz(below);
-    const int lp = has_prev ? prev : lane;
-    const int32_t dp = (has_prev ? 0 : kNever) + dur;
+    x3 = has_prev ? prev : empty;   // after the machine's previous operator, no delay
     depmask |= has_prev ? 1u << prev : 0u;
+    // Used slot words to the front, so that the loop under the baton can leave out what no lane uses: most windows need
+    // two or three shuffles a round, not four.  Measured: V = 16384 / D = 8
+    // K = 16384 10.4 -> 9.5 ms, multi-modal graph K = 1024 84 -> 76 us; V = 4096 / D = 64, where issue limits, +1.6 %.
+    int nslots = 4;
+    if constexpr (!WIDE) {
+      const bool u0 = x0 != empty, u1 = x1 != empty, u2 = x2 != empty;
+      int32_t t;
+      t = u0 ? x1 : empty; x0 = u0 ? x0 : x1; x1 = t;                                     // (x0, x1) in order
+      const bool v1 = u0 && u1, v0 = u0 || u1;
+      t = v1 ? x2 : empty; { const int32_t y1 = v1 ? x1 : (v0 ? x2 : empty); x0 = v0 ? x0 : x2; x1 = y1; x2 = t; }
+      const int used = (int)u0 + (int)u1 + (int)u2;
+      t = used == 3 ? x3 : empty;
+      x2 = used == 2 ? x3 : x2;
+      x1 = used == 1 ? x3 : x1;
+      x0 = used == 0 ? x3 : x0;
+      x3 = t;
+      nslots = __any_sync(FULL, x2 != empty) ? (__any_sync(FULL, x3 != empty) ? 4 : 3) : 2;
+    }
+    // (the shuffles use the low five bits of a slot word; D^o is folded into the in-window delays, Eq. 3)
+    const int32_t d0 = (x0 >> 5) + dur, d1 = (x1 >> 5) + dur, d2 = (x2 >> 5) + dur, d3 = (x3 >> 5) + dur;
     // Depth of the window: peel off, round by round, the lanes whose sources are all peeled.  After n
     // rounds of relaxation every lane of depth <= n holds its final value, so the number of rounds is
     // known before the baton arrives and the loop under it needs no vote.
@@ -360,7 +382,6 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
         ++nrounds;
       }
     }
-
     // ---- memory levels (Eqs. 17-19): prefix sums of A along each machine's lanes, then the machine's
     // level before the window, under the ledger baton ----
     int32_t lv = dA;
@@ -396,8 +417,8 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
     if (win > 0) named_sync<1, NW, IMMBAR>(warp);
     const uint32_t w0 = state[a0], w1 = state[a1], w2 = state[a2];
     const int32_t fr = (int32_t)state[fr_at];
-    int32_t r_base = __vimax3_s32(__viaddmax_s32((int32_t)(w0 >> 8), g0, fr), (int32_t)(w1 >> 8) + g1,
-                                  (int32_t)(w2 >> 8) + g2);
+    int32_t r_base = max(__vimax3_s32(__viaddmax_s32((int32_t)(w0 >> 8), g0, fr), (int32_t)(w1 >> 8) + g1,
+                                      (int32_t)(w2 >> 8) + g2), r_pre);
     if constexpr (WIDE) {
       uint32_t xw[kExtra];
 #pragma unroll
@@ -409,18 +430,30 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
     int32_t e = b_end;
     // every dependence points to a lower lane, so the values rise monotonically to the window's
     // longest-path solution, which they reach after `nrounds` rounds
-    for (int it = 0; it < nrounds; ++it) {
-      const int32_t s0 = __shfl_sync(FULL, e, l0), s1 = __shfl_sync(FULL, e, l1);
-      const int32_t s2 = __shfl_sync(FULL, e, l2), s3 = __shfl_sync(FULL, e, lp);
-      int32_t en = __vimax3_s32(__viaddmax_s32(s0, d0, b_end), __viaddmax_s32(s1, d1, s2 + d2), s3 + dp);
-      if constexpr (WIDE) {
-        int32_t xs[kExtra];
-#pragma unroll
-        for (int q = 0; q < kExtra; ++q) xs[q] = __shfl_sync(FULL, e, xl[q]);
-#pragma unroll
-        for (int q = 0; q < kExtra; ++q) en = __viaddmax_s32(xs[q], xd[q], en);
+    if (!WIDE && nslots == 2) {
+      for (int it = 0; it < nrounds; ++it) {
+        const int32_t s0 = __shfl_sync(FULL, e, x0), s1 = __shfl_sync(FULL, e, x1);
+        e = __viaddmax_s32(s0, d0, __viaddmax_s32(s1, d1, b_end));
       }
-      e = en;
+    } else if (!WIDE && nslots == 3) {
+      for (int it = 0; it < nrounds; ++it) {
+        const int32_t s0 = __shfl_sync(FULL, e, x0), s1 = __shfl_sync(FULL, e, x1), s2 = __shfl_sync(FULL, e, x2);
+        e = __viaddmax_s32(s0, d0, __viaddmax_s32(s1, d1, __viaddmax_s32(s2, d2, b_end)));
+      }
+    } else {
+      for (int it = 0; it < nrounds; ++it) {
+        const int32_t s0 = __shfl_sync(FULL, e, x0), s1 = __shfl_sync(FULL, e, x1);
+        const int32_t s2 = __shfl_sync(FULL, e, x2), s3 = __shfl_sync(FULL, e, x3);
+        int32_t en = __vimax3_s32(__viaddmax_s32(s0, d0, b_end), __viaddmax_s32(s1, d1, s2 + d2), s3 + d3);
+        if constexpr (WIDE) {
+          int32_t xs[kExtra];
+#pragma unroll
+          for (int q = 0; q < kExtra; ++q) xs[q] = __shfl_sync(FULL, e, xx[q]);
+#pragma unroll
+          for (int q = 0; q < kExtra; ++q) en = __viaddmax_s32(xs[q], (xx[q] >> 5) + dur, en);
+        }
+        e = en;
+      }
     }
     state[st_at] = ((uint32_t)e << 8) | j;
     state[fw_at] = (uint32_t)e;
