@@ -98,12 +98,14 @@ template <int NW, bool BY_POS, int CLS, bool TIMES, bool STAGED, bool WIDE>
 __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, const uint8_t* __restrict__ nblob,
                                                                int64_t K, const uint8_t* __restrict__ assign,
                                                                const uint16_t* __restrict__ order, pe_outputs out,
-                                                               uint32_t flags, TeamStrides sd) {
+                                                               uint32_t flags, TeamStrides sd,
+                                                               const uint32_t* __restrict__ cls_rows) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   static_assert(NW >= 2 && NW <= 6, "two named barriers per warp (numbers 1 .. 2 NW), barrier 0 is the block's");
   constexpr uint32_t FULL = 0xFFFFFFFFu;
-  constexpr bool TWO_CLASS = CLS == 2;
-  constexpr bool NEED_CLS = CLS != 0;
+  constexpr bool TWO_CLASS = CLS >= 2;
+  constexpr bool CLS_BITS = CLS == 3;   // two classes, every pair connected, at most 32 machines: bit x of cls_rows[j]
+  constexpr bool NEED_CLS = CLS == 1 || CLS == 2;
   constexpr int NT = NW * 32;
   constexpr bool IMMBAR = NW < 6;   // six warps per block go with large states, where few blocks fit anyway
   constexpr int32_t kNever = -(1 << 25);   // delay of an empty slot: never wins the maximum (times stay below 2^23)
@@ -241,6 +243,21 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
   uint32_t o_cur = load_order(warp), o_nxt = load_order(warp + NW);
   uint4 rec_nxt = __ldg(gp.ops + min(o_cur, vmax));
   const uint32_t none = (uint32_t)V;
+  // WIDE: incoming edges 1.. (two classes) or 2.. (one class) of the next window's operators, requested all at once when
+  // their record has arrived, so that no round trip to L2 per edge is in the set-up
+  constexpr int kList = !WIDE ? 1 : (TWO_CLASS ? 7 : 6);
+  uint2 listed[kList];
+  auto request_edges = [&](const uint4& r) {
+    if constexpr (WIDE) {
+      const int n = (int)(r.y >> 24);
+#pragma unroll
+      for (int q = 0; q < kList; ++q) {
+        if (TWO_CLASS) listed[q] = n > 1 + q ? __ldg(reinterpret_cast<const uint2*>(gp.edges) + r.x + 1 + q) : make_uint2(none, 0u);
+        else listed[q] = make_uint2(n > 3 && n > 2 + q ? __ldg(gp.edges + r.x + 2 + q) : none, 0u);
+      }
+    }
+  };
+  request_edges(rec_nxt);
 
   for (int win = warp; win < nwin; win += NW) {
     const int base = win * 32;
@@ -262,6 +279,7 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
       if (!BY_POS) dev_max = max(dev_max, jr);
       if ((own >> 8) != ((kTeamPending >> 8) | (uint32_t)k)) st |= PE_STATUS_ORDER_INVALID;   // repeated operator
     }
+    const uint32_t crow = CLS_BITS ? __ldg(cls_rows + j) : 0u;
     const int indeg = (int)(rec.y >> 24);
     const int32_t dur = act ? (int32_t)(rec.y & 0xFFFFu) : 0;
     const int32_t dA = act ? (int32_t)(rec.y << 8) >> 24 : 0;
@@ -290,6 +308,7 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
       const uint32_t w = state[p];
       const uint32_t xp = w & 0xFFu;
       uint32_t delay = lo >> 16;
+      if (CLS_BITS) delay = __funnelshift_r(crow, crow, w) & 1u ? hi : delay;   // (shift amount modulo 32: the machine)
       if (NEED_CLS) {
         const uint32_t cl = gp.cls[min(xp, dmax) * D + j];
         if (TWO_CLASS) delay = cl == 1u ? hi : delay;
@@ -319,30 +338,29 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
 #pragma unroll
     for (int q = 0; q < kExtra; ++q) { xa[q] = none; xg[q] = kNever; xx[q] = empty; }
     classify(rec.z, rec.w, a0, g0, x0);
-    if (TWO_CLASS) {
+    if constexpr (WIDE) {
+      a1 = none; a2 = none; g1 = kNever; g2 = kNever; x1 = empty; x2 = empty;
+      if (TWO_CLASS) {
+        if (indeg > 1) classify(listed[0].x, listed[0].y, a1, g1, x1);
+        if (indeg > 2) classify(listed[1].x, listed[1].y, a2, g2, x2);
+      } else {
+        // with more than three incoming edges the record's first word is the edge list's slot, not edge 2
+        classify(rec.w, 0u, a1, g1, x1);
+        classify(indeg > 3 ? listed[0].x : rec.x, 0u, a2, g2, x2);
+      }
+#pragma unroll
+      for (int q = 0; q < kExtra; ++q)
+        if (indeg > 3 + q) classify(listed[q + (TWO_CLASS ? 2 : 1)].x, listed[q + (TWO_CLASS ? 2 : 1)].y, xa[q], xg[q], xx[q]);
+    } else if (TWO_CLASS) {
       a1 = none; a2 = none; g1 = kNever; g2 = kNever; x1 = empty; x2 = empty;
       const uint2* ed = reinterpret_cast<const uint2*>(gp.edges) + rec.x;
       if (indeg > 1) { const uint2 e1 = __ldg(ed + 1); classify(e1.x, e1.y, a1, g1, x1); }
       if (indeg > 2) { const uint2 e2 = __ldg(ed + 2); classify(e2.x, e2.y, a2, g2, x2); }
-      if constexpr (WIDE) {
-#pragma unroll
-        for (int q = 0; q < kExtra; ++q)
-          if (indeg > 3 + q) { const uint2 eq = __ldg(ed + 3 + q); classify(eq.x, eq.y, xa[q], xg[q], xx[q]); }
-      }
     } else {
       classify(rec.w, 0u, a1, g1, x1);
-      if constexpr (WIDE) {
-        // with more than three incoming edges the record's first word is the edge list's slot, not edge 2
-        const uint32_t* ed = gp.edges + rec.x;
-        const bool many = indeg > 3;
-        classify(many ? __ldg(ed + 2) : rec.x, 0u, a2, g2, x2);
-#pragma unroll
-        for (int q = 0; q < kExtra; ++q)
-          if (indeg > 3 + q) classify(__ldg(ed + 3 + q), 0u, xa[q], xg[q], xx[q]);
-      } else {
-        classify(rec.x, 0u, a2, g2, x2);
-      }
+      classify(rec.x, 0u, a2, g2, x2);
     }
+    request_edges(rec_nxt);
     if (!act) {
       st = st_before; depmask = 0; r_pre = 0; a0 = a1 = a2 = none; x0 = x1 = x2 = empty;
 #pragma unroll
@@ -355,7 +373,7 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
     // two or three shuffles a round, not four.  Measured: V = 16384 / D = 8
     // K = 16384 10.4 -> 9.5 ms, multi-modal graph K = 1024 84 -> 76 us; V = 4096 / D = 64, where issue limits, +1.6 %.
     int nslots = 4;
-    if constexpr (!WIDE) {
+    {
       const bool u0 = x0 != empty, u1 = x1 != empty, u2 = x2 != empty;
       int32_t t;
       t = u0 ? x1 : empty; x0 = u0 ? x0 : x1; x1 = t;                                     // (x0, x1) in order
@@ -367,7 +385,7 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
       x1 = used == 1 ? x3 : x1;
       x0 = used == 0 ? x3 : x0;
       x3 = t;
-      nslots = __any_sync(FULL, x2 != empty) ? (__any_sync(FULL, x3 != empty) ? 4 : 3) : 2;
+      if (!WIDE) nslots = __any_sync(FULL, x2 != empty) ? (__any_sync(FULL, x3 != empty) ? 4 : 3) : 2;
     }
     // (the shuffles use the low five bits of a slot word; D^o is folded into the in-window delays, Eq. 3)
     const int32_t d0 = (x0 >> 5) + dur, d1 = (x1 >> 5) + dur, d2 = (x2 >> 5) + dur, d3 = (x3 >> 5) + dur;
@@ -375,11 +393,23 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
     // rounds of relaxation every lane of depth <= n holds its final value, so the number of rounds is
     // known before the baton arrives and the loop under it needs no vote.
     int nrounds = 0;
+    uint32_t wide_rounds = 0;
     {
       uint32_t done = __ballot_sync(FULL, depmask == 0);
+      int depth = 0;
       while (done != FULL) {
+        if (WIDE) depth += (int)(~done >> lane & 1u);
         done = __ballot_sync(FULL, (depmask & ~done) == 0);
         ++nrounds;
+      }
+      if constexpr (WIDE) {
+        // A lane's sources are final when `depth - 1` rounds are done, and values only rise: a lane with more than two
+        // sources in the window needs the others in round `depth` alone.  So most rounds shuffle two slots, and only
+        // those marked here all nine (MoE graph, 14 rounds and 2.3 such lanes a window: 126 -> 44 shuffles).
+        bool many = x2 != empty;
+#pragma unroll
+        for (int q = 0; q < kExtra; ++q) many = many || xx[q] != empty;
+        wide_rounds = __reduce_or_sync(FULL, many ? 1u << ((depth - 1) & 31) : 0u);
       }
     }
     // ---- memory levels (Eqs. 17-19): prefix sums of A along each machine's lanes, then the machine's
@@ -440,15 +470,22 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
         const int32_t s0 = __shfl_sync(FULL, e, x0), s1 = __shfl_sync(FULL, e, x1), s2 = __shfl_sync(FULL, e, x2);
         e = __viaddmax_s32(s0, d0, __viaddmax_s32(s1, d1, __viaddmax_s32(s2, d2, b_end)));
       }
-    } else {
+    } else if (!WIDE) {
       for (int it = 0; it < nrounds; ++it) {
         const int32_t s0 = __shfl_sync(FULL, e, x0), s1 = __shfl_sync(FULL, e, x1);
         const int32_t s2 = __shfl_sync(FULL, e, x2), s3 = __shfl_sync(FULL, e, x3);
-        int32_t en = __vimax3_s32(__viaddmax_s32(s0, d0, b_end), __viaddmax_s32(s1, d1, s2 + d2), s3 + d3);
-        if constexpr (WIDE) {
+        e = __vimax3_s32(__viaddmax_s32(s0, d0, b_end), __viaddmax_s32(s1, d1, s2 + d2), s3 + d3);
+      }
+    } else {
+      for (int it = 0; it < nrounds; ++it) {
+        const int32_t s0 = __shfl_sync(FULL, e, x0), s1 = __shfl_sync(FULL, e, x1);
+        int32_t en = __viaddmax_s32(s0, d0, __viaddmax_s32(s1, d1, e));
+        if (wide_rounds >> it & 1u) {
+          const int32_t s2 = __shfl_sync(FULL, e, x2), s3 = __shfl_sync(FULL, e, x3);
           int32_t xs[kExtra];
 #pragma unroll
           for (int q = 0; q < kExtra; ++q) xs[q] = __shfl_sync(FULL, e, xx[q]);
+          en = __vimax3_s32(en, s2 + d2, s3 + d3);
 #pragma unroll
           for (int q = 0; q < kExtra; ++q) en = __viaddmax_s32(xs[q], (xx[q] >> 5) + dur, en);
         }

@@ -21,13 +21,14 @@ struct TeamCall {
 
 template <int NW, bool BY_POS, int CLS>
 int launch3(const TeamCall& t) {
+  const uint32_t* cls_rows = CLS == 3 ? reinterpret_cast<const uint32_t*>(t.g->d_tblob + t.g->tview.cls_row) : nullptr;
   auto go = [&](auto kern) -> int {
     if (!set_smem(kern, t.p->smem)) return PE_ERR_CUDA;
     // the state is all these blocks need from the SM's memory: ask for the largest shared-memory carve-out
     // (a hint; without it the default carve-out can hold fewer blocks than shared memory would allow)
     cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     kern<<<(unsigned)t.kc, NW * 32, t.p->smem, t.stream>>>(t.g->nview, t.g->d_nblob, t.K, t.assign, t.order, t.out, t.flags,
-                                                            t.sd);
+                                                            t.sd, cls_rows);
     return PE_OK;
   };
   const bool wide = t.g->max_indeg > 3;   // operators with four to eight incoming edges
@@ -40,12 +41,16 @@ int launch3(const TeamCall& t) {
 
 template <int NW>
 int launch_team_nw(const TeamCall& t, bool by_pos) {
-  const int cls = t.g->nview.L == 2 ? 2 : (t.g->nview.need_cls ? 1 : 0);
+  // the class of a pair is a bit of a row word where the tile encoding has those (no table read per edge; multi-modal and
+  // MoE graphs)
+  const int cls = t.g->nview.L == 2 ? (t.g->tile_ok && t.g->tview.cls_kind == 2 ? 3 : 2) : (t.g->nview.need_cls ? 1 : 0);
   if (by_pos) {
+    if (cls == 3) return launch3<NW, true, 3>(t);
     if (cls == 2) return launch3<NW, true, 2>(t);
     if (cls == 1) return launch3<NW, true, 1>(t);
     return launch3<NW, true, 0>(t);
   }
+  if (cls == 3) return launch3<NW, false, 3>(t);
   if (cls == 2) return launch3<NW, false, 2>(t);
   if (cls == 1) return launch3<NW, false, 1>(t);
   return launch3<NW, false, 0>(t);
