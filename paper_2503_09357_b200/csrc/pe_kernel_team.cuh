@@ -477,19 +477,29 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
         e = __vimax3_s32(__viaddmax_s32(s0, d0, b_end), __viaddmax_s32(s1, d1, s2 + d2), s3 + d3);
       }
     } else {
-      for (int it = 0; it < nrounds; ++it) {
-        const int32_t s0 = __shfl_sync(FULL, e, x0), s1 = __shfl_sync(FULL, e, x1);
-        int32_t en = __viaddmax_s32(s0, d0, __viaddmax_s32(s1, d1, e));
-        if (wide_rounds >> it & 1u) {
-          const int32_t s2 = __shfl_sync(FULL, e, x2), s3 = __shfl_sync(FULL, e, x3);
-          int32_t xs[kExtra];
-#pragma unroll
-          for (int q = 0; q < kExtra; ++q) xs[q] = __shfl_sync(FULL, e, xx[q]);
-          en = __vimax3_s32(en, s2 + d2, s3 + d3);
-#pragma unroll
-          for (int q = 0; q < kExtra; ++q) en = __viaddmax_s32(xs[q], (xx[q] >> 5) + dur, en);
+      int it = 0;
+      for (uint32_t marks = wide_rounds;; marks &= marks - 1u) {
+        const int stop = marks ? __ffs((int)marks) - 1 : nrounds;
+        for (; it < stop; ++it) {
+          const int32_t s0 = __shfl_sync(FULL, e, x0), s1 = __shfl_sync(FULL, e, x1);
+          e = __viaddmax_s32(s0, d0, __viaddmax_s32(s1, d1, e));
         }
-        e = en;
+        if (marks == 0u) break;
+        const int32_t s0 = __shfl_sync(FULL, e, x0), s1 = __shfl_sync(FULL, e, x1);
+        const int32_t s2 = __shfl_sync(FULL, e, x2), s3 = __shfl_sync(FULL, e, x3);
+        int32_t xs[kExtra];
+#pragma unroll
+        for (int q = 0; q < kExtra; ++q) xs[q] = __shfl_sync(FULL, e, xx[q]);
+        int32_t ea = __viaddmax_s32(s0, d0, e), eb = __viaddmax_s32(s1, d1, s2 + d2);
+        ea = __viaddmax_s32(s3, d3, ea);
+#pragma unroll
+        for (int q = 0; q < kExtra; ++q) {
+          const int32_t t = (xx[q] >> 5) + dur;
+          if (q & 1) ea = __viaddmax_s32(xs[q], t, ea);
+          else eb = __viaddmax_s32(xs[q], t, eb);
+        }
+        e = max(ea, eb);
+        ++it;
       }
     }
     state[st_at] = ((uint32_t)e << 8) | j;
