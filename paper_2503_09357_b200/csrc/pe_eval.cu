@@ -407,9 +407,11 @@ static double team_us(const pe_graph* g, int64_t K) {
   const double rate = g->max_indeg > 3 ? 20000.0 : (width < 24.0 ? 32000.0 : (g->D < 32 ? 42000.0 : 51000.0));
   return 10.0 + 0.026 * V + V * (double)K / rate;
 }
-static double lane_us(const pe_graph* g, int64_t K, const Plan& lane) {
+// (times by operator leave in a pass of their own: multi-modal graph K = 65536 3505 against 2844 us of TEAM)
+static double lane_us(const pe_graph* g, int64_t K, uint32_t flags, const Plan& lane) {
   const double V = g->V, rounds = (double)K / ((double)lane.tile_resident * g->sm_count);
-  return 8.0 + (g->max_indeg > 3 ? 0.15 : 0.103) * V * (rounds > 1.0 ? rounds : 1.0);
+  const double us = (g->max_indeg > 3 ? 0.15 : 0.103) * V * (rounds > 1.0 ? rounds : 1.0);
+  return 8.0 + ((flags & PE_TIMES_BY_OP) ? 1.35 : 1.0) * us;
 }
 
 // Exclusive channels: a lane per candidate (~0.3 us a position where the channel words leave few lanes per SM) or the
@@ -455,7 +457,7 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
       const bool has_s = plan_shared(g, K, allow_compact, p) && (p->tiled || p->threads >= 48);
       const bool has_t = plan_team(g, K, allow_compact, &tm);
       if (has_s && !p->tiled) return PE_OK;
-      if (has_s && (!has_t || lane_us(g, K, *p) <= team_us(g, K)) && (has_t || p->tile_resident >= 28)) return PE_OK;
+      if (has_s && (!has_t || lane_us(g, K, flags, *p) <= team_us(g, K)) && (has_t || p->tile_resident >= 28)) return PE_OK;
       if (has_t) { *p = tm; return PE_OK; }
       const bool has_w = plan_warp(g, K, flags, allow_compact, &w);
       const bool has_g = plan_global(g, K, flags, allow_compact, &gl);

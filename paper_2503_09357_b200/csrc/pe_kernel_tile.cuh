@@ -400,18 +400,11 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
       const uint32_t bz = HET ? dv.y + dur_het : __dp2a_lo(r4.x, 1u, dv.y);                     // + D^o_i (low half)
       sts_state<S16>(st_a + i * pitch, e);
       sts128(dv_a + j * dpitch, make_uint4(e, bz, (uint32_t)lv, (uint32_t)max((int32_t)dv.w, lv)));
-      if (TIMES) {
-        if (TIMES == 1) {
-          *reinterpret_cast<int32_t*>(start_b) = (int32_t)(rt >> jb);
-          *reinterpret_cast<int32_t*>(finish_b) = (int32_t)(e >> jb);
-          start_b += K4;
-          finish_b += K4;
-        } else {
-          const uint32_t io = min(i, vlast - 1u);
-          const size_t at = (size_t)io * K4;
-          *reinterpret_cast<int32_t*>(start_b + at) = (int32_t)(rt >> jb);
-          *reinterpret_cast<int32_t*>(finish_b + at) = (int32_t)(e >> jb);
-        }
+      if (TIMES == 1) {
+        *reinterpret_cast<int32_t*>(start_b) = (int32_t)(rt >> jb);
+        *reinterpret_cast<int32_t*>(finish_b) = (int32_t)(e >> jb);
+        start_b += K4;
+        finish_b += K4;
       }
       if (!BY_POS) {   // a repetition right behind: its own word was read before this step's store
         if (i_n == i) own_n = 0u;
@@ -465,6 +458,22 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
     }
 
     // ---- results of the tile ----
+    if (TIMES == 2) {
+      // Times by operator: the state words hold every end time, so they leave row by row here; a store per step would
+      // touch 32 rows at once (bidirectional pipeline K = 65536: 879 -> 212 us; V = 256 / D = 8 K = 2^20: 9.2 -> 1.6 ms).
+#pragma unroll 4
+      for (int i = 0; i < V; ++i) {
+        const uint32_t w = lds_state<S16>(st_a + (uint32_t)i * pitch), d16 = lds32(rec_a + (uint32_t)i * 16u) & 0xFFFFu;
+        const int32_t fin = (int32_t)(w >> jb);
+        const int32_t d = HET ? (int32_t)lds16(durm_a + ((uint32_t)i * (uint32_t)D + min(w & jmask, dmax)) * 2u) : (int32_t)(S16 ? d16 >> jb : d16);
+        if (cand) {
+          *reinterpret_cast<int32_t*>(start_b) = fin - d;
+          *reinterpret_cast<int32_t*>(finish_b) = fin;
+        }
+        start_b += K4;
+        finish_b += K4;
+      }
+    }
     if (own_min < unsched) st |= PE_STATUS_ORDER_INVALID;   // an operator twice, or an entry that is no operator
     // a machine's end times rise: the largest last one is the makespan (formed here, not in the loop below: 1185 against
     // 1248 us at V = 256, D = 8)
