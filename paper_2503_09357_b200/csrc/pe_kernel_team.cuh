@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(NW * 32) pe_eval_team_kernel(PeNarrowView g, c
     if (win + 1 < nwin) named_arrive<1, NW, IMMBAR>(next_warp);
 
     // ---- after the baton has gone: outputs ----
-    z = max(z, e);
+    if (act) z = max(z, e);   // (the gather of a lane beyond the end still carries a delay into operator 0)
     if (TIMES && act) {
       const uint32_t row = by_op_times ? i : (uint32_t)k;
       const size_t at = STAGED ? (size_t)row : (size_t)row * sd.out_row;
