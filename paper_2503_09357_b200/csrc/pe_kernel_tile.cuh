@@ -457,6 +457,9 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
       for (int u = 0; u < kRing; ++u) { ring[u] = nxt[u]; if (BY_POS) aring[u] = anxt[u]; }
     }
 
+    // The loop wrote its words through asm that names no memory; the results read them through ordinary loads.
+    __syncwarp();
+
     // ---- results of the tile ----
     if (TIMES == 2) {
       // Times by operator: the state words hold every end time, so they leave row by row here; a store per step would
