@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
   const int32_t* cap = reinterpret_cast<const int32_t*>(smem_raw + g.cap);
 
   const uint32_t pitch = (uint32_t)P * 4u;   // bytes of a row of words
-  const int ml = lane < P ? lane : P - 1;    // lanes beyond the tile do what its last lane does: same addresses, same values
+  const int ml = lane < P ? lane : P - 1;    // (lanes beyond the tile have no column: they only copy, and sit out the main loop)
   const uint32_t vlast = (uint32_t)V, dmax = (uint32_t)(D - 1);
   uint8_t* st_base = S16 ? smem_raw + sh.off_state + (uint32_t)(warp >> 1) * sh.state_bytes + (uint32_t)ml * 4u + (uint32_t)(warp & 1) * 2u
                          : smem_raw + sh.off_state + (uint32_t)warp * sh.state_bytes + (uint32_t)ml * 4u;
@@ -422,7 +422,9 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
     // copies 1517 us (11 more instructions a step).  With exclusive channels or durations by machine the step is so
     // long that sixteen of them unrolled overflow the instruction cache: blocks of 8 (238 -> 185 us and 138 -> 113 us on
     // the bidirectional pipeline, K = 16384).
-    for (int kb = 0; kb < V; kb += kRing) {
+    // Lanes beyond the tile stay out: they would read and write the last lane's words, and after a branch nothing keeps
+    // them in step with it.
+    for (int kb = write ? 0 : V; kb < V; kb += kRing) {
       ord_b += (size_t)kRing * K2;
       asg_b += (size_t)kRing * K1;
       uint32_t nxt[kRing], anxt[kRing];
@@ -457,7 +459,8 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
       for (int u = 0; u < kRing; ++u) { ring[u] = nxt[u]; if (BY_POS) aring[u] = anxt[u]; }
     }
 
-    // The loop wrote its words through asm that names no memory; the results read them through ordinary loads.
+    // The lanes that sat out come back.  The loop wrote its words through asm that names no memory; the results read them
+    // through ordinary loads.
     __syncwarp();
 
     // ---- results of the tile ----

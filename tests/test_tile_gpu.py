@@ -29,7 +29,7 @@ def chain_graph(V, D, indeg, classes, scale, seed=0):
 @pytest.mark.parametrize("V,D,indeg,classes,scale,K", [
     (15, 3, 2, 1, 4, 31), (16, 3, 2, 1, 4, 33), (17, 4, 3, 1, 4, 64), (47, 8, 3, 1, 200, 128), (48, 8, 2, 2, 200, 129),
     (49, 40, 3, 2, 30, 96), (63, 32, 5, 2, 30, 97), (65, 5, 6, 1, 300, 1), (80, 6, 3, 3, 30, 4740), (1500, 8, 3, 1, 40, 300),
-    (1600, 8, 2, 2, 40, 299)])
+    (1600, 8, 2, 2, 40, 299), (1200, 8, 6, 3, 9, 301), (1100, 12, 6, 1, 9, 200)])
 def test_tile_edges_match_the_oracle(V, D, indeg, classes, scale, K):
     import torch
     if not torch.cuda.is_available():
