@@ -15,10 +15,11 @@
 //   * times are kept and compared in packed form, time << jb | machine.  A maximum over packed words is
 //     a maximum over times (the machine bits only break ties), so a source costs: address, load,
 //     same-machine test, delay select, fused add-max;
-//   * validity costs two instructions a step: an operator that is not scheduled yet holds a time field
-//     beyond every reachable time, which the makespan accumulator sees; a repeated operator finds its
-//     own word scheduled; an entry that is no operator is clamped to the sentinel row V, which counts as
-//     scheduled.
+//   * validity costs one instruction a step: an operator that is not scheduled yet holds a time field
+//     beyond every reachable time, which reaches the machine's last end time; a repeated operator does not
+//     find exactly the unscheduled word (behind a missing source it finds a later time, so a comparison with
+//     scheduled words alone would let repetitions add up until the packed time wraps); an entry that is no
+//     operator is clamped to the sentinel row V, which counts as scheduled.
 // Measured on B200 (before: the thread-per-candidate kernel this one replaces, 92 instructions and ~370 cycles a
 // step at V = 256; now 68 and ~230): V = 256 / D = 8, K = 2^20: 1.85 -> 1.19 ms; bidirectional pipeline (V = 480),
 // K = 65536: 352 -> 166 us, with durations by machine, K = 16384: 490 -> 113 us (generic kernel before); multi-modal
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
 
     // ---- main loop ----
     uint32_t st = 0;
-    uint32_t own_min = 0xFFFFFFFFu, dev_max = 0;
+    uint32_t own_max = 0, dev_max = 0;   // own_max: the word a position finds for its operator, less `unsched`
     uint8_t* start_b = reinterpret_cast<uint8_t*>(out.start) + (size_t)cc * 4;     // this position's row
     uint8_t* finish_b = reinterpret_cast<uint8_t*>(out.finish) + (size_t)cc * 4;
 
@@ -328,7 +329,7 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
       uint32_t dur_het = 0;
       if (HET) dur_het = lds16(durm_a + (i * (uint32_t)D + j) * 2u);
       if (BY_POS) own = lds_state<S16>(st_a + i * pitch);
-      own_min = min(own_min, own);
+      own_max = max(own_max, own - unsched);
       // the next position's operator
       const uint32_t i_n = min(o_next, vlast);
       const uint4 rec_n = lds128(rec_a + i_n * 16u);
@@ -480,7 +481,7 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
         finish_b += K4;
       }
     }
-    if (own_min < unsched) st |= PE_STATUS_ORDER_INVALID;   // an operator twice, or an entry that is no operator
+    if (own_max > jmask) st |= PE_STATUS_ORDER_INVALID;   // an operator twice, or an entry that is no operator
     // a machine's end times rise: the largest last one is the makespan (formed here, not in the loop below: 1185 against
     // 1248 us at V = 256, D = 8)
     uint32_t z = 0;
@@ -489,7 +490,7 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
     if (BY_POS) {
       if (dev_max > dmax) st |= PE_STATUS_ASSIGN_RANGE;
       // entries at positions that hold no operator are not consulted
-      if (dev_max > dmax && own_min < unsched) {
+      if (dev_max > dmax && own_max > jmask) {
         st &= ~(uint32_t)PE_STATUS_ASSIGN_RANGE;
         for (int k = 0; k < V; ++k)
           if ((uint32_t)order[(size_t)k * (size_t)K + cc] < (uint32_t)V && (uint32_t)assign[(size_t)k * (size_t)K + cc] > dmax)

@@ -53,3 +53,34 @@ def test_tile_edges_match_the_oracle(V, D, indeg, classes, scale, K):
             gu.check(g, w, a, order, flags=flags | pe.PE_VARIANT_SHARED, label=f"flags {flags}")
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("by_pos", [False, True])
+@pytest.mark.parametrize("dur,scale", [(65535, 1), (255, 0)])
+def test_repetitions_behind_a_missing_source_are_flagged(dur, scale, by_pos):
+    """Operator 0 is placed again and again ahead of its predecessor: every repetition adds its duration to a time that
+    is beyond all reachable ones, until the packed word wraps into the reachable range.  `repeat` covers the count (129)
+    at which that happens, with 32-bit words (dur 65535) and, where the time bound allows, 16-bit words (dur 255)."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2503_09357_b200 import binding as pe
+    V, D, K = 310, 2, 300
+    w = ck.problem(V, [(1, 0)], np.where(np.arange(V) == 0, dur, scale), D, comm=0)
+    w.assign_mode, w.group = "per_op", None
+    assign = np.ones((V, K), np.uint8)
+    assign[0] = 0
+    order = np.repeat((2 + np.arange(V) % (V - 2)).astype(np.uint16)[:, None], K, axis=1)
+    for c in range(K):
+        repeat = 2 + c // 2
+        if c % 2:
+            order[V - repeat:, c] = 0                   # one after the other at the end,
+        else:
+            order[V - 2 * repeat + 1::2, c] = 0         # or with another operator in between
+    a = np.take_along_axis(assign, order.astype(np.int64), axis=0) if by_pos else assign
+    g = pe.Graph(w)
+    try:
+        gpu, ref = gu.check(g, w, a, order, flags=pe.PE_VARIANT_SHARED | (pe.PE_ASSIGN_BY_POS if by_pos else 0))
+        assert (ref["status"] & pe.PE_STATUS_ORDER_INVALID).all()
+    finally:
+        g.close()
