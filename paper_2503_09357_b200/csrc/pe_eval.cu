@@ -234,8 +234,9 @@ static inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; 
 
 // exclusive: PE_COMM_EXCLUSIVE - the compact kernel keeps one more word per machine pair and candidate;
 // the generic shared-state kernel does not offer it.
-static bool plan_shared(const pe_graph* g, int64_t K, bool allow_compact, Plan* p, bool exclusive = false) {
-  if (allow_compact && plan_tile(g, K, exclusive, p)) return true;
+static bool plan_shared(const pe_graph* g, int64_t K, uint32_t flags, bool allow_compact, Plan* p) {
+  const bool exclusive = (flags & PE_COMM_EXCLUSIVE) != 0;
+  if (allow_compact && plan_tile(g, K, (flags & PE_ASSIGN_BY_POS) != 0, exclusive, p)) return true;
   if (g->time_bound >= kPackedTimeLimit) return false;
   p->compact = false;
   if (exclusive) return false;
@@ -434,7 +435,7 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
   const uint32_t want = flags & PE_VARIANT_MASK;
   if (g->hetero) {   // machine-dependent durations: the generic one-thread-per-candidate kernels
     if (want == PE_VARIANT_WARP || want == PE_VARIANT_TEAM) return PE_ERR_UNSUPPORTED;
-    if (!(flags & PE_COMM_EXCLUSIVE) && want != PE_VARIANT_GLOBAL && plan_shared(g, K, allow_compact, p) &&
+    if (!(flags & PE_COMM_EXCLUSIVE) && want != PE_VARIANT_GLOBAL && plan_shared(g, K, flags, allow_compact, p) &&
         (p->tiled || p->threads >= 48 || want == PE_VARIANT_SHARED))
       return PE_OK;
     if (want == PE_VARIANT_SHARED) return PE_ERR_UNSUPPORTED;
@@ -444,7 +445,7 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
     // exclusive channels: the compact shared-state kernel where a block of candidates still fits with one
     // more word per machine pair each, else the generic global-state kernel
     if (want == PE_VARIANT_AUTO || want == PE_VARIANT_SHARED) {
-      if (plan_shared(g, K, allow_compact, p, true) && (want == PE_VARIANT_SHARED || lane_pays_exclusive(g, K, *p))) return PE_OK;
+      if (plan_shared(g, K, flags, allow_compact, p) && (want == PE_VARIANT_SHARED || lane_pays_exclusive(g, K, *p))) return PE_OK;
       if (want == PE_VARIANT_SHARED) return PE_ERR_UNSUPPORTED;
       *p = Plan();
     }
@@ -454,7 +455,7 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
   switch (want) {
     case PE_VARIANT_AUTO: {
       Plan w, gl, tm;
-      const bool has_s = plan_shared(g, K, allow_compact, p) && (p->tiled || p->threads >= 48);
+      const bool has_s = plan_shared(g, K, flags, allow_compact, p) && (p->tiled || p->threads >= 48);
       const bool has_t = plan_team(g, K, allow_compact, &tm);
       if (has_s && !p->tiled) return PE_OK;
       if (has_s && (!has_t || lane_us(g, K, flags, *p) <= team_us(g, K)) && (has_t || p->tile_resident >= 28)) return PE_OK;
@@ -470,13 +471,13 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
       const bool warp_wins = w.threads >= 4 * 32 || (w.threads >= 3 * 32 && has_g && gl.smem == 0);
       if (has_w && (warp_wins || !has_g || !gl.compact)) { *p = w; return PE_OK; }
       if (has_g && gl.compact) { *p = gl; return PE_OK; }
-      if (plan_shared(g, K, allow_compact, p)) return PE_OK;
+      if (plan_shared(g, K, flags, allow_compact, p)) return PE_OK;
       if (has_w) { *p = w; return PE_OK; }
       if (has_g) { *p = gl; return PE_OK; }
       return PE_ERR_UNSUPPORTED;
     }
     case PE_VARIANT_GLOBAL: return plan_global(g, K, flags, allow_compact, p) ? PE_OK : PE_ERR_UNSUPPORTED;
-    case PE_VARIANT_SHARED: return plan_shared(g, K, allow_compact, p) ? PE_OK : PE_ERR_UNSUPPORTED;
+    case PE_VARIANT_SHARED: return plan_shared(g, K, flags, allow_compact, p) ? PE_OK : PE_ERR_UNSUPPORTED;
     case PE_VARIANT_WARP: return plan_warp(g, K, flags, allow_compact, p) ? PE_OK : PE_ERR_UNSUPPORTED;
     case PE_VARIANT_TEAM: return plan_team(g, K, allow_compact, p) ? PE_OK : PE_ERR_UNSUPPORTED;
     default: return PE_ERR_UNSUPPORTED;

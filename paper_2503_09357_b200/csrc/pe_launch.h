@@ -48,7 +48,7 @@ static bool set_smem(Kern kern, size_t bytes) {
 }
 
 // pe_eval_tile_kernel (plan variant SHARED over the tile encoding).
-bool plan_tile(const pe_graph* g, int64_t K, bool exclusive, Plan* p);
+bool plan_tile(const pe_graph* g, int64_t K, bool by_pos, bool exclusive, Plan* p);
 int launch_tile(const pe_graph* g, const Plan& p, bool by_pos, int64_t K, const uint8_t* assign, const uint16_t* order,
                 uint32_t flags, const pe_outputs& out, cudaStream_t stream);
 

@@ -8,7 +8,7 @@ inline size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
 }
 
 // Block shape: W warps of P lanes that together use the shared memory of an SM.
-bool plan_tile(const pe_graph* g, int64_t K, bool exclusive, Plan* p) {
+bool plan_tile(const pe_graph* g, int64_t K, bool by_pos, bool exclusive, Plan* p) {
   if (!g->tile_ok || K >= ((int64_t)1 << 26)) return false;   // (row pitches times the ring length are 32-bit)
   if (g->hetero && exclusive) return false;
   const PeTileView& tv = g->tview;
@@ -27,13 +27,24 @@ bool plan_tile(const pe_graph* g, int64_t K, bool exclusive, Plan* p) {
     const size_t states = mode == kTileS16 ? (W + 1) / 2 : W;
     return fixed + W * per + states * up16(P * 4 * rows);
   };
+  // The time of a round (all resident tiles, V positions) is that of one step as long as every warp has a scheduler to
+  // itself and rises from the fifth warp on, more where narrow rows meet in the same banks, and once more beyond
+  // kTileWarps, where a step has half the registers; the largest number of candidates per unit of that is taken.
+  // Measured, ns a step by W x P (by operator): V = 961 / D = 8 2x24 87, 3x16 84, 4x12 90, 6x8 110, 8x4 111, 12x4 164,
+  // 13x4 195; V = 256 / D = 8 3x32 102, 4x32 105, 5x32 129, 6x32 145, 7x28 198, 8x24 186; V = 480, 16-bit words 4x32 105,
+  // 5x32 123, 6x32 128, 7x24 140, 8x24 157; V = 64 16x32 51 us in all (K = 200000), 8x32 59.  By-operator machine ids are
+  // read four candidates at a time: a width that is no multiple of four costs 40 to 50 % there (V = 961 2x24 87, 2x26 131)
+  // and nothing by position (101 and 100; V = 684 / D = 6 3x24 105, 4x19 107).
+  const size_t grain = by_pos ? 1 : 4;
   size_t bestW = 0, bestP = 0;
   double best = 0;
-  for (size_t W = 1; W <= 16; ++W)
-    for (size_t P = 32; P >= 4; P -= 4)
+  for (size_t W = 1; W <= 2 * kTileWarps; ++W)
+    for (size_t P = 32; P >= 4; P -= grain)
       if (bytes(W, P) <= g->smem_optin) {
-        // rows of fewer than 32 words spread a warp's gathers over the banks unevenly
-        const double score = (double)(W * P) * (P == 32 ? 1.0 : 0.9);
+        double round = W <= 4 ? 1.0 : 1.0 + 0.14 * (double)(W - 4);
+        if (W > 4 && P < 32) round /= 0.9;
+        if (W > kTileWarps) round /= 0.88;
+        const double score = (double)(W * P) / round;
         if (score > best) { best = score; bestW = W; bestP = P; }
         break;
       }

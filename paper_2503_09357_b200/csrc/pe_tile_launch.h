@@ -21,7 +21,7 @@ template <int CLS, int EDGES, bool BY_POS, int MODE>
 int launch_tile3(const TileCall& t) {
   const Plan& p = *t.p;
   TileShape sh = p.tile;
-  sh.vector_init = !BY_POS && t.K % 4 == 0 && ((uintptr_t)t.assign & 3u) == 0;
+  sh.vector_init = !BY_POS && sh.lanes % 4 == 0 && t.K % 4 == 0 && ((uintptr_t)t.assign & 3u) == 0;
   auto go = [&](auto kern) -> int {
     if (!set_smem(kern, p.smem)) return PE_ERR_CUDA;
     kern<<<(unsigned)p.grid, p.threads, p.smem, t.stream>>>(t.g->tview, t.g->d_tblob, t.K, t.assign, t.order, t.out,

@@ -4,8 +4,10 @@
 
 namespace pe {
 
+constexpr int kTileWarps = 8;   // warps of a block (twice as many where operators are few)
+
 struct TileShape {
-  int lanes;            // P, candidates per tile (multiple of 4)
+  int lanes;            // P, candidates per tile (4 to 32)
   int jbits;            // machine bits of a state word (8 with 32-bit words)
   int64_t tiles;        // ceil(K / P)
   uint32_t off_dev;     // byte offsets in shared memory: machine records of warp 0, weight sums, state words, channels
