@@ -102,8 +102,12 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // of a pair is a bit of a row word.
 // EDGES: 2 / 3 = no operator has more incoming edges, all inline; 0 = inline edges, then the edge list.
 // TIMES: 0 = none, 1 = by position, 2 = by operator.
-template <int CLS, int EDGES, bool BY_POS, int TIMES, int MODE>
-__global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const uint8_t* __restrict__ blob, int64_t K,
+// WARPS: largest number of warps of a block.  With kTileWarps a thread may use the registers that a request block of
+// sixteen positions needs without spilling (128 registers and 4 to 12 bytes of spills with twice as many warps: V = 1024 /
+// D = 64 K = 65536 1110 -> 1038 us by operator and, with blocks of 16 instead of 8, 1178 -> 954 by position; multi-modal
+// graph 2434 -> 2310 and 2337 -> 2121; V = 256 / D = 8 K = 2^20 1205 -> 1163 and 1249 -> 1032).
+template <int CLS, int EDGES, bool BY_POS, int TIMES, int MODE, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) pe_eval_tile_kernel(PeTileView g, const uint8_t* __restrict__ blob, int64_t K,
                                                            const uint8_t* __restrict__ assign,
                                                            const uint16_t* __restrict__ order, pe_outputs out, int* err,
                                                            TileShape sh) {
@@ -111,7 +115,13 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
   constexpr uint32_t FULL = 0xFFFFFFFFu;
   constexpr bool S16 = MODE == kTileS16, EXCL = MODE == kTileExcl, HET = MODE == kTileHet;
   using StateT = typename std::conditional<S16, uint16_t, uint32_t>::type;
-  constexpr int kRing = BY_POS || EXCL || HET ? 8 : 16;   // order entries (and by-position machine ids) per request
+  // Order entries (and by-position machine ids) per request.  A step with branches, or with channels or durations by
+  // machine, is so long that sixteen of them are no longer inlined or overflow the instruction cache.
+  constexpr bool kRoomy = WARPS <= kTileWarps, kStraight = !EXCL && !HET && CLS != 1 && EDGES != 0;
+  constexpr bool kEight = kRoomy ? !kStraight || (BY_POS && TIMES == 1 && CLS == 0 && EDGES == 2 && !S16) : BY_POS || EXCL || HET;
+  constexpr int kRing = kEight ? 8 : 16;
+  // Whether a step carries stores that are never executed (see there).
+  constexpr bool kIdleStores = kRoomy && kStraight && TIMES != 1 && !(TIMES == 0 && !BY_POS && CLS == 0 && (S16 || EDGES == 2));
   constexpr int NIN = CLS == 0 ? (EDGES == 2 ? 2 : 3) : 2;   // edges that the record carries inline
   const int V = g.V, D = g.D;
   const int lane = threadIdx.x & 31;
@@ -401,6 +411,14 @@ __global__ void __launch_bounds__(512) pe_eval_tile_kernel(PeTileView g, const u
       const uint32_t bz = HET ? dv.y + dur_het : __dp2a_lo(r4.x, 1u, dv.y);                     // + D^o_i (low half)
       sts_state<S16>(st_a + i * pitch, e);
       sts128(dv_a + j * dpitch, make_uint4(e, bz, (uint32_t)lv, (uint32_t)max((int32_t)dv.w, lv)));
+      if (kIdleStores)
+        // Without any store to global memory in the step the compiler lets the block's requests share a scoreboard with
+        // the step's shared-memory loads, and every block waits for DRAM; with a store, executed or not, it does not.
+        // Measured (us, without / with): V = 1024 / D = 64 K = 32768 by position 630 / 541, times by operator 950 / 807;
+        // multi-modal graph K = 30000 by operator 1360 / 1163, by position 1378 / 1014; bidirectional pipeline K = 65536
+        // by position 172 / 133.  (Left out of the forms where it costs: V = 480 by operator 137 / 145.)
+        asm volatile("{.reg .pred p; setp.lt.s32 p, %3, 0; @p st.global.u32 [%0], %1; @p st.global.u32 [%0], %2;}"
+                     ::"l"(start_b), "r"(rt), "r"(e), "r"(sh.lanes) : "memory");
       if (TIMES == 1) {
         *reinterpret_cast<int32_t*>(start_b) = (int32_t)(rt >> jb);
         *reinterpret_cast<int32_t*>(finish_b) = (int32_t)(e >> jb);

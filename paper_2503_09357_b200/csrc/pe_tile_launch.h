@@ -17,8 +17,8 @@ struct TileCall {
   cudaStream_t stream;
 };
 
-template <int CLS, int EDGES, bool BY_POS, int MODE>
-int launch_tile3(const TileCall& t) {
+template <int CLS, int EDGES, bool BY_POS, int MODE, int WARPS>
+int launch_tile4(const TileCall& t) {
   const Plan& p = *t.p;
   TileShape sh = p.tile;
   sh.vector_init = !BY_POS && sh.lanes % 4 == 0 && t.K % 4 == 0 && ((uintptr_t)t.assign & 3u) == 0;
@@ -28,9 +28,18 @@ int launch_tile3(const TileCall& t) {
                                                              t.g->d_error, sh);
     return PE_OK;
   };
-  if (!t.out.start) return go(pe_eval_tile_kernel<CLS, EDGES, BY_POS, 0, MODE>);
-  if (t.flags & PE_TIMES_BY_OP) return go(pe_eval_tile_kernel<CLS, EDGES, BY_POS, 2, MODE>);
-  return go(pe_eval_tile_kernel<CLS, EDGES, BY_POS, 1, MODE>);
+  if (!t.out.start) return go(pe_eval_tile_kernel<CLS, EDGES, BY_POS, 0, MODE, WARPS>);
+  if (t.flags & PE_TIMES_BY_OP) return go(pe_eval_tile_kernel<CLS, EDGES, BY_POS, 2, MODE, WARPS>);
+  return go(pe_eval_tile_kernel<CLS, EDGES, BY_POS, 1, MODE, WARPS>);
+}
+
+template <int CLS, int EDGES, bool BY_POS, int MODE>
+int launch_tile3(const TileCall& t) {
+  // More registers gain nothing for a step with channels (within 3 %), and by position for one with branches or with
+  // durations by machine (V = 480 K = 32768 172 us with 128 registers, 178 with more; MoE graph 102 and 109).
+  constexpr bool kBoth = MODE != kTileExcl && !(BY_POS && (MODE == kTileHet || CLS == 1 || EDGES == 0));
+  if (kBoth && t.p->threads <= 32 * kTileWarps) return launch_tile4<CLS, EDGES, BY_POS, MODE, kBoth ? kTileWarps : 2 * kTileWarps>(t);
+  return launch_tile4<CLS, EDGES, BY_POS, MODE, 2 * kTileWarps>(t);
 }
 
 // EDGES specialisations (two or three inline edges and nothing else) exist for the modes that carry the main path.
