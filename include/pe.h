@@ -132,7 +132,8 @@ typedef struct {
 /* Bytes of device workspace pe_eval_batch needs for K candidates with these flags (may be 0). */
 size_t pe_workspace_bytes(const pe_graph* g, int64_t K, uint32_t flags);
 
-/* Which kernel variant (PE_VARIANT_*) a call with these arguments runs; negative = error code. */
+/* Which kernel variant (PE_VARIANT_*) a call with these arguments, 16-bit orders and start and finish wanted runs;
+ * negative = error code. */
 int pe_eval_variant(const pe_graph* g, int64_t K, uint32_t flags);
 
 /* Evaluate K candidates.  Asynchronous on `cuda_stream` (a cudaStream_t; NULL = default stream);

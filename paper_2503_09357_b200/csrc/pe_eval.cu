@@ -315,11 +315,15 @@ static bool plan_team(const pe_graph* g, int64_t K, bool allow_compact, Plan* p)
   // (measured at V = 4096 / D = 64: 4.46e10 with two warps, 4.36e10 with four, 3.3e10 with six; the MoE graph:
   // 2.03e10 against 1.96e10 and 1.63e10).
   // A batch that leaves SMs with fewer blocks than fit is bound by the latency of one block: more warps then.
+  // (Operators with more than three sources need more registers a thread, so fewer blocks of many warps fit: small batches
+  // of the MoE graphs, us with two / four / six warps: V = 2816 K = 1036 179 / 219 / 213, K = 888 155 / 142 / 201; V = 528
+  // K = 592 33 / 29 / 46.)
   size_t per_sm = (g->smem_per_sm ? g->smem_per_sm : g->smem_optin) / (smem + 1024);
   const size_t fair = (size_t)((K + g->sm_count - 1) / g->sm_count);
+  const size_t fewer = g->max_indeg > 3 && fair < per_sm ? 1 : 0;
   if (per_sm > fair) per_sm = fair;
   if (per_sm < 1) per_sm = 1;
-  const int nw = per_sm <= 4 ? 6 : (per_sm <= 7 ? 4 : 2);
+  const int nw = per_sm <= 4 - fewer ? 6 : (per_sm <= 7 - fewer ? 4 : 2);
   const size_t by_barriers = (size_t)64 / (nw == 6 ? 16 : 2 * nw + 1);
   if (per_sm > by_barriers) per_sm = by_barriers;
   if (per_sm * nw * 32 > 2048) per_sm = 2048 / (nw * 32);
@@ -395,24 +399,45 @@ static bool plan_global(const pe_graph* g, int64_t K, uint32_t flags, bool allow
   return true;
 }
 
-// Which of a lane (SHARED over the tile encoding), a block of warps (TEAM) and, for graphs that TEAM does not serve, a
-// warp per candidate is done first.  A lane takes ~0.1 us a position however few candidates there are, an SM holds
-// tile_resident of them; a block of warps takes ~0.026 us a position, and all SMs together evaluate `rate` positions a
-// microsecond, the fewer the deeper a window of 32 positions is (few operators per level of the graph, few machines) and
-// the more sources an operator has.  Measured (lane / team, us): V = 480 K = 1023 50 / 29, K = 3551 50 / 77; V = 1536
-// K = 1024 197 / 84, K = 65536 2554 / 3149; V = 1024 D = 8 K = 1000 105 / 49, K = 3000 92 / 107; V = 1024 D = 64
-// K = 524288 8578 / 10558; V = 1600 D = 64 K = 65536 2752 / 2030; V = 2116 D = 8 K = 65536 4186 / 3354; MoE graph
-// K = 16384 6200 / 2080.
-static double team_us(const pe_graph* g, int64_t K) {
-  const double V = g->V, width = V / g->levels;
-  const double rate = g->max_indeg > 3 ? 20000.0 : (width < 24.0 ? 32000.0 : (g->D < 32 ? 42000.0 : 51000.0));
-  return 10.0 + 0.026 * V + V * (double)K / rate;
+// AUTO takes the kernel that is estimated to be done first: a lane (SHARED over the tile encoding), a block of warps
+// (TEAM) or a warp (WARP) per candidate.  `times`: the call wants start and finish.  All figures in us, measured with
+// inputs and outputs in DRAM.
+//
+// A lane takes ~0.08 us a position however few candidates there are (0.18 where operators have more than three sources),
+// rounds of all resident tiles follow each other, and times by operator leave in a pass of their own.  Measured (estimate /
+// time): V = 1024 D = 64 K = 28036 432 / 461; V = 1369 D = 32 K = 14000 354 / 373; V = 1296 D = 8 K = 65536 1385 / 1215;
+// multi-modal graph V = 1536 K = 28036 894 / 1029.
+static double lane_us(const pe_graph* g, uint32_t flags, bool times, const Plan& lane) {
+  const double V = g->V, warps = lane.threads / 32;
+  const double step = (g->max_indeg > 3 ? 0.18 : (times ? 0.081 : 0.083)) * (warps > 4 ? 1.0 + 0.14 * (warps - 4.0) : 1.0);
+  return 5.0 + 0.012 * V + step * V * (double)lane.tile_rounds * (times && (flags & PE_TIMES_BY_OP) ? 1.55 : 1.0);
 }
-// (times by operator leave in a pass of their own: multi-modal graph K = 65536 3505 against 2844 us of TEAM)
-static double lane_us(const pe_graph* g, int64_t K, uint32_t flags, const Plan& lane) {
-  const double V = g->V, rounds = (double)K / ((double)lane.tile_resident * g->sm_count);
-  const double us = (g->max_indeg > 3 ? 0.15 : 0.103) * V * (rounds > 1.0 ? rounds : 1.0);
-  return 8.0 + ((flags & PE_TIMES_BY_OP) ? 1.35 : 1.0) * us;
+// A block of warps takes ~0.02 us a position, and all SMs together evaluate `rate` positions a microsecond, the fewer the
+// deeper a window of 32 positions is (few operators per level of the graph, few machines) and the more sources an operator
+// has; without staging copies every access touches a sector of its own.  Measured: V = 1600 D = 64 K = 14000 479 / 480,
+// without times 385 / 380; V = 1369 D = 32 K = 28036 841 / 828; MoE graph V = 2816 K = 16384 2121 / 1850; multi-modal
+// graph V = 2304 K = 28036 1960 / 1950; bidirectional pipeline V = 480 K = 2000 (direct) 53 / 61.
+static double team_us(const pe_graph* g, int64_t K, bool times, bool staged) {
+  const double V = g->V, width = V / g->levels;
+  double rate;
+  if (g->max_indeg > 3) rate = times ? 22500.0 : 25000.0;
+  else if (width < 24.0) rate = times ? 34000.0 : 38000.0;
+  else if (g->D < 32) rate = times ? 42000.0 : 48500.0;
+  else if (g->D < 64) rate = times ? 48000.0 : 58500.0;
+  else rate = times ? 51500.0 : 64500.0;
+  if (!staged) return 10.0 + 0.024 * V + V * (double)K / std::min(rate, 30000.0);
+  return 14.0 + (times ? 0.02 : 0.015) * V + V * (double)K / rate;
+}
+// A warp per candidate: rounds of all resident warps, a step of which takes the longer the more of them issue.  It comes
+// first only where whole levels of the graph fill its windows, enough warps fit and the rows of a batch are short enough
+// for its strided accesses.  Measured: V = 1600 D = 64 K = 3500 124 / 120, K = 7000 243 / 239; V = 1024 D = 64 K = 14000
+// without times 219 / 230; V = 1920 D = 16 K = 3500 176 / 168; at K = 65536 it takes up to 1.3 times as long a round.
+static double warp_us(const pe_graph* g, int64_t K, bool times, const Plan& w) {
+  const double V = g->V, n = w.threads / 32;
+  if (!w.compact || n < 20.0 || g->max_indeg > 3 || V / g->levels < 56.0 || K > 32768) return 1e30;
+  const int64_t per_round = (int64_t)(w.threads / 32) * g->sm_count;
+  const double step = (times ? 0.036 + 0.0016 * n : 0.028 + 0.0013 * n) * (g->D < 32 ? (times ? 1.2 : 1.35) : 1.0);
+  return 5.0 + step * V * (double)((K + per_round - 1) / per_round);
 }
 
 // Exclusive channels: a lane per candidate (~0.3 us a position where the channel words leave few lanes per SM) or the
@@ -427,8 +452,8 @@ static bool lane_pays_exclusive(const pe_graph* g, int64_t K, const Plan& lane) 
 }
 
 // allow_compact: the call can use the compact-graph kernels (u16 orders; start and finish both
-// wanted or both absent).  Size queries pass true and false and take the larger workspace.
-static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_compact, Plan* p) {
+// wanted or both absent).  times: start and finish are wanted.  Size queries take the largest workspace of all forms.
+static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_compact, bool times, Plan* p) {
   if (!g || K < 0) return PE_ERR_INVALID_ARG;
   if (flags & ~(uint32_t)(PE_ASSIGN_BY_POS | PE_TIMES_BY_OP | PE_COMM_EXCLUSIVE | PE_VARIANT_MASK)) return PE_ERR_INVALID_ARG;
   *p = Plan();
@@ -458,9 +483,15 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
       const bool has_s = plan_shared(g, K, flags, allow_compact, p) && (p->tiled || p->threads >= 48);
       const bool has_t = plan_team(g, K, allow_compact, &tm);
       if (has_s && !p->tiled) return PE_OK;
-      if (has_s && (!has_t || lane_us(g, K, flags, *p) <= team_us(g, K)) && (has_t || p->tile_resident >= 28)) return PE_OK;
-      if (has_t) { *p = tm; return PE_OK; }
       const bool has_w = plan_warp(g, K, flags, allow_compact, &w);
+      if (has_t) {
+        const double by_lane = has_s ? lane_us(g, flags, times, *p) : 1e30, by_team = team_us(g, K, times, tm.staged);
+        const double by_warp = has_w ? warp_us(g, K, times, w) : 1e30;
+        if (by_lane <= by_team && by_lane <= by_warp) return PE_OK;
+        *p = by_team <= by_warp ? tm : w;
+        return PE_OK;
+      }
+      if (has_s && p->tile_resident >= 28) return PE_OK;   // (28 lanes of the multi-modal graph beat 28 warps: 1029 / 1218 us)
       const bool has_g = plan_global(g, K, flags, allow_compact, &gl);
       // Graphs that TEAM does not serve (operators with more than eight sources, 32-bit orders, one of the times only):
       // a warp per candidate (state on chip) wins while at least four warps fit on an SM; for the largest graphs the
@@ -554,15 +585,18 @@ static int launch_typed(const pe_graph* g, const Plan& p, int64_t K, const uint8
 }  // namespace pe
 
 extern "C" size_t pe_workspace_bytes(const pe_graph* g, int64_t K, uint32_t flags) {
-  pe::Plan a, b;
-  const size_t wa = pe::make_plan(g, K, flags, true, &a) == PE_OK ? a.workspace : 0;
-  const size_t wb = pe::make_plan(g, K, flags, false, &b) == PE_OK ? b.workspace : 0;
-  return wa > wb ? wa : wb;
+  size_t most = 0;
+  for (const bool compact : {true, false})
+    for (const bool times : {true, false}) {
+      pe::Plan p;
+      if (pe::make_plan(g, K, flags, compact, times, &p) == PE_OK) most = std::max(most, p.workspace);
+    }
+  return most;
 }
 
 extern "C" int pe_eval_variant(const pe_graph* g, int64_t K, uint32_t flags) {
   pe::Plan p;
-  const int rc = pe::make_plan(g, K, flags, true, &p);
+  const int rc = pe::make_plan(g, K, flags, true, true, &p);
   return rc != PE_OK ? rc : p.variant;
 }
 
@@ -580,7 +614,7 @@ static int eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, const void*
   if (order_bytes == 2 && g->V > 65536) return PE_ERR_INVALID_ARG;
   pe::Plan p;
   const bool allow_compact = order_bytes == 2 && ((out->start != nullptr) == (out->finish != nullptr));
-  const int rc = pe::make_plan(g, K, flags, allow_compact, &p);
+  const int rc = pe::make_plan(g, K, flags, allow_compact, out->start != nullptr, &p);
   if (rc != PE_OK) return rc;
   if (K == 0) return PE_OK;
   if (!assign || !order) return PE_ERR_INVALID_ARG;

@@ -26,6 +26,7 @@ struct Plan {
   bool tiled = false;
   int tile_mode = 0;
   int tile_resident = 0;    // candidates an SM holds at once
+  int64_t tile_rounds = 0;  // tiles that a warp evaluates one after the other
   int64_t grid = 0;
   TileShape tile = {};
   // TEAM: inputs and times go through candidate-major staging copies in the workspace, a chunk of candidates at a time

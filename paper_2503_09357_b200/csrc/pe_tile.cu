@@ -54,6 +54,7 @@ bool plan_tile(const pe_graph* g, int64_t K, bool by_pos, bool exclusive, Plan* 
   const int64_t tiles = (K + (int64_t)bestP - 1) / (int64_t)bestP;
   const int64_t sms = g->sm_count;
   const int64_t rounds = (tiles + sms * (int64_t)bestW - 1) / (sms * (int64_t)bestW);
+  p->tile_rounds = rounds;
   if (rounds > 0) {
     const int64_t w = (tiles + sms * rounds - 1) / (sms * rounds);
     if (w < (int64_t)bestW) bestW = (size_t)w;

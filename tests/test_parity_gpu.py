@@ -552,3 +552,20 @@ def test_two_host_threads_share_a_graph(pe):
         assert not errors, errors
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("by_pos", [False, True])
+@pytest.mark.parametrize("V,D,K", [(1600, 64, 300), (1600, 64, 3500), (1024, 64, 5000), (784, 64, 2000)])
+def test_automatic_choice_with_and_without_times(pe, V, D, K, by_pos):
+    """Around the sizes where a lane, a warp and a block of warps per candidate take about the same time the choice
+    depends on the batch and on whether start and finish are wanted; the workspace of the size query serves both."""
+    w = wl.make_config(5, V=V, D=D)
+    assign, order = wl.make_candidates(w, K=K)
+    a = wl.assign_by_pos(assign, order) if by_pos else assign
+    g = pe.Graph(w)
+    try:
+        for want_times in (True, False):
+            gu.check(g, w, a, order, flags=pe.PE_ASSIGN_BY_POS if by_pos else 0, want_times=want_times,
+                     label=f"V {V} K {K} times {want_times}")
+    finally:
+        g.close()
