@@ -619,9 +619,16 @@ static int eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, const void*
   if (K == 0) return PE_OK;
   if (!assign || !order) return PE_ERR_INVALID_ARG;
   if ((K + p.threads - 1) / p.threads > (int64_t)INT_MAX) return PE_ERR_INVALID_ARG;
-  if (p.variant == PE_VARIANT_TEAM && p.staged && direct_ok && (!workspace || workspace_bytes < p.workspace)) {
-    p.staged = false;
-    p.workspace = 0;
+  if (p.variant == PE_VARIANT_TEAM && p.staged && (!workspace || workspace_bytes < p.workspace)) {
+    // The automatic choice may need a workspace for a small batch and none for a large one (a lane per candidate): a
+    // caller who sized it for the largest batch has none for the smaller ones either.
+    pe::Plan large;
+    if (!direct_ok && (flags & PE_VARIANT_MASK) == PE_VARIANT_AUTO)
+      direct_ok = pe::make_plan(g, (int64_t)1 << 24, flags, allow_compact, out->start != nullptr, &large) == PE_OK && large.workspace == 0;
+    if (direct_ok) {
+      p.staged = false;
+      p.workspace = 0;
+    }
   }
   if (p.workspace > 0 && (!workspace || workspace_bytes < p.workspace)) return PE_ERR_WORKSPACE;
   int prev = -1;

@@ -569,3 +569,28 @@ def test_automatic_choice_with_and_without_times(pe, V, D, K, by_pos):
                      label=f"V {V} K {K} times {want_times}")
     finally:
         g.close()
+
+
+def test_a_workspace_for_the_largest_batch_serves_smaller_ones(pe):
+    """V = 1024, D = 8: large batches run without workspace (a lane per candidate), small ones would stage copies in one."""
+    import torch
+    from oracle import pe_oracle as orc
+    w = wl.make_config(5, V=1024, D=8)
+    g = pe.Graph(w)
+    try:
+        assert pe.pe_workspace_bytes(g.handle, 65536, 0) == 0
+        for K in (1024, 2048):
+            assert pe.pe_workspace_bytes(g.handle, K, 0) > 0 and g.variant(K) == "team"
+            assign, order = wl.make_candidates(w, K=K)
+            out = g.alloc_outputs(K)
+            outs = pe.make_outputs(**{k: v.data_ptr() for k, v in out.items()})
+            a = torch.from_numpy(assign).cuda(); o = torch.from_numpy(gu.as_signed(order)).cuda()
+            assert pe.pe_eval_batch(g.handle, K, a.data_ptr(), o.data_ptr(), 2, 0, outs, 0, 0, 0) == pe.PE_OK
+            torch.cuda.synchronize()
+            res = {k: v.cpu().numpy() for k, v in out.items()}
+            res["status"] = res["status"].view(np.uint32)
+            gu.compare(res, orc.evaluate(w, assign, order, threads=gu.CPU_THREADS), f"K {K} without workspace")
+            # asked for by name the kernel still wants its workspace
+            assert pe.pe_eval_batch(g.handle, K, a.data_ptr(), o.data_ptr(), 2, pe.PE_VARIANT_TEAM, outs, 0, 0, 0) == pe.PE_ERR_WORKSPACE
+    finally:
+        g.close()
