@@ -336,16 +336,26 @@ __global__ void __launch_bounds__(kTopkBlock) pe_topk_write_kernel(int64_t K, co
   }
 }
 
-__global__ void pe_topk_fill_kernel(int32_t* out_index, int32_t k) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < k; i += gridDim.x * blockDim.x) out_index[i] = -1;
+__global__ void pe_topk_fill_kernel(int32_t* out_index, int64_t from, int64_t k) {
+  for (int64_t i = from + blockIdx.x * blockDim.x + threadIdx.x; i < k; i += gridDim.x * blockDim.x) out_index[i] = -1;
+}
+static void fill_rest(int32_t* out_index, int64_t from, int64_t k, cudaStream_t stream) {   // entries from .. k - 1
+  if (k <= from) return;
+  const int64_t want = (k - from + 255) / 256;
+  pe_topk_fill_kernel<<<(unsigned)(want < 256 ? want : 256), 256, 0, stream>>>(out_index, from, k);
 }
 
 // The whole selection in one block, for batches whose keys fit in shared memory.  Bound by the latency of a few block
 // barriers (a launch of its own per step, eleven in all, cost ~2 us each).  The histogram covers the range the values
-// have, not 32 bits: most batches need one or two rounds, and neighbouring values do not meet in one bin.
+// have, not 32 bits: most batches need one or two rounds, and neighbouring values do not meet in one bin.  Entries that
+// cannot be filled are set to -1 up to `fill`; one block writes ~60 GB/s, so lists beyond kOneFill leave the rest to a
+// launch with more blocks (K = 4096: k = 262144 22.6 -> 11.4 us, k = 4194304 272 -> 14.4 us; k = 40000 would take 10.4
+// instead of 8.3 us that way).
+constexpr int32_t kOneFill = 65536;
 __global__ void __launch_bounds__(1024) pe_topk_one_kernel(int K, const int32_t* __restrict__ makespan,
                                                            const uint32_t* __restrict__ status, uint32_t reject_mask, int32_t k,
-                                                           int32_t* __restrict__ out_index, int32_t* __restrict__ out_count) {
+                                                           int32_t fill, int32_t* __restrict__ out_index,
+                                                           int32_t* __restrict__ out_count) {
   extern __shared__ unsigned int keys[];   // makespan, or kNone where the candidate does not qualify
   constexpr unsigned int kNone = 0xFFFFFFFFu, FULL = 0xFFFFFFFFu;
   __shared__ unsigned int hist[kTopkBins];
@@ -434,7 +444,7 @@ __global__ void __launch_bounds__(1024) pe_topk_one_kernel(int K, const int32_t*
       before_b += better;
       before_e += equal;
     }
-  for (int i = (int)all + t; i < k; i += 1024) out_index[i] = -1;
+  for (int i = (int)all + t; i < fill; i += 1024) out_index[i] = -1;
   if (t == 0) *out_count = (int32_t)all;
 }
 
@@ -475,12 +485,16 @@ extern "C" int pe_select_topk(int64_t K, const int32_t* makespan, const uint32_t
     int ret = PE_OK;
     const size_t bytes = sizeof(unsigned int) * (size_t)(K > 0 ? K : 1);
     if (!pe::set_smem(pe::pe_topk_one_kernel, bytes)) ret = PE_ERR_CUDA;
-    else pe::pe_topk_one_kernel<<<1, 1024, bytes, stream>>>((int)K, makespan, status, reject_mask, k, out_index, out_count);
+    else {
+      const int32_t fill = k < pe::kOneFill ? k : pe::kOneFill;
+      pe::fill_rest(out_index, fill, k, stream);
+      pe::pe_topk_one_kernel<<<1, 1024, bytes, stream>>>((int)K, makespan, status, reject_mask, k, fill, out_index, out_count);
+    }
     if (cudaGetLastError() != cudaSuccess) ret = PE_ERR_CUDA;
     if (prev != attr.device) cudaSetDevice(prev);
     return ret;
   }
-  if (k > 0) pe::pe_topk_fill_kernel<<<(k + 255) / 256 > 256 ? 256 : (k + 255) / 256, 256, 0, stream>>>(out_index, k);
+  pe::fill_rest(out_index, 0, k, stream);
   pe::pe_topk_init_kernel<<<1, 256, 0, stream>>>(st, hist, (unsigned int)k);
   const int shifts[3] = {21, 10, 0}, bits[3] = {11, 11, 10};
   for (int p = 0; p < 3; ++p) {

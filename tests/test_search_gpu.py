@@ -80,3 +80,24 @@ def test_search_reaches_the_zero_bubble_of_the_two_stage_bidirectional_pipeline(
                   f"(Section V-A: best found PP/2-1 = {PP // 2 - 1}, DualPipe 2(PP/2-1) = {2 * (PP // 2 - 1)})")
         finally:
             g.close()
+
+
+@pytest.mark.parametrize("K,k", [(1, 5), (1000, 65535), (1000, 65537), (30000, 100001), (32768, 65536), (40000, 100000)])
+def test_topk_lists_longer_than_the_batch_are_padded(K, k):
+    """Every entry behind the qualifying candidates is -1, on both sides of the batch size that one block handles."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2503_09357_b200 import binding as pe
+    rs = np.random.RandomState(K)
+    mk = torch.from_numpy(rs.randint(0, 500, K).astype(np.int32)).cuda()
+    status = rs.randint(0, 3, K).astype(np.int32)
+    st = torch.from_numpy(status).cuda()
+    idx = torch.full((k,), 7, dtype=torch.int32, device="cuda"); cnt = torch.empty(1, dtype=torch.int32, device="cuda")
+    n = pe.pe_select_topk_workspace_bytes(K)
+    ws = torch.empty(max(n, 16), dtype=torch.uint8, device="cuda")
+    assert pe.pe_select_topk(K, mk.data_ptr(), st.data_ptr(), 0xFFFFFFFF, k, idx.data_ptr(), cnt.data_ptr(), ws.data_ptr(), n,
+                             torch.cuda.current_stream().cuda_stream) == pe.PE_OK
+    want = np.flatnonzero(status == 0)                                    # everything that qualifies, by index
+    got = idx.cpu().numpy()
+    assert int(cnt.item()) == len(want) and np.array_equal(got[:len(want)], want) and (got[len(want):] == -1).all()
