@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kLaneThreads) pe_decode_lane_kernel(PeFwdView 
         bad = bad || i[u] >= (uint32_t)V;
         const uint32_t op = min(i[u], (uint32_t)(V - 1));
         const uint32_t missing = head[op] >> 24;
-        bad = bad || word[op * kLaneThreads] != 0xFFFFu;   // twice (rank and count are never both 255: 255 missing need a 256th operator)
+        bad = bad || word[op * kLaneThreads] != 0xFFFFu;   // twice (0xFFFF is also what 255 missing at rank 255 make, but that is the last entry: nothing follows that could meet it)
         lst[r * kLaneThreads] = (uint8_t)op;
         word[op * kLaneThreads] = (uint16_t)(missing << 8 | (uint32_t)r);
         if (missing == 0u) add((uint32_t)r);
@@ -472,11 +472,18 @@ static bool plan_decode_lane(const pe_graph* g, int64_t K, DecodePlan* p) {
   if (V > 256 || E > 65535 || !g->fview.short_lists) return false;
   const size_t bytes = V * 4 + (V + 31) / 32 * kLaneThreads * 4 + V * kLaneThreads * 3 + (E + 3) / 4 * 4;
   if (bytes > g->smem_optin) return false;
-  // A lane takes ~0.1 us a placement and ~0.3 us a successor however few candidates there are; the warp kernel places
-  // ~18000 operators a microsecond.  Measured (lane / warp, us): V = 64 K = 8192 46 / 39, K = 32768 48 / 129; V = 256
-  // K = 8192 179 / 132, K = 32768 187 / 449, K = 131072 757 / 1706; tiny pipeline (one successor an operator)
-  // K = 1024 25 / 18, K = 8192 25 / 38.
-  if (0.1 * (double)V + 0.3 * (double)E > 6.0 + (double)V * (double)K / 18000.0) return false;
+  // A lane takes ~0.1 us a placement and ~0.3 us a successor, less (~0.12 us) for those beyond two an operator, which come
+  // without a placement of their own, however few candidates there are; the candidates that fit on chip go through in
+  // rounds.  The warp kernel places ~18000 operators a microsecond, the fewer the more successors they have.  Measured (lane
+  // / warp, us): V = 64, E = 56 K = 8192 28 / 39, K = 32768 31 / 126; V = 256, E = 483 K = 8192 181 / 135, K = 32768 188 /
+  // 446; V = 64, E = 819 K = 16384 108 / 88, K = 65536 122 / 311; V = 256, E = 6200 K = 65536 1696 / 1463; V = 128, E = 4146
+  // K = 131072 893 / 1667.
+  const double dV = (double)V, dE = (double)E, paired = std::min(dE, 2.0 * dV);
+  const int64_t resident = (int64_t)(g->smem_per_sm / (bytes + 1024)) * kLaneThreads * g->sm_count;
+  const double rounds = resident > 0 ? (double)((K + resident - 1) / resident) : 1e30;
+  const double by_lane = (0.1 * dV + 0.3 * paired + 0.12 * (dE - paired)) * rounds;
+  const double by_warp = 6.0 + dV * (double)K * (55.0 + 1.4 * dE / dV) * 1e-6;
+  if (by_lane > by_warp) return false;
   p->shared = p->lane = true;
   p->threads = kLaneThreads;
   p->smem = bytes;
