@@ -685,20 +685,22 @@ extern "C" int pe_eval_batch_host(pe_graph* g, int64_t K, const uint8_t* host_as
   // directions use separate DMA engines).  A chunk of Kc candidates lives in the staging buffers
   // as a dense [rows][Kc] block at element offset rows * first; the strided host side is handled
   // by 2-D copies.
-  // Shorter chunks shorten the ramp before the first download and after the last upload (the first and the last chunk
-  // are half the others for the same reason), but every chunk costs launches, and narrow rows copy more slowly.
+  // Shorter chunks shorten the ramp before the first download and after the last upload (up to eight chunks the first and
+  // the last are half the others for the same reason), but every chunk costs launches, and narrow rows copy more slowly.
   // Measured (ms, 1 / 3 / 5 / 8 / 16 chunks): MoE graph K = 16384 (500 MB moved) 11.3 / 8.5 / 8.2 / 8.5 / 8.8,
   // bidirectional pipeline K = 65536 (350 MB) 6.6 / 5.4 / 5.3 / 5.3 / 6.1, K = 8192 (44 MB) 0.88 / 0.81 / 0.84 / 0.93 /
-  // 1.09, K = 1024 (5 MB) 0.18 / 0.20 / 0.25 / 0.31 / 0.46; V = 16384 K = 65536 (12 GB): 16 beat 8 and 4.
+  // 1.09, K = 1024 (5 MB) 0.18 / 0.20 / 0.25 / 0.31 / 0.46; V = 16384 K = 65536 (12 GB): 16 beat 8 and 4, and sixteen
+  // equal ones (167) beat half-length first and last ones (184 on the same box).
   const size_t moved = V * Ks * (1 + ob + (host_out->start ? 4 : 0) + (host_out->finish ? 4 : 0));
   int nchunks = moved < ((size_t)24 << 20) ? 1 : (moved < ((size_t)64 << 20) ? 3 : 5);
-  if (K >= 32768) nchunks = 8;   // (rows stay wide)
+  if (K >= 32768) nchunks = 8;   // (the count that batches this wide have always had; below 24 MB fewer may be faster)
   if (moved >= ((size_t)4 << 30)) nchunks = 16;
   if (nchunks > (K + 63) / 64) nchunks = (int)((K + 63) / 64);
   int64_t begin[pe_graph::kMaxChunks + 1];
-  const int64_t halves = nchunks > 3 ? 2 * nchunks - 2 : 2 * nchunks;
+  const bool half_ends = nchunks > 3 && nchunks <= 8;
+  const int64_t halves = half_ends ? 2 * nchunks - 2 : 2 * nchunks;
   for (int q = 0; q <= nchunks; ++q) {
-    const int64_t at = nchunks > 3 ? (q == 0 ? 0 : 2 * q - 1) : 2 * q;
+    const int64_t at = half_ends ? (q == 0 ? 0 : 2 * q - 1) : 2 * q;
     begin[q] = q == nchunks ? K : K * at / halves / 64 * 64;
   }
   std::lock_guard<std::mutex> lock(g->host_mutex);

@@ -594,3 +594,34 @@ def test_a_workspace_for_the_largest_batch_serves_smaller_ones(pe):
             assert pe.pe_eval_batch(g.handle, K, a.data_ptr(), o.data_ptr(), 2, pe.PE_VARIANT_TEAM, outs, 0, 0, 0) == pe.PE_ERR_WORKSPACE
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("config,kw,K", [(2, {}, 16001), (5, dict(V=1024, D=8), 5000), (2, {}, 40001), (5, dict(V=4096, D=64), 96000)])
+def test_host_buffer_chunks_match_the_resident_batch(pe, config, kw, K):
+    """Five chunks with half-length ends; three chunks that stage copies by themselves but find no workspace, because the
+    whole batch needs none; eight chunks; sixteen equal ones.  Compared with pe_eval_batch on the same candidates."""
+    import torch
+    w = wl.make_config(config, **kw)
+    g = pe.Graph(w)
+    try:
+        gen = torch.Generator(device="cuda"); gen.manual_seed(K)
+        lists = torch.empty((w.num_ops, K), dtype=torch.int16, device="cuda")
+        for c in range(0, K, 8000):
+            n = min(8000, K - c)
+            lists[:, c:c + n] = torch.rand((n, w.num_ops), device="cuda", generator=gen).argsort(dim=1).to(torch.int16).t()
+        order, status = g.decode_priority(lists)
+        del lists
+        assign = torch.randint(0, w.num_devices, (w.num_ops, K), dtype=torch.uint8, device="cuda", generator=gen)
+        want = {k: v.cpu() for k, v in g.eval_batch(assign, order).items()}
+        h_a, h_o = assign.cpu().pin_memory(), order.cpu().pin_memory()
+        d_out = g.alloc_outputs(K)
+        h_out = {k: torch.full(v.shape, -7, dtype=v.dtype).pin_memory() for k, v in d_out.items()}
+        host, dev = (pe.make_outputs(**{k: v.data_ptr() for k, v in x.items()}) for x in (h_out, d_out))
+        n = pe.pe_workspace_bytes(g.handle, K, 0)
+        ws = torch.empty(max(n, 256), dtype=torch.uint8, device="cuda")
+        assert pe.pe_eval_batch_host(g.handle, K, h_a.data_ptr(), h_o.data_ptr(), 2, 0, host, assign.data_ptr(), order.data_ptr(),
+                                     dev, ws.data_ptr() if n else 0, n, torch.cuda.current_stream().cuda_stream) == pe.PE_OK
+        for k, v in want.items():
+            assert torch.equal(h_out[k], v), k
+    finally:
+        g.close()
