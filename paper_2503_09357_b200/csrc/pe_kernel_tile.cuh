@@ -43,9 +43,13 @@ constexpr int kTilePlain = 0;   // 32-bit state words
 constexpr int kTileS16 = 1;     // 16-bit state words
 constexpr int kTileExcl = 2;    // PE_COMM_EXCLUSIVE: the end of the last transfer per channel, [machine pair][P]
 constexpr int kTileHet = 3;     // durations by machine
+constexpr int kTileLong = 4;    // 32-bit state words, time bounds up to kPackedTimeLimit
+constexpr int kTileExclLong = 5;
 
-constexpr int64_t kTileTimeLimit = 0x7F0000;        // 32-bit words: end times stay below this
+constexpr int64_t kTileTimeLimit = 0x7FFFFF;        // 32-bit words: end times stay below this
 constexpr uint32_t kTileUnscheduled = 0x7FFFFF00u;  // | machine; sums with a delay and a duration do not wrap
+// Longer times leave no room above them: such a sum may wrap, so the words of the sources themselves are tested.
+constexpr uint32_t kTileUnscheduledLong = 0xFFFFFF00u;
 
 // Shared-memory accesses of the main loop by 32-bit address, in program order: the loads of a step go out before
 // its stores, those that the previous step's stores may feed first.
@@ -113,7 +117,9 @@ __global__ void __launch_bounds__(32 * WARPS) pe_eval_tile_kernel(PeTileView g, 
                                                            TileShape sh) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   constexpr uint32_t FULL = 0xFFFFFFFFu;
-  constexpr bool S16 = MODE == kTileS16, EXCL = MODE == kTileExcl, HET = MODE == kTileHet;
+  constexpr bool S16 = MODE == kTileS16, EXCL = MODE == kTileExcl || MODE == kTileExclLong, HET = MODE == kTileHet;
+  constexpr bool LONG = MODE == kTileLong || MODE == kTileExclLong;
+  constexpr uint32_t kUnsched32 = LONG ? kTileUnscheduledLong : kTileUnscheduled;
   using StateT = typename std::conditional<S16, uint16_t, uint32_t>::type;
   // Order entries (and by-position machine ids) per request.  A step with branches, or with channels or durations by
   // machine, is so long that sixteen of them are no longer inlined or overflow the instruction cache.
@@ -130,7 +136,7 @@ __global__ void __launch_bounds__(32 * WARPS) pe_eval_tile_kernel(PeTileView g, 
   const int P = sh.lanes;
   const uint32_t jb = S16 ? (uint32_t)sh.jbits : 8u;
   const uint32_t jmask = (1u << jb) - 1u;
-  const uint32_t unsched = S16 ? ((0xFFFFu >> jb) << jb) : kTileUnscheduled;
+  const uint32_t unsched = S16 ? ((0xFFFFu >> jb) << jb) : kUnsched32;
 
   {
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + g.bytes);
@@ -239,8 +245,8 @@ __global__ void __launch_bounds__(32 * WARPS) pe_eval_tile_kernel(PeTileView g, 
             raw_bad |= x[q] ^ xc;
             if (mine && row < V)
               sts128(words_a + (uint32_t)row * pitch,
-                     make_uint4(__byte_perm(xc, kTileUnscheduled, 0x7650), __byte_perm(xc, kTileUnscheduled, 0x7651),
-                                __byte_perm(xc, kTileUnscheduled, 0x7652), __byte_perm(xc, kTileUnscheduled, 0x7653)));
+                     make_uint4(__byte_perm(xc, kUnsched32, 0x7650), __byte_perm(xc, kUnsched32, 0x7651),
+                                __byte_perm(xc, kUnsched32, 0x7652), __byte_perm(xc, kUnsched32, 0x7653)));
           }
           __syncwarp();
         }
@@ -301,6 +307,7 @@ __global__ void __launch_bounds__(32 * WARPS) pe_eval_tile_kernel(PeTileView g, 
 
     // ---- main loop ----
     uint32_t st = 0;
+    uint32_t src_max = 0;                // LONG: largest word of a source
     uint32_t own_max = 0, dev_max = 0;   // own_max: the word a position finds for its operator, less `unsched`
     uint8_t* start_b = reinterpret_cast<uint8_t*>(out.start) + (size_t)cc * 4;     // this position's row
     uint8_t* finish_b = reinterpret_cast<uint8_t*>(out.finish) + (size_t)cc * 4;
@@ -352,6 +359,7 @@ __global__ void __launch_bounds__(32 * WARPS) pe_eval_tile_kernel(PeTileView g, 
       };
       // one source: its packed end time plus the delay that applies (Eqs. 11-13)
       auto source = [&](uint32_t pp, uint32_t ww, uint32_t dd) -> uint32_t {
+        if (LONG) src_max = max(src_max, ww);
         const bool same = ((ww ^ j) & jmask) == 0u;
         uint32_t d;
         bool channel = true;
@@ -504,7 +512,7 @@ __global__ void __launch_bounds__(32 * WARPS) pe_eval_tile_kernel(PeTileView g, 
     // 1248 us at V = 256, D = 8)
     uint32_t z = 0;
     for (int j = 0; j < D; ++j) z = max(z, (uint32_t)dev((uint32_t)j).x);
-    if (z >= unsched) st |= PE_STATUS_ORDER_INVALID;        // an operator ahead of one of its predecessors
+    if ((LONG ? src_max : z) >= unsched) st |= PE_STATUS_ORDER_INVALID;   // an operator ahead of one of its predecessors
     if (BY_POS) {
       if (dev_max > dmax) st |= PE_STATUS_ASSIGN_RANGE;
       // entries at positions that hold no operator are not consulted

@@ -9,7 +9,7 @@ inline size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 // Block shape: W warps of P lanes that together use the shared memory of an SM.
 bool plan_tile(const pe_graph* g, int64_t K, bool by_pos, bool exclusive, Plan* p) {
-  if (!g->tile_ok || K >= ((int64_t)1 << 26)) return false;   // (row pitches times the ring length are 32-bit)
+  if (!g->tile_ok || K >= ((int64_t)1 << 30)) return false;   // (row pitches in bytes are 32-bit)
   if (g->hetero && exclusive) return false;
   const PeTileView& tv = g->tview;
   int jb = 1;
@@ -18,7 +18,10 @@ bool plan_tile(const pe_graph* g, int64_t K, bool by_pos, bool exclusive, Plan* 
   if (g->hetero) mode = kTileHet;
   else if (exclusive) mode = kTileExcl;
   else if (jb < 16 && g->time_bound < ((int64_t)1 << (16 - jb)) - 1) mode = kTileS16;
-  if (mode != kTileS16 && g->time_bound >= kTileTimeLimit) return false;
+  if (mode != kTileS16 && g->time_bound >= kTileTimeLimit) {
+    if (g->hetero || g->time_bound >= kPackedTimeLimit) return false;
+    mode = exclusive ? kTileExclLong : kTileLong;
+  }
   const size_t fixed = up16((size_t)tv.bytes + 8);
   if (fixed >= g->smem_optin) return false;
   const size_t D = (size_t)g->D, rows = (size_t)g->V + 1;
@@ -92,6 +95,8 @@ int launch_tile(const pe_graph* g, const Plan& p, bool by_pos, int64_t K, const 
     case kTileS16: return by_pos ? launch_tile_pos_s16(t) : launch_tile_op_s16(t);
     case kTileExcl: return by_pos ? launch_tile_pos_excl(t) : launch_tile_op_excl(t);
     case kTileHet: return by_pos ? launch_tile_pos_het(t) : launch_tile_op_het(t);
+    case kTileLong:
+    case kTileExclLong: return by_pos ? launch_tile_pos_long(t) : launch_tile_op_long(t);
     default: return PE_ERR_UNSUPPORTED;
   }
 }

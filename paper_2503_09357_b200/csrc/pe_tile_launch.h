@@ -37,7 +37,7 @@ template <int CLS, int EDGES, bool BY_POS, int MODE>
 int launch_tile3(const TileCall& t) {
   // More registers gain nothing for a step with channels (within 3 %), and by position for one with branches or with
   // durations by machine (V = 480 K = 32768 172 us with 128 registers, 178 with more; MoE graph 102 and 109).
-  constexpr bool kBoth = MODE != kTileExcl && !(BY_POS && (MODE == kTileHet || CLS == 1 || EDGES == 0));
+  constexpr bool kBoth = MODE != kTileExcl && MODE != kTileExclLong && !(BY_POS && (MODE == kTileHet || CLS == 1 || EDGES == 0));
   if (kBoth && t.p->threads <= 32 * kTileWarps) return launch_tile4<CLS, EDGES, BY_POS, MODE, kBoth ? kTileWarps : 2 * kTileWarps>(t);
   return launch_tile4<CLS, EDGES, BY_POS, MODE, 2 * kTileWarps>(t);
 }
@@ -63,9 +63,11 @@ int launch_tile_op_plain(const TileCall& t);
 int launch_tile_op_s16(const TileCall& t);
 int launch_tile_op_excl(const TileCall& t);
 int launch_tile_op_het(const TileCall& t);
+int launch_tile_op_long(const TileCall& t);
 int launch_tile_pos_plain(const TileCall& t);
 int launch_tile_pos_s16(const TileCall& t);
 int launch_tile_pos_excl(const TileCall& t);
 int launch_tile_pos_het(const TileCall& t);
+int launch_tile_pos_long(const TileCall& t);
 
 }  // namespace pe

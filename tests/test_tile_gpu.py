@@ -84,3 +84,63 @@ def test_repetitions_behind_a_missing_source_are_flagged(dur, scale, by_pos):
         assert (ref["status"] & pe.PE_STATUS_ORDER_INVALID).all()
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("top,classes,indeg", [(0x7FFFFE, 1, 3), (0x7FFFFF, 1, 3), (0xFFFEFF, 1, 2), (0xFFFEFF, 2, 5), (0xFFFEFF, 3, 3)])
+def test_time_bounds_up_to_24_bits(top, classes, indeg):
+    """Sum of durations and delays just below and at the bound from which a sum with the unscheduled word may wrap, and at
+    the largest that fits a packed word: the lane kernel still serves them, with and without exclusive channels."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2503_09357_b200 import binding as pe
+    V, D, K = 300, 5, 130
+    w = chain_graph(V, D, indeg, classes, 2, seed=top % 97)
+    w.comm[:] = w.comm * 3000
+    rest = top - int(w.comm.max(axis=1).sum())
+    w.dur = np.full(V, rest // V, np.int32)
+    w.dur[V - 1] += rest - int(w.dur.sum())
+    assert w.dur.max() <= 65535 and int(w.dur.sum()) + int(w.comm.max(axis=1).sum()) == top
+    assign, order = wl.make_candidates(w, K=K)
+    order[5, 3] = order[4, 3]
+    order[:, 6] = order[::-1, 6].copy()
+    order[7, 9] = 65535
+    order[-140:, 12] = order[-141, 12]
+    g = pe.Graph(w)
+    try:
+        for flags in (0, pe.PE_ASSIGN_BY_POS, pe.PE_COMM_EXCLUSIVE, pe.PE_ASSIGN_BY_POS | pe.PE_COMM_EXCLUSIVE):
+            a = assign
+            if flags & pe.PE_ASSIGN_BY_POS:
+                a = np.take_along_axis(assign, np.minimum(order, V - 1).astype(np.int64), axis=0)
+            gu.check(g, w, a, order, flags=flags | pe.PE_VARIANT_SHARED, label=f"flags {flags}")
+            gu.check(g, w, a, order, flags=flags | pe.PE_VARIANT_SHARED | pe.PE_TIMES_BY_OP, label=f"flags {flags} by op")
+            gu.check(g, w, a, order, flags=flags, label=f"auto {flags}")
+    finally:
+        g.close()
+
+
+def test_more_candidates_than_2_to_the_26():
+    """Row pitches in bytes near the top of 32 bits' halves; two operators, so that the result can be written down."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2503_09357_b200 import binding as pe
+    K = (1 << 26) + 37
+    w = ck.problem(2, [], [3, 5], 2)
+    g = pe.Graph(w)
+    try:
+        gen = torch.Generator(device="cuda"); gen.manual_seed(1)
+        assign = torch.randint(0, 2, (2, K), dtype=torch.uint8, device="cuda", generator=gen)
+        order = torch.randint(0, 2, (1, K), dtype=torch.int16, device="cuda", generator=gen)
+        order = torch.cat([order, 1 - order])
+        for flags in (pe.PE_VARIANT_SHARED, pe.PE_VARIANT_SHARED | pe.PE_TIMES_BY_OP | pe.PE_COMM_EXCLUSIVE):
+            out = g.eval_batch(assign, order, flags=flags)
+            same = assign[0] == assign[1]
+            assert int(out["status"].abs().max()) == 0
+            assert torch.equal(out["makespan"], torch.where(same, 8, 5).to(torch.int32))
+            first = order[0] if not flags & pe.PE_TIMES_BY_OP else torch.zeros_like(order[0])
+            ahead = same & (order[0] != first)
+            want = torch.where(first == 0, 3, 5).to(torch.int32) + torch.where(ahead, torch.where(first == 0, 5, 3), 0).to(torch.int32)
+            assert torch.equal(out["finish"][0], want)
+    finally:
+        g.close()
