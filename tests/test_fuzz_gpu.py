@@ -68,3 +68,39 @@ def test_random_problems_match_the_oracle_in_every_variant(seed):
             assert np.array_equal(dorder.cpu().numpy().view(np.uint16), ref_order), f"seed {seed} decode {bit}"
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("seed", range(12))
+def test_random_problems_with_permuted_operator_ids(seed):
+    """The same problems with the operators renumbered: edges then run both ways in the numbering and operator 0 has
+    predecessors."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2503_09357_b200 import binding as pe
+    rs = np.random.RandomState(5000 + seed)
+    w = random_problem(rs)
+    V = w.num_ops
+    new = rs.permutation(V).astype(np.int32)                  # new id of every operator
+    if w.num_edges and rs.rand() < 0.7:                       # an operator with predecessors becomes operator 0
+        last = int(w.edge_dst[rs.randint(w.num_edges)])
+        new[np.flatnonzero(new == 0)[0]], new[last] = new[last], 0
+    old = np.argsort(new)
+    w.edge_src, w.edge_dst = new[w.edge_src], new[w.edge_dst]
+    w.dur, w.mem_delta = w.dur[old].copy(), w.mem_delta[old].copy()
+    if w.mem_weight is not None:
+        w.mem_weight = w.mem_weight[old].copy()
+    w.comm = w.comm * int(rs.choice([1, 100]))
+    K = int(rs.choice([1, 31, 97, 200]))
+    assign, order = wl.make_candidates(w, K=K, seed=seed)
+    base = int(rs.choice([0, pe.PE_ASSIGN_BY_POS, pe.PE_TIMES_BY_OP, pe.PE_ASSIGN_BY_POS | pe.PE_TIMES_BY_OP]))
+    a = wl.assign_by_pos(assign, order) if base & pe.PE_ASSIGN_BY_POS else assign
+    g = pe.Graph(w)
+    try:
+        for name, bit in (("auto", 0), ("global", pe.PE_VARIANT_GLOBAL), ("shared", pe.PE_VARIANT_SHARED),
+                          ("warp", pe.PE_VARIANT_WARP), ("team", pe.PE_VARIANT_TEAM), ("exclusive", pe.PE_COMM_EXCLUSIVE)):
+            if pe.pe_eval_variant(g.handle, K, base | bit) < 0:
+                continue
+            gu.check(g, w, a, order, flags=base | bit, want_times=bool(rs.rand() < 0.8), label=f"seed {seed} {name}")
+    finally:
+        g.close()

@@ -497,9 +497,9 @@ def test_many_sources_of_one_operator_inside_its_window(pe):
 
 @pytest.mark.parametrize("K", [333, 332])
 def test_team_kernel_with_and_without_staging_copies(pe, K):
-    """The block-per-candidate kernel reads the interleaved arrays directly when K is not a multiple of 4 (K = 333)
-    and goes through candidate-major staging copies otherwise (K = 332); both, in every layout, on a graph large
-    enough for it to be the automatic choice, and on the MoE graph (operators with eight incoming edges)."""
+    """The block-per-candidate kernel in every layout, with an odd batch and one that is a multiple of four: through
+    candidate-major staging copies on a graph of 4096 operators, and on the interleaved arrays directly on the MoE graph
+    (operators with eight incoming edges), whose batches are below 2^20 operator-evaluations."""
     for w in (wl.make_config(5, V=4096, D=8), wl.make_config(3)):
         assign, order = wl.make_candidates(w, K=K)
         g = pe.Graph(w)
@@ -623,5 +623,62 @@ def test_host_buffer_chunks_match_the_resident_batch(pe, config, kw, K):
                                      dev, ws.data_ptr() if n else 0, n, torch.cuda.current_stream().cuda_stream) == pe.PE_OK
         for k, v in want.items():
             assert torch.equal(h_out[k], v), k
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("config,kw,K", [(5, dict(V=4096, D=8), 200), (5, dict(V=4096, D=8), 201), (3, {}, 400), (3, {}, 401)])
+def test_team_kernel_on_the_other_side_of_the_staging_limit(pe, config, kw, K):
+    """V = 4096 without staging copies and the MoE graph with them, in every layout."""
+    w = wl.make_config(config, **kw)
+    assign, order = wl.make_candidates(w, K=K)
+    g = pe.Graph(w)
+    try:
+        staged = pe.pe_workspace_bytes(g.handle, K, pe.PE_VARIANT_TEAM) > 0
+        assert staged == (config == 3) == (w.num_ops * K >= 1 << 20)
+        for base in (0, pe.PE_ASSIGN_BY_POS, pe.PE_TIMES_BY_OP, pe.PE_ASSIGN_BY_POS | pe.PE_TIMES_BY_OP):
+            a = wl.assign_by_pos(assign, order) if base & pe.PE_ASSIGN_BY_POS else assign
+            gu.check(g, w, a, order, flags=base | pe.PE_VARIANT_TEAM, label=f"team K={K} flags={base}")
+        gu.check(g, w, assign, order, flags=pe.PE_VARIANT_TEAM, want_times=False, label=f"team K={K} summary")
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("by_pos,by_op_times,want_times", [(False, False, True), (True, True, True), (True, False, False)])
+def test_team_kernel_odd_batch_of_several_chunks(pe, by_pos, by_op_times, want_times):
+    """V = 16384 with an odd batch of more than two chunks: the unaligned transpositions start inside the rows, both halves
+    of the workspace and the side streams are used.  The same batch without workspace runs directly; both must agree,
+    and every 101st candidate with the oracle."""
+    import torch
+    from oracle import pe_oracle as orc
+    w = wl.make_config(5, V=16384, D=8)
+    K = 7107
+    g = pe.Graph(w)
+    try:
+        gen = torch.Generator(device="cuda"); gen.manual_seed(5)
+        lists = torch.rand((K, w.num_ops), device="cuda", generator=gen).argsort(dim=1).to(torch.int16).t().contiguous()
+        order, _ = g.decode_priority(lists)
+        assign = torch.randint(0, w.num_devices, (w.num_ops, K), dtype=torch.uint8, device="cuda", generator=gen)
+        flags = (pe.PE_ASSIGN_BY_POS if by_pos else 0) | (pe.PE_TIMES_BY_OP if by_op_times else 0)
+        a = assign.gather(0, order.long() & 0xFFFF) if by_pos else assign
+        need = pe.pe_workspace_bytes(g.handle, K, flags | pe.PE_VARIANT_TEAM)
+        assert 0 < need < K * w.num_ops * 11                     # two halves that hold fewer candidates than the batch
+        res = []
+        for ws_bytes in (need, 0):
+            out = g.alloc_outputs(K, want_times)
+            outs = pe.make_outputs(**{k: v.data_ptr() for k, v in out.items()})
+            ws = torch.empty(max(ws_bytes, 256), dtype=torch.uint8, device="cuda")
+            assert pe.pe_eval_batch(g.handle, K, a.data_ptr(), order.data_ptr(), 2, flags | pe.PE_VARIANT_TEAM, outs,
+                                    ws.data_ptr() if ws_bytes else 0, ws_bytes, torch.cuda.current_stream().cuda_stream) == pe.PE_OK
+            torch.cuda.synchronize()
+            res.append(out)
+        for k in res[0]:
+            assert torch.equal(res[0][k], res[1][k]), k
+        pick = torch.arange(0, K, 101, device="cuda")
+        part = {k: (v[pick] if v.dim() == 1 else v[:, pick]).cpu().numpy() for k, v in res[0].items()}
+        part["status"] = part["status"].view(np.uint32)
+        ref = orc.evaluate(w, a[:, pick].contiguous().cpu().numpy(), order[:, pick].contiguous().cpu().numpy().view(np.uint16),
+                           flags=flags & 7, want_times=want_times, threads=gu.CPU_THREADS)
+        gu.compare(part, ref, "slice")
     finally:
         g.close()

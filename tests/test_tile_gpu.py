@@ -144,3 +144,34 @@ def test_more_candidates_than_2_to_the_26():
             assert torch.equal(out["finish"][0], want)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("V,D,indeg,classes,scale,K,hetero", [
+    (48, 8, 2, 2, 4, 129, False), (49, 40, 3, 2, 30, 96, False), (256, 8, 3, 1, 4, 4741, False), (1500, 8, 3, 1, 40, 301, False),
+    (65, 5, 6, 1, 300, 33, True), (80, 6, 3, 3, 30, 300, True), (700, 12, 2, 2, 30, 201, True)])
+def test_every_form_runs_on_the_lane_kernel(V, D, indeg, classes, scale, K, hetero):
+    """Every layout of assignments and times on the lane kernel itself: the shared variant needs no workspace and, unlike
+    the generic kernel behind the same name, serves batches whose times are both wanted or both absent."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2503_09357_b200 import binding as pe
+    w = chain_graph(V, D, indeg, classes, scale, seed=7)
+    if hetero:
+        w.dur_by_machine = np.random.RandomState(V).randint(0, scale, (V, D)).astype(np.int32)
+    assign, order = wl.make_candidates(w, K=K)
+    order[5, 3] = order[4, 3]
+    order[7, 9] = 65535
+    assign[int(order[V // 2, 11]), 11] = 255
+    a_pos = np.take_along_axis(assign, np.minimum(order, V - 1).astype(np.int64), axis=0)
+    g = pe.Graph(w)
+    try:
+        base = (0, pe.PE_TIMES_BY_OP, pe.PE_ASSIGN_BY_POS, pe.PE_ASSIGN_BY_POS | pe.PE_TIMES_BY_OP)
+        exclusive = () if hetero or D > 32 or V > 1000 else tuple(f | pe.PE_COMM_EXCLUSIVE for f in base)
+        for flags in base + exclusive:
+            assert pe.pe_eval_variant(g.handle, K, flags | pe.PE_VARIANT_SHARED) == pe.PE_VARIANT_SHARED
+            for want_times in (True, False):
+                gu.check(g, w, a_pos if flags & pe.PE_ASSIGN_BY_POS else assign, order, flags=flags | pe.PE_VARIANT_SHARED,
+                         want_times=want_times, label=f"flags {flags} times {want_times}")
+    finally:
+        g.close()
