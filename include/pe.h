@@ -105,8 +105,8 @@ enum {
                                   warps prepare windows of the order side by side and only the recurrence of
                                   Eqs. 3, 7-8, 11-13 runs window after window.  For graphs with in-degree <= 8 and
                                   16-bit orders, with start and finish both wanted or both absent; otherwise
-                                  PE_ERR_UNSUPPORTED.  Uses workspace (staging copies) from K = 64 on; a K that is no multiple of 4
-                                  also runs, slower, without it */
+                                  PE_ERR_UNSUPPORTED.  Uses workspace (staging copies) from K = 64 and V * K = 2^20
+                                  on; a K that is no multiple of 4 also runs, slower, without it */
   PE_VARIANT_MASK = 15u << 8
 };
 
@@ -142,7 +142,8 @@ int pe_eval_variant(const pe_graph* g, int64_t K, uint32_t flags);
  *   order       device, [V*K] by-pos pi_c[k] at k*K + c; uint16_t if order_bytes == 2 (V <= 65536), uint32_t if 4
  *   out         outputs wanted (struct read during the call)
  *   workspace   device scratch of at least pe_workspace_bytes() bytes, 256-byte aligned; contents are
- *               overwritten; calls running concurrently must not share it
+ *               overwritten; calls running concurrently must not share it.  A workspace sized for the largest
+ *               batch of a program also serves its smaller ones
  * Precondition: every candidate's order is a topological permutation and every machine id < D;
  * violations are flagged per candidate in `status` and never index out of bounds. */
 int pe_eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, const void* order, int order_bytes, uint32_t flags,

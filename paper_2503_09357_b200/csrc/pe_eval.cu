@@ -416,7 +416,8 @@ static double lane_us(const pe_graph* g, uint32_t flags, bool times, const Plan&
 // deeper a window of 32 positions is (few operators per level of the graph, few machines) and the more sources an operator
 // has; without staging copies every access touches a sector of its own.  Measured: V = 1600 D = 64 K = 14000 479 / 480,
 // without times 385 / 380; V = 1369 D = 32 K = 28036 841 / 828; MoE graph V = 2816 K = 16384 2121 / 1850; multi-modal
-// graph V = 2304 K = 28036 1960 / 1950; bidirectional pipeline V = 480 K = 2000 (direct) 53 / 61.
+// graph V = 2304 K = 28036 1960 / 1950; direct: V = 480 K = 2000 56 / 61,
+// V = 576 K = 256 26 / 26, V = 64 K = 1024 10.2 / 9.2 (a lane: 11.0 / 10.2).
 static double team_us(const pe_graph* g, int64_t K, bool times, bool staged) {
   const double V = g->V, width = V / g->levels;
   double rate;
@@ -425,7 +426,7 @@ static double team_us(const pe_graph* g, int64_t K, bool times, bool staged) {
   else if (g->D < 32) rate = times ? 42000.0 : 48500.0;
   else if (g->D < 64) rate = times ? 48000.0 : 58500.0;
   else rate = times ? 51500.0 : 64500.0;
-  if (!staged) return 10.0 + 0.024 * V + V * (double)K / std::min(rate, 30000.0);
+  if (!staged) return 6.0 + 0.024 * V + V * (double)K / std::min(rate, 25000.0);
   return 14.0 + (times ? 0.02 : 0.015) * V + V * (double)K / rate;
 }
 // A warp per candidate: rounds of all resident warps, a step of which takes the longer the more of them issue.  It comes
@@ -446,7 +447,7 @@ static double warp_us(const pe_graph* g, int64_t K, bool times, const Plan& w) {
 // K = 16384 2049 / 2743; V = 400 D = 64 K = 8192 939 / 1348.
 static bool lane_pays_exclusive(const pe_graph* g, int64_t K, const Plan& lane) {
   if (!lane.tiled) return lane.threads >= 48;
-  if (lane.tile_resident >= 16) return true;
+  if (lane.tile_resident >= 16) return true;   // (multi-modal graph V = 1536, sixteen lanes: 1.71 against 2.74 ms at K = 16384)
   const double rounds = (double)K / ((double)lane.tile_resident * g->sm_count);
   return 0.3 * (rounds > 1.0 ? rounds : 1.0) < std::max(2.4, (double)K / 4500.0);
 }
@@ -458,7 +459,10 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
   if (flags & ~(uint32_t)(PE_ASSIGN_BY_POS | PE_TIMES_BY_OP | PE_COMM_EXCLUSIVE | PE_VARIANT_MASK)) return PE_ERR_INVALID_ARG;
   *p = Plan();
   const uint32_t want = flags & PE_VARIANT_MASK;
-  if (g->hetero) {   // machine-dependent durations: the generic one-thread-per-candidate kernels
+  // Machine-dependent durations: a lane per candidate wherever the tile encoding fits, however few lanes that leaves (V = 1369
+  // D = 64, four a SM: K = 4000 983 us against 6415 of the generic global-state kernel, K = 65536 15.4 against 27.2 ms; MoE
+  // graph K = 16384 12.0 against 22.6 ms), else the generic kernels.
+  if (g->hetero) {
     if (want == PE_VARIANT_WARP || want == PE_VARIANT_TEAM) return PE_ERR_UNSUPPORTED;
     if (!(flags & PE_COMM_EXCLUSIVE) && want != PE_VARIANT_GLOBAL && plan_shared(g, K, flags, allow_compact, p) &&
         (p->tiled || p->threads >= 48 || want == PE_VARIANT_SHARED))
@@ -467,8 +471,8 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
     return plan_global(g, K, flags, false, p) ? PE_OK : PE_ERR_UNSUPPORTED;
   }
   if (flags & PE_COMM_EXCLUSIVE) {
-    // exclusive channels: the compact shared-state kernel where a block of candidates still fits with one
-    // more word per machine pair each, else the generic global-state kernel
+    // exclusive channels: a lane per candidate with one more word per machine pair, or the global-state kernel (the
+    // compact one where the graph has that encoding)
     if (want == PE_VARIANT_AUTO || want == PE_VARIANT_SHARED) {
       if (plan_shared(g, K, flags, allow_compact, p) && (want == PE_VARIANT_SHARED || lane_pays_exclusive(g, K, *p))) return PE_OK;
       if (want == PE_VARIANT_SHARED) return PE_ERR_UNSUPPORTED;
@@ -515,6 +519,15 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
   }
 }
 
+// A call whose kernel the library chooses among lanes, warps and blocks of warps.
+static bool auto_choice(const pe_graph* g, int64_t K, uint32_t flags) {
+  return g && K >= 0 && (flags & PE_VARIANT_MASK) == PE_VARIANT_AUTO && !(flags & PE_COMM_EXCLUSIVE) && !g->hetero;
+}
+// Whether that choice needs no workspace for arbitrarily large batches.
+static bool large_batches_need_none(const pe_graph* g, uint32_t flags, bool times) {
+  Plan large;
+  return make_plan(g, (int64_t)1 << 24, flags, true, times, &large) == PE_OK && large.workspace == 0;
+}
 
 template <typename OrderT, bool BY_POS>
 static int launch_typed(const pe_graph* g, const Plan& p, int64_t K, const uint8_t* assign, const void* order,
@@ -591,6 +604,11 @@ extern "C" size_t pe_workspace_bytes(const pe_graph* g, int64_t K, uint32_t flag
       pe::Plan p;
       if (pe::make_plan(g, K, flags, compact, times, &p) == PE_OK) most = std::max(most, p.workspace);
     }
+  // Smaller batches than this one may stage copies where it does not (see eval_batch): room for those of K candidates.
+  pe::Plan tm;
+  if (pe::auto_choice(g, K, flags) && pe::plan_team(g, K, true, &tm) && tm.workspace > most &&
+      !(pe::large_batches_need_none(g, flags, true) && pe::large_batches_need_none(g, flags, false)))
+    most = tm.workspace;
   return most;
 }
 
@@ -622,9 +640,8 @@ static int eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, const void*
   if (p.variant == PE_VARIANT_TEAM && p.staged && (!workspace || workspace_bytes < p.workspace)) {
     // The automatic choice may need a workspace for a small batch and none for a large one (a lane per candidate): a
     // caller who sized it for the largest batch has none for the smaller ones either.
-    pe::Plan large;
-    if (!direct_ok && (flags & PE_VARIANT_MASK) == PE_VARIANT_AUTO)
-      direct_ok = pe::make_plan(g, (int64_t)1 << 24, flags, allow_compact, out->start != nullptr, &large) == PE_OK && large.workspace == 0;
+    if (!direct_ok && pe::auto_choice(g, K, flags))
+      direct_ok = pe::large_batches_need_none(g, flags, true) && pe::large_batches_need_none(g, flags, false);
     if (direct_ok) {
       p.staged = false;
       p.workspace = 0;

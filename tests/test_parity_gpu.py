@@ -682,3 +682,17 @@ def test_team_kernel_odd_batch_of_several_chunks(pe, by_pos, by_op_times, want_t
         gu.compare(part, ref, "slice")
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("V,D", [(1600, 64), (1024, 64), (1156, 64), (1024, 8), (256, 8)])
+def test_workspace_sizes_cover_smaller_batches(pe, V, D):
+    """Under the automatic choice a workspace for K candidates is enough for any fewer: the sizes do not fall, unless large
+    batches need none at all (smaller ones then run without)."""
+    w = wl.make_config(5, V=V, D=D)
+    g = pe.Graph(w)
+    try:
+        sizes = [64, 300, 700, 1024, 1500, 2000, 3500, 5000, 7000, 14000, 28036, 65536]
+        need = [pe.pe_workspace_bytes(g.handle, K, 0) for K in sizes]
+        assert need[-1] == 0 or need == sorted(need), dict(zip(sizes, need))
+    finally:
+        g.close()
