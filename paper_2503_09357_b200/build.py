@@ -9,7 +9,7 @@ CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libpe.so")
 SOURCES = ["pe_graph.cu", "pe_eval.cu", "pe_tile.cu"] + [f"pe_tile_{l}_{m}.cu" for l in ("op", "pos")
                                                          for m in ("plain", "s16", "excl", "het", "long")] + [
-    "pe_lane.cu", "pe_lane_op.cu", "pe_lane_pos.cu", "pe_warp2.cu", "pe_warp2_op.cu", "pe_warp2_pos.cu", "pe_team.cu",
+    "pe_slot.cu", "pe_slot_plain.cu", "pe_slot_excl.cu", "pe_slot_excl16.cu", "pe_slot_het.cu", "pe_lane.cu", "pe_lane_op.cu", "pe_lane_pos.cu", "pe_warp2.cu", "pe_warp2_op.cu", "pe_warp2_pos.cu", "pe_team.cu",
     "pe_team_nw2.cu", "pe_team_nw4.cu", "pe_team_nw6.cu", "pe_select.cu", "pe_decode.cu", "pe_coarsen.cu"]
 OBJ_DIR = os.path.join(_HERE, "_build")
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

@@ -452,9 +452,33 @@ static bool lane_pays_exclusive(const pe_graph* g, int64_t K, const Plan& lane) 
   return 0.3 * (rounds > 1.0 ? rounds : 1.0) < std::max(2.4, (double)K / 4500.0);
 }
 
+// The slot kernels: the gather takes ~430000 positions a microsecond, start and finish by operator 250000 (odd batches a
+// quarter longer), a step of the recurrence `base` or, with many warps on an SM, `per_warp` for each.  Measured (estimate /
+// time, us): multi-modal graph V = 1536 K = 4096 144 / 132, K = 65536 493 / 476, with exclusive channels K = 16384 549 / 507,
+// with durations by machine K = 65536 493 / 607; MoE graph V = 2816 K = 4096 523 / 511, K = 16384 607 / 734, times by operator
+// 795 / 894; pipeline V = 64 K = 16384 20 / 19, K = 65536 40 / 40.
+static double slot_us(const pe_graph* g, int64_t K, uint32_t flags, bool times, const Plan& s) {
+  const double V = g->V, cells = V * (double)K, warps = s.threads / 32;
+  const bool listed = g->sview.max_sources > (g->sview.cls_kind == 0 ? 3 : 2);
+  double base = listed ? (g->sview.max_sources <= 8 ? 0.172 : 0.3) : (g->sview.max_sources == 1 ? 0.06 : 0.075);
+  if (s.exclusive) base = listed ? 0.58 : 0.155;
+  if (g->hetero) base += 0.012;
+  const double step = std::max(base, (listed ? 0.021 : 0.0105) * warps), odd = K % 4 != 0 ? 1.25 : 1.0;
+  return 11.0 + odd * cells / 430e3 + V * step * (double)s.tile_rounds + (double)K * (g->D * 3.2e-6 + 1.3e-4) +
+         (times && (flags & PE_TIMES_BY_OP) ? 3.0 + odd * cells / 250e3 : 0.0);
+}
+// Estimated time of a plan that the automatic choice has made among the other kernels (a lane per candidate takes longer with
+// channel words, V = 1536 K = 1024 250 us, or durations by machine, 170 us).
+static double plan_us(const pe_graph* g, int64_t K, uint32_t flags, bool times, const Plan& p) {
+  if (p.variant == PE_VARIANT_TEAM) return team_us(g, K, times, p.staged);
+  if (p.variant == PE_VARIANT_WARP && p.compact) return warp_us(g, K, times, p);
+  if (p.tiled) return lane_us(g, flags, times, p) * (p.exclusive ? 2.0 : (g->hetero && g->max_indeg <= 3 ? 1.3 : 1.0));
+  return 1e30;
+}
+
 // allow_compact: the call can use the compact-graph kernels (u16 orders; start and finish both
 // wanted or both absent).  times: start and finish are wanted.  Size queries take the largest workspace of all forms.
-static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_compact, bool times, Plan* p) {
+static int plan_others(const pe_graph* g, int64_t K, uint32_t flags, bool allow_compact, bool times, Plan* p) {
   if (!g || K < 0) return PE_ERR_INVALID_ARG;
   if (flags & ~(uint32_t)(PE_ASSIGN_BY_POS | PE_TIMES_BY_OP | PE_COMM_EXCLUSIVE | PE_VARIANT_MASK)) return PE_ERR_INVALID_ARG;
   *p = Plan();
@@ -519,14 +543,25 @@ static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_co
   }
 }
 
+// allow_slot: the workspace is not known to be too small for the slot kernels.
+static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_compact, bool times, Plan* p, bool allow_slot = true) {
+  const int rc = plan_others(g, K, flags, allow_compact, times, p);
+  if (rc != PE_OK || !allow_slot || !allow_compact || K == 0 || (flags & PE_VARIANT_MASK) != PE_VARIANT_AUTO) return rc;
+  const double others = plan_us(g, K, flags, times, *p);
+  if (!g->slot_ok || others < 1.08 * (11.0 + (double)g->V * ((double)K / 430e3 + 0.06))) return PE_OK;   // (no plan to be made)
+  Plan s;
+  if (plan_slot(g, K, flags, times, &s) && 1.08 * slot_us(g, K, flags, times, s) < others) *p = s;
+  return PE_OK;
+}
+
 // A call whose kernel the library chooses among lanes, warps and blocks of warps.
 static bool auto_choice(const pe_graph* g, int64_t K, uint32_t flags) {
   return g && K >= 0 && (flags & PE_VARIANT_MASK) == PE_VARIANT_AUTO && !(flags & PE_COMM_EXCLUSIVE) && !g->hetero;
 }
-// Whether that choice needs no workspace for arbitrarily large batches.
+// Whether that choice, apart from the slot kernels, needs no workspace for arbitrarily large batches.
 static bool large_batches_need_none(const pe_graph* g, uint32_t flags, bool times) {
   Plan large;
-  return make_plan(g, (int64_t)1 << 24, flags, true, times, &large) == PE_OK && large.workspace == 0;
+  return make_plan(g, (int64_t)1 << 24, flags, true, times, &large, false) == PE_OK && large.workspace == 0;
 }
 
 template <typename OrderT, bool BY_POS>
@@ -539,6 +574,13 @@ static int launch_typed(const pe_graph* g, const Plan& p, int64_t K, const uint8
   if (p.compact) {
     if (sizeof(OrderT) != 2) return PE_ERR_INVALID_ARG;
     const uint16_t* ord16 = static_cast<const uint16_t*>(order);
+    if (p.slot) {
+      int64_t n = 0;
+      const int rc = launch_slot(g, p, BY_POS, K, assign, ord16, flags, out, workspace, stream, &n);
+      if (rc != PE_OK) return rc;
+      g_launches.fetch_add(n, std::memory_order_relaxed);
+      return cudaGetLastError() == cudaSuccess ? PE_OK : PE_ERR_CUDA;
+    }
     if (p.tiled) {
       const int rc = launch_tile(g, p, BY_POS, K, assign, ord16, flags, out, stream);
       if (rc != PE_OK) return rc;
@@ -607,8 +649,10 @@ extern "C" size_t pe_workspace_bytes(const pe_graph* g, int64_t K, uint32_t flag
   // Smaller batches than this one may stage copies where it does not (see eval_batch): room for those of K candidates.
   pe::Plan tm;
   if (pe::auto_choice(g, K, flags) && pe::plan_team(g, K, true, &tm) && tm.workspace > most &&
-      !(pe::large_batches_need_none(g, flags, true) && pe::large_batches_need_none(g, flags, false)))
+      (g->slot_ok || !(pe::large_batches_need_none(g, flags, true) && pe::large_batches_need_none(g, flags, false))))
     most = tm.workspace;
+  pe::Plan sl;
+  if (g && K > 0 && (flags & PE_VARIANT_MASK) == PE_VARIANT_AUTO && pe::plan_slot(g, K, flags, true, &sl) && sl.workspace > most) most = sl.workspace;
   return most;
 }
 
@@ -632,7 +676,11 @@ static int eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, const void*
   if (order_bytes == 2 && g->V > 65536) return PE_ERR_INVALID_ARG;
   pe::Plan p;
   const bool allow_compact = order_bytes == 2 && ((out->start != nullptr) == (out->finish != nullptr));
-  const int rc = pe::make_plan(g, K, flags, allow_compact, out->start != nullptr, &p);
+  int rc = pe::make_plan(g, K, flags, allow_compact, out->start != nullptr, &p);
+  if (rc == PE_OK && p.slot && (!workspace || workspace_bytes < p.workspace)) {   // the other kernels ask for less
+    p = pe::Plan();
+    rc = pe::make_plan(g, K, flags, allow_compact, out->start != nullptr, &p, false);
+  }
   if (rc != PE_OK) return rc;
   if (K == 0) return PE_OK;
   if (!assign || !order) return PE_ERR_INVALID_ARG;

@@ -93,6 +93,66 @@ int check_desc(const pe_graph_desc* d, int64_t* time_bound, int64_t* mem_bound, 
   return PE_OK;
 }
 
+// Slots for the slot encoding: operator s takes over the slot of operator p when all successors of p are s or ancestors of
+// s (their readings are over in every topological order by then); preferably that of one of its predecessors.  version[s]:
+// operators of its slot up to and including s, at most `longest`.  Returns the number of slots, or -1 when more than `most`
+// are needed.
+int32_t share_slots(int32_t V, const std::vector<int32_t>& sptr, const std::vector<int32_t>& succ, const PeOpRec* ops,
+                    const int32_t* pred, int32_t most, int32_t longest, std::vector<int32_t>* slot, std::vector<int32_t>* version) {
+  slot->assign(V, -1);
+  version->assign(V, 0);
+  const size_t words = ((size_t)V + 63) / 64;
+  std::vector<int32_t> deg(V), stack, tail;   // tail: last operator of every slot
+  std::vector<int32_t> unread(V), idle;       // successors of an operator still to come; slots whose tail has none
+  for (int32_t i = 0; i < V; ++i) unread[i] = sptr[i + 1] - sptr[i];
+  std::vector<uint64_t> anc((size_t)V * words, 0);
+  for (int32_t i = V - 1; i >= 0; --i) {
+    deg[i] = ops[i].indeg;
+    if (deg[i] == 0) stack.push_back(i);
+  }
+  while (!stack.empty()) {   // depth first: a chain of operators is followed to its end
+    const int32_t s = stack.back();
+    stack.pop_back();
+    uint64_t* a = anc.data() + (size_t)s * words;
+    const int32_t first = ops[s].edge_begin, last = ops[s].edge_begin + ops[s].indeg;
+    for (int32_t q = first; q < last; ++q) {
+      const uint64_t* b = anc.data() + (size_t)pred[q] * words;
+      for (size_t w = 0; w < words; ++w) a[w] |= b[w];
+      a[pred[q] / 64] |= 1ull << (pred[q] % 64);
+    }
+    auto free_for_s = [&](int32_t t) {   // every successor of the slot's tail is s or an ancestor of s
+      const int32_t p = tail[t];
+      if ((*version)[p] == longest || sptr[p] == sptr[p + 1]) return false;
+      for (int32_t q = sptr[p]; q < sptr[p + 1]; ++q)
+        if (succ[q] != s && !(a[succ[q] / 64] >> (succ[q] % 64) & 1u)) return false;
+      return true;
+    };
+    int32_t take = -1;
+    for (int32_t q = first; q < last && take < 0; ++q)
+      if (tail[(*slot)[pred[q]]] == pred[q] && free_for_s((*slot)[pred[q]])) take = (*slot)[pred[q]];
+    for (size_t t = 0; t < idle.size() && take < 0; ++t)
+      if (free_for_s(idle[t])) {
+        take = idle[t];
+        idle.erase(idle.begin() + (std::ptrdiff_t)t);
+      }
+    if (take < 0) {
+      if ((int32_t)tail.size() == most) return -1;
+      take = (int32_t)tail.size();
+      tail.push_back(s);
+      (*version)[s] = 1;
+    } else {
+      (*version)[s] = (*version)[tail[take]] + 1;
+      tail[take] = s;
+    }
+    (*slot)[s] = take;
+    for (int32_t q = first; q < last; ++q)
+      if (--unread[pred[q]] == 0 && tail[(*slot)[pred[q]]] == pred[q]) idle.push_back((*slot)[pred[q]]);
+    for (int32_t q = sptr[s]; q < sptr[s + 1]; ++q)
+      if (--deg[succ[q]] == 0) stack.push_back(succ[q]);
+  }
+  return (int32_t)tail.size();
+}
+
 std::vector<cudaEvent_t*> team_events(pe_graph* g) {
   return {&g->team_fork,    &g->team_join[0], &g->team_join[1], &g->team_join[2], &g->team_in[0],
           &g->team_in[1],   &g->team_done[0], &g->team_done[1], &g->team_back[0], &g->team_back[1]};
@@ -287,6 +347,109 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
       for (int64_t q = 0; q < (int64_t)V * D; ++q) ((uint16_t*)(tblob.data() + tv.durm))[q] = (uint16_t)d->dur_by_machine[q];
   }
 
+  // slot encoding
+  std::vector<uint8_t> sblob;
+  g->slot_ok = false;
+  g->d_sblob = nullptr;
+  std::memset(&g->sview, 0, sizeof(g->sview));
+  int64_t asum = 0;
+  int32_t longest_field = 1;   // of the durations and delays
+  for (int32_t i = 0; i < V; ++i) {
+    asum += std::abs((int64_t)ops[i].mem_delta);
+    for (int32_t j = 0; j < (g->hetero ? D : 1); ++j)
+      longest_field = std::max(longest_field, g->hetero ? d->dur_by_machine[(size_t)i * D + j] : ops[i].dur);
+  }
+  for (int64_t q = 0; q < (int64_t)E * L; ++q) longest_field = std::max(longest_field, comm[q]);
+  int vbits = 8;
+  while (vbits > 0 && (tb >= (int64_t)1 << (24 - vbits) || (int64_t)longest_field << vbits > 65535)) --vbits;
+  if (tile && V <= 4096 && asum < 32768 && vbits >= 4) {
+    std::vector<int32_t> sptr(V + 1, 0), succ(E), slot, version;
+    for (int32_t b = 0; b < E; ++b) sptr[d->edge_src[b] + 1]++;
+    for (int32_t i = 0; i < V; ++i) sptr[i + 1] += sptr[i];
+    std::vector<int32_t> fill(sptr.begin(), sptr.end() - 1);
+    for (int32_t b = 0; b < E; ++b) succ[fill[d->edge_src[b]]++] = d->edge_dst[b];
+    const int32_t n = share_slots(V, sptr, succ, ops, pred, V / 4, (1 << (vbits - 1)) - 1, &slot, &version);
+    if (n >= 0) {
+      g->slot_ok = true;
+      PeSlotView& sv = g->sview;
+      sv.V = V; sv.E = E; sv.D = D; sv.nslots = n;
+      sv.has_weight = g->has_weight ? 1 : 0;
+      sv.cls_kind = g->tview.cls_kind;
+      sv.vbits = vbits;
+      struct Source { uint32_t slot, c0, c1; };   // delays << vbits | version, per class
+      std::vector<std::vector<Source>> sources(V + 1);
+      std::vector<uint8_t> own_first(V + 1, 0);
+      sv.max_sources = 0;
+      for (int32_t i = 0; i < V; ++i) {
+        const uint32_t before = (uint32_t)version[i] - 1u;
+        bool chained = false;
+        for (int32_t q = ops[i].edge_begin; q < ops[i].edge_begin + ops[i].indeg; ++q)
+          chained = chained || (slot[pred[q]] == slot[i] && version[pred[q]] == version[i] - 1);
+        if (!chained) { sources[i].push_back({(uint32_t)slot[i], before, before}); own_first[i] = 1; }
+        for (int32_t q = ops[i].edge_begin; q < ops[i].edge_begin + ops[i].indeg; ++q) {
+          const uint32_t v = (uint32_t)version[pred[q]], c0 = (uint32_t)comm[(size_t)q * L], c1 = L == 2 ? (uint32_t)comm[(size_t)q * L + 1] : c0;
+          sources[i].push_back({(uint32_t)slot[pred[q]], c0 << vbits | v, c1 << vbits | v});
+        }
+        sv.max_sources = std::max(sv.max_sources, (int32_t)sources[i].size());
+      }
+      std::vector<uint32_t> list, list_at(V + 1, 0), rec((size_t)(V + 1) * 4, 0);
+      const bool padded = sv.max_sources <= 8;   // six places an operator, places without a source name row nslots
+      const Source none = {(uint32_t)n, 0u, 0u};
+      auto add_list = [&](const std::vector<Source>& src, size_t from) {
+        const size_t count = padded ? 6 : src.size() - from;
+        for (size_t q = 0; q < count; ++q) {
+          const Source& x = from + q < src.size() ? src[from + q] : none;
+          const uint32_t mark = q + 1 == count ? 0x1000u : 0u;
+          if (sv.cls_kind == 0) list.push_back(x.c0 << 16 | mark | x.slot);
+          else { list.push_back(mark | x.slot); list.push_back(x.c0 | x.c1 << 16); }
+        }
+        while (padded && list.size() % 4 != 0) list.push_back((uint32_t)n);
+      };
+      for (int32_t i = 0; i <= V; ++i) {   // (record V stands for entries that are no operator)
+        uint32_t* r = rec.data() + 4 * (size_t)i;
+        const std::vector<Source>& src = sources[i];
+        const uint32_t own = i < V ? (uint32_t)slot[i] : (uint32_t)n + 1u;
+        auto get = [&](size_t q) { return q < src.size() ? src[q] : none; };
+        r[0] = (own & 0xFFu) << 16;
+        if (i < V) r[0] |= (uint32_t)(uint8_t)(int8_t)ops[i].mem_delta << 24 | (uint32_t)(g->hetero ? 0 : ops[i].dur) << vbits | (uint32_t)version[i];
+        if (sv.cls_kind == 0) {
+          auto edge = [&](size_t q) { return get(q).c0 << 16 | get(q).slot; };
+          r[1] = edge(0) | (own >> 8) << 12;
+          r[2] = edge(1) | (src.size() > 3 ? 0x1000u : 0u) | (own_first[i] ? 0x2000u : 0u);
+          r[3] = src.size() > 3 ? (uint32_t)list.size() : edge(2);
+          if (src.size() > 3) add_list(src, 2);
+        } else {
+          r[1] = get(0).slot | (own >> 8) << 12 | get(1).slot << 16 | (src.size() > 2 ? 0x10000000u : 0u) | (own_first[i] ? 0x20000000u : 0u);
+          r[2] = get(0).c0 | get(0).c1 << 16;
+          r[3] = get(1).c0 | get(1).c1 << 16;
+          list_at[i] = (uint32_t)(list.size() / 2);
+          if (src.size() > 2) add_list(src, 2);
+        }
+      }
+      std::vector<uint16_t> dur16(V), durm16(g->hetero ? (size_t)(V + 1) * D : 0, 0);
+      for (int32_t i = 0; i < V; ++i) dur16[i] = (uint16_t)ops[i].dur;
+      if (g->hetero)
+        for (size_t q = 0; q < (size_t)V * D; ++q) durm16[q] = (uint16_t)(d->dur_by_machine[q] << vbits);
+      auto put = [&](const void* at, size_t bytes) {
+        const size_t off = sblob.size();
+        sblob.resize(align16(off + bytes), 0);
+        if (bytes) std::memcpy(sblob.data() + off, at, bytes);
+        return (uint32_t)off;
+      };
+      sv.ops = put(rec.data(), rec.size() * 4);
+      sv.list = put(list.data(), list.size() * 4);
+      sv.list_at = put(list_at.data(), list.empty() || sv.cls_kind == 0 ? 0 : list_at.size() * 4);
+      sv.cls = put(tblob.data() + g->tview.cls, sv.cls_kind == 1 ? (size_t)D * D : 0);
+      sv.cls_row = put(tblob.data() + g->tview.cls_row, sv.cls_kind == 2 ? (size_t)D * 4 : 0);
+      sv.cap = put(cap, (size_t)D * 4);
+      sv.durm = put(durm16.data(), durm16.size() * 2);
+      sv.bytes = (uint32_t)sblob.size();
+      sv.dur = put(dur16.data(), (size_t)V * 2);
+      sv.weight = put(d->mem_weight, g->has_weight ? (size_t)V * 4 : 0);
+      sv.total = (uint32_t)sblob.size();
+    }
+  }
+
   // forward view (successor lists) for priority-list decoding
   std::vector<uint8_t> fblob;
   g->fwd_ok = V <= 65536 && mdeg <= 255;
@@ -358,7 +521,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
     all.insert(all.end(), part.begin(), part.end());
     return at;
   };
-  const size_t at_blob = place(blob), at_n = place(nblob), at_t = place(tblob), at_f = place(fblob);
+  const size_t at_blob = place(blob), at_n = place(nblob), at_t = place(tblob), at_f = place(fblob), at_s = place(sblob);
   const size_t at_err = place(std::vector<uint8_t>(256, 0));
   int prev = -1, sms = 0, optin = 0, per_sm = 0;
   bool ok = cudaGetDevice(&prev) == cudaSuccess && cudaSetDevice(cuda_device) == cudaSuccess &&
@@ -376,6 +539,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
       g->d_nblob = narrow ? base + at_n : nullptr;
       g->d_tblob = tile ? base + at_t : nullptr;
       g->d_fwd = g->fwd_ok ? base + at_f : nullptr;
+      g->d_sblob = g->slot_ok ? base + at_s : nullptr;
       g->d_error = reinterpret_cast<int*>(base + at_err);
     }
     if (ok) {

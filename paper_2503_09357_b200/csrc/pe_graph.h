@@ -90,6 +90,40 @@ struct PeTileView {
   uint32_t bytes;      // total, multiple of 16
 };
 
+// Slot encoding, for graphs through which few results are alive at a time (see pe_kernel_slot.cuh): operators share
+// `nslots` state words.  Built when the tile encoding exists, V <= 4096, V / 4 slots are enough, the levels without weights
+// stay below 2^15, and durations, delays and the time bound leave `vbits` >= 4 bits for versions: times are kept in units of
+// 2^vbits, a field below stands for `value << vbits | version`.  One 16-byte record per operator, and record V for entries
+// that are no operator:
+//   x = (uint8)A << 24 | own slot (low byte) << 16 | dur, own version;  bits 12..15 of y = own slot >> 8
+//   one class, every pair connected (cls_kind 0):  y, z, w = sources 0, 1, 2 as (delay, version) << 16 | slot; bit 12 of z:
+//     more than three sources, w = place of source 2 in the list ((delay, version) << 16 | last << 12 | slot); bit 13: see below
+//   otherwise:  y = slot 0 | slot 1 << 16 | more than two sources << 28,  z, w = source 0, 1:  (delay, version) of class 0 |
+//     of class 1 << 16;  list_at[operator] = place of source 2 in the list ({last << 12 | slot, as z}); bit 29 of y: see below
+// Sources are the incoming edges.  An operator whose slot was not held by one of its predecessors has its own slot in front
+// of them, with the version of the operator that held it and no delay (that operator is an ancestor, or there was none):
+// bit 13 / 29.  With at most eight sources an operator's part of the list has six places (eight words or twelve).
+// Slot nslots stands for missing sources (it holds "ended at 0", version 0), nslots + 1 takes words that nobody reads.
+struct PeSlotView {
+  int32_t V, E, D;
+  int32_t nslots;
+  int32_t vbits;
+  int32_t has_weight;
+  int32_t cls_kind;    // as in PeTileView
+  int32_t max_sources;
+  uint32_t ops;        // uint4[V + 1]
+  uint32_t list;       // uint32[] or uint2[]
+  uint32_t list_at;    // uint32[V + 1] (class kinds 1 and 2 with a list)
+  uint32_t cls;        // uint8[D*D] (kind 1)
+  uint32_t cls_row;    // uint32[D] (kind 2)
+  uint32_t cap;        // int32[D]
+  uint32_t durm;       // uint16[(V + 1)*D], << vbits (heterogeneous machines)
+  uint32_t bytes;      // of the arrays above, which the recurrence keeps in shared memory; multiple of 16
+  uint32_t dur;        // uint16[V]
+  uint32_t weight;     // int32[V] if has_weight
+  uint32_t total;      // multiple of 16
+};
+
 // Forward view of the DAG for priority-list decoding, built when V <= 65536 and no operator has more than
 // 255 incoming edges.  Parallel edges count once (a predecessor is placed once).  One record per operator of
 // rec_bytes / 2 uint16: {n, successors 0 .. inl - 1, V} with inl = rec_bytes / 2 - 2, places without a successor hold V;
@@ -123,6 +157,9 @@ struct pe_graph {
   bool tile_ok;        // the tile encoding exists
   PeTileView tview;
   uint8_t* d_tblob;    // device copy of the tile encoding (nullptr if !tile_ok)
+  bool slot_ok;        // the slot encoding exists
+  PeSlotView sview;
+  uint8_t* d_sblob;    // device copy of the slot encoding (nullptr if !slot_ok)
   bool fwd_ok;         // the forward view exists
   PeFwdView fview;
   uint8_t* d_fwd;      // device copy of the forward view (nullptr if !fwd_ok)

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "pe_graph.h"
+#include "pe_slot_shape.h"
 #include "pe_tile_shape.h"
 
 namespace pe {
@@ -29,6 +30,13 @@ struct Plan {
   int64_t tile_rounds = 0;  // tiles that a warp evaluates one after the other
   int64_t grid = 0;
   TileShape tile = {};
+  // SHARED over the slot encoding (pe_eval_slot_kernel; tile_mode, tile_resident, tile_rounds as above): candidates of a
+  // chunk, row pitch and offsets of the workspace arrays, candidates per block of the kernels around it
+  bool slot = false;
+  int64_t slot_chunk = 0, slot_pitch = 0;
+  size_t slot_off_status = 0, slot_off_wsum = 0, slot_off_words = 0;
+  int slot_gather = 0, slot_times = 0;
+  SlotShape slot_shape = {};
   // TEAM: inputs and times go through candidate-major staging copies in the workspace, a chunk of candidates at a time
   bool staged = false;
   int64_t team_chunk = 0;   // candidates per chunk
@@ -52,6 +60,12 @@ static bool set_smem(Kern kern, size_t bytes) {
 bool plan_tile(const pe_graph* g, int64_t K, bool by_pos, bool exclusive, Plan* p);
 int launch_tile(const pe_graph* g, const Plan& p, bool by_pos, int64_t K, const uint8_t* assign, const uint16_t* order,
                 uint32_t flags, const pe_outputs& out, cudaStream_t stream);
+
+// pe_eval_slot_kernel (plan variant SHARED over the slot encoding) with the kernels around it; needs plan.workspace.
+// Adds the number of kernels it launched to *launches.
+bool plan_slot(const pe_graph* g, int64_t K, uint32_t flags, bool times, Plan* p);
+int launch_slot(const pe_graph* g, const Plan& p, bool by_pos, int64_t K, const uint8_t* assign, const uint16_t* order,
+                uint32_t flags, const pe_outputs& out, void* workspace, cudaStream_t stream, int64_t* launches);
 
 // pe_eval_lane_kernel (plan variant GLOBAL over the compact encoding; state in `gstate`).
 int launch_lane(const pe_graph* g, const Plan& p, bool by_pos, int64_t K, const uint8_t* assign, const uint16_t* order,

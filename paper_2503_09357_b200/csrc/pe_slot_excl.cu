@@ -1,0 +1,6 @@
+// Instantiations of pe_eval_slot_kernel: exclusive channels, 32-bit channel words.
+#include "pe_slot_launch.h"
+
+namespace pe {
+int launch_slot_excl(const SlotCall& t) { return launch_slot_mode<kSlotExcl>(t); }
+}  // namespace pe
