@@ -7,7 +7,7 @@
 // one of smallest rank comes next (Kahn's algorithm with the ranks as priorities).  The result is
 // a topological order of G_m, i.e. a valid `order` argument of pe_eval_batch.
 //
-// The set of available operators is kept by rank.  Two kernels:
+// The set of available operators is kept by rank.  Kernels:
 //
 // Warp per candidate (pe_decode_warp_kernel; per-operator state on chip).  Placing an operator is a chain of
 // dependent steps (smallest rank -> operator -> successors -> their counts -> new ranks), so the work is spread
@@ -31,6 +31,8 @@
 // with one summary word in a register; 3.1 bytes of state per operator (rank and missing predecessors in 16 bits, the
 // list in 8) let up to ~1000 candidates share an SM and hide the chain of a placement, bitmap -> list -> successor
 // list -> counts, about five shared-memory round trips.
+//
+// Lane per candidate with a pool (pe_decode_pool_kernel, see there): graphs that a few chains of operators cover.
 //
 // Thread per candidate (pe_decode_kernel; for graphs whose per-candidate state does not fit on chip, V above
 // ~55000, or on request).  The bitmap has two summary levels above it (one bit per 32-bit word of the level below;
@@ -432,9 +434,175 @@ __global__ void __launch_bounds__(kLaneThreads) pe_decode_lane_kernel(PeFwdView 
   }
 }
 
+// Shared-memory accesses by 32-bit address, in program order.
+__device__ __forceinline__ uint32_t smem_get8(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t smem_get16(uint32_t a) {
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t smem_get32(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint2 smem_get64(uint32_t a) {
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint4 smem_get128(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void smem_put8(uint32_t a, uint32_t v) { asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v)); }
+__device__ __forceinline__ void smem_put16(uint32_t a, uint32_t v) { asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v)); }
+__device__ __forceinline__ void smem_put32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v)); }
+__device__ __forceinline__ void smem_put32_if(uint32_t a, uint32_t v, bool on) {
+  asm volatile("{.reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u32 [%0], %1;}" ::"r"(a), "r"(v), "r"((uint32_t)on));
+}
+__device__ __forceinline__ void smem_put128(uint32_t a, uint4 v) {
+  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
+}
+
+// Shape of a pe_decode_pool_kernel launch: warps take tiles of `lanes` candidates.
+struct PoolShape {
+  int lanes;
+  int64_t tiles;
+  uint32_t off_state;     // state of warp 0: pool, ranks, counts
+  uint32_t state_bytes;   // per warp
+  uint32_t off_rank, off_cnt;
+};
+
+// Lane per candidate with a pool (pe_decode_pool_kernel): graphs that at most 32 chains cover (two operators
+// of a chain, one an ancestor of the other, are never available together).  The available operators stand in shared memory, [place / 4][lane][4], as rank << 17 |
+// place << 12 | operator; a lane reads all places to find the smallest rank, three instructions for four places.
+//   rank[i]   u16 [operator][lane]: rank of operator i
+//   cnt[j]    u8 [join][lane]: predecessors still missing, less one, of the operators that have several; row num_joins
+//             stands for all others (always 0), row num_joins + 1 takes what they write
+// Every turn of the loop hands one successor of the operator placed last its "one predecessor fewer" and, once that
+// operator's list is used up, places the next one.  A turn has no branch (32 candidates would take every side of each: a
+// first version with them took 730 cycles a turn), and the pool is read while the successor's rank is on its way: what
+// is released in this turn is compared with what was in the pool before.
+// What bounds it: the chain operator -> record -> rank of its successor, two shared-memory round trips, with the few warps
+// that fit (2 bytes an operator and candidate): ~110 ns a turn.  Measured (us, warp kernel or lane kernel with a bitmap
+// before): multi-modal graph V = 1536 K = 8192 834 -> 195, K = 64 228 -> 193; MoE graph V = 2816 K = 8192 2879 -> 1232;
+// pipeline V = 256 K = 16384 103 -> 45.
+template <int QUADS>
+__global__ void __launch_bounds__(512, 1) pe_decode_pool_kernel(PeFwdView f, const uint8_t* __restrict__ fblob, int64_t K,
+                                                                const uint16_t* __restrict__ list, uint16_t* __restrict__ order,
+                                                                uint32_t* __restrict__ status, PoolShape sh, int* err) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int V = f.V, P = sh.lanes;
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), nwarps = blockDim.x >> 5;
+  {
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + f.pool_bytes);
+    if (!stage_blob(smem_raw, fblob + f.prec, f.pool_bytes, bar, err)) return;
+  }
+  const uint32_t smem_a = smem_u32(smem_raw), more_a = smem_a + f.pmore;
+  const uint16_t* roots = reinterpret_cast<const uint16_t*>(smem_raw + f.roots);
+  const uint8_t* first = smem_raw + f.joins;
+  const uint32_t mine = smem_a + sh.off_state + (uint32_t)warp * sh.state_bytes;
+  const uint32_t pool_a = mine + (uint32_t)lane * 16u, qpitch = (uint32_t)P * 16u;   // bytes of a row of four places
+  const uint32_t rank_a = mine + sh.off_rank + (uint32_t)lane * 2u, rpitch = (uint32_t)P * 2u;
+  const uint32_t cnt_a = mine + sh.off_cnt + (uint32_t)lane, cpitch = (uint32_t)P;
+  auto place_at = [&](uint32_t t) { return pool_a + (t >> 2) * qpitch + (t & 3u) * 4u; };
+  const uint32_t K2 = (uint32_t)K * 2u, joins = (uint32_t)f.num_joins, vlast = (uint32_t)(V - 1);
+
+  for (int64_t tile = (int64_t)warp * gridDim.x + blockIdx.x; tile < sh.tiles; tile += (int64_t)nwarps * gridDim.x) {
+    const int64_t c = tile * P + lane;
+    if (lane >= P || c >= K) continue;   // (the lanes of a warp have nothing to do with each other)
+#pragma unroll
+    for (int q = 0; q < QUADS; ++q) smem_put128(pool_a + (uint32_t)q * qpitch, make_uint4(kNoKey, kNoKey, kNoKey, kNoKey));
+    for (int i = 0; i < V; ++i) smem_put16(rank_a + (uint32_t)i * rpitch, 0xFFFFu);
+    for (uint32_t j = 0; j < joins + 1u; ++j) smem_put8(cnt_a + j * cpitch, j < joins ? (uint32_t)first[j] : 0u);
+
+    // the list: the operators' ranks; an operator twice, or an entry that is none, leaves another one out
+    {
+      const uint8_t* at = reinterpret_cast<const uint8_t*>(list + c);
+      constexpr int kBatch = 64;   // (few warps: what is in flight decides; rows of 16 took 40 us at V = 1536)
+      int r0 = 0;
+      for (; r0 + kBatch <= V; r0 += kBatch) {
+        uint32_t i[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) i[u] = __ldg(reinterpret_cast<const uint16_t*>(at + (uint64_t)(uint32_t)(r0 + u) * K2));
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u)
+          if (i[u] < (uint32_t)V) smem_put16(rank_a + i[u] * rpitch, (uint32_t)(r0 + u));
+      }
+#pragma unroll 8
+      for (; r0 < V; ++r0) {
+        const uint32_t i = __ldg(reinterpret_cast<const uint16_t*>(at + (uint64_t)(uint32_t)r0 * K2));
+        if (i < (uint32_t)V) smem_put16(rank_a + i * rpitch, (uint32_t)r0);
+      }
+    }
+    uint32_t most = 0;
+#pragma unroll 16
+    for (int i = 0; i < V; ++i) most = max(most, smem_get16(rank_a + (uint32_t)i * rpitch));
+    const bool bad = most == 0xFFFFu;
+    if (status) status[c] = bad ? (uint32_t)PE_STATUS_ORDER_INVALID : 0u;
+    if (bad) continue;   // not a permutation: the order of this candidate stays unwritten
+
+    uint32_t open = f.num_roots < 32 ? ~0u << f.num_roots : 0u;   // free places
+    for (uint32_t t = 0; t < (uint32_t)f.num_roots; ++t) {
+      const uint32_t i = roots[t];
+      smem_put32(place_at(t), smem_get16(rank_a + i * rpitch) << 17 | t << 12 | i);
+    }
+    uint8_t* out = reinterpret_cast<uint8_t*>(order + c);
+    int k = 0;
+    uint32_t left = 0, succ = 0xFFFF0000u, more = more_a;   // of the operator placed last: successors to come, the next one, where the others are
+    for (int it = 0; it < f.turns + 1 && k < V; ++it) {     // (one turn a successor, one for an operator without, one to begin with)
+      const bool has = left != 0u;
+      const uint32_t s = succ & 0xFFFFu, j = succ >> 16;
+      const bool join = j != 0xFFFFu;
+      const uint32_t r = smem_get16(rank_a + s * rpitch);
+      const uint32_t m = smem_get8(cnt_a + (join ? j : joins) * cpitch);
+      const uint32_t succ_more = smem_get32(more);
+      uint4 p[QUADS];
+#pragma unroll
+      for (int q = 0; q < QUADS; ++q) p[q] = smem_get128(pool_a + (uint32_t)q * qpitch);
+      smem_put8(cnt_a + (join && has ? j : joins + 1u) * cpitch, m - 1u);
+      const bool freed = has && m == 0u;
+      const uint32_t t = (uint32_t)__ffs((int)open) - 1u;
+      const uint32_t fresh = r << 17 | t << 12 | s;
+      smem_put32_if(place_at(t & 31u), fresh, freed);
+      open = freed ? open & (open - 1u) : open;
+      left -= has ? 1u : 0u;
+      succ = succ_more;
+      more += has ? 4u : 0u;
+      uint32_t rest[QUADS];
+#pragma unroll
+      for (int q = 0; q < QUADS; ++q) rest[q] = min(min(p[q].x, p[q].y), min(p[q].z, p[q].w));
+#pragma unroll
+      for (int q = 1; q < QUADS; ++q) rest[0] = min(rest[0], rest[q]);
+      const uint32_t key = min(rest[0], freed ? fresh : kNoKey);
+      const bool pop = left == 0u;   // (some operator is available until the last one is placed)
+      const uint32_t i = min(key & 0xFFFu, vlast), at = (key >> 12) & 31u;
+      smem_put32_if(place_at(at), kNoKey, pop);
+      const uint2 rec = smem_get64(smem_a + i * 8u);
+      if (pop) *reinterpret_cast<uint16_t*>(out) = (uint16_t)i;
+      out += pop ? K2 : 0u;
+      k += pop ? 1 : 0;
+      open |= pop ? 1u << at : 0u;
+      succ = pop ? rec.x : succ;
+      left = pop ? rec.y >> 24 : left;
+      more = pop ? more_a + (rec.y & 0xFFFFFFu) * 4u : more;
+    }
+  }
+}
+
 struct DecodePlan {
   bool shared = false;      // per-operator state on chip
-  bool lane = false;        // pe_decode_lane_kernel, otherwise pe_decode_warp_kernel
+  bool lane = false;        // pe_decode_lane_kernel
+  bool pool = false;        // pe_decode_pool_kernel, otherwise pe_decode_warp_kernel
+  PoolShape shape = {};
+  int64_t grid = 0;
+  double us = 1e30;         // estimated time
   bool rec_smem = false;    // operator records in shared memory
   int threads = 0;
   uint32_t words = 0;       // shared words per warp
@@ -464,6 +632,11 @@ static bool plan_decode_warp(const pe_graph* g, int64_t K, DecodePlan* p) {
     p->smem = bytes;
   }
   p->shared = best > 0;
+  // bound by issue, or by the chain of a placement (longer where the records are not on chip)
+  const double dV = (double)V, dK = (double)K, per_sm = std::max(1.0, dK / (double)g->sm_count);
+  if (best > 0)
+    p->us = 6.0 + std::max(dV * dK * (55.0 + 1.4 * g->fview.E / dV) * 1e-6,
+                           dV * (p->rec_smem ? 0.142 : 0.33) * per_sm / std::min(per_sm, (double)best));
   return p->shared;
 }
 
@@ -484,9 +657,46 @@ static bool plan_decode_lane(const pe_graph* g, int64_t K, DecodePlan* p) {
   const double by_lane = (0.1 * dV + 0.3 * paired + 0.12 * (dE - paired)) * rounds;
   const double by_warp = 6.0 + dV * (double)K * (55.0 + 1.4 * dE / dV) * 1e-6;
   if (by_lane > by_warp) return false;
+  p->us = by_lane;
   p->shared = p->lane = true;
   p->threads = kLaneThreads;
   p->smem = bytes;
+  return true;
+}
+
+// Measured (estimate / time, us): V = 1536 K = 8192 182 / 195, K = 16384 357 / 390; V = 2304 K = 4096 289 / 463; V = 2816
+// K = 4096 581 / 619.
+static bool plan_decode_pool(const pe_graph* g, int64_t K, DecodePlan* p) {
+  const PeFwdView& f = g->fview;
+  if (!f.pool_bytes || K < 1 || K >= ((int64_t)1 << 30)) return false;
+  const size_t V = (size_t)g->V, fixed = ((size_t)f.pool_bytes + 8 + 15) / 16 * 16;
+  auto bytes = [&](size_t P) { return (P * (4 * (size_t)f.places + 2 * V + (size_t)f.num_joins + 2) + 15) / 16 * 16; };
+  size_t bestW = 0, bestP = 0;
+  for (size_t W = 1; W <= 16; ++W)
+    for (size_t P = 32; P >= 4; P -= 4)
+      if (fixed + W * bytes(P) <= g->smem_optin) {
+        if (W * P > bestW * bestP) { bestW = W; bestP = P; }
+        break;
+      }
+  if (bestW == 0) return false;
+  const int64_t sms = g->sm_count, tiles = (K + (int64_t)bestP - 1) / (int64_t)bestP;
+  const int64_t rounds = (tiles + sms * (int64_t)bestW - 1) / (sms * (int64_t)bestW);
+  const int64_t w = (tiles + sms * rounds - 1) / (sms * rounds);
+  if (w < (int64_t)bestW) bestW = (size_t)w;
+  const double turn = std::max(0.085 + 0.001 * f.places, 0.03 * (double)bestW);
+  p->us = 8.0 + (0.012 * (double)V + turn * (double)f.turns) * (double)rounds;
+  p->shared = p->pool = true;
+  p->rec_smem = false;
+  p->threads = (int)(32 * bestW);
+  p->grid = std::min(tiles, sms);
+  PoolShape& sh = p->shape;
+  sh.lanes = (int)bestP;
+  sh.tiles = tiles;
+  sh.off_state = (uint32_t)fixed;
+  sh.state_bytes = (uint32_t)bytes(bestP);
+  sh.off_rank = (uint32_t)(bestP * 4 * (size_t)f.places);
+  sh.off_cnt = sh.off_rank + (uint32_t)((bestP * 2 * V + 3) / 4 * 4);
+  p->smem = fixed + bestW * bytes(bestP);
   return true;
 }
 
@@ -495,7 +705,10 @@ static bool decode_plan(const pe_graph* g, int64_t K, uint32_t flags, DecodePlan
   const uint32_t want = flags & PE_VARIANT_MASK;
   const size_t V = (size_t)g->V, n0 = (V + 31) / 32, n1 = (n0 + 31) / 32;
   if (want == PE_VARIANT_AUTO || want == PE_VARIANT_SHARED) {
-    if (plan_decode_lane(g, K, p) || plan_decode_warp(g, K, p)) return true;
+    DecodePlan pool;
+    if (!plan_decode_lane(g, K, p)) plan_decode_warp(g, K, p);
+    if (plan_decode_pool(g, K, &pool) && pool.us < p->us) *p = pool;
+    if (p->shared) return true;
     if (want == PE_VARIANT_SHARED) return false;
   }
   if (want != PE_VARIANT_AUTO && want != PE_VARIANT_GLOBAL) return false;
@@ -546,6 +759,10 @@ extern "C" int pe_decode_priority(pe_graph* g, int64_t K, const void* list, int 
     auto kern = pe::pe_decode_lane_kernel;
     if (!pe::set_smem(kern, p.smem)) ret = PE_ERR_CUDA;
     else kern<<<(unsigned)((K + p.threads - 1) / p.threads), p.threads, p.smem, stream>>>(g->fview, g->d_fwd, K, list16, order16, status);
+  } else if (p.pool) {
+    auto kern = g->fview.places <= 8 ? pe::pe_decode_pool_kernel<2> : (g->fview.places <= 16 ? pe::pe_decode_pool_kernel<4> : (g->fview.places <= 24 ? pe::pe_decode_pool_kernel<6> : pe::pe_decode_pool_kernel<8>));
+    if (!pe::set_smem(kern, p.smem)) ret = PE_ERR_CUDA;
+    else kern<<<(unsigned)p.grid, p.threads, p.smem, stream>>>(g->fview, g->d_fwd, K, list16, order16, status, p.shape, g->d_error);
   } else if (p.shared) {
     const int64_t nw = p.threads / 32;
     auto kern = p.rec_smem ? pe::pe_decode_warp_kernel<true> : pe::pe_decode_warp_kernel<false>;

@@ -93,38 +93,86 @@ int check_desc(const pe_graph_desc* d, int64_t* time_bound, int64_t* mem_bound, 
   return PE_OK;
 }
 
-// Slots for the slot encoding: operator s takes over the slot of operator p when all successors of p are s or ancestors of
-// s (their readings are over in every topological order by then); preferably that of one of its predecessors.  version[s]:
-// operators of its slot up to and including s, at most `longest`.  Returns the number of slots, or -1 when more than `most`
-// are needed.
-int32_t share_slots(int32_t V, const std::vector<int32_t>& sptr, const std::vector<int32_t>& succ, const PeOpRec* ops,
-                    const int32_t* pred, int32_t most, int32_t longest, std::vector<int32_t>* slot, std::vector<int32_t>* version) {
-  slot->assign(V, -1);
-  version->assign(V, 0);
-  const size_t words = ((size_t)V + 63) / 64;
-  std::vector<int32_t> deg(V), stack, tail;   // tail: last operator of every slot
-  std::vector<int32_t> unread(V), idle;       // successors of an operator still to come; slots whose tail has none
-  for (int32_t i = 0; i < V; ++i) unread[i] = sptr[i + 1] - sptr[i];
-  std::vector<uint64_t> anc((size_t)V * words, 0);
+// Ancestors of every operator as rows of bits, and a topological order that follows a chain of operators to its end.
+struct Ancestors {
+  size_t words = 0;
+  std::vector<uint64_t> bits;
+  std::vector<int32_t> sptr, succ, order;   // successors (with repetitions) in CSR form
+  bool of(int32_t i, int32_t a) const { return bits[(size_t)i * words + (size_t)(a / 64)] >> (a % 64) & 1u; }
+};
+Ancestors find_ancestors(int32_t V, const PeOpRec* ops, const int32_t* pred) {
+  Ancestors a;
+  a.words = ((size_t)V + 63) / 64;
+  a.bits.assign((size_t)V * a.words, 0);
+  a.sptr.assign(V + 1, 0);
+  const int32_t E = ops[V - 1].edge_begin + ops[V - 1].indeg;
+  for (int32_t q = 0; q < E; ++q) a.sptr[pred[q] + 1]++;
+  for (int32_t i = 0; i < V; ++i) a.sptr[i + 1] += a.sptr[i];
+  a.succ.resize(E);
+  std::vector<int32_t> fill(a.sptr.begin(), a.sptr.end() - 1), deg(V), stack;
+  for (int32_t i = 0; i < V; ++i)
+    for (int32_t q = ops[i].edge_begin; q < ops[i].edge_begin + ops[i].indeg; ++q) a.succ[fill[pred[q]]++] = i;
   for (int32_t i = V - 1; i >= 0; --i) {
     deg[i] = ops[i].indeg;
     if (deg[i] == 0) stack.push_back(i);
   }
-  while (!stack.empty()) {   // depth first: a chain of operators is followed to its end
+  while (!stack.empty()) {
     const int32_t s = stack.back();
     stack.pop_back();
-    uint64_t* a = anc.data() + (size_t)s * words;
-    const int32_t first = ops[s].edge_begin, last = ops[s].edge_begin + ops[s].indeg;
-    for (int32_t q = first; q < last; ++q) {
-      const uint64_t* b = anc.data() + (size_t)pred[q] * words;
-      for (size_t w = 0; w < words; ++w) a[w] |= b[w];
-      a[pred[q] / 64] |= 1ull << (pred[q] % 64);
+    a.order.push_back(s);
+    uint64_t* row = a.bits.data() + (size_t)s * a.words;
+    for (int32_t q = ops[s].edge_begin; q < ops[s].edge_begin + ops[s].indeg; ++q) {
+      const uint64_t* b = a.bits.data() + (size_t)pred[q] * a.words;
+      for (size_t w = 0; w < a.words; ++w) row[w] |= b[w];
+      row[pred[q] / 64] |= 1ull << (pred[q] % 64);
     }
+    for (int32_t q = a.sptr[s]; q < a.sptr[s + 1]; ++q)
+      if (--deg[a.succ[q]] == 0) stack.push_back(a.succ[q]);
+  }
+  return a;
+}
+
+// Chains (of operators each of which is an ancestor of the next) that cover all operators: at most as many operators are
+// available at once.  -1 when more than `most` are needed.
+int32_t cover_by_chains(const Ancestors& anc, const PeOpRec* ops, const int32_t* pred, int32_t most) {
+  std::vector<int32_t> tail, chain(anc.order.size(), -1);
+  for (const int32_t s : anc.order) {
+    int32_t take = -1;
+    for (int32_t q = ops[s].edge_begin; q < ops[s].edge_begin + ops[s].indeg && take < 0; ++q)
+      if (tail[chain[pred[q]]] == pred[q]) take = chain[pred[q]];
+    for (int32_t t = 0; t < (int32_t)tail.size() && take < 0; ++t)
+      if (anc.of(s, tail[t])) take = t;
+    if (take < 0) {
+      if ((int32_t)tail.size() == most) return -1;
+      take = (int32_t)tail.size();
+      tail.push_back(s);
+    }
+    tail[take] = s;
+    chain[s] = take;
+  }
+  return (int32_t)tail.size();
+}
+
+// Slots for the slot encoding: operator s takes over the slot of operator p when all successors of p are s or ancestors of
+// s (their readings are over in every topological order by then); preferably that of one of its predecessors.  version[s]:
+// operators of its slot up to and including s, at most `longest`.  Returns the number of slots, or -1 when more than `most`
+// are needed.
+int32_t share_slots(const Ancestors& anc, const PeOpRec* ops, const int32_t* pred, int32_t most, int32_t longest,
+                    std::vector<int32_t>* slot, std::vector<int32_t>* version) {
+  const std::vector<int32_t>&sptr = anc.sptr, &succ = anc.succ;
+  const int32_t V = (int32_t)anc.order.size();
+  slot->assign(V, -1);
+  version->assign(V, 0);
+  std::vector<int32_t> tail;              // last operator of every slot
+  std::vector<int32_t> unread(V), idle;   // successors of an operator still to come; slots whose tail has none
+  for (int32_t i = 0; i < V; ++i) unread[i] = sptr[i + 1] - sptr[i];
+  for (const int32_t s : anc.order) {
+    const int32_t first = ops[s].edge_begin, last = ops[s].edge_begin + ops[s].indeg;
     auto free_for_s = [&](int32_t t) {   // every successor of the slot's tail is s or an ancestor of s
       const int32_t p = tail[t];
       if ((*version)[p] == longest || sptr[p] == sptr[p + 1]) return false;
       for (int32_t q = sptr[p]; q < sptr[p + 1]; ++q)
-        if (succ[q] != s && !(a[succ[q] / 64] >> (succ[q] % 64) & 1u)) return false;
+        if (succ[q] != s && !anc.of(s, succ[q])) return false;
       return true;
     };
     int32_t take = -1;
@@ -147,8 +195,6 @@ int32_t share_slots(int32_t V, const std::vector<int32_t>& sptr, const std::vect
     (*slot)[s] = take;
     for (int32_t q = first; q < last; ++q)
       if (--unread[pred[q]] == 0 && tail[(*slot)[pred[q]]] == pred[q]) idle.push_back((*slot)[pred[q]]);
-    for (int32_t q = sptr[s]; q < sptr[s + 1]; ++q)
-      if (--deg[succ[q]] == 0) stack.push_back(succ[q]);
   }
   return (int32_t)tail.size();
 }
@@ -347,6 +393,9 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
       for (int64_t q = 0; q < (int64_t)V * D; ++q) ((uint16_t*)(tblob.data() + tv.durm))[q] = (uint16_t)d->dur_by_machine[q];
   }
 
+  Ancestors anc;
+  if (V <= 4096) anc = find_ancestors(V, ops, pred);
+
   // slot encoding
   std::vector<uint8_t> sblob;
   g->slot_ok = false;
@@ -363,12 +412,8 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
   int vbits = 8;
   while (vbits > 0 && (tb >= (int64_t)1 << (24 - vbits) || (int64_t)longest_field << vbits > 65535)) --vbits;
   if (tile && V <= 4096 && asum < 32768 && vbits >= 4) {
-    std::vector<int32_t> sptr(V + 1, 0), succ(E), slot, version;
-    for (int32_t b = 0; b < E; ++b) sptr[d->edge_src[b] + 1]++;
-    for (int32_t i = 0; i < V; ++i) sptr[i + 1] += sptr[i];
-    std::vector<int32_t> fill(sptr.begin(), sptr.end() - 1);
-    for (int32_t b = 0; b < E; ++b) succ[fill[d->edge_src[b]]++] = d->edge_dst[b];
-    const int32_t n = share_slots(V, sptr, succ, ops, pred, V / 4, (1 << (vbits - 1)) - 1, &slot, &version);
+    std::vector<int32_t> slot, version;
+    const int32_t n = share_slots(anc, ops, pred, V / 4, (1 << (vbits - 1)) - 1, &slot, &version);
     if (n >= 0) {
       g->slot_ok = true;
       PeSlotView& sv = g->sview;
@@ -498,12 +543,49 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
       }
     }
     fv.V = V; fv.E = (int32_t)usucc.size();
+    // pool kernel: joins, roots, successors
+    std::vector<uint8_t> pool;
+    const int32_t chains = fv.short_lists && V <= 4096 ? cover_by_chains(anc, ops, pred, 32) : -1;
+    if (chains >= 0) {
+      std::vector<uint32_t> join(V, 0xFFFFu), prec((size_t)V * 2, 0), pmore;
+      std::vector<uint8_t> joins;
+      std::vector<uint16_t> roots;
+      int32_t leaves = 0;
+      for (int32_t i = 0; i < V; ++i) {
+        if (uindeg[i] > 1) { join[i] = (uint32_t)joins.size(); joins.push_back((uint8_t)(uindeg[i] - 1)); }
+        if (uindeg[i] == 0) roots.push_back((uint16_t)i);
+      }
+      for (int32_t i = 0; i < V; ++i) {
+        const uint32_t n = uptr[i + 1] - uptr[i];
+        leaves += n == 0 ? 1 : 0;
+        auto entry = [&](uint32_t q) { return (uint32_t)usucc[q] | join[usucc[q]] << 16; };
+        prec[2 * (size_t)i] = n > 0 ? entry(uptr[i]) : 0u;
+        prec[2 * (size_t)i + 1] = n << 24 | (uint32_t)pmore.size();
+        for (uint32_t q = 1; q < n; ++q) pmore.push_back(entry(uptr[i] + q));
+      }
+      fv.num_roots = (int32_t)roots.size(); fv.num_joins = (int32_t)joins.size();
+      fv.places = (chains + 7) / 8 * 8;
+      fv.turns = (int32_t)usucc.size() + leaves;
+      auto put = [&](const void* from, size_t n) {
+        const size_t off = pool.size();
+        pool.resize(align16(off + n), 0);
+        if (n) std::memcpy(pool.data() + off, from, n);
+        return (uint32_t)off;
+      };
+      pmore.push_back(0xFFFF0000u);   // (read, not used, behind the last successor of an operator)
+      put(prec.data(), prec.size() * 4);
+      fv.pmore = put(pmore.data(), pmore.size() * 4);
+      fv.roots = put(roots.data(), roots.size() * 2);
+      fv.joins = put(joins.data(), joins.size());
+      fv.pool_bytes = (uint32_t)pool.size();
+    }
     uint64_t fat = 0;
     fv.ptr = (uint32_t)fat;   fat = align16(fat + (uint64_t)(V + 1) * 4);
     fv.succ = (uint32_t)fat;  fat = align16(fat + (uint64_t)usucc.size() * 2);
     fv.indeg = (uint32_t)fat; fat = align16(fat + (uint64_t)V);
     fv.rec = (uint32_t)fat;   fat = align16(fat + (uint64_t)V * fv.rec_bytes);
     fv.more = (uint32_t)fat;  fat = align16(fat + (uint64_t)more.size() * 2);
+    fv.prec = (uint32_t)fat;  fat = align16(fat + pool.size());
     fblob.assign((size_t)fat, 0);
     auto put = [&](uint32_t at, const void* from, size_t n) { if (n) std::memcpy(fblob.data() + at, from, n); };
     put(fv.ptr, uptr.data(), (size_t)(V + 1) * 4);
@@ -511,6 +593,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
     put(fv.indeg, uindeg.data(), (size_t)V);
     put(fv.rec, rec.data(), (size_t)V * fv.rec_bytes);
     put(fv.more, more.data(), more.size() * 2);
+    put(fv.prec, pool.data(), pool.size());
   }
 
   // one allocation and one copy for all encodings (each on a 256-byte boundary), the status word last

@@ -138,6 +138,18 @@ struct PeFwdView {
   uint32_t rec_bytes;   // 16, or 32 where a fiftieth of the operators has 7 to 14 successors
   uint32_t more;   // uint16[]
   int32_t short_lists;  // no operator has more than 255 successors
+  // For pe_decode_pool_kernel (pool_bytes 0: absent; V <= 4096, at most 32 chains cover all operators, at most 255 successors
+  // an operator); offsets below count from
+  // prec, one block that is copied to shared memory.  A successor is operator | its place among the joins << 16 (0xFFFF: it has
+  // one predecessor); prec: {first successor, how many << 24 | the others' place in pmore}.
+  int32_t num_roots, num_joins;
+  int32_t places;       // of the pool: chains that cover the operators, a multiple of 8
+  int32_t turns;        // of the kernel's loop: successors, and operators without one
+  uint32_t prec;        // uint2[V]
+  uint32_t pmore;       // uint32[]
+  uint32_t roots;       // uint16[num_roots]
+  uint32_t joins;       // uint8[num_joins]: predecessors less one
+  uint32_t pool_bytes;  // multiple of 16
 };
 
 struct pe_graph {
