@@ -672,10 +672,12 @@ static bool plan_decode_pool(const pe_graph* g, int64_t K, DecodePlan* p) {
   const size_t V = (size_t)g->V, fixed = ((size_t)f.pool_bytes + 8 + 15) / 16 * 16;
   auto bytes = [&](size_t P) { return (P * (4 * (size_t)f.places + 2 * V + (size_t)f.num_joins + 2) + 15) / 16 * 16; };
   size_t bestW = 0, bestP = 0;
+  double best = 0;
   for (size_t W = 1; W <= 16; ++W)
     for (size_t P = 32; P >= 4; P -= 4)
       if (fixed + W * bytes(P) <= g->smem_optin) {
-        if (W * P > bestW * bestP) { bestW = W; bestP = P; }
+        const double score = (double)(W * P) / (W <= 4 ? 1.0 : 1.0 + 0.14 * (double)(W - 4));   // (narrow tiles of many warps cost)
+        if (score > best) { best = score; bestW = W; bestP = P; }
         break;
       }
   if (bestW == 0) return false;

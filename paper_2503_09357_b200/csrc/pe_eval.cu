@@ -454,16 +454,17 @@ static bool lane_pays_exclusive(const pe_graph* g, int64_t K, const Plan& lane) 
 
 // The slot kernels: the gather takes ~430000 positions a microsecond, start and finish by operator 250000 (odd batches a
 // quarter longer), a step of the recurrence `base` or, with many warps on an SM, `per_warp` for each.  Measured (estimate /
-// time, us): multi-modal graph V = 1536 K = 4096 144 / 132, K = 65536 493 / 476, with exclusive channels K = 16384 549 / 507,
+// time, us): multi-modal graph V = 1536 K = 4096 144 / 132, K = 65536 493 / 476, with exclusive channels K = 16384 416 / 468,
 // with durations by machine K = 65536 493 / 607; MoE graph V = 2816 K = 4096 523 / 511, K = 16384 607 / 734, times by operator
 // 795 / 894; pipeline V = 64 K = 16384 20 / 19, K = 65536 40 / 40.
 static double slot_us(const pe_graph* g, int64_t K, uint32_t flags, bool times, const Plan& s) {
   const double V = g->V, cells = V * (double)K, warps = s.threads / 32;
   const bool listed = g->sview.max_sources > (g->sview.cls_kind == 0 ? 3 : 2);
   double base = listed ? (g->sview.max_sources <= 8 ? 0.172 : 0.3) : (g->sview.max_sources == 1 ? 0.06 : 0.075);
-  if (s.exclusive) base = listed ? 0.58 : 0.155;
+  if (g->sview.marks) base = g->sview.max_sources == 1 ? 0.07 : 0.087;
+  if (s.exclusive) base = listed ? 0.4 : 0.11;
   if (g->hetero) base += 0.012;
-  const double step = std::max(base, (listed ? 0.021 : 0.0105) * warps), odd = K % 4 != 0 ? 1.25 : 1.0;
+  const double step = std::max(base, (listed ? 0.021 : (g->sview.marks ? 0.0135 : 0.0105)) * warps), odd = K % 4 != 0 ? 1.25 : 1.0;
   return 11.0 + odd * cells / 430e3 + V * step * (double)s.tile_rounds + (double)K * (g->D * 3.2e-6 + 1.3e-4) +
          (times && (flags & PE_TIMES_BY_OP) ? 3.0 + odd * cells / 250e3 : 0.0);
 }
@@ -646,13 +647,14 @@ extern "C" size_t pe_workspace_bytes(const pe_graph* g, int64_t K, uint32_t flag
       pe::Plan p;
       if (pe::make_plan(g, K, flags, compact, times, &p) == PE_OK) most = std::max(most, p.workspace);
     }
+  pe::Plan sl;
+  const bool slots = g && K > 0 && (flags & PE_VARIANT_MASK) == PE_VARIANT_AUTO && pe::plan_slot(g, K, flags, true, &sl);
   // Smaller batches than this one may stage copies where it does not (see eval_batch): room for those of K candidates.
   pe::Plan tm;
   if (pe::auto_choice(g, K, flags) && pe::plan_team(g, K, true, &tm) && tm.workspace > most &&
-      (g->slot_ok || !(pe::large_batches_need_none(g, flags, true) && pe::large_batches_need_none(g, flags, false))))
+      (slots || !(pe::large_batches_need_none(g, flags, true) && pe::large_batches_need_none(g, flags, false))))
     most = tm.workspace;
-  pe::Plan sl;
-  if (g && K > 0 && (flags & PE_VARIANT_MASK) == PE_VARIANT_AUTO && pe::plan_slot(g, K, flags, true, &sl) && sl.workspace > most) most = sl.workspace;
+  if (slots && sl.workspace > most) most = sl.workspace;
   return most;
 }
 

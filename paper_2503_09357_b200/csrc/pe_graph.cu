@@ -155,9 +155,10 @@ int32_t cover_by_chains(const Ancestors& anc, const PeOpRec* ops, const int32_t*
 
 // Slots for the slot encoding: operator s takes over the slot of operator p when all successors of p are s or ancestors of
 // s (their readings are over in every topological order by then); preferably that of one of its predecessors.  version[s]:
-// operators of its slot up to and including s, at most `longest`.  Returns the number of slots, or -1 when more than `most`
-// are needed.
-int32_t share_slots(const Ancestors& anc, const PeOpRec* ops, const int32_t* pred, int32_t most, int32_t longest,
+// operators of its slot up to and including s, at most `longest`.  marks: an operator without successors leaves a mark in the
+// slot of a predecessor (version 0; one mark a holder) where one is free to take it.  Returns the number of slots, or -1 when
+// more than `most` are needed.
+int32_t share_slots(const Ancestors& anc, const PeOpRec* ops, const int32_t* pred, int32_t most, int32_t longest, bool marks,
                     std::vector<int32_t>* slot, std::vector<int32_t>* version) {
   const std::vector<int32_t>&sptr = anc.sptr, &succ = anc.succ;
   const int32_t V = (int32_t)anc.order.size();
@@ -165,9 +166,15 @@ int32_t share_slots(const Ancestors& anc, const PeOpRec* ops, const int32_t* pre
   version->assign(V, 0);
   std::vector<int32_t> tail;              // last operator of every slot
   std::vector<int32_t> unread(V), idle;   // successors of an operator still to come; slots whose tail has none
+  std::vector<uint8_t> marked(V, 0);
   for (int32_t i = 0; i < V; ++i) unread[i] = sptr[i + 1] - sptr[i];
   for (const int32_t s : anc.order) {
     const int32_t first = ops[s].edge_begin, last = ops[s].edge_begin + ops[s].indeg;
+    if (marks && sptr[s] == sptr[s + 1]) {
+      for (int32_t q = first; q < last && (*slot)[s] < 0; ++q)
+        if (!marked[pred[q]]) { marked[pred[q]] = 1; (*slot)[s] = (*slot)[pred[q]]; }
+      if ((*slot)[s] >= 0) continue;   // (its predecessor has a successor that is nobody's ancestor: the slot stays with it)
+    }
     auto free_for_s = [&](int32_t t) {   // every successor of the slot's tail is s or an ancestor of s
       const int32_t p = tail[t];
       if ((*version)[p] == longest || sptr[p] == sptr[p + 1]) return false;
@@ -413,7 +420,12 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
   while (vbits > 0 && (tb >= (int64_t)1 << (24 - vbits) || (int64_t)longest_field << vbits > 65535)) --vbits;
   if (tile && V <= 4096 && asum < 32768 && vbits >= 4) {
     std::vector<int32_t> slot, version;
-    const int32_t n = share_slots(anc, ops, pred, V / 4, (1 << (vbits - 1)) - 1, &slot, &version);
+    bool marks = false;
+    int32_t n = share_slots(anc, ops, pred, V / 4, (1 << (vbits - 1)) - 1, false, &slot, &version);
+    if (n < 0 && g->tview.cls_kind == 0 && mdeg <= 3) {
+      marks = true;
+      n = share_slots(anc, ops, pred, (int32_t)(0.65 * V), (1 << (vbits - 2)) - 1, true, &slot, &version);
+    }
     if (n >= 0) {
       g->slot_ok = true;
       PeSlotView& sv = g->sview;
@@ -421,6 +433,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
       sv.has_weight = g->has_weight ? 1 : 0;
       sv.cls_kind = g->tview.cls_kind;
       sv.vbits = vbits;
+      sv.marks = marks ? 1 : 0;
       struct Source { uint32_t slot, c0, c1; };   // delays << vbits | version, per class
       std::vector<std::vector<Source>> sources(V + 1);
       std::vector<uint8_t> own_first(V + 1, 0);
@@ -430,7 +443,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
         bool chained = false;
         for (int32_t q = ops[i].edge_begin; q < ops[i].edge_begin + ops[i].indeg; ++q)
           chained = chained || (slot[pred[q]] == slot[i] && version[pred[q]] == version[i] - 1);
-        if (!chained) { sources[i].push_back({(uint32_t)slot[i], before, before}); own_first[i] = 1; }
+        if (!chained && !marks) { sources[i].push_back({(uint32_t)slot[i], before, before}); own_first[i] = 1; }
         for (int32_t q = ops[i].edge_begin; q < ops[i].edge_begin + ops[i].indeg; ++q) {
           const uint32_t v = (uint32_t)version[pred[q]], c0 = (uint32_t)comm[(size_t)q * L], c1 = L == 2 ? (uint32_t)comm[(size_t)q * L + 1] : c0;
           sources[i].push_back({(uint32_t)slot[pred[q]], c0 << vbits | v, c1 << vbits | v});
@@ -456,7 +469,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
         const uint32_t own = i < V ? (uint32_t)slot[i] : (uint32_t)n + 1u;
         auto get = [&](size_t q) { return q < src.size() ? src[q] : none; };
         r[0] = (own & 0xFFu) << 16;
-        if (i < V) r[0] |= (uint32_t)(uint8_t)(int8_t)ops[i].mem_delta << 24 | (uint32_t)(g->hetero ? 0 : ops[i].dur) << vbits | (uint32_t)version[i];
+        if (i < V) r[0] |= (uint32_t)(uint8_t)(int8_t)ops[i].mem_delta << 24 | (uint32_t)(g->hetero ? 0 : ops[i].dur) << vbits | (version[i] > 0 ? (uint32_t)version[i] : 1u << (vbits - 1));
         if (sv.cls_kind == 0) {
           auto edge = [&](size_t q) { return get(q).c0 << 16 | get(q).slot; };
           r[1] = edge(0) | (own >> 8) << 12;

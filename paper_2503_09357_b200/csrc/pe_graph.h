@@ -91,7 +91,8 @@ struct PeTileView {
 };
 
 // Slot encoding, for graphs through which few results are alive at a time (see pe_kernel_slot.cuh): operators share
-// `nslots` state words.  Built when the tile encoding exists, V <= 4096, V / 4 slots are enough, the levels without weights
+// `nslots` state words.  Built when the tile encoding exists, V <= 4096, V / 4 slots are enough (with `marks`, for one class
+// and at most three incoming edges: 0.65 V), the levels without weights
 // stay below 2^15, and durations, delays and the time bound leave `vbits` >= 4 bits for versions: times are kept in units of
 // 2^vbits, a field below stands for `value << vbits | version`.  One 16-byte record per operator, and record V for entries
 // that are no operator:
@@ -102,12 +103,14 @@ struct PeTileView {
 //     of class 1 << 16;  list_at[operator] = place of source 2 in the list ({last << 12 | slot, as z}); bit 29 of y: see below
 // Sources are the incoming edges.  An operator whose slot was not held by one of its predecessors has its own slot in front
 // of them, with the version of the operator that held it and no delay (that operator is an ancestor, or there was none):
-// bit 13 / 29.  With at most eight sources an operator's part of the list has six places (eight words or twelve).
+// bit 13 / 29.  With `marks` there are no such sources: every operator reads its own slot besides, and one without successors
+// has the slot of a predecessor and the top bit of `version` instead of one.  With at most eight sources an operator's part of the list has six places (eight words or twelve).
 // Slot nslots stands for missing sources (it holds "ended at 0", version 0), nslots + 1 takes words that nobody reads.
 struct PeSlotView {
   int32_t V, E, D;
   int32_t nslots;
   int32_t vbits;
+  int32_t marks;
   int32_t has_weight;
   int32_t cls_kind;    // as in PeTileView
   int32_t max_sources;

@@ -20,6 +20,9 @@
 // reads the word of its own slot (as a predecessor's, or as one source more): a slot's operators are then executed one
 // after the other, each once at most, and never before a predecessor.  V positions that pass are therefore a topological
 // permutation, and every topological permutation passes.
+// Graphs with many operators that nobody follows (OWN; random graphs, the bidirectional pipeline): such an operator needs no
+// word, only a bit that says it has been executed.  That is the top bit of the version field of one of its predecessors, whose
+// slot it leaves otherwise as it is; all operators then read the word of their own slot besides their sources'.
 //
 // State word: (time << vbits | version) << 8 | machine.
 //
@@ -297,12 +300,15 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
 }
 
 // A step: machine record {end of the machine's last operator (packed), level << 16 | peak} and the words of the sources come
-// from shared memory, everything else of the position was fetched during the step before.
+// from shared memory, everything else of the position was fetched during the step before.  (With the busy time in the record,
+// 12 bytes, the gather is free of atomics, but fewer candidates fit: multi-modal graph K = 65536 474 -> 525 us, MoE graph
+// K = 16381 922 -> 903.)
 // CLS: 0 = one link class, every pair connected; 1 = class table; 2 = two classes, every pair connected, at most 32 machines.
 // EDGES: no operator has more sources (1 to 3 with one class, 2 otherwise), all inline; 8 = inline ones, then six places of
 // the list; 0 = inline ones, then the list.
 // TIMES: 0 = none, 1 = by position, 2 = words for pe_slot_times_kernel.
-template <int CLS, int EDGES, int TIMES, int MODE>
+// OWN: see above (one link class, EDGES 1 to 3, no channels).
+template <int CLS, int EDGES, int TIMES, int MODE, bool OWN>
 __global__ void __launch_bounds__(32 * kSlotWarps, 1) pe_eval_slot_kernel(PeSlotView g, const uint8_t* __restrict__ blob, int64_t K,
                                                                        int64_t n, const uint4* __restrict__ entries, int64_t pitch_e,
                                                                        const uint32_t* __restrict__ status, const int32_t* __restrict__ wsum,
@@ -322,7 +328,7 @@ __global__ void __launch_bounds__(32 * kSlotWarps, 1) pe_eval_slot_kernel(PeSlot
     if (!stage_blob(smem_raw, blob, g.bytes, bar, err)) return;
   }
   const int32_t* cap = reinterpret_cast<const int32_t*>(smem_raw + g.cap);
-  const uint32_t tshift = 8u + (uint32_t)g.vbits, tmask = ~0u << tshift;   // time field of a packed word
+  const uint32_t tshift = 8u + (uint32_t)g.vbits, tmask = ~0u << tshift, mark = 1u << (tshift - 1u);   // time field of a packed word, top bit of its version
   const uint32_t pitch = (uint32_t)P * 4u, dpitch = (uint32_t)P * 8u;
   const int ml = lane < P ? lane : P - 1;
   const bool mine = lane < P;
@@ -370,7 +376,7 @@ __global__ void __launch_bounds__(32 * kSlotWarps, 1) pe_eval_slot_kernel(PeSlot
     }
     __syncwarp();
 
-    uint32_t st = 0, bad = 0;   // bad: differences between versions found and expected, among other bits
+    uint32_t st = 0, bad = 0, marked = 0;   // bad: differences between versions found and expected, among other bits
     uint8_t* start_b = TIMES == 1 ? reinterpret_cast<uint8_t*>(out.start + cc) : reinterpret_cast<uint8_t*>(words + cc);
     uint8_t* finish_b = TIMES == 1 ? reinterpret_cast<uint8_t*>(out.finish + cc) : nullptr;
     uint32_t ent = mine ? cur[0].x : 0u;
@@ -391,6 +397,8 @@ __global__ void __launch_bounds__(32 * kSlotWarps, 1) pe_eval_slot_kernel(PeSlot
       }
 #pragma unroll
       for (int q = 0; q < NIN; ++q) w[q] = lds32(st_a + p[q] * pitch);
+      const uint32_t own_a = st_a + (((r4.x >> 16) & 0xFFu) | ((r4.y >> 4) & 0xF00u)) * pitch;
+      const uint32_t w_own = OWN ? lds32(own_a) : 0u;
       const uint2 dv = lds64(dv_a + j * dpitch);
       uint32_t crow = 0;
       if (CLS == 2) crow = lds32(row_a + j * 4u);
@@ -422,19 +430,20 @@ __global__ void __launch_bounds__(32 * kSlotWarps, 1) pe_eval_slot_kernel(PeSlot
           }
         }
         if (EXCL) {
-          // the transfer starts when its source has ended (Eq. 13) and the channel is free (Eq. 14), lasts D^c (Eq. 11)
-          if (!same && pp != nslots && channel && real) {
-            const uint32_t ch = ch_a + (min(ww & 0xFFu, dmax) * (uint32_t)D + j) * chpitch;
-            if (CH16) {
-              const uint32_t t_end = max(ww >> tshift, lds16(ch)) + (d >> tshift);
-              sts_state<true>(ch, t_end);
-              return t_end << tshift;
-            }
-            const uint32_t t_end = max(ww & tmask, lds32(ch)) + (d & tmask);
+          // the transfer starts when its source has ended (Eq. 13) and the channel is free (Eq. 14), lasts D^c (Eq. 11).
+          // Sources that need no channel take the word behind the last one: 32 candidates would take both sides of a branch.
+          const bool moves = !same && pp != nslots && channel && real;
+          const uint32_t ch = ch_a + (moves ? (ww & 0xFFu) * (uint32_t)D + j : (uint32_t)(D * D)) * chpitch;
+          uint32_t t_end;
+          if (CH16) {
+            t_end = max(ww >> tshift, lds16(ch)) + (d >> tshift);
+            sts_state<true>(ch, t_end);
+            t_end <<= tshift;
+          } else {
+            t_end = max(ww & tmask, lds32(ch)) + (d & tmask);
             sts_state<false>(ch, t_end);
-            return t_end;
           }
-          return ww;
+          return moves ? t_end : ww;
         }
         return ww + (same ? 0u : d);
       };
@@ -487,15 +496,20 @@ __global__ void __launch_bounds__(32 * kSlotWarps, 1) pe_eval_slot_kernel(PeSlot
           }
         }
       }
-      uint32_t durj = __byte_perm(r4.x, j, 0x5104);   // D^o, the own version and the machine (Eq. 3)
-      if (HET) durj += dur_het << 8;
+      const uint32_t durj = __byte_perm(r4.x, j, 0x5104);   // D^o, the own version and the machine (Eq. 3)
       const uint32_t rt = r & tmask;
-      const uint32_t e = rt + durj;
+      const uint32_t e = HET ? rt + durj + (dur_het << 8) : rt + durj;
       // + A_i (byte 3 of the record) on the level; the peak follows it (Eqs. 17-19)
       const uint32_t lv = dv.y + ((uint32_t)__dp4a((int32_t)r4.x, 0x01000000, 0) << 16);
       const uint32_t lp = max_s16x2(lv, __byte_perm(lv, 0u, 0x3232));
-      const uint32_t own = ((r4.x >> 16) & 0xFFu) | ((r4.y >> 4) & 0xF00u);
-      sts_state<false>(st_a + own * pitch, e);
+      if (OWN) {
+        const bool last = (durj & mark) != 0u;   // nobody follows it
+        if (last) marked |= w_own;
+        else bad |= (w_own + 0x100u) ^ durj;
+        sts_state<false>(own_a, last ? w_own | mark : e);
+      } else {
+        sts_state<false>(own_a, e);
+      }
       sts64(dv_a + j * dpitch, make_uint2(e, lp));
       if (TIMES == 1) {
         *reinterpret_cast<int32_t*>(start_b) = (int32_t)(rt >> tshift);
@@ -533,7 +547,7 @@ __global__ void __launch_bounds__(32 * kSlotWarps, 1) pe_eval_slot_kernel(PeSlot
     }
     __syncwarp();
 
-    if (bad & ~tmask & ~0xFFu) st |= PE_STATUS_ORDER_INVALID;
+    if ((bad & (mark - 0x100u)) | (marked & mark)) st |= PE_STATUS_ORDER_INVALID;
     uint32_t z = 0;
     st |= status[cc];
     for (int j = 0; j < D; ++j) {

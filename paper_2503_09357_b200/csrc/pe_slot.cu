@@ -65,18 +65,23 @@ bool plan_slot(const pe_graph* g, int64_t K, uint32_t flags, bool times, Plan* p
   const bool by_op_times = times && (flags & PE_TIMES_BY_OP) != 0;
   if (g->hetero && exclusive) return false;
   const PeSlotView& sv = g->sview;
+  // Larger graphs with marks gain less by operator, and programs run their large batches without a workspace.
+  if (sv.marks && (exclusive || (!by_pos && !g->hetero && g->V > 512))) return false;
   p->slot_gather = (int)tile_width(g, [&](size_t C) { return gather_smem(g, by_pos, C); });
   p->slot_times = (int)tile_width(g, [&](size_t C) { return (size_t)(g->V + 1) * C * 4; });
   if (p->slot_gather == 0 || p->slot_times == 0) return false;
   const int mode = g->hetero ? kSlotHet : (!exclusive ? kSlotPlain : (g->time_bound < 65536 ? kSlotExcl16 : kSlotExcl));
   const size_t fixed = up16((size_t)sv.bytes + 8), D = (size_t)g->D, rows = (size_t)sv.nslots + 2;
-  const size_t chan = exclusive ? D * D * (mode == kSlotExcl16 ? 2 : 4) : 0;
+  const size_t chan = exclusive ? (D * D + 1) * (mode == kSlotExcl16 ? 2 : 4) : 0;
   auto bytes = [&](size_t W, size_t P) { return fixed + W * (P * 16 * kSlotQuads + up16(P * 8 * D) + up16(P * chan) + up16(P * 4 * rows)); };
   size_t bestW = 0, bestP = 0;
+  double best = 0;
   for (size_t W = 1; W <= (size_t)kSlotWarps; ++W)
     for (size_t P = 32; P >= 4; P -= 4)
       if (bytes(W, P) <= g->smem_optin) {
-        if (W * P > bestW * bestP) { bestW = W; bestP = P; }
+        // (from seven warps on a step takes the longer the more there are)
+        const double score = (double)(W * P) / std::max(1.0, (double)W / 7.0) * (1.0 + 1e-3 * (double)W);
+        if (score > best) { best = score; bestW = W; bestP = P; }
         break;
       }
   if (bestW == 0) return false;
@@ -101,7 +106,7 @@ bool plan_slot(const pe_graph* g, int64_t K, uint32_t flags, bool times, Plan* p
     const int64_t w = (tiles + sms * rounds - 1) / (sms * rounds);
     if (w < (int64_t)bestW) bestW = (size_t)w;
   }
-  p->tile_rounds = chunk > 0 ? rounds * ((K + chunk - 1) / chunk) : 0;
+  p->tile_rounds = chunk > 0 ? rounds * (K / chunk) + (K % chunk + wave - 1) / wave : 0;
   p->variant = PE_VARIANT_SHARED;
   p->compact = true;
   p->slot = true;

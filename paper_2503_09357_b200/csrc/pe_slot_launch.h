@@ -23,7 +23,7 @@ struct SlotCall {
   cudaStream_t stream;
 };
 
-template <int CLS, int EDGES, int MODE>
+template <int CLS, int EDGES, int MODE, bool OWN = false>
 int launch_slot3(const SlotCall& t) {
   auto go = [&](auto kern) -> int {
     if (!set_smem(kern, t.p->smem)) return PE_ERR_CUDA;
@@ -31,26 +31,35 @@ int launch_slot3(const SlotCall& t) {
                                                                  t.wsum, t.words, t.out, t.g->d_error, t.shape);
     return PE_OK;
   };
-  if (!t.out.start) return go(pe_eval_slot_kernel<CLS, EDGES, 0, MODE>);
-  if (t.words) return go(pe_eval_slot_kernel<CLS, EDGES, 2, MODE>);
-  return go(pe_eval_slot_kernel<CLS, EDGES, 1, MODE>);
+  if (!t.out.start) return go(pe_eval_slot_kernel<CLS, EDGES, 0, MODE, OWN>);
+  if (t.words) return go(pe_eval_slot_kernel<CLS, EDGES, 2, MODE, OWN>);
+  return go(pe_eval_slot_kernel<CLS, EDGES, 1, MODE, OWN>);
 }
 
 template <int MODE>
 int launch_slot_mode(const SlotCall& t) {
   const PeSlotView& v = t.g->sview;
   constexpr bool kPlain = MODE == kSlotPlain, kExcl = MODE == kSlotExcl || MODE == kSlotExcl16;
-  const bool eight = !kExcl && v.max_sources <= 8;
+  if constexpr (!kExcl) {
+    if (v.marks) {
+      if (v.max_sources <= 1) return launch_slot3<0, 1, MODE, true>(t);
+      if (v.max_sources == 2) return launch_slot3<0, 2, MODE, true>(t);
+      return launch_slot3<0, 3, MODE, true>(t);
+    }
+  } else if (v.marks) {
+    return PE_ERR_UNSUPPORTED;
+  }
+  const bool eight = v.max_sources <= 8;
   if (v.cls_kind == 0) {
     if (kPlain && v.max_sources <= 1) return launch_slot3<0, kPlain ? 1 : 0, MODE>(t);
     if (!kExcl && v.max_sources <= 2) return launch_slot3<0, kExcl ? 0 : 2, MODE>(t);
     if (kPlain && v.max_sources <= 3) return launch_slot3<0, kPlain ? 3 : 0, MODE>(t);
-    if (eight) return launch_slot3<0, kExcl ? 0 : 8, MODE>(t);
+    if (eight) return launch_slot3<0, 8, MODE>(t);
     return launch_slot3<0, 0, MODE>(t);
   }
   if (v.cls_kind == 2) {
     if (v.max_sources <= 2) return launch_slot3<2, 2, MODE>(t);
-    if (eight) return launch_slot3<2, kExcl ? 0 : 8, MODE>(t);
+    if (eight) return launch_slot3<2, 8, MODE>(t);
     return launch_slot3<2, 0, MODE>(t);
   }
   return launch_slot3<1, 0, MODE>(t);
