@@ -129,7 +129,9 @@ typedef struct {
   uint32_t* status;  /* [K]   PE_STATUS_* bits */
 } pe_outputs;
 
-/* Bytes of device workspace pe_eval_batch needs for K candidates with these flags (may be 0). */
+/* Bytes of device workspace for pe_eval_batch with K candidates and these flags (may be 0).  Under PE_VARIANT_AUTO part of
+ * it may be optional: given less, a batch that the slot kernels would have taken runs by another kernel, where that one
+ * needs no more than what is given. */
 size_t pe_workspace_bytes(const pe_graph* g, int64_t K, uint32_t flags);
 
 /* Which kernel variant (PE_VARIANT_*) a call with these arguments, 16-bit orders and start and finish wanted runs;

@@ -565,6 +565,18 @@ static bool large_batches_need_none(const pe_graph* g, uint32_t flags, bool time
   return make_plan(g, (int64_t)1 << 24, flags, true, times, &large, false) == PE_OK && large.workspace == 0;
 }
 
+// Workspace of the slot kernels where the automatic choice takes them: for this batch, else for the largest of its half, its
+// quarter, ... for which it does.  (It grows with the batch; a batch that would need more than it is given takes another kernel.)
+static size_t slot_workspace(const pe_graph* g, int64_t K, uint32_t flags) {
+  size_t most = 0;
+  for (int64_t k = K; k > 0 && most == 0; k /= 2)
+    for (const bool times : {true, false}) {
+      Plan p;
+      if (make_plan(g, k, flags, true, times, &p) == PE_OK && p.slot) most = std::max(most, p.workspace);
+    }
+  return most;
+}
+
 template <typename OrderT, bool BY_POS>
 static int launch_typed(const pe_graph* g, const Plan& p, int64_t K, const uint8_t* assign, const void* order,
                         uint32_t flags, const pe_outputs& out, void* workspace, cudaStream_t stream) {
@@ -645,16 +657,17 @@ extern "C" size_t pe_workspace_bytes(const pe_graph* g, int64_t K, uint32_t flag
   for (const bool compact : {true, false})
     for (const bool times : {true, false}) {
       pe::Plan p;
-      if (pe::make_plan(g, K, flags, compact, times, &p) == PE_OK) most = std::max(most, p.workspace);
+      const int rc = pe::make_plan(g, K, flags, compact, times, &p);
+      if (rc == PE_ERR_INVALID_ARG) return 0;
+      if (rc == PE_OK) most = std::max(most, p.workspace);
     }
-  pe::Plan sl;
-  const bool slots = g && K > 0 && (flags & PE_VARIANT_MASK) == PE_VARIANT_AUTO && pe::plan_slot(g, K, flags, true, &sl);
-  // Smaller batches than this one may stage copies where it does not (see eval_batch): room for those of K candidates.
+  // Smaller batches than this one may stage copies, or take the slot kernels, where it does not (see eval_batch): room for
+  // those of K candidates.
   pe::Plan tm;
   if (pe::auto_choice(g, K, flags) && pe::plan_team(g, K, true, &tm) && tm.workspace > most &&
-      (slots || !(pe::large_batches_need_none(g, flags, true) && pe::large_batches_need_none(g, flags, false))))
+      !(pe::large_batches_need_none(g, flags, true) && pe::large_batches_need_none(g, flags, false)))
     most = tm.workspace;
-  if (slots && sl.workspace > most) most = sl.workspace;
+  if (g && g->slot_ok) most = std::max(most, pe::slot_workspace(g, K, flags));
   return most;
 }
 

@@ -1,0 +1,69 @@
+"""Where the automatic choice takes the slot kernels, and what it asks for them."""
+import numpy as np
+import pytest
+
+from paper_2503_09357_b200 import workloads as wl
+from tests import gpu_util as gu
+
+pytestmark = pytest.mark.gpu
+
+
+def binding():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2503_09357_b200 import binding as pe
+    return pe
+
+
+def launches(pe, g, w, K, flags=0, want_times=True, workspace=None):
+    """Kernels that one call launches, checked against the oracle."""
+    assign, order = wl.make_candidates(w, K=K)
+    if flags & pe.PE_ASSIGN_BY_POS:
+        assign = np.take_along_axis(assign, order.astype(np.int64), axis=0)
+    if workspace is None:
+        before = pe.pe_kernel_launches()
+        gu.check(g, w, assign, order, flags=flags, want_times=want_times)
+        return pe.pe_kernel_launches() - before
+    import torch
+    from oracle import pe_oracle as orc
+    out = g.alloc_outputs(K, want_times)
+    before = pe.pe_kernel_launches()
+    g.eval_batch(torch.from_numpy(assign).cuda(), torch.from_numpy(gu.as_signed(order)).cuda(), flags=flags, out=out, workspace=workspace)
+    torch.cuda.synchronize()
+    n = pe.pe_kernel_launches() - before
+    res = {k: v.cpu().numpy() for k, v in out.items()}
+    res["status"] = res["status"].view(np.uint32)
+    gu.compare(res, orc.evaluate(w, assign, order, flags=flags & 7, want_times=want_times, threads=gu.CPU_THREADS))
+    return n
+
+
+@pytest.mark.parametrize("config,kw,K", [(1, {}, 1024), (5, dict(V=256, D=8), 1 << 20), (2, {}, 65536)])
+def test_batches_that_never_take_the_slot_kernels_ask_for_nothing(config, kw, K):
+    pe = binding()
+    g = pe.Graph(wl.make_config(config, **kw))
+    try:
+        assert pe.pe_workspace_bytes(g.handle, K, 0) == 0
+        assert pe.pe_workspace_bytes(g.handle, K, 1 << 20) == 0   # (flags that no call accepts)
+    finally:
+        g.close()
+
+
+def test_workspace_is_what_the_slot_kernels_use():
+    """Multi-modal graph: 4 bytes a position and a status word, a candidate."""
+    pe = binding()
+    w = wl.make_config(4)
+    V, K = w.num_ops, 8192
+    g = pe.Graph(w)
+    try:
+        per = V * 4 + 4 + (w.num_devices * 4 if w.mem_weight is not None else 0)
+        import torch
+        n = pe.pe_workspace_bytes(g.handle, K, 0)
+        assert K * per <= n <= K * per + 4096
+        ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+        # the workspace of the largest batch serves the smaller ones, whichever kernel they take
+        for k, want in ((K, 2), (4097, None), (1001, None), (64, None), (1, None)):
+            got = launches(pe, g, w, k, workspace=(ws, n))
+            assert want is None or got == want
+    finally:
+        g.close()
