@@ -433,12 +433,18 @@ static double team_us(const pe_graph* g, int64_t K, bool times, bool staged) {
 // first only where whole levels of the graph fill its windows, enough warps fit and the rows of a batch are short enough
 // for its strided accesses.  Measured: V = 1600 D = 64 K = 3500 124 / 120, K = 7000 243 / 239; V = 1024 D = 64 K = 14000
 // without times 219 / 230; V = 1920 D = 16 K = 3500 176 / 168; at K = 65536 it takes up to 1.3 times as long a round.
-static double warp_us(const pe_graph* g, int64_t K, bool times, const Plan& w) {
+// With more than three sources an operator (a window is then resolved in rounds from the state in shared memory) a step takes
+// 0.205 us whatever the number of warps: MoE graph with sixteen experts V = 2432 K = 148 503 / 522, K = 4096 1002 / 1059,
+// K = 16384 3994 / 4181, V = 3648 K = 1000 753 / 714, K = 16384 10475 / 9893.
+static double warp_rounds_us(const pe_graph* g, int64_t K, bool times, const Plan& w) {
   const double V = g->V, n = w.threads / 32;
-  if (!w.compact || n < 20.0 || g->max_indeg > 3 || V / g->levels < 56.0 || K > 32768) return 1e30;
   const int64_t per_round = (int64_t)(w.threads / 32) * g->sm_count;
-  const double step = (times ? 0.036 + 0.0016 * n : 0.028 + 0.0013 * n) * (g->D < 32 ? (times ? 1.2 : 1.35) : 1.0);
+  const double step = !w.compact || g->max_indeg > 3 ? 0.205 : (times ? 0.036 + 0.0016 * n : 0.028 + 0.0013 * n) * (g->D < 32 ? (times ? 1.2 : 1.35) : 1.0);
   return 5.0 + step * V * (double)((K + per_round - 1) / per_round);
+}
+static double warp_us(const pe_graph* g, int64_t K, bool times, const Plan& w) {
+  if (!w.compact || w.threads < 20 * 32 || g->max_indeg > 3 || (double)g->V / g->levels < 56.0 || K > 32768) return 1e30;
+  return warp_rounds_us(g, K, times, w);
 }
 
 // Exclusive channels: a lane per candidate (~0.3 us a position where the channel words leave few lanes per SM) or the
@@ -469,10 +475,14 @@ static double slot_us(const pe_graph* g, int64_t K, uint32_t flags, bool times, 
          (times && (flags & PE_TIMES_BY_OP) ? 3.0 + odd * cells / 250e3 : 0.0);
 }
 // Estimated time of a plan that the automatic choice has made among the other kernels (a lane per candidate takes longer with
-// channel words, V = 1536 K = 1024 250 us, or durations by machine, 170 us).
+// channel words, V = 1536 K = 1024 250 us, or durations by machine, 170 us; the global-state kernel with exclusive channels
+// V = 2816 K = 16384 10253 / 12118, K = 32768 20505 / 14992, the generic one for durations by machine V = 1369 D = 64 K = 4000
+// 6434 / 6415, K = 65536 35887 / 27200, MoE graph K = 16384 18455 / 22600).  Where 48 lanes of the generic kernel fit, the tile
+// kernel does too.
 static double plan_us(const pe_graph* g, int64_t K, uint32_t flags, bool times, const Plan& p) {
   if (p.variant == PE_VARIANT_TEAM) return team_us(g, K, times, p.staged);
-  if (p.variant == PE_VARIANT_WARP && p.compact) return warp_us(g, K, times, p);
+  if (p.variant == PE_VARIANT_WARP) return warp_rounds_us(g, K, times, p);
+  if (p.variant == PE_VARIANT_GLOBAL) return (double)g->V * std::max(p.compact ? 2.4 : 4.7, (double)K / (p.compact ? 4500.0 : 2500.0));
   if (p.tiled) return lane_us(g, flags, times, p) * (p.exclusive ? 2.0 : (g->hetero && g->max_indeg <= 3 ? 1.3 : 1.0));
   return 1e30;
 }

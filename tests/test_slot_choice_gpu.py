@@ -67,3 +67,15 @@ def test_workspace_is_what_the_slot_kernels_use():
             assert want is None or got == want
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("K,kernels", [(148, 1), (1000, 1), (9472, 2)])
+def test_small_batches_of_operators_with_many_sources_take_a_warp_each(K, kernels):
+    """Sixteen sources an operator: a lane walks them one after the other (955 us at any small K), a warp side by side (522)."""
+    pe = binding()
+    w = wl.make_config(3, layers=16, experts=16, microbatches=4)
+    g = pe.Graph(w)
+    try:
+        assert launches(pe, g, w, K) == kernels
+    finally:
+        g.close()
