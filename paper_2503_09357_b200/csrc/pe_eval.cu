@@ -12,6 +12,7 @@
 #include <utility>
 #include <algorithm>
 #include <climits>
+#include <cmath>
 #include <cstdio>
 
 #include "pe_device.cuh"
@@ -459,20 +460,35 @@ static bool lane_pays_exclusive(const pe_graph* g, int64_t K, const Plan& lane) 
 }
 
 // The slot kernels: the gather takes ~430000 positions a microsecond, start and finish by operator 250000 (odd batches a
-// quarter longer), a step of the recurrence `base` or, with many warps on an SM, `per_warp` for each.  Measured (estimate /
-// time, us): multi-modal graph V = 1536 K = 4096 144 / 132, K = 65536 493 / 476, with exclusive channels K = 16384 416 / 468,
-// with durations by machine K = 65536 493 / 607; MoE graph V = 2816 K = 4096 523 / 511, K = 16384 607 / 734, times by operator
-// 795 / 894; pipeline V = 64 K = 16384 20 / 19, K = 65536 40 / 40.
+// quarter longer), those by position cost the recurrence one for 1.4 million (4 million where it is slower itself).  A step of
+// the recurrence takes the longer the more sources an operator has (with up to eight the list is read at once, beyond it is
+// walked) and, from five or so warps on an SM on, the more there are.  Over 1065 calls of the graphs of workloads/graphs.py the
+// estimate is 9 % below the time at most (12 % below 100 us) and up to 25 % above it (a few candidates with long lists: up to
+// three times as long).  Measured (estimate / time, us): multi-modal graph V = 1536 K = 1024 131 / 128, K = 32768 287 / 282, with
+// exclusive channels K = 16384 520 / 499, with durations by machine K = 32768 311 / 321; MoE graph V = 2816 K = 4096 526 / 521,
+// K = 32768 845 / 849, times by operator 1196 / 1185, with exclusive channels K = 8192 760 / 769, with durations by machine
+// K = 16384 745 / 749, with sixteen experts V = 2432 K = 16384 1050 / 1137; layered V = 1024 D = 8 K = 131072 1508 / 1510;
+// pipeline V = 64 K = 65536 41 / 40, with exclusive channels K = 4096 25 / 26.
 static double slot_us(const pe_graph* g, int64_t K, uint32_t flags, bool times, const Plan& s) {
-  const double V = g->V, cells = V * (double)K, warps = s.threads / 32;
-  const bool listed = g->sview.max_sources > (g->sview.cls_kind == 0 ? 3 : 2);
-  double base = listed ? (g->sview.max_sources <= 8 ? 0.172 : 0.3) : (g->sview.max_sources == 1 ? 0.06 : 0.075);
-  if (g->sview.marks) base = g->sview.max_sources == 1 ? 0.07 : 0.087;
-  if (s.exclusive) base = listed ? 0.4 : 0.11;
-  if (g->hetero) base += 0.012;
-  const double step = std::max(base, (listed ? 0.021 : (g->sview.marks ? 0.0135 : 0.0105)) * warps), odd = K % 4 != 0 ? 1.25 : 1.0;
-  return 11.0 + odd * cells / 430e3 + V * step * (double)s.tile_rounds + (double)K * (g->D * 3.2e-6 + 1.3e-4) +
-         (times && (flags & PE_TIMES_BY_OP) ? 3.0 + odd * cells / 250e3 : 0.0);
+  const double V = g->V, cells = V * (double)K, warps = s.threads / 32, sources = g->sview.max_sources;
+  const bool listed = sources > (g->sview.cls_kind == 0 ? 3 : 2), by_op = times && (flags & PE_TIMES_BY_OP);
+  double step;
+  if (listed) {
+    step = sources <= 8 ? 0.172 : 0.024 * sources * std::sqrt(s.slot_shape.lanes / 32.0);
+    step = step * (s.exclusive ? 1.41 : 1.0) + (s.exclusive ? 0.009 : 0.0125) * std::max(0.0, warps - 4.0) + (g->hetero ? 0.008 : 0.0);
+  } else if (g->sview.marks) {
+    step = sources == 1 ? (warps > 4 ? 0.074 : 0.071) : (warps > 4 ? 0.087 : 0.075);
+    if (g->hetero) step += warps > 4 ? 0.02 : 0.007;
+  } else if (s.exclusive) {
+    step = std::max(warps > 3 ? 0.138 : 0.112, 0.0186 * warps);
+  } else if (g->hetero) {
+    step = std::max(0.082, 0.013 * warps);
+  } else {
+    step = std::max(sources == 1 ? 0.06 : 0.075, 0.009 * warps);
+  }
+  const double odd = K % 4 != 0 ? 1.25 : 1.0;
+  return (s.exclusive ? 16.0 : 11.0) + odd * cells / 430e3 + V * step * (double)s.tile_rounds + (double)K * (g->D * 3.2e-6 + 1.3e-4) +
+         (by_op ? 5.0 + odd * cells / 250e3 : (times ? cells / (listed ? 4e6 : 1.4e6) : 0.0));
 }
 // Estimated time of a plan that the automatic choice has made among the other kernels (a lane per candidate takes longer with
 // channel words, V = 1536 K = 1024 250 us, or durations by machine, 170 us; the global-state kernel with exclusive channels

@@ -79,3 +79,16 @@ def test_small_batches_of_operators_with_many_sources_take_a_warp_each(K, kernel
         assert launches(pe, g, w, K) == kernels
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("K", [148, 4096])
+def test_exclusive_channels_of_the_tiny_pipeline_stay_with_the_lane_kernel(K):
+    """One launch (20 us) instead of two (24 us)."""
+    pe = binding()
+    w = wl.make_config(1)
+    g = pe.Graph(w)
+    try:
+        for times in (True, False):
+            assert launches(pe, g, w, K, pe.PE_COMM_EXCLUSIVE, times) == 1
+    finally:
+        g.close()
