@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(32 * kSlotWarps, 1) pe_eval_slot_kernel(PeSlot
     __syncwarp();
     if (mine) {
       request(0);
-      for (uint32_t q = 0; q < nslots + 1u; ++q) sts_state<false>(st_a + q * pitch, 0u);
+      for (uint32_t q = 0; q < nslots + 2u; ++q) sts_state<false>(st_a + q * pitch, 0u);
       for (int j = 0; j < D; ++j) sts64(dv_a + (uint32_t)j * dpitch, make_uint2(0u, 0u));
       if (EXCL)
         for (int q = 0; q < D * D; ++q) sts_state<CH16>(ch_a + (uint32_t)q * chpitch, 0u);
