@@ -65,7 +65,12 @@ bool plan_slot(const pe_graph* g, int64_t K, uint32_t flags, bool times, Plan* p
   const bool by_op_times = times && (flags & PE_TIMES_BY_OP) != 0;
   if (g->hetero && exclusive) return false;
   const PeSlotView& sv = g->sview;
-  // Larger graphs with marks gain less by operator, and programs run their large batches without a workspace.
+  // Marks: no kernel with channels.  By operator on one kind of machine such graphs of any size ran without a workspace before
+  // there were slot kernels, and programs with large graphs count on that (4 bytes a position and candidate: 268 MB for V = 1024
+  // K = 65536); up to 512 operators the workspace is small enough to ask for.  It is no limit of the kernels.  Measured (us, a
+  // lane per candidate / slot kernels): taken, V = 484 D = 64 K = 16384 107 / 73, K = 131072 604 / 503; refused, V = 529 D = 64
+  // K = 16384 104 / 93, K = 131072 688 / 644, V = 1024 D = 8 K = 65536 807 / 751, V = 1024 D = 64 K = 131072 1960 / 1506,
+  // bidirectional pipeline V = 960 K = 131072 1403 / 922.
   if (sv.marks && (exclusive || (!by_pos && !g->hetero && g->V > 512))) return false;
   p->slot_gather = (int)tile_width(g, [&](size_t C) { return gather_smem(g, by_pos, C); });
   p->slot_times = (int)tile_width(g, [&](size_t C) { return (size_t)(g->V + 1) * C * 4; });

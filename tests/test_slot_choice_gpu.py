@@ -92,3 +92,16 @@ def test_exclusive_channels_of_the_tiny_pipeline_stay_with_the_lane_kernel(K):
             assert launches(pe, g, w, K, pe.PE_COMM_EXCLUSIVE, times) == 1
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("V,D,by_pos,kernels", [(484, 64, False, 2), (529, 64, False, 1), (1024, 64, True, 2)])
+def test_larger_graphs_with_marks_need_no_workspace_by_operator(V, D, by_pos, kernels):
+    pe = binding()
+    w = wl.make_config(5, V=V, D=D)
+    flags = pe.PE_ASSIGN_BY_POS if by_pos else 0
+    g = pe.Graph(w)
+    try:
+        assert launches(pe, g, w, 16384, flags) == kernels
+        assert (pe.pe_workspace_bytes(g.handle, 16384, flags) == 0) == (kernels == 1)
+    finally:
+        g.close()
