@@ -632,11 +632,13 @@ static bool plan_decode_warp(const pe_graph* g, int64_t K, DecodePlan* p) {
     p->smem = bytes;
   }
   p->shared = best > 0;
-  // bound by issue, or by the chain of a placement (longer where the records are not on chip)
-  const double dV = (double)V, dK = (double)K, per_sm = std::max(1.0, dK / (double)g->sm_count);
+  // bound by issue, or by the chain of a placement (longer where the records are not on chip).  Measured (estimate / time, us):
+  // V = 64 K = 64 16.9 / 16.4, V = 704 K = 256 111 / 119, V = 1536 K = 1024 233 / 240, K = 16384 1426 / 1524; records not on
+  // chip: V = 2304 K = 256 479 / 479, V = 2816 K = 256 692 / 682, K = 8192 2865 / 2785.
+  const double dV = (double)V, dK = (double)K, dE = (double)g->fview.E, per_sm = std::max(1.0, dK / (double)g->sm_count);
   if (best > 0)
-    p->us = 6.0 + std::max(dV * dK * (55.0 + 1.4 * g->fview.E / dV) * 1e-6,
-                           dV * (p->rec_smem ? 0.142 : 0.33) * per_sm / std::min(per_sm, (double)best));
+    p->us = 7.5 + std::max(dV * dK * (55.0 + 1.4 * dE / dV) * 1e-6,
+                           (p->rec_smem ? 0.147 * dV : 0.145 * dV + 0.06 * dE) * per_sm / std::min(per_sm, (double)best));
   return p->shared;
 }
 
@@ -664,8 +666,9 @@ static bool plan_decode_lane(const pe_graph* g, int64_t K, DecodePlan* p) {
   return true;
 }
 
-// Measured (estimate / time, us): V = 1536 K = 8192 182 / 195, K = 16384 357 / 390; V = 2304 K = 4096 289 / 463; V = 2816
-// K = 4096 581 / 619.
+// A turn is a chain of shared-memory round trips, longer with more places to read, and bound by issue from five warps on an SM
+// on.  Measured (estimate / time, us): V = 64 K = 1024 15.2 / 14.3, K = 65536 28 / 27; V = 704 (MoE) K = 8192 143 / 137; V = 1536
+// K = 8192 196 / 199, K = 16384 384 / 389; V = 2304 K = 4096 309 / 315; V = 2816 K = 4096 627 / 633, K = 16384 2484 / 2510.
 static bool plan_decode_pool(const pe_graph* g, int64_t K, DecodePlan* p) {
   const PeFwdView& f = g->fview;
   if (!f.pool_bytes || K < 1 || K >= ((int64_t)1 << 30)) return false;
@@ -685,7 +688,7 @@ static bool plan_decode_pool(const pe_graph* g, int64_t K, DecodePlan* p) {
   const int64_t rounds = (tiles + sms * (int64_t)bestW - 1) / (sms * (int64_t)bestW);
   const int64_t w = (tiles + sms * rounds - 1) / (sms * rounds);
   if (w < (int64_t)bestW) bestW = (size_t)w;
-  const double turn = std::max(0.085 + 0.001 * f.places, 0.03 * (double)bestW);
+  const double turn = std::max(0.092 + 0.0011 * f.places, 0.021 * (double)bestW);
   p->us = 8.0 + (0.012 * (double)V + turn * (double)f.turns) * (double)rounds;
   p->shared = p->pool = true;
   p->rec_smem = false;
@@ -709,7 +712,7 @@ static bool decode_plan(const pe_graph* g, int64_t K, uint32_t flags, DecodePlan
   if (want == PE_VARIANT_AUTO || want == PE_VARIANT_SHARED) {
     DecodePlan pool;
     if (!plan_decode_lane(g, K, p)) plan_decode_warp(g, K, p);
-    if (plan_decode_pool(g, K, &pool) && pool.us < p->us) *p = pool;
+    if (plan_decode_pool(g, K, &pool) && 1.08 * pool.us < p->us) *p = pool;   // (what the estimates are off by)
     if (p->shared) return true;
     if (want == PE_VARIANT_SHARED) return false;
   }
