@@ -718,7 +718,8 @@ static int eval_batch(pe_graph* g, int64_t K, const uint8_t* assign, const void*
   pe::Plan p;
   const bool allow_compact = order_bytes == 2 && ((out->start != nullptr) == (out->finish != nullptr));
   int rc = pe::make_plan(g, K, flags, allow_compact, out->start != nullptr, &p);
-  if (rc == PE_OK && p.slot && (!workspace || workspace_bytes < p.workspace)) {   // the other kernels ask for less
+  // (the other kernels ask for less, and most of them have no use for a workspace, however it is aligned)
+  if (rc == PE_OK && p.slot && (!workspace || workspace_bytes < p.workspace || ((uintptr_t)workspace & 15u) != 0)) {
     p = pe::Plan();
     rc = pe::make_plan(g, K, flags, allow_compact, out->start != nullptr, &p, false);
   }

@@ -105,3 +105,19 @@ def test_larger_graphs_with_marks_need_no_workspace_by_operator(V, D, by_pos, ke
         assert (pe.pe_workspace_bytes(g.handle, 16384, flags) == 0) == (kernels == 1)
     finally:
         g.close()
+
+
+def test_an_unaligned_workspace_is_left_alone():
+    """The slot kernels use 16-byte accesses; other kernels run where the workspace does not allow for those."""
+    import torch
+    pe = binding()
+    w = wl.make_config(4, microbatches=4)
+    K = 16384
+    g = pe.Graph(w)
+    try:
+        n = pe.pe_workspace_bytes(g.handle, K, 0)
+        ws = torch.empty(n + 256, dtype=torch.uint8, device="cuda")
+        assert launches(pe, g, w, K, workspace=(ws, n)) == 2
+        assert launches(pe, g, w, K, workspace=(ws[8:], n)) == 1
+    finally:
+        g.close()
