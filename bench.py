@@ -36,31 +36,31 @@ for _V, _D in wl.SWEEP_POINTS:
 DEFAULT_WORKLOAD = "random_layered_V16384_D64"   # the largest configuration: sweep point V=16384, D=64, K=65536
 
 FALLBACK_HBM_GBS = 6650.0
-# the kernel each variant runs for graphs that have a compact encoding (all benchmark workloads do)
-KERNEL_OF_VARIANT = {"shared": "pe_eval_tile_kernel", "global": "pe_eval_lane_kernel",
-                     "warp": "pe_eval_warp2_kernel", "team": "pe_eval_team_kernel"}
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per operator-evaluation of the evaluation kernel
-# from an ncu capture, keyed by kernel variant, valid only while the sources that kernel is built from hash to
+# from an ncu capture, keyed by kernel, valid only while the sources that kernel is built from hash to
 # the value recorded with it.  Reported as null when those sources have changed since the capture.
 KERNEL_SOURCES = {
-    "team": ("pe_kernel_team.cuh", "pe_team.cu", "pe_team_launch.h", "pe_transpose.cuh"),
-    "warp": ("pe_kernel_warp2.cuh", "pe_warp2_launch.h", "pe_device.cuh", "pe_kernel_lane.cuh"),
-    "global": ("pe_kernel_lane.cuh", "pe_lane_launch.h", "pe_device.cuh"),
-    "shared": ("pe_kernel_tile.cuh", "pe_tile_launch.h", "pe_device.cuh"),
+    "pe_eval_team_kernel": ("pe_kernel_team.cuh", "pe_team.cu", "pe_team_launch.h", "pe_transpose.cuh"),
+    "pe_eval_warp2_kernel": ("pe_kernel_warp2.cuh", "pe_warp2_launch.h", "pe_device.cuh", "pe_kernel_lane.cuh"),
+    "pe_eval_lane_kernel": ("pe_kernel_lane.cuh", "pe_lane_launch.h", "pe_device.cuh"),
+    "pe_eval_tile_kernel": ("pe_kernel_tile.cuh", "pe_tile_launch.h", "pe_device.cuh"),
+    "pe_eval_slot_kernel": ("pe_kernel_slot.cuh", "pe_slot.cu", "pe_slot_launch.h", "pe_slot_shape.h", "pe_kernel_tile.cuh",
+                            "pe_device.cuh"),
 }
 NCU_TRAFFIC = {
-    # variant: (hash of its sources at capture time, DRAM bytes per operator-evaluation, captured workload)
-    "team": ("698c9fc757a7e542", 10.13, "random_layered_V16384_D64 at K = 3552 (one chunk), scaled by operator-evaluations; "
-                        "the staging transpositions around the kernel move another 22 B per operator-evaluation"),
+    # kernel: (hash of its sources at capture time, DRAM bytes per operator-evaluation, captured workload)
+    "pe_eval_team_kernel": ("698c9fc757a7e542", 10.13, "random_layered_V16384_D64 at K = 3552 (one chunk), scaled by "
+                            "operator-evaluations; the staging transpositions around the kernel move another 22 B per "
+                            "operator-evaluation"),
 }
 
 
-def kernel_source_hash(variant):
-    """Hash of the sources the kernel of `variant` is built from."""
+def kernel_source_hash(kernel):
+    """Hash of the sources an evaluation kernel is built from."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2503_09357_b200", "csrc")
-    for name in KERNEL_SOURCES.get(variant, ()):
+    for name in KERNEL_SOURCES.get(kernel, ()):
         with open(os.path.join(csrc, name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -247,7 +247,8 @@ def time_exclusive(pe, name, dev, local_rank, stream, op_budget, want_times, ste
         torch.cuda.synchronize(dev)
         times.append(e0.elapsed_time(e1))
     ms = statistics.mean(times)
-    rec = {"workload": name, "V": oV, "D": oD, "K": oK, "kernel_variant": og.variant(oK, flags), "ms": ms,
+    rec = {"workload": name, "V": oV, "D": oD, "K": oK, "kernel_variant": og.variant(oK, flags),
+           "kernel": pe.pe_eval_kernel(og.handle, oK, flags), "ms": ms,
            "op_evals_per_s": oK * oV / (ms * 1e-3), "gbs": compulsory_bytes(oV, oD, oK, 2, want_times) / (ms * 1e-3) / 1e9}
     og.close()
     return rec
@@ -292,7 +293,7 @@ def run_ours(args):
     t_gen = time.perf_counter() - t_gen
 
     g = pe.Graph(w, device=local_rank)
-    variant = g.variant(K, flags)
+    variant, kernel = g.variant(K, flags), pe.pe_eval_kernel(g.handle, K, flags)
     d_assign = h_assign.to(dev, non_blocking=True)
     d_order = h_order.to(dev, non_blocking=True)
     d_out = g.alloc_outputs(K, want_times)
@@ -423,7 +424,7 @@ def run_ours(args):
             ms = statistics.mean(times)
             oalg = compulsory_bytes(ow.num_ops, ow.num_devices, oK, 2, want_times)
             others.append({"workload": name, "V": ow.num_ops, "D": ow.num_devices, "K": oK,
-                           "kernel_variant": og.variant(oK, flags), "ms": ms,
+                           "kernel_variant": og.variant(oK, flags), "kernel": pe.pe_eval_kernel(og.handle, oK, flags), "ms": ms,
                            "op_evals_per_s": oK * ow.num_ops / (ms * 1e-3),
                            "gbs": oalg / (ms * 1e-3) / 1e9})
             og.close()
@@ -448,8 +449,8 @@ def run_ours(args):
         alg = compulsory_bytes(V, D, K, obytes, want_times)
         achieved = alg / (kms * 1e-3) / 1e9
         traffic = None
-        rec = NCU_TRAFFIC.get(variant)
-        if rec and rec[0] == kernel_source_hash(variant):
+        rec = NCU_TRAFFIC.get(kernel)
+        if rec and rec[0] == kernel_source_hash(kernel):
             traffic = rec[1] * K * V
         cpu = None
         parity = None
@@ -469,7 +470,7 @@ def run_ours(args):
                        "l2": "inputs and outputs larger than L2" if alg > 252e6 else "working set below 2x L2: not flushed",
                        "candidate_generation_s": round(t_gen, 1)},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                         "traffic": traffic, "peak_source": f"of {peak_src}", "kernel": KERNEL_OF_VARIANT[variant],
+                         "traffic": traffic, "peak_source": f"of {peak_src}", "kernel": kernel,
                          "kernel_ms": kms, "algorithmic_bytes_per_launch": alg},
             "e2e": {"value": e2e_value, "unit": "op-evals/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "steps": e2e_steps},

@@ -44,7 +44,7 @@ enum {
   PE_ERR_RANGE = -3,       /* negative duration / communication / weight, edge endpoint or link class out of range */
   PE_ERR_OVERFLOW = -4,    /* sum(dur) + sum_e max_l comm, or sum|A| + sum W, does not fit in int32 */
   PE_ERR_CUDA = -5,        /* a CUDA runtime call failed (no device, out of memory, launch error) */
-  PE_ERR_WORKSPACE = -6,   /* workspace pointer NULL or smaller than pe_workspace_bytes() */
+  PE_ERR_WORKSPACE = -6,   /* workspace NULL or smaller than the kernel needs (pe_workspace_bytes() is enough for every kernel) */
   PE_ERR_TIMEOUT = -7,     /* a bounded device-side wait expired (reported by pe_graph_poll_error) */
   PE_ERR_UNSUPPORTED = -8, /* the requested kernel variant cannot run this problem size */
   PE_ERR_SCRATCH_LIMIT = -9 /* pe_eval_batch_noalloc: the batch needs more than PE_NOALLOC_SCRATCH_BYTES of scratch */
@@ -69,8 +69,8 @@ typedef struct {
                                   the duration a machine index): operator i lasts dur_by_machine[i*D + j] >= 0 on
                                   machine j, D^o_i of Eq. 3 becoming D^o_{i,x_i}; NULL = homogeneous (`dur` applies).
                                   `dur` must still be given (it is ignored by the evaluation when this is set).
-                                  Such graphs are evaluated by the one-thread-per-candidate kernels
-                                  (PE_VARIANT_SHARED / PE_VARIANT_GLOBAL); PE_VARIANT_WARP and PE_VARIANT_TEAM return
+                                  Such graphs are evaluated by the one-thread-per-candidate kernels (PE_VARIANT_SHARED /
+                                  PE_VARIANT_GLOBAL and the slot kernels of PE_VARIANT_AUTO); PE_VARIANT_WARP and PE_VARIANT_TEAM return
                                   PE_ERR_UNSUPPORTED for them. */
 } pe_graph_desc;
 
@@ -93,13 +93,20 @@ enum {
                             each other in the order in which their receiving operators appear in pi (as pi fixes y),
                             those into one operator in the order of the edge list; the transfer of (i1, i2) starts
                             at max(e_i1, end of the channel's previous transfer) (Eqs. 13, 14), lasts D^c (Eq. 11),
-                            and i2 starts no earlier than its end (Eq. 12).  Offered by the shared-state kernel (no
-                            workspace) and the global-state kernel (D*D*K*4 more bytes of workspace), not by
-                            PE_VARIANT_WARP; ask pe_workspace_bytes with the same flags. */
-  /* Kernel variant (bits 8..11); 0 lets the library choose from (V, E, D, L) and the device. */
-  PE_VARIANT_AUTO = 0u << 8,
+                            and i2 starts no earlier than its end (Eq. 12).  Offered by the shared-state kernels
+                            (PE_VARIANT_SHARED: no workspace; the slot kernels of PE_VARIANT_AUTO use some) and the
+                            global-state kernel (D*D*K*4 more bytes of workspace), not by PE_VARIANT_WARP and
+                            PE_VARIANT_TEAM; ask pe_workspace_bytes with the same flags. */
+  /* Kernel variant (bits 8..11); 0 lets the library choose from (V, E, D, L), K, the outputs wanted, the workspace given and
+   * the device. */
+  PE_VARIANT_AUTO = 0u << 8,   /* besides the variants below it has the slot kernels: one thread per candidate, state words in
+                                  shared memory that operators share where the graph keeps few results alive, a gather
+                                  kernel in front (and one behind for PE_TIMES_BY_OP).  They need workspace, about 4*V*K bytes
+                                  (8*V*K with start and finish by operator), a batch above 2^30 bytes of it going through in
+                                  chunks.  pe_eval_variant calls them PE_VARIANT_SHARED; forced, that is the kernel without
+                                  workspace */
   PE_VARIANT_GLOBAL = 1u << 8, /* one thread per candidate, finish-time state in the caller's workspace */
-  PE_VARIANT_SHARED = 2u << 8, /* one thread per candidate, finish-time state in shared memory */
+  PE_VARIANT_SHARED = 2u << 8, /* one thread per candidate, a state word for every operator in shared memory */
   PE_VARIANT_WARP = 3u << 8,   /* one warp per candidate, finish-time state in shared memory */
   PE_VARIANT_TEAM = 4u << 8,   /* one block of several warps per candidate, finish-time state in shared memory; the
                                   warps prepare windows of the order side by side and only the recurrence of
@@ -137,6 +144,11 @@ size_t pe_workspace_bytes(const pe_graph* g, int64_t K, uint32_t flags);
 /* Which kernel variant (PE_VARIANT_*) a call with these arguments, 16-bit orders and start and finish wanted runs;
  * negative = error code. */
 int pe_eval_variant(const pe_graph* g, int64_t K, uint32_t flags);
+
+/* Name of the kernel that evaluates the candidates of such a call, given the workspace of pe_workspace_bytes()
+ * ("pe_eval_slot_kernel", ...; a static string); NULL where pe_eval_variant returns an error code.  It tells the kernels of
+ * one variant apart. */
+const char* pe_eval_kernel(const pe_graph* g, int64_t K, uint32_t flags);
 
 /* Evaluate K candidates.  Asynchronous on `cuda_stream` (a cudaStream_t; NULL = default stream);
  * never synchronises.  K = 0 is a successful no-op.

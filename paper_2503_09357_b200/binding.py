@@ -55,6 +55,8 @@ _lib.pe_workspace_bytes.restype = ctypes.c_size_t
 _lib.pe_workspace_bytes.argtypes = [_P, ctypes.c_int64, ctypes.c_uint32]
 _lib.pe_eval_variant.restype = ctypes.c_int
 _lib.pe_eval_variant.argtypes = [_P, ctypes.c_int64, ctypes.c_uint32]
+_lib.pe_eval_kernel.restype = ctypes.c_char_p
+_lib.pe_eval_kernel.argtypes = [_P, ctypes.c_int64, ctypes.c_uint32]
 _lib.pe_eval_batch.restype = ctypes.c_int
 _lib.pe_eval_batch.argtypes = [_P, ctypes.c_int64, _P, _P, ctypes.c_int, ctypes.c_uint32, ctypes.POINTER(pe_outputs),
                                _P, ctypes.c_size_t, _P]
@@ -183,6 +185,12 @@ def pe_workspace_bytes(handle, K: int, flags: int = 0) -> int:
 
 def pe_eval_variant(handle, K: int, flags: int = 0) -> int:
     return int(_lib.pe_eval_variant(handle, int(K), int(flags)))
+
+
+def pe_eval_kernel(handle, K: int, flags: int = 0):
+    """Name of the kernel that evaluates such a batch, None where the call is refused."""
+    name = _lib.pe_eval_kernel(handle, int(K), int(flags))
+    return None if name is None else name.decode()
 
 
 def make_outputs(start=0, finish=0, makespan=0, busy=0, peak_mem=0, status=0):

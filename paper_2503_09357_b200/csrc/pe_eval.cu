@@ -703,6 +703,19 @@ extern "C" int pe_eval_variant(const pe_graph* g, int64_t K, uint32_t flags) {
   return rc != PE_OK ? rc : p.variant;
 }
 
+extern "C" const char* pe_eval_kernel(const pe_graph* g, int64_t K, uint32_t flags) {
+  pe::Plan p;
+  if (pe::make_plan(g, K, flags, true, true, &p) != PE_OK) return nullptr;
+  if (p.slot) return "pe_eval_slot_kernel";
+  if (p.tiled) return "pe_eval_tile_kernel";
+  switch (p.variant) {
+    case PE_VARIANT_TEAM: return "pe_eval_team_kernel";
+    case PE_VARIANT_WARP: return p.compact ? "pe_eval_warp2_kernel" : "pe_eval_warp_kernel";
+    case PE_VARIANT_GLOBAL: return p.compact ? "pe_eval_lane_kernel" : "pe_eval_global_kernel";
+    default: return "pe_eval_shared_kernel";
+  }
+}
+
 namespace pe { extern std::atomic<int64_t> g_decode_launches; }
 extern "C" int64_t pe_kernel_launches(void) {
   return pe::g_launches.load(std::memory_order_relaxed) + pe::g_decode_launches.load(std::memory_order_relaxed);

@@ -121,3 +121,20 @@ def test_an_unaligned_workspace_is_left_alone():
         assert launches(pe, g, w, K, workspace=(ws[8:], n)) == 1
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("config,kw,K,flag,kernel,n", [
+    (4, {}, 8192, None, "pe_eval_slot_kernel", 2), (3, {}, 8192, "PE_TIMES_BY_OP", "pe_eval_slot_kernel", 3),
+    (4, {}, 8192, "PE_VARIANT_SHARED", "pe_eval_tile_kernel", 1), (4, {}, 64, None, "pe_eval_team_kernel", 1),
+    (4, {}, 64, "PE_VARIANT_WARP", "pe_eval_warp2_kernel", 1), (4, {}, 64, "PE_VARIANT_GLOBAL", "pe_eval_lane_kernel", 1)])
+def test_the_kernel_that_is_named_is_the_one_that_runs(config, kw, K, flag, kernel, n):
+    pe = binding()
+    w = wl.make_config(config, **kw)
+    g = pe.Graph(w)
+    try:
+        flags = getattr(pe, flag) if flag else 0
+        assert pe.pe_eval_kernel(g.handle, K, flags) == kernel
+        assert launches(pe, g, w, K, flags) == n
+        assert pe.pe_eval_kernel(g.handle, K, 1 << 20) is None
+    finally:
+        g.close()
