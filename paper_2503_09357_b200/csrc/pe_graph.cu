@@ -400,8 +400,11 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
       for (int64_t q = 0; q < (int64_t)V * D; ++q) ((uint16_t*)(tblob.data() + tv.durm))[q] = (uint16_t)d->dur_by_machine[q];
   }
 
-  Ancestors anc;
-  if (V <= 4096) anc = find_ancestors(V, ops, pred);
+  Ancestors anc;   // (dense graphs that no encoding below serves take as long to find them as for all the rest)
+  auto ancestors = [&]() -> const Ancestors& {
+    if (anc.words == 0) anc = find_ancestors(V, ops, pred);
+    return anc;
+  };
 
   // slot encoding
   std::vector<uint8_t> sblob;
@@ -421,7 +424,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
   if (tile && V <= 4096 && asum < 32768 && vbits >= 4) {
     std::vector<int32_t> slot, version;
     bool marks = false;
-    int32_t n = share_slots(anc, ops, pred, V / 4, (1 << (vbits - 1)) - 1, false, &slot, &version);
+    int32_t n = share_slots(ancestors(), ops, pred, V / 4, (1 << (vbits - 1)) - 1, false, &slot, &version);
     if (n < 0 && g->tview.cls_kind == 0 && mdeg <= 3) {
       marks = true;
       n = share_slots(anc, ops, pred, (int32_t)(0.65 * V), (1 << (vbits - 2)) - 1, true, &slot, &version);
@@ -558,7 +561,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
     fv.V = V; fv.E = (int32_t)usucc.size();
     // pool kernel: joins, roots, successors
     std::vector<uint8_t> pool;
-    const int32_t chains = fv.short_lists && V <= 4096 ? cover_by_chains(anc, ops, pred, 32) : -1;
+    const int32_t chains = fv.short_lists && V <= 4096 ? cover_by_chains(ancestors(), ops, pred, 32) : -1;
     if (chains >= 0) {
       std::vector<uint32_t> join(V, 0xFFFFu), prec((size_t)V * 2, 0), pmore;
       std::vector<uint8_t> joins;
