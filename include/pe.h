@@ -43,7 +43,7 @@ enum {
   PE_ERR_CYCLE = -2,       /* the edge list is not a DAG */
   PE_ERR_RANGE = -3,       /* negative duration / communication / weight, edge endpoint or link class out of range */
   PE_ERR_OVERFLOW = -4,    /* sum(dur) + sum_e max_l comm, or sum|A| + sum W, does not fit in int32 */
-  PE_ERR_CUDA = -5,        /* a CUDA runtime call failed (no device, out of memory, launch error) */
+  PE_ERR_CUDA = -5,        /* a CUDA runtime call failed (no device, out of memory, launch error), or the host has no memory */
   PE_ERR_WORKSPACE = -6,   /* workspace NULL or smaller than the kernel needs (pe_workspace_bytes() is enough for every kernel) */
   PE_ERR_TIMEOUT = -7,     /* a bounded device-side wait expired (reported by pe_graph_poll_error) */
   PE_ERR_UNSUPPORTED = -8, /* the requested kernel variant cannot run this problem size */

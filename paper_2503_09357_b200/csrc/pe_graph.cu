@@ -3,7 +3,8 @@
 #include <climits>
 #include <cstdlib>
 #include <cstring>
-#include <new>
+#include <exception>
+#include <memory>
 #include <vector>
 
 #include "pe_device.cuh"
@@ -211,21 +212,15 @@ std::vector<cudaEvent_t*> team_events(pe_graph* g) {
           &g->team_in[1],   &g->team_done[0], &g->team_done[1], &g->team_back[0], &g->team_back[1]};
 }
 
-}  // namespace
-
-extern "C" int pe_graph_validate(const pe_graph_desc* desc) { return check_desc(desc, nullptr, nullptr, nullptr, nullptr); }
-
-extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph** out) {
-  if (!out) return PE_ERR_INVALID_ARG;
-  *out = nullptr;
+int create(const pe_graph_desc* d, int cuda_device, pe_graph** out) {
   int64_t tb = 0, mb = 0;
   int32_t mdeg = 0, levels = 1;
   const int rc = check_desc(d, &tb, &mb, &mdeg, &levels);
   if (rc != PE_OK) return rc;
   const int32_t V = d->num_ops, E = d->num_edges, D = d->num_devices, L = d->num_link_classes;
 
-  pe_graph* g = new (std::nothrow) pe_graph();
-  if (!g) return PE_ERR_INVALID_ARG;
+  std::unique_ptr<pe_graph> owner(new pe_graph());
+  pe_graph* const g = owner.get();
   g->V = V; g->E = E; g->D = D; g->L = L;
   g->device = cuda_device;
   g->has_weight = d->mem_weight != nullptr;
@@ -242,7 +237,7 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
   lay.cls = (uint32_t)at;    at = align16(at + (uint64_t)D * D);
   lay.cap = (uint32_t)at;    at = align16(at + (uint64_t)D * 4);
   lay.durm = (uint32_t)at;   at = align16(at + (g->hetero ? (uint64_t)V * D * 4 : 0));
-  if (at > 0x7FFFFFF0ull) { delete g; return PE_ERR_INVALID_ARG; }
+  if (at > 0x7FFFFFF0ull) return PE_ERR_INVALID_ARG;
   lay.bytes = (uint32_t)at;
 
   // by-predecessor CSR: incoming edges of operator i occupy slots edge_begin .. edge_begin + indeg
@@ -674,11 +669,30 @@ extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph
       if (g->ev_done[q]) cudaEventDestroy(g->ev_done[q]);
     }
     cudaGetLastError();
-    delete g;
     return PE_ERR_CUDA;
   }
-  *out = g;
+  *out = owner.release();
   return PE_OK;
+}
+
+}  // namespace
+
+extern "C" int pe_graph_validate(const pe_graph_desc* desc) {
+  try {
+    return check_desc(desc, nullptr, nullptr, nullptr, nullptr);
+  } catch (const std::exception&) {   // (no memory for the scratch arrays)
+    return PE_ERR_CUDA;
+  }
+}
+
+extern "C" int pe_graph_create(const pe_graph_desc* d, int cuda_device, pe_graph** out) {
+  if (!out) return PE_ERR_INVALID_ARG;
+  *out = nullptr;
+  try {
+    return create(d, cuda_device, out);
+  } catch (const std::exception&) {
+    return PE_ERR_CUDA;
+  }
 }
 
 extern "C" int pe_destroy(pe_graph* g) {
