@@ -44,9 +44,9 @@ KERNEL_SOURCES = {
     "pe_eval_team_kernel": ("pe_kernel_team.cuh", "pe_team.cu", "pe_team_launch.h", "pe_transpose.cuh"),
     "pe_eval_warp2_kernel": ("pe_kernel_warp2.cuh", "pe_warp2_launch.h", "pe_device.cuh", "pe_kernel_lane.cuh"),
     "pe_eval_lane_kernel": ("pe_kernel_lane.cuh", "pe_lane_launch.h", "pe_device.cuh"),
-    "pe_eval_tile_kernel": ("pe_kernel_tile.cuh", "pe_tile_launch.h", "pe_device.cuh"),
+    "pe_eval_tile_kernel": ("pe_kernel_tile.cuh", "pe_tile_launch.h", "pe_smem.cuh", "pe_device.cuh"),
     "pe_eval_slot_kernel": ("pe_kernel_slot.cuh", "pe_slot.cu", "pe_slot_launch.h", "pe_slot_shape.h", "pe_kernel_tile.cuh",
-                            "pe_device.cuh"),
+                            "pe_smem.cuh", "pe_device.cuh"),
 }
 NCU_TRAFFIC = {
     # kernel: (hash of its sources at capture time, DRAM bytes per operator-evaluation, captured workload)

@@ -46,6 +46,7 @@
 #include "pe_device.cuh"
 #include "pe_graph.h"
 #include "pe_launch.h"
+#include "pe_smem.cuh"
 
 namespace pe {
 
@@ -434,42 +435,6 @@ __global__ void __launch_bounds__(kLaneThreads) pe_decode_lane_kernel(PeFwdView 
   }
 }
 
-// Shared-memory accesses by 32-bit address, in program order.
-__device__ __forceinline__ uint32_t smem_get8(uint32_t a) {
-  uint32_t v;
-  asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint32_t smem_get16(uint32_t a) {
-  uint16_t v;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint32_t smem_get32(uint32_t a) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint2 smem_get64(uint32_t a) {
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint4 smem_get128(uint32_t a) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ void smem_put8(uint32_t a, uint32_t v) { asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v)); }
-__device__ __forceinline__ void smem_put16(uint32_t a, uint32_t v) { asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v)); }
-__device__ __forceinline__ void smem_put32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v)); }
-__device__ __forceinline__ void smem_put32_if(uint32_t a, uint32_t v, bool on) {
-  asm volatile("{.reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u32 [%0], %1;}" ::"r"(a), "r"(v), "r"((uint32_t)on));
-}
-__device__ __forceinline__ void smem_put128(uint32_t a, uint4 v) {
-  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
-}
-
 // Shape of a pe_decode_pool_kernel launch: warps take tiles of `lanes` candidates.
 struct PoolShape {
   int lanes;
@@ -518,9 +483,9 @@ __global__ void __launch_bounds__(512, 1) pe_decode_pool_kernel(PeFwdView f, con
     const int64_t c = tile * P + lane;
     if (lane >= P || c >= K) continue;   // (the lanes of a warp have nothing to do with each other)
 #pragma unroll
-    for (int q = 0; q < QUADS; ++q) smem_put128(pool_a + (uint32_t)q * qpitch, make_uint4(kNoKey, kNoKey, kNoKey, kNoKey));
-    for (int i = 0; i < V; ++i) smem_put16(rank_a + (uint32_t)i * rpitch, 0xFFFFu);
-    for (uint32_t j = 0; j < joins + 1u; ++j) smem_put8(cnt_a + j * cpitch, j < joins ? (uint32_t)first[j] : 0u);
+    for (int q = 0; q < QUADS; ++q) sts128(pool_a + (uint32_t)q * qpitch, make_uint4(kNoKey, kNoKey, kNoKey, kNoKey));
+    for (int i = 0; i < V; ++i) sts16(rank_a + (uint32_t)i * rpitch, 0xFFFFu);
+    for (uint32_t j = 0; j < joins + 1u; ++j) sts8(cnt_a + j * cpitch, j < joins ? (uint32_t)first[j] : 0u);
 
     // the list: the operators' ranks; an operator twice, or an entry that is none, leaves another one out
     {
@@ -533,17 +498,17 @@ __global__ void __launch_bounds__(512, 1) pe_decode_pool_kernel(PeFwdView f, con
         for (int u = 0; u < kBatch; ++u) i[u] = __ldg(reinterpret_cast<const uint16_t*>(at + (uint64_t)(uint32_t)(r0 + u) * K2));
 #pragma unroll
         for (int u = 0; u < kBatch; ++u)
-          if (i[u] < (uint32_t)V) smem_put16(rank_a + i[u] * rpitch, (uint32_t)(r0 + u));
+          if (i[u] < (uint32_t)V) sts16(rank_a + i[u] * rpitch, (uint32_t)(r0 + u));
       }
 #pragma unroll 8
       for (; r0 < V; ++r0) {
         const uint32_t i = __ldg(reinterpret_cast<const uint16_t*>(at + (uint64_t)(uint32_t)r0 * K2));
-        if (i < (uint32_t)V) smem_put16(rank_a + i * rpitch, (uint32_t)r0);
+        if (i < (uint32_t)V) sts16(rank_a + i * rpitch, (uint32_t)r0);
       }
     }
     uint32_t most = 0;
 #pragma unroll 16
-    for (int i = 0; i < V; ++i) most = max(most, smem_get16(rank_a + (uint32_t)i * rpitch));
+    for (int i = 0; i < V; ++i) most = max(most, lds16(rank_a + (uint32_t)i * rpitch));
     const bool bad = most == 0xFFFFu;
     if (status) status[c] = bad ? (uint32_t)PE_STATUS_ORDER_INVALID : 0u;
     if (bad) continue;   // not a permutation: the order of this candidate stays unwritten
@@ -551,7 +516,7 @@ __global__ void __launch_bounds__(512, 1) pe_decode_pool_kernel(PeFwdView f, con
     uint32_t open = f.num_roots < 32 ? ~0u << f.num_roots : 0u;   // free places
     for (uint32_t t = 0; t < (uint32_t)f.num_roots; ++t) {
       const uint32_t i = roots[t];
-      smem_put32(place_at(t), smem_get16(rank_a + i * rpitch) << 17 | t << 12 | i);
+      sts32(place_at(t), lds16(rank_a + i * rpitch) << 17 | t << 12 | i);
     }
     uint8_t* out = reinterpret_cast<uint8_t*>(order + c);
     int k = 0;
@@ -560,17 +525,17 @@ __global__ void __launch_bounds__(512, 1) pe_decode_pool_kernel(PeFwdView f, con
       const bool has = left != 0u;
       const uint32_t s = succ & 0xFFFFu, j = succ >> 16;
       const bool join = j != 0xFFFFu;
-      const uint32_t r = smem_get16(rank_a + s * rpitch);
-      const uint32_t m = smem_get8(cnt_a + (join ? j : joins) * cpitch);
-      const uint32_t succ_more = smem_get32(more);
+      const uint32_t r = lds16(rank_a + s * rpitch);
+      const uint32_t m = lds8(cnt_a + (join ? j : joins) * cpitch);
+      const uint32_t succ_more = lds32(more);
       uint4 p[QUADS];
 #pragma unroll
-      for (int q = 0; q < QUADS; ++q) p[q] = smem_get128(pool_a + (uint32_t)q * qpitch);
-      smem_put8(cnt_a + (join && has ? j : joins + 1u) * cpitch, m - 1u);
+      for (int q = 0; q < QUADS; ++q) p[q] = lds128(pool_a + (uint32_t)q * qpitch);
+      sts8(cnt_a + (join && has ? j : joins + 1u) * cpitch, m - 1u);
       const bool freed = has && m == 0u;
       const uint32_t t = (uint32_t)__ffs((int)open) - 1u;
       const uint32_t fresh = r << 17 | t << 12 | s;
-      smem_put32_if(place_at(t & 31u), fresh, freed);
+      sts32_if(place_at(t & 31u), fresh, freed);
       open = freed ? open & (open - 1u) : open;
       left -= has ? 1u : 0u;
       succ = succ_more;
@@ -583,8 +548,8 @@ __global__ void __launch_bounds__(512, 1) pe_decode_pool_kernel(PeFwdView f, con
       const uint32_t key = min(rest[0], freed ? fresh : kNoKey);
       const bool pop = left == 0u;   // (some operator is available until the last one is placed)
       const uint32_t i = min(key & 0xFFFu, vlast), at = (key >> 12) & 31u;
-      smem_put32_if(place_at(at), kNoKey, pop);
-      const uint2 rec = smem_get64(smem_a + i * 8u);
+      sts32_if(place_at(at), kNoKey, pop);
+      const uint2 rec = lds64(smem_a + i * 8u);
       if (pop) *reinterpret_cast<uint16_t*>(out) = (uint16_t)i;
       out += pop ? K2 : 0u;
       k += pop ? 1 : 0;

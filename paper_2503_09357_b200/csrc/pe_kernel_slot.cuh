@@ -287,18 +287,6 @@ constexpr int kSlotExcl = 1;     // PE_COMM_EXCLUSIVE: the end of the last trans
 constexpr int kSlotExcl16 = 2;   // the same in 16 bits (time bounds below 2^16)
 constexpr int kSlotHet = 3;      // durations by machine
 
-__device__ __forceinline__ uint2 lds64(uint32_t a) {
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ void sts64(uint32_t a, uint2 v) {
-  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y));
-}
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-
 // A step: machine record {end of the machine's last operator (packed), level << 16 | peak} and the words of the sources come
 // from shared memory, everything else of the position was fetched during the step before.  (With the busy time in the record,
 // 12 bytes, the gather is free of atomics, but fewer candidates fit: multi-modal graph K = 65536 474 -> 525 us, MoE graph

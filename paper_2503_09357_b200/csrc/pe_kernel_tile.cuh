@@ -34,6 +34,7 @@
 #include <type_traits>
 
 #include "pe_device.cuh"
+#include "pe_smem.cuh"
 #include "pe_tile_shape.h"
 
 namespace pe {
@@ -51,40 +52,6 @@ constexpr uint32_t kTileUnscheduled = 0x7FFFFF00u;  // | machine; sums with a de
 // Longer times leave no room above them: such a sum may wrap, so the words of the sources themselves are tested.
 constexpr uint32_t kTileUnscheduledLong = 0xFFFFFF00u;
 
-// Shared-memory accesses of the main loop by 32-bit address, in program order: the loads of a step go out before
-// its stores, those that the previous step's stores may feed first.
-template <bool S16>
-__device__ __forceinline__ uint32_t lds_state(uint32_t a) {
-  uint32_t v;
-  if constexpr (S16) {
-    uint16_t h;
-    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(h) : "r"(a));
-    v = h;
-  } else {
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-  }
-  return v;
-}
-template <bool S16>
-__device__ __forceinline__ void sts_state(uint32_t a, uint32_t v) {
-  if constexpr (S16) asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v));
-  else asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v));
-}
-__device__ __forceinline__ uint4 lds128(uint32_t a) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ void sts128(uint32_t a, uint4 v) {
-  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
-}
-__device__ __forceinline__ uint32_t lds32(uint32_t a) { return lds_state<false>(a); }
-__device__ __forceinline__ uint32_t lds16(uint32_t a) { return lds_state<true>(a); }
-__device__ __forceinline__ uint32_t lds8(uint32_t a) {
-  uint32_t v;
-  asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
 // Order entries and by-position machine ids: volatile, so that a block's requests stay in front of its steps.
 __device__ __forceinline__ uint32_t ldg_u16(const void* p) {
   uint16_t v;
@@ -96,10 +63,6 @@ __device__ __forceinline__ uint32_t ldg_u8(const void* p) {
   asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // CLS: 0 = one link class, every pair connected; 1 = class table in shared memory (one or two classes,
 // pairs without a channel possible); 2 = two classes, every pair connected, at most 32 machines: the class
