@@ -459,48 +459,73 @@ static bool lane_pays_exclusive(const pe_graph* g, int64_t K, const Plan& lane) 
   return 0.3 * (rounds > 1.0 ? rounds : 1.0) < std::max(2.4, (double)K / 4500.0);
 }
 
-// The slot kernels: the gather takes ~430000 positions a microsecond, start and finish by operator 250000 (odd batches a
-// quarter longer), those by position cost the recurrence one for 1.4 million (4 million where it is slower itself).  A step of
+// How often a warp meets an operator with more sources than its record holds: the more copies of the model run side by side
+// (microbatches; a layer with that many experts has their number + 3 operators on four levels), the less its lanes agree.
+static double list_share(const pe_graph* g) {
+  return 1.0 - std::exp(-0.69 * std::max(0.5, 4.0 * g->V / g->levels / (g->sview.max_sources + 3.0)));
+}
+// The slot kernels: the gather takes ~467000 positions a microsecond, start and finish by operator 269000 (odd batches a
+// quarter longer), those by position cost the recurrence one for 1.53 million (3.1 million where it is slower itself).  A step of
 // the recurrence takes the longer the more sources an operator has (with up to eight the list is read at once, beyond it is
-// walked) and, from five or so warps on an SM on, the more there are.  Over 1065 calls of the graphs of workloads/graphs.py the
-// estimate is 9 % below the time at most (12 % below 100 us) and up to 25 % above it (a few candidates with long lists: up to
-// three times as long).  Measured (estimate / time, us): multi-modal graph V = 1536 K = 1024 131 / 128, K = 32768 287 / 282, with
-// exclusive channels K = 16384 520 / 499, with durations by machine K = 32768 311 / 321; MoE graph V = 2816 K = 4096 526 / 521,
-// K = 32768 845 / 849, times by operator 1196 / 1185, with exclusive channels K = 8192 760 / 769, with durations by machine
-// K = 16384 745 / 749, with sixteen experts V = 2432 K = 16384 1050 / 1137; layered V = 1024 D = 8 K = 131072 1508 / 1510;
-// pipeline V = 64 K = 65536 41 / 40, with exclusive channels K = 4096 25 / 26.
+// walked) and, from five or so warps on an SM on, the more there are.
+// The constants of this function and of lane_plan_us are fitted to 34931 calls of random graphs, sizes, layouts and options: the
+// estimates are within 12 % of the time for nine calls in ten, within 20 % for 98 in a hundred.  With the margin that make_plan
+// takes, the choice loses 5 % (and 2 us) or more to what it leaves out in 3 calls of a hundred, and is that much slower than
+// without slot kernels in 2 of a thousand.  Measured (estimate / time, us): multi-modal graph V = 1536 K = 1024 128 / 128,
+// K = 32768 279 / 282, with exclusive channels K = 16384 464 / 501, with durations by machine K = 32768 319 / 321; MoE graph
+// V = 2816 K = 4096 532 / 521, K = 32768 844 / 847, times by operator 1162 / 1183, with exclusive channels K = 8192 798 / 769,
+// with durations by machine K = 16384 721 / 747, with sixteen experts V = 2432 K = 16384 1049 / 1134; layered V = 1024 D = 8
+// K = 131072 1594 / 1519; pipeline V = 64 K = 65536 44 / 42, with exclusive channels K = 4096 25 / 26; bidirectional pipeline
+// V = 480 K = 65536 190 / 185.
 static double slot_us(const pe_graph* g, int64_t K, uint32_t flags, bool times, const Plan& s) {
-  const double V = g->V, cells = V * (double)K, warps = s.threads / 32, sources = g->sview.max_sources;
+  const double V = g->V, cells = V * (double)K, warps = s.threads / 32, sources = g->sview.max_sources, lanes = s.slot_shape.lanes;
   const bool listed = sources > (g->sview.cls_kind == 0 ? 3 : 2), by_op = times && (flags & PE_TIMES_BY_OP);
+  const double over4 = std::max(0.0, warps - 4.0);
   double step;
   if (listed) {
-    step = sources <= 8 ? 0.172 : 0.024 * sources * std::sqrt(s.slot_shape.lanes / 32.0);
-    step = step * (s.exclusive ? 1.41 : 1.0) + (s.exclusive ? 0.009 : 0.0125) * std::max(0.0, warps - 4.0) + (g->hetero ? 0.008 : 0.0);
+    step = sources <= 8 ? (sources <= 4 ? 0.2185 : 0.1855) * list_share(g) * std::pow(lanes / 32.0, 0.107) : 0.024 * sources * std::sqrt(lanes / 32.0);
+    step = s.exclusive ? 1.595 * step + 0.0128 * over4 : step * (1.0 + 0.08 * over4);
+    if (g->hetero) step += 0.0104;
   } else if (g->sview.marks) {
-    step = sources == 1 ? (warps > 4 ? 0.074 : 0.071) : (warps > 4 ? 0.087 : 0.075);
-    if (g->hetero) step += warps > 4 ? 0.02 : 0.007;
+    step = sources == 1 ? (warps > 4 ? 0.0789 : 0.0652) : (warps > 4 ? 0.0958 : 0.0791);
+    if (g->hetero) step += warps > 4 ? 0.0098 : 0.0051;
   } else if (s.exclusive) {
-    step = std::max(warps > 3 ? 0.138 : 0.112, 0.0186 * warps);
+    step = sources == 1 ? 0.16 + 0.0049 * over4 : 0.115 + 0.0078 * over4;
   } else if (g->hetero) {
-    step = std::max(0.082, 0.013 * warps);
+    step = (sources == 1 ? 0.0686 : 0.0816) + 0.0071 * over4;
   } else {
-    step = std::max(sources == 1 ? 0.06 : 0.075, 0.009 * warps);
+    step = (sources == 1 ? 0.0552 : 0.0728) + 0.0042 * std::max(0.0, warps - 6.0);
   }
-  const double odd = K % 4 != 0 ? 1.25 : 1.0;
-  return (s.exclusive ? 16.0 : 11.0) + odd * cells / 430e3 + V * step * (double)s.tile_rounds + (double)K * (g->D * 3.2e-6 + 1.3e-4) +
-         (by_op ? 5.0 + odd * cells / 250e3 : (times ? cells / (listed ? 4e6 : 1.4e6) : 0.0));
+  const double around = cells * (K % 4 != 0 ? 1.24 : 1.0) * (flags & PE_ASSIGN_BY_POS ? 0.937 : 1.0);   // gather, times by operator
+  return 12.0 + (listed ? 1.5 : 0.0) + (s.exclusive ? 0.76 : 0.0) + around / 467e3 + V * step * (double)s.tile_rounds +
+         (double)K * (g->D * 0.71e-6 + 2.19e-4) + (by_op ? 4.8 + around / 269e3 : (times ? cells / (listed ? 3.1e6 : 1.53e6) : 0.0));
 }
-// Estimated time of a plan that the automatic choice has made among the other kernels (a lane per candidate takes longer with
-// channel words, V = 1536 K = 1024 250 us, or durations by machine, 170 us; the global-state kernel with exclusive channels
-// V = 2816 K = 16384 10253 / 12118, K = 32768 20505 / 14992, the generic one for durations by machine V = 1369 D = 64 K = 4000
-// 6434 / 6415, K = 65536 35887 / 27200, MoE graph K = 16384 18455 / 22600).  Where 48 lanes of the generic kernel fit, the tile
-// kernel does too.
+// A lane per candidate, where the slot kernels are the alternative (lane_us, which compares lanes with warps and blocks of warps,
+// knows neither odd rows nor channel words nor durations by machine).
+static double lane_plan_us(const pe_graph* g, int64_t K, uint32_t flags, bool times, const Plan& p) {
+  const double V = g->V, cells = V * (double)K, warps = p.threads / 32, lanes = p.tile_resident / std::max(1.0, warps);
+  const bool many = g->max_indeg > 3, by_pos = (flags & PE_ASSIGN_BY_POS) != 0;
+  const double D = g->D;
+  double step = g->max_indeg <= 1 ? 0.0786 : (g->max_indeg == 2 ? 0.0822 : 0.08);
+  step *= std::pow(std::min(D, 16.0) / 16.0, 0.032) * std::pow(std::max(D, 16.0) / 16.0, 0.063) * std::pow(std::min(lanes, 32.0) / 32.0, 0.084);
+  if (many) step = (g->max_indeg == 4 ? 0.223 : 0.25) * list_share(g) * std::pow(lanes / 32.0, lanes < 16.0 ? 0.2 : 0.072) * (warps > 4 ? 1.137 : 1.0);
+  if (p.tile_mode == kTileS16) step *= 0.925 * (by_pos ? 0.906 : 1.0) * (1.0 + 0.017 * std::max(0.0, warps - 4.0));
+  if (p.exclusive) step *= (g->max_indeg <= 1 ? 2.385 : (many ? 2.0 : 2.05)) * (1.0 + 0.03 * std::max(0.0, warps - 4.0));
+  else step *= (g->hetero ? (many ? 0.99 : 1.314) : 1.0) * (1.0 + 0.019 * std::min(4.0, std::max(0.0, warps - 4.0)) + 0.106 * std::max(0.0, warps - 8.0));
+  if (times) step *= flags & PE_TIMES_BY_OP ? (many || p.exclusive ? 1.235 : 1.49) : 1.03;
+  if (by_pos) step *= 0.932;
+  const double odd = K % 4 != 0 && !by_pos ? (p.exclusive ? 1.094 : (many ? 1.13 : 1.164)) : 1.0;
+  return (8.9 + 0.0051 * V + V * step * (double)p.tile_rounds + cells * (times ? 1.5e-6 : 1.19e-6)) * odd;
+}
+// Estimated time of a plan that the automatic choice has made among the other kernels (the global-state kernel with exclusive
+// channels V = 2816 K = 16384 10253 / 12118, K = 32768 20505 / 14992, the generic one for durations by machine V = 1369 D = 64
+// K = 4000 6434 / 6415, K = 65536 35887 / 27200, MoE graph K = 16384 18455 / 22600).  Where 48 lanes of the generic kernel fit, the
+// tile kernel does too.
 static double plan_us(const pe_graph* g, int64_t K, uint32_t flags, bool times, const Plan& p) {
   if (p.variant == PE_VARIANT_TEAM) return team_us(g, K, times, p.staged);
   if (p.variant == PE_VARIANT_WARP) return warp_rounds_us(g, K, times, p);
   if (p.variant == PE_VARIANT_GLOBAL) return (double)g->V * std::max(p.compact ? 2.4 : 4.7, (double)K / (p.compact ? 4500.0 : 2500.0));
-  if (p.tiled) return lane_us(g, flags, times, p) * (p.exclusive ? 2.0 : (g->hetero && g->max_indeg <= 3 ? 1.3 : 1.0));
-  return 1e30;
+  return p.tiled ? lane_plan_us(g, K, flags, times, p) : 1e30;
 }
 
 // allow_compact: the call can use the compact-graph kernels (u16 orders; start and finish both
@@ -574,10 +599,11 @@ static int plan_others(const pe_graph* g, int64_t K, uint32_t flags, bool allow_
 static int make_plan(const pe_graph* g, int64_t K, uint32_t flags, bool allow_compact, bool times, Plan* p, bool allow_slot = true) {
   const int rc = plan_others(g, K, flags, allow_compact, times, p);
   if (rc != PE_OK || !allow_slot || !allow_compact || K == 0 || (flags & PE_VARIANT_MASK) != PE_VARIANT_AUTO) return rc;
+  if (!g->slot_ok) return PE_OK;
   const double others = plan_us(g, K, flags, times, *p);
-  if (!g->slot_ok || others < 1.08 * (11.0 + (double)g->V * ((double)K / 430e3 + 0.06))) return PE_OK;   // (no plan to be made)
+  if (others < 1.05 * (12.0 + (double)g->V * ((double)K / 500e3 + 0.055))) return PE_OK;   // (no plan to be made)
   Plan s;
-  if (plan_slot(g, K, flags, times, &s) && 1.08 * slot_us(g, K, flags, times, s) < others) *p = s;
+  if (plan_slot(g, K, flags, times, &s) && 1.05 * slot_us(g, K, flags, times, s) < others) *p = s;
   return PE_OK;
 }
 

@@ -39,14 +39,6 @@
 
 namespace pe {
 
-// MODE of the kernel
-constexpr int kTilePlain = 0;   // 32-bit state words
-constexpr int kTileS16 = 1;     // 16-bit state words
-constexpr int kTileExcl = 2;    // PE_COMM_EXCLUSIVE: the end of the last transfer per channel, [machine pair][P]
-constexpr int kTileHet = 3;     // durations by machine
-constexpr int kTileLong = 4;    // 32-bit state words, time bounds up to kPackedTimeLimit
-constexpr int kTileExclLong = 5;
-
 constexpr int64_t kTileTimeLimit = 0x7FFFFF;        // 32-bit words: end times stay below this
 constexpr uint32_t kTileUnscheduled = 0x7FFFFF00u;  // | machine; sums with a delay and a duration do not wrap
 // Longer times leave no room above them: such a sum may wrap, so the words of the sources themselves are tested.

@@ -6,6 +6,14 @@ namespace pe {
 
 constexpr int kTileWarps = 8;   // warps of a block (twice as many where operators are few)
 
+// MODE of the kernel (Plan::tile_mode)
+constexpr int kTilePlain = 0;   // 32-bit state words
+constexpr int kTileS16 = 1;     // 16-bit state words
+constexpr int kTileExcl = 2;    // PE_COMM_EXCLUSIVE: the end of the last transfer per channel, [machine pair][P]
+constexpr int kTileHet = 3;     // durations by machine
+constexpr int kTileLong = 4;    // 32-bit state words, time bounds up to kPackedTimeLimit
+constexpr int kTileExclLong = 5;
+
 struct TileShape {
   int lanes;            // P, candidates per tile (4 to 32)
   int jbits;            // machine bits of a state word (8 with 32-bit words)

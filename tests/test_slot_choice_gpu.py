@@ -38,8 +38,9 @@ def launches(pe, g, w, K, flags=0, want_times=True, workspace=None):
     return n
 
 
-@pytest.mark.parametrize("config,kw,K", [(1, {}, 1024), (5, dict(V=256, D=8), 1 << 20), (2, {}, 65536)])
+@pytest.mark.parametrize("config,kw,K", [(1, {}, 1024), (5, dict(V=256, D=8), 1 << 20), (1, {}, 65536)])
 def test_batches_that_never_take_the_slot_kernels_ask_for_nothing(config, kw, K):
+    """(Half a batch of the bidirectional pipeline at K = 65536 may take them: K = 32768 without times.)"""
     pe = binding()
     g = pe.Graph(wl.make_config(config, **kw))
     try:
