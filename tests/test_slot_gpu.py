@@ -116,3 +116,46 @@ def test_chains_longer_than_the_versions_and_batches_without_workspace():
         gu.compare(res, ref, "no workspace")
     finally:
         g.close()
+
+
+def forked_chains(V, D, scale):
+    """Chains side by side that fork every twenty operators; the branch ends after eight.  One source an operator, and the word
+    that its slot held before where a branch begins."""
+    rs = np.random.RandomState(V)
+    edges, ends, i = [], [-1] * 6, 0
+    while i < V:
+        for c in range(6):
+            for step in range(20):
+                if i >= V:
+                    break
+                if ends[c] >= 0:
+                    edges.append((ends[c], i))
+                ends[c] = i
+                i += 1
+                if step == 10:
+                    at = ends[c]
+                    for _ in range(8):
+                        if i < V:
+                            edges.append((at, i))
+                            at = i
+                            i += 1
+    w = ck.problem(V, edges, rs.randint(0, scale, V), D, comm=rs.randint(0, scale, (len(edges), 1)), A=rs.randint(-4, 5, V),
+                   cap=rs.randint(5, 60, D))
+    w.assign_mode, w.group = "per_op", None
+    return w
+
+
+@pytest.mark.parametrize("V,width,fan,classes,D,scale,K", [
+    (1000, 12, 1, 1, 16, 30, 9000), (1000, 0, 0, 1, 24, 30, 9002), (1001, 12, 2, 1, 32, 30, 9001), (1003, 12, 6, 1, 8, 9, 9003),
+    (1004, 10, 14, 1, 7, 9, 16004), (1005, 16, 1, 2, 32, 30, 8004), (1006, 8, 7, 2, 16, 20, 9006), (1007, 10, 12, 2, 5, 9, 16000),
+    (1009, 12, 9, 3, 6, 30, 16009), (1300, 12, 1, 3, 20, 30, 5000)])
+def test_every_call_goes_through_the_slot_kernels(V, width, fan, classes, D, scale, K):
+    """Graphs that leave a lane per candidate few lanes: all sixteen forms (layouts, times, exclusive channels) of one, two,
+    three, up to eight and more sources over one link class, two of them and a class table."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2503_09357_b200 import binding as pe
+    w = narrow_graph(V, width, fan, classes, D, scale) if width else forked_chains(V, D, scale)
+    forms = (0, pe.PE_TIMES_BY_OP, pe.PE_ASSIGN_BY_POS, pe.PE_ASSIGN_BY_POS | pe.PE_TIMES_BY_OP)
+    assert check_all(pe, w, K, forms, exclusive=True) == 16
