@@ -455,9 +455,10 @@ struct PoolShape {
 // first version with them took 730 cycles a turn), and the pool is read while the successor's rank is on its way: what
 // is released in this turn is compared with what was in the pool before.
 // What bounds it: the chain operator -> record -> rank of its successor, two shared-memory round trips, with the few warps
-// that fit (2 bytes an operator and candidate): ~110 ns a turn.  Measured (us, warp kernel or lane kernel with a bitmap
-// before): multi-modal graph V = 1536 K = 8192 834 -> 195, K = 64 228 -> 193; MoE graph V = 2816 K = 8192 2879 -> 1232;
-// pipeline V = 256 K = 16384 103 -> 45.
+// that fit (2 bytes an operator and candidate): 249 cycles a turn, set-up included, at V = 1536 K = 8192 (two warps on an SM, 109
+// instructions and 38 shared-memory wavefronts a turn, 45 % of the issue slots of the schedulers that have a warp).  Measured
+// (us, warp kernel or lane kernel with a bitmap before): multi-modal graph V = 1536 K = 8192 834 -> 199, K = 64 231 -> 192; MoE
+// graph V = 2816 K = 8192 2785 -> 1258; pipeline V = 256 K = 16384 100 -> 41, V = 64 K = 1024 18 -> 14.
 template <int QUADS>
 __global__ void __launch_bounds__(512, 1) pe_decode_pool_kernel(PeFwdView f, const uint8_t* __restrict__ fblob, int64_t K,
                                                                 const uint16_t* __restrict__ list, uint16_t* __restrict__ order,

@@ -3,7 +3,7 @@
 // Operators share state words ("slots").  Operator s takes over the slot of operator p when every successor of p is s or
 // an ancestor of s: in any topological order all readers of p's end time are then through when s is scheduled.  The
 // assignment of slots depends on the graph alone (made once in pe_graph_create), and a pipeline or a layered model graph
-// needs few of them: 26 for the 1536 operators of the multi-modal graph.  So the per-candidate state shrinks from 4 bytes an
+// needs few of them: 24 for the 1536 operators of the multi-modal graph.  So the per-candidate state shrinks from 4 bytes an
 // operator to a few hundred bytes, and an SM holds hundreds of candidates instead of 14 to 60.
 //
 // The machine of an operator has no place in such a state, so the batch goes through two kernels:
@@ -26,12 +26,17 @@
 //
 // State word: (time << vbits | version) << 8 | machine.
 //
-// What bounds them: the recurrence the chain of a step (~160 cycles, half of them shared-memory round trips) up to four
-// warps on an SM, then shared-memory wavefronts (20 a step, ten of them for the operator record); the gather instructions (22
-// a position) and DRAM.  Measured on B200 (us, lane kernel with a word per operator, block of warps or global state before):
-// multi-modal graph V = 1536 K = 65536 2305 -> 475, K = 16384 594 -> 208, with durations by machine K = 65536 4630 -> 607,
-// with exclusive channels K = 16384 1711 -> 506; MoE graph V = 2816 K = 16384 1852 -> 734, times by operator K = 16381 1916
-// -> 1047, with durations by machine K = 16384 11878 -> 652.
+// What bounds them (counters of one launch, multi-modal graph V = 1536 K = 16384): the recurrence the chain of a step up to four
+// warps on an SM (174 cycles a step, 58 instructions, 35 % of the issue slots, 43 % of the shared-memory pipe), then
+// shared-memory wavefronts: 20.6 a step, 7 of them bank conflicts, mostly of the operator records.  The gather instructions
+// and shared memory: 22 instructions and 8 wavefronts for 32 positions, 68 % of the pipe, 29 % of the DRAM rate (53 us for 25
+// million positions).  Times by operator DRAM: 53 % of its rate (82 us).  The MoE graph takes 120 instructions and 30
+// wavefronts a step, exclusive channels 79 and 22.5, marks (V = 1024 by position) 72 and 14.
+// Measured on B200 (us, lane kernel with a word per operator, block of warps or global state before): multi-modal graph
+// V = 1536 K = 65536 2304 -> 475 (gather 178, recurrence 274), K = 16384 594 -> 210, with durations by machine K = 32768 2320 ->
+// 321, with exclusive channels K = 16384 1714 -> 467 (52, 413); MoE graph V = 2816 K = 16384 1850 -> 600, times by operator
+// K = 16381 1918 -> 919 (118, 494, 305), with durations by machine K = 16384 11890 -> 748; V = 1024 D = 64 by position K = 2^19
+// 7315 -> 5955 (980, 5090).
 #pragma once
 #include "pe_kernel_tile.cuh"
 #include "pe_slot_shape.h"
@@ -340,7 +345,7 @@ __global__ void __launch_bounds__(32 * kSlotWarps, 1) pe_eval_slot_kernel(PeSlot
     const uint8_t* ent_b = reinterpret_cast<const uint8_t*>(entries) + cc * 16;
     // The words of a block of positions are brought to shared memory by asynchronous copies, each lane its own, while the
     // block before is worked on.  (Loads into registers share a scoreboard with the step's shared-memory loads: every
-    // block then waited for DRAM.  Multi-modal graph K = 8192 158 -> 140 us, with exclusive channels K = 16384 593 -> 429.)
+    // block then waited for DRAM.  Multi-modal graph K = 8192 158 -> 140 us when this was made.)
     uint4 cur[kSlotQuads];
     auto request = [&](int q0) {
 #pragma unroll
