@@ -105,7 +105,8 @@ struct PeTileView {
 // of them, with the version of the operator that held it and no delay (that operator is an ancestor, or there was none):
 // bit 13 / 29.  With `marks` there are no such sources: every operator reads its own slot besides, and one without successors
 // has the slot of a predecessor and the top bit of `version` instead of one.  With at most eight sources an operator's part of the list has six places (eight words or twelve).
-// Slot nslots stands for missing sources (it holds "ended at 0", version 0), nslots + 1 is that of entries that are no operator.
+// Slot nslots stands for missing sources (it holds "ended at 0", version 0), nslots + 1 is that of entries
+// that are no operator (not initialised: their candidate is flagged already).
 struct PeSlotView {
   int32_t V, E, D;
   int32_t nslots;
